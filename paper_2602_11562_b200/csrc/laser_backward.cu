@@ -1112,8 +1112,12 @@ int backward_t(const Plan& p, const T* items, const int32_t* lengths, const T* c
   // ---- forward, kept in fp32: projections and H' (the FP32-ALU forward kernels), then the GSTA layers
   char* mma_scratch = ws + p.total + s.total;
   const bool mma = tensor && sta_bwd_mma_supported(p);     // (users with very few candidates keep the FP32 gate kernels)
+  const bool stream = tensor && backward_stream_supported(p);   // one candidate per user: no keys or values of the items
   const bool attn_mma = mma && gsta_attn_mma_supported(p); // the recomputed GSTA attention on the MMAs as well
-  if (tensor) {
+  if (stream) {
+    BWD_OK(gemm<T, T>(gx, N, dqk, d, cands, d, false, Wq, dqk, false, Qf, dqk, p.inv_gamma, false, false));
+    BWD_OK(backward_stream_forward(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, s.Hp, ws, mma_scratch, st));
+  } else if (tensor) {
     // (sta_fwd_mma writes every row of H' that is read later: all candidates of every non-empty segment)
     if (!(mma && sta_fwd_mma_supported(p))) LASER_CUDA_OK(cudaMemsetAsync(s.Hp, 0, (size_t)N * Lp * d * sizeof(float), st));
     // projections as three matrix products over all rows (padding rows included: their K and V are never read)
@@ -1210,10 +1214,20 @@ int backward_t(const Plan& p, const T* items, const int32_t* lengths, const T* c
   }
 
   // ---- backward through the segment aggregation and the gates
-  LASER_CUDA_OK(cudaMemsetAsync(s.dQf, 0, (size_t)N * dqk * sizeof(float), st));
-  LASER_CUDA_OK(cudaMemsetAsync(s.dK, 0, UL * dqk * sizeof(float), st));
-  LASER_CUDA_OK(cudaMemsetAsync(s.dV, 0, UL * d * sizeof(float), st));
-  if (mma) {
+  const float* p_sums = nullptr;
+  if (stream) {
+    BWD_OK(backward_stream(p, items, lengths, cand_offsets, Wv, s.dHp, d_items, dWv, &p_sums, ws, mma_scratch, st));
+    // d(q_h / gamma) = p_h W_k[:, h];  dW_k[:, h] += p_h^T q_h / gamma, every head
+    const int dqh = p.dqh;
+    BWD_OK(gemm<float, T>(gx, N, dqh, d, p_sums, H * d, false, Wk, dqk, false, s.dQf, dqk, 1.f, false, false, H, d, dqh, dqh));
+    BWD_OK(gemm<float, float>(gx, d, dqh, N, p_sums, H * d, true, Qf, dqk, false, dWk, dqk, 1.f, true, true, H, d, dqh, dqh));
+  } else {
+    LASER_CUDA_OK(cudaMemsetAsync(s.dQf, 0, (size_t)N * dqk * sizeof(float), st));
+    LASER_CUDA_OK(cudaMemsetAsync(s.dK, 0, UL * dqk * sizeof(float), st));
+    LASER_CUDA_OK(cudaMemsetAsync(s.dV, 0, UL * d * sizeof(float), st));
+  }
+  if (stream) {
+  } else if (mma) {
     // (with the attention on the MMAs and at least one layer, dH' has arrived in bf16 already)
     BWD_OK(sta_bwd_mma(p, attn_mma && M > 0 ? nullptr : s.dHp, lengths, cand_offsets, s.dQf, s.dK, s.dV, mma_scratch, st));
   } else {
@@ -1235,10 +1249,12 @@ int backward_t(const Plan& p, const T* items, const int32_t* lengths, const T* c
   // ---- backward through the projections (Qf = T W_q / gamma)
   BWD_OK(gemm<T, float>(gx, d, dqk, N, cands, d, true, s.dQf, dqk, false, dWq, dqk, p.inv_gamma, true, true));
   BWD_OK(gemm<float, T>(gx, N, d, dqk, s.dQf, dqk, false, Wq, dqk, true, s.dT, d, p.inv_gamma, true, false));
-  BWD_OK(gemm<T, float>(gx, d, dqk, (int)UL, items, d, true, s.dK, dqk, false, dWk, dqk, 1.f, true, true));
-  BWD_OK(gemm<T, float>(gx, d, d, (int)UL, items, d, true, s.dV, d, false, dWv, d, 1.f, true, true));
-  BWD_OK(gemm<float, T>(gx, (int)UL, d, dqk, s.dK, dqk, false, Wk, dqk, true, d_items, d, 1.f, false, false));
-  BWD_OK(gemm<float, T>(gx, (int)UL, d, d, s.dV, d, false, Wv, d, true, d_items, d, 1.f, true, false));
+  if (!stream) {
+    BWD_OK(gemm<T, float>(gx, d, dqk, (int)UL, items, d, true, s.dK, dqk, false, dWk, dqk, 1.f, true, true));
+    BWD_OK(gemm<T, float>(gx, d, d, (int)UL, items, d, true, s.dV, d, false, dWv, d, 1.f, true, true));
+    BWD_OK(gemm<float, T>(gx, (int)UL, d, dqk, s.dK, dqk, false, Wk, dqk, true, d_items, d, 1.f, false, false));
+    BWD_OK(gemm<float, T>(gx, (int)UL, d, d, s.dV, d, false, Wv, d, true, d_items, d, 1.f, true, false));
+  }
   LASER_CUDA_OK(cudaMemcpyAsync(d_cands, s.dT, Nd * sizeof(float), cudaMemcpyDeviceToDevice, st));
 #undef BWD_OK
   LASER_CUDA_OK(cudaGetLastError());
@@ -1247,7 +1263,7 @@ int backward_t(const Plan& p, const T* items, const int32_t* lengths, const T* c
 
 }  // namespace
 
-size_t backward_scratch_bytes(const Plan& p) { return carve_scratch(p, nullptr).total + sta_bwd_mma_scratch_bytes(p); }
+size_t backward_scratch_bytes(const Plan& p) { return carve_scratch(p, nullptr).total + sta_bwd_mma_scratch_bytes(p) + backward_stream_scratch_bytes(p); }
 
 bool backward_tensor_supported(const Plan& p) { return p.dtype == LASER_BF16; }
 

@@ -144,6 +144,25 @@ int stream_sta(const Plan& p, const void* items, const int32_t* lengths, const v
                const void* Wq, const void* Wk, const void* Wv, void* Hprime, char* ws, cudaStream_t st,
                const void* Wg_images);
 
+// u [U, H, d] (fp32) = W_k[:, h] (t W_q)_h / gamma for the candidate of every user (zero rows without one), and the users'
+// launch order, longest first; scratch: stream_fold_bytes(p).
+size_t stream_fold_bytes(const Plan& p);
+const int* stream_fold_order(const Plan& p, const char* scratch);   // null: index order
+int stream_fold(const Plan& p, const int32_t* lengths, const void* cands, const int32_t* cand_offsets, const void* Wq,
+                const void* Wk, const void* Wv, float* u, char* scratch, int* status, cudaStream_t st);
+
+// Backward pass of batches with at most one candidate per user (laser_backward_stream.cu).  _forward recomputes H' (fp32,
+// rows of non-empty segments only); the other writes every row of d_items, adds to dWv and leaves
+// p_h = sum_n de_{n,h} x_n, from which the gradients of the query side and of W_k follow, in *p_sums [N, H, d].
+bool backward_stream_supported(const Plan& p);
+size_t backward_stream_scratch_bytes(const Plan& p);
+int backward_stream_forward(const Plan& p, const void* items, const int32_t* lengths, const void* cands,
+                            const int32_t* cand_offsets, const void* Wq, const void* Wk, const void* Wv, float* Hp, char* ws,
+                            char* scratch, cudaStream_t st);
+int backward_stream(const Plan& p, const void* items, const int32_t* lengths, const int32_t* cand_offsets, const void* Wv,
+                    const float* dHp, float* d_items, float* dWv, const float** p_sums, char* ws, char* scratch,
+                    cudaStream_t st);
+
 // Multi-resolution feature fusion (laser_fusion.cu); uses only the status word of the workspace.
 int fusion_forward(const Plan& p, const void* Hprime, const void* z, const int32_t* lengths, const int32_t* cand_offsets,
                    int num_recent, void* fused, char* ws, cudaStream_t st);

@@ -373,6 +373,26 @@ int launch_stream(const StreamParams& P, cudaStream_t st) {
   return LASER_OK;
 }
 
+int launch_pre(const StreamParams& P, cudaStream_t st) {
+  const int user_warps = (P.U + 15) / 16;
+  const dim3 grid((user_warps + kPreWarps - 1) / kPreWarps + 2 + (P.order ? 1 : 0)), block(kPreWarps * 32);
+  LaunchScope ls("stream_pre", st);
+  cudaError_t e;
+  switch (P.d / 16) {
+    case 1: e = launch_chained(stream_pre_kernel<1>, grid, block, 0, st, P, user_warps); break;
+    case 2: e = launch_chained(stream_pre_kernel<2>, grid, block, 0, st, P, user_warps); break;
+    case 3: e = launch_chained(stream_pre_kernel<3>, grid, block, 0, st, P, user_warps); break;
+    case 4: e = launch_chained(stream_pre_kernel<4>, grid, block, 0, st, P, user_warps); break;
+    case 5: e = launch_chained(stream_pre_kernel<5>, grid, block, 0, st, P, user_warps); break;
+    case 6: e = launch_chained(stream_pre_kernel<6>, grid, block, 0, st, P, user_warps); break;
+    case 7: e = launch_chained(stream_pre_kernel<7>, grid, block, 0, st, P, user_warps); break;
+    case 8: e = launch_chained(stream_pre_kernel<8>, grid, block, 0, st, P, user_warps); break;
+    default: return LASER_ERR_UNSUPPORTED;
+  }
+  LASER_CUDA_OK(e);
+  return LASER_OK;
+}
+
 }  // namespace
 
 bool stream_supported(const Plan& p) {
@@ -394,6 +414,27 @@ static bool stream_wants_order(const Plan& p) {
   int dev = 0, sms = 148;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   return p.U > 4 * sms;
+}
+
+size_t stream_fold_bytes(const Plan& p) {       // the W_v image (a by-product), the users' order and its sort keys
+  return align_up((size_t)p.d * p.d * 2) + 2 * align_up((size_t)p.U * sizeof(int));
+}
+const int* stream_fold_order(const Plan& p, const char* scratch) {
+  return stream_wants_order(p) ? reinterpret_cast<const int*>(scratch + align_up((size_t)p.d * p.d * 2)) : nullptr;
+}
+int stream_fold(const Plan& p, const int32_t* lengths, const void* cands, const int32_t* cand_offsets, const void* Wq,
+                const void* Wk, const void* Wv, float* u, char* scratch, int* status, cudaStream_t st) {
+  StreamParams P = {};
+  P.U = p.U; P.L = p.L; P.d = p.d; P.dqk = p.dqk; P.H = p.H; P.S = p.S; P.Lp = p.Lp; P.N = p.N; P.M = p.M;
+  P.inv_gamma = p.inv_gamma;
+  P.cands = (const bf16*)cands; P.Wq = (const bf16*)Wq; P.Wk = (const bf16*)Wk; P.Wv = (const bf16*)Wv;
+  P.lengths = lengths; P.cand_offsets = cand_offsets;
+  P.u = u;
+  P.imgv = reinterpret_cast<uint4*>(scratch);
+  P.order = const_cast<int*>(stream_fold_order(p, scratch));
+  P.order_keys = P.order ? P.order + align_up((size_t)p.U * sizeof(int)) / sizeof(int) : nullptr;
+  P.status = status;
+  return launch_pre(P, st);
 }
 
 int stream_sta(const Plan& p, const void* items, const int32_t* lengths, const void* cands, const int32_t* cand_offsets,
@@ -423,25 +464,8 @@ int stream_sta(const Plan& p, const void* items, const int32_t* lengths, const v
                                      align_up((size_t)p.d * p.d * 2));
     P.order_keys = P.order + p.U;
   }
-  {
-    const int user_warps = (p.U + 15) / 16;
-    const dim3 grid((user_warps + kPreWarps - 1) / kPreWarps + 2 + (P.order ? 1 : 0)), block(kPreWarps * 32);
-    LaunchScope ls("stream_pre", st);
-    cudaError_t e;
-    switch (p.d / 16) {
-      case 1: e = launch_chained(stream_pre_kernel<1>, grid, block, 0, st, P, user_warps); break;
-      case 2: e = launch_chained(stream_pre_kernel<2>, grid, block, 0, st, P, user_warps); break;
-      case 3: e = launch_chained(stream_pre_kernel<3>, grid, block, 0, st, P, user_warps); break;
-      case 4: e = launch_chained(stream_pre_kernel<4>, grid, block, 0, st, P, user_warps); break;
-      case 5: e = launch_chained(stream_pre_kernel<5>, grid, block, 0, st, P, user_warps); break;
-      case 6: e = launch_chained(stream_pre_kernel<6>, grid, block, 0, st, P, user_warps); break;
-      case 7: e = launch_chained(stream_pre_kernel<7>, grid, block, 0, st, P, user_warps); break;
-      case 8: e = launch_chained(stream_pre_kernel<8>, grid, block, 0, st, P, user_warps); break;
-      default: return LASER_ERR_UNSUPPORTED;
-    }
-    LASER_CUDA_OK(e);
-  }
-  int rc;
+  int rc = launch_pre(P, st);
+  if (rc != LASER_OK) return rc;
   switch (p.d / 16) {
     case 1: rc = launch_stream<1>(P, st); break;
     case 2: rc = launch_stream<2>(P, st); break;

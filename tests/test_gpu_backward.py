@@ -161,3 +161,34 @@ def test_backward_rejects_a_short_workspace():
     ws = torch.empty(P.laser_backward_workspace_bytes(b.cfg) - 256, dtype=torch.uint8, device="cuda")
     with pytest.raises(P.LaserError):
         P.laser_backward(b.cfg, *b.args(), b.Wg, torch.zeros((w.N, 32), device="cuda"), workspace=ws)
+
+
+# one candidate per user (laser_backward_stream.cu): partial row groups and segments, one to eight heads, blocks that share
+# a user, and more users than one wave of blocks
+STREAM_CASES = [
+    dict(U=5, C=1, L=75, d=16, H=1, S=75, M=1, dtype="bf16", lengths=[75, 16, 17, 1, 0], emb_std="inv_sqrt_d"),
+    dict(U=3, C=1, L=1100, d=128, H=8, S=17, M=1, dtype="bf16", lengths=[1100, 1099, 16]),
+    dict(U=2, C=1, L=400, d=96, H=3, S=10, M=2, dtype="bf16", lengths=[400, 211]),
+    dict(U=640, C=1, L=40, d=64, H=2, S=10, M=2, dtype="bf16"),
+]
+
+
+@pytest.mark.parametrize("case", range(len(STREAM_CASES)))
+def test_backward_one_candidate_matches_oracle(case):
+    worst = _check(STREAM_CASES[case], 1300 + case, P.PATH_AUTO, 2e-3, want_kernel=False)
+    print("backward, one candidate per user, worst error / largest entry:", {k: f"{v:.2e}" for k, v in worst.items()})
+
+
+def test_backward_users_without_a_candidate():
+    w = make_custom(U=6, C=1, L=50, d=64, H=2, S=10, M=1, dtype="bf16", seed=1310)
+    offs = np.array([0, 1, 1, 2, 3, 3, 4], dtype=np.int32)          # users 1 and 4 have none
+    s = w.spec
+    args = (w.items, w.lengths, w.cands[:4], offs, w.Wq, w.Wk, w.Wv, w.Wg)
+    dz = np.random.default_rng(3).standard_normal((4, s.d)).astype(np.float32)
+    ref = backward_oracle.backward(*args, s.S, s.H, dz.astype(np.float64), w.gamma, w.tau)
+    b = P.DeviceBatch.from_numpy(items=w.items, lengths=w.lengths, cands=w.cands[:4], cand_offsets=offs, Wq=w.Wq, Wk=w.Wk,
+                                 Wv=w.Wv, Wg=w.Wg, S=s.S, H=s.H, M=s.M, dtype="bf16", gamma=w.gamma, tau=w.tau)
+    got = P.laser_backward(b.cfg, *b.args(), b.Wg, torch.from_numpy(dz).cuda())
+    for k, r in ref.items():
+        assert np.max(np.abs(got[k].cpu().numpy() - r)) <= 2e-3 * np.max(np.abs(r)), k
+    assert not got["d_items"][1].any() and not got["d_items"][4].any()
