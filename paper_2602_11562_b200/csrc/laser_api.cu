@@ -3,6 +3,8 @@
 #include <string.h>
 
 #include <algorithm>
+#include <atomic>
+#include <mutex>
 
 #include "laser_common.cuh"
 
@@ -32,6 +34,45 @@ LaunchScope::LaunchScope(const char* name, cudaStream_t st) : st_(st), slot_(-1)
 }
 LaunchScope::~LaunchScope() {
   if (slot_ >= 0) cudaEventRecord(g_prof_ev[2 * slot_ + 1], st_);
+}
+
+constexpr int kMaxDevices = 64;
+int device_sms() {
+  static std::atomic<int> known[kMaxDevices];
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 148;
+  if (dev < kMaxDevices && (n = known[dev].load(std::memory_order_relaxed)) > 0) return n;
+  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) return 148;
+  if (dev < kMaxDevices) known[dev].store(n, std::memory_order_relaxed);
+  return n;
+}
+
+// One slot per (kernel, device), open addressing (a full table only costs a repeated driver call).  The attribute is raised
+// under a lock and never lowered, so that threads with launches of different sizes do not undo each other's.
+cudaError_t allow_smem_ptr(const void* kernel, int bytes) {
+  struct Slot {
+    std::atomic<uintptr_t> key;
+    std::atomic<int> bytes;
+  };
+  constexpr unsigned kSlots = 1024;
+  static Slot slots[kSlots];
+  int dev = 0;
+  const cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const uintptr_t key = reinterpret_cast<uintptr_t>(kernel) ^ ((uintptr_t)dev << 56);
+  Slot* mine = nullptr;
+  for (unsigned i = 0; i < 16 && !mine; ++i) {
+    Slot& s = slots[((key >> 4) * 0x9E3779B97F4A7C15ull >> 32) + i & (kSlots - 1)];
+    uintptr_t empty = 0;
+    if (s.key.load(std::memory_order_acquire) == key || s.key.compare_exchange_strong(empty, key) || empty == key) mine = &s;
+  }
+  if (mine && mine->bytes.load(std::memory_order_acquire) >= bytes) return cudaSuccess;
+  static std::mutex raise;
+  const std::lock_guard<std::mutex> lock(raise);
+  if (mine && mine->bytes.load(std::memory_order_acquire) >= bytes) return cudaSuccess;
+  const cudaError_t rc = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (rc == cudaSuccess && mine) mine->bytes.store(bytes, std::memory_order_release);
+  return rc;
 }
 
 static int resolve_path(const Plan& p, int requested) {
@@ -132,6 +173,7 @@ static int clear_status(const Plan& p, char* ws, cudaStream_t st) {
   return LASER_OK;
 }
 
+// Every path's first kernel clears the status word (its block 0, before anything reports into it).
 // Wg_images: GSTA weights whose images the STA set-up may build on the side (null when GSTA does not follow).
 static int run_sta(const Plan& p, const void* items, const int32_t* lengths, const void* cands,
                    const int32_t* cand_offsets, const void* Wq, const void* Wk, const void* Wv, void* Hp, char* ws,
@@ -157,12 +199,10 @@ static int run_gsta(const Plan& p, const void* Hp, const int32_t* lengths, const
 static int forward_impl(const Plan& p, const void* items, const int32_t* lengths, const void* cands,
                         const int32_t* cand_offsets, const void* Wq, const void* Wk, const void* Wv, const void* Wg,
                         void* Hprime, void* z, char* ws, cudaStream_t st) {
-  int rc = clear_status(p, ws, st);
-  if (rc != LASER_OK) return rc;
-  if (p.N == 0) return LASER_OK;
+  if (p.N == 0) return clear_status(p, ws, st);       // (with work to do, STA's first kernel clears the status word)
   void* Hp = Hprime ? Hprime : (void*)(ws + p.off_hp);
   const bool side_images = p.M > 0 && p.path != LASER_PATH_SIMT && gsta_mma_supported(p);
-  rc = run_sta(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, Hp, ws, st, side_images ? Wg : nullptr);
+  const int rc = run_sta(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, Hp, ws, st, side_images ? Wg : nullptr);
   if (rc != LASER_OK) return rc;
   return run_gsta(p, Hp, lengths, cand_offsets, cands, Wg, z, ws, st, side_images);
 }
@@ -191,8 +231,7 @@ int laser_sta_forward(const laser_config* cfg, const void* items, const int32_t*
   if (p.N > 0 && (rc = check_ptrs({items, cands, Wq, Wk, Wv, Hprime})) != LASER_OK) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   char* ws = static_cast<char*>(workspace);
-  if ((rc = clear_status(p, ws, st)) != LASER_OK) return rc;
-  if (p.N == 0) return LASER_OK;
+  if (p.N == 0) return clear_status(p, ws, st);
   return run_sta(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, Hprime, ws, st, nullptr);
 }
 
@@ -300,8 +339,7 @@ int laser_sta_softmax_forward(const laser_config* cfg, const void* items, const 
   if (p.N > 0 && (rc = check_ptrs({items, cands, Wq, Wk, Wv, Hprime})) != LASER_OK) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   char* ws = static_cast<char*>(workspace);
-  if ((rc = clear_status(p, ws, st)) != LASER_OK) return rc;
-  if (p.N == 0) return LASER_OK;
+  if (p.N == 0) return clear_status(p, ws, st);
   if (p.path == LASER_PATH_TENSOR)
     return tensor_sta(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, Hprime, ws, st, nullptr, true);
   return simt_sta_softmax(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, Hprime, ws, st);
@@ -400,8 +438,7 @@ int laser_forward_ffn(const laser_config* cfg, const void* items, const int32_t*
   if (Hprime && !aligned16(Hprime)) return LASER_ERR_INVALID_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   char* ws = static_cast<char*>(workspace);
-  if ((rc = clear_status(p, ws, st)) != LASER_OK) return rc;
-  if (p.N == 0) return LASER_OK;
+  if (p.N == 0) return clear_status(p, ws, st);
   void* Hp = Hprime ? Hprime : (void*)(ws + p.off_hp);
   const bool side_images = p.M > 0 && p.path != LASER_PATH_SIMT && gsta_mma_supported(p);
   rc = run_sta(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, Hp, ws, st, side_images ? Wgsta : nullptr);

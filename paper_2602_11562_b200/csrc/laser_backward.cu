@@ -361,13 +361,6 @@ rows_gemm_kernel(int M, int K, const TA* __restrict__ A, int lda, const TB* __re
   }
 }
 
-int bwd_sm_count() {
-  int dev = 0, n = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return 148;
-  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) return 148;
-  return n;
-}
-
 template <typename TA, typename TB>
 bool rows_gemm_fits(int M, int N, int K, const TA* A, int lda, const float* C, int ldc) {
   constexpr int per16 = 16 / (int)sizeof(TA);
@@ -381,11 +374,11 @@ int launch_rows_gemm(cudaStream_t st, int M, int K, const TA* A, int lda, const 
                      float alpha, bool accumulate, bf16* C16 = nullptr) {
   const size_t smem = (size_t)K * (N + 8) * sizeof(uint32_t) + 2 * (size_t)kRowsTile * RowsPitch<TA>::elems(K) * sizeof(TA);
   auto kernel = rows_gemm_kernel<TA, TB, N>;
-  LASER_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  LASER_CUDA_OK(allow_smem(kernel, smem));
   const int n_tiles = (M + kRowsTile - 1) / kRowsTile;
   const int per_sm = smem <= 100 * 1024 ? 2 : 1;
   LaunchScope ls("bwd_gemm_rows", st);
-  kernel<<<std::min(n_tiles, per_sm * bwd_sm_count()), kGemmThreads, smem, st>>>(M, K, A, lda, B, ldb, tb ? 1 : 0, C, C16, ldc,
+  kernel<<<std::min(n_tiles, per_sm * device_sms()), kGemmThreads, smem, st>>>(M, K, A, lda, B, ldb, tb ? 1 : 0, C, C16, ldc,
                                                                               alpha, accumulate ? 1 : 0, n_tiles);
   LASER_CUDA_OK(cudaGetLastError());
   return LASER_OK;
@@ -487,8 +480,8 @@ int launch_cols_gemm(cudaStream_t st, int R, const TA* A, int lda, const TB* B, 
   constexpr int AP = MO + 16 / (int)sizeof(TA) * 2, BPT = N + 32 / (int)sizeof(TB);
   const size_t smem = 2 * 32 * ((size_t)AP * sizeof(TA) + (size_t)BPT * sizeof(TB));
   auto kernel = cols_gemm_kernel<TA, TB, MO, N>;
-  LASER_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  const int blocks_max = 2 * bwd_sm_count();
+  LASER_CUDA_OK(allow_smem(kernel, smem));
+  const int blocks_max = 2 * device_sms();
   const int per = ((R + blocks_max - 1) / blocks_max + 31) / 32 * 32;
   LaunchScope ls("bwd_gemm_cols", st);
   kernel<<<(R + per - 1) / per, kGemmThreads, smem, st>>>(R, A, lda, B, ldb, C, ldc, alpha, per);
@@ -979,82 +972,6 @@ __global__ void sta_bwd_kernel(const float* __restrict__ Qf, const float* __rest
   }
 }
 
-// H' in fp32 for the backward's forward recomputation, head widths known at compile time: one block per (segment, 32
-// candidates, user), thread (candidate, head) with its query slice and its accumulators in registers; the segment's
-// items pass through shared memory 32 at a time and every lane reads them as 128-bit broadcasts.  (Other head widths
-// use the forward's own FP32 kernel.)
-template <int DQH, int DVH>
-__global__ void sta_fwd32_kernel(const float* __restrict__ Qf, const float* __restrict__ Kf, const float* __restrict__ Vf,
-                                 const int* __restrict__ lengths, const int* __restrict__ cand_offsets,
-                                 float* __restrict__ Hp, int L, int d, int dqk, int H, int S, int Lp, int N) {
-  extern __shared__ __align__(16) float sm[];
-  float* Ks = sm;                        // [32][dqk]
-  float* Vs = Ks + kChunk * dqk;         // [32][d]
-  const int u = blockIdx.z, seg = blockIdx.x;
-  const int len = lengths[u], off0 = cand_offsets[u], off1 = cand_offsets[u + 1];
-  if (len < 0 || len > L || off0 < 0 || off1 < off0 || off1 > N) return;
-  const int c0 = off0 + blockIdx.y * 32;
-  if (c0 >= off1) return;
-  const int tid = threadIdx.x, nt = blockDim.x, ci = tid & 31, h = tid >> 5, c = c0 + ci;
-  const bool live = c < off1 && h < H;
-  float q[DQH], acc[DVH];
-#pragma unroll
-  for (int a = 0; a < DQH / 4; ++a) {
-    const float4 x = live ? reinterpret_cast<const float4*>(Qf + (size_t)c * dqk + h * DQH)[a] : make_float4(0.f, 0.f, 0.f, 0.f);
-    q[4 * a] = x.x; q[4 * a + 1] = x.y; q[4 * a + 2] = x.z; q[4 * a + 3] = x.w;
-  }
-#pragma unroll
-  for (int v = 0; v < DVH; ++v) acc[v] = 0.f;
-  const int n_begin = seg * S, n_end = min(min(n_begin + S, L), len);
-  for (int nb = n_begin; nb < n_end; nb += kChunk) {
-    const int cnt = min(kChunk, n_end - nb);
-    __syncthreads();
-    for (int i = tid; i < cnt * dqk / 4; i += nt)
-      reinterpret_cast<float4*>(Ks)[i] = reinterpret_cast<const float4*>(Kf + ((size_t)u * L + nb) * dqk)[i];
-    for (int i = tid; i < cnt * d / 4; i += nt)
-      reinterpret_cast<float4*>(Vs)[i] = reinterpret_cast<const float4*>(Vf + ((size_t)u * L + nb) * d)[i];
-    __syncthreads();
-    if (live) {
-      for (int n = 0; n < cnt; ++n) {
-        const float4* kp = reinterpret_cast<const float4*>(Ks + n * dqk + h * DQH);
-        const float4* vp = reinterpret_cast<const float4*>(Vs + n * d + h * DVH);
-        float e = 0.f;
-#pragma unroll
-        for (int a = 0; a < DQH / 4; ++a) {
-          const float4 x = kp[a];
-          e = fmaf(q[4 * a], x.x, e); e = fmaf(q[4 * a + 1], x.y, e); e = fmaf(q[4 * a + 2], x.z, e); e = fmaf(q[4 * a + 3], x.w, e);
-        }
-        const float g = 1.f / (1.f + expf(-e));
-#pragma unroll
-        for (int v = 0; v < DVH / 4; ++v) {
-          const float4 x = vp[v];
-          acc[4 * v] = fmaf(g, x.x, acc[4 * v]); acc[4 * v + 1] = fmaf(g, x.y, acc[4 * v + 1]);
-          acc[4 * v + 2] = fmaf(g, x.z, acc[4 * v + 2]); acc[4 * v + 3] = fmaf(g, x.w, acc[4 * v + 3]);
-        }
-      }
-    }
-  }
-  if (live) {
-    float4* out = reinterpret_cast<float4*>(Hp + ((size_t)c * Lp + seg) * d + h * DVH);
-#pragma unroll
-    for (int v = 0; v < DVH / 4; ++v) out[v] = make_float4(acc[4 * v], acc[4 * v + 1], acc[4 * v + 2], acc[4 * v + 3]);
-  }
-}
-
-template <int DQH, int DVH>
-int launch_sta_fwd32(const Plan& p, const float* Qf, const float* Kf, const float* Vf, const int32_t* lengths,
-                     const int32_t* cand_offsets, float* Hp, cudaStream_t st) {
-  const size_t smem = (size_t)kChunk * (p.dqk + p.d) * sizeof(float);
-  const int ctiles = (p.maxC + 31) / 32;
-  if (p.U > 65535 || ctiles > 65535 || smem > 200 * 1024) return LASER_ERR_UNSUPPORTED;
-  LASER_CUDA_OK(cudaFuncSetAttribute(sta_fwd32_kernel<DQH, DVH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  LaunchScope ls("bwd_sta_fwd", st);
-  sta_fwd32_kernel<DQH, DVH><<<dim3(p.Lp, ctiles, p.U), 32 * p.H, smem, st>>>(Qf, Kf, Vf, lengths, cand_offsets, Hp, p.L,
-                                                                               p.d, p.dqk, p.H, p.S, p.Lp, p.N);
-  LASER_CUDA_OK(cudaGetLastError());
-  return LASER_OK;
-}
-
 struct BwdScratch {
   float *Hp, *dHp, *T, *Q, *Qt, *A, *Mh, *dT, *dM, *dQt, *dQ, *dQf, *dK, *dV;
   size_t total;
@@ -1138,15 +1055,11 @@ int backward_t(const Plan& p, const T* items, const int32_t* lengths, const T* c
     }
     if (mma) BWD_OK(sta_mma_operands(p, Qf, kv_ready ? nullptr : Kf, kv_ready ? nullptr : Vf, mma_scratch, st));
     if (mma && sta_fwd_mma_supported(p)) BWD_OK(sta_fwd_mma(p, lengths, cand_offsets, attn_mma ? nullptr : s.Hp, attn_mma, mma_scratch, st));
-    else if (p.dqh == 16 && dvh == 16 && p.H <= 32) BWD_OK(launch_sta_fwd32<16, 16>(p, Qf, Kf, Vf, lengths, cand_offsets, s.Hp, st));
-    else if (p.dqh == 16 && dvh == 32 && p.H <= 32) BWD_OK(launch_sta_fwd32<16, 32>(p, Qf, Kf, Vf, lengths, cand_offsets, s.Hp, st));
+    else if (p.dqh == 16 && (dvh == 16 || dvh == 32 || dvh == 64) && p.H <= 32) BWD_OK(simt_attend_f32(p, lengths, cand_offsets, s.Hp, ws, st));
     else BWD_OK(simt_sta_f32(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, s.Hp, ws, st));
-  } else if (p.dqh == 16 && (dvh == 16 || dvh == 32) && p.H <= 32) {
-    // (a candidate tile of a user with more candidates than max_cands_per_user declares would stay unwritten: zero first)
-    LASER_CUDA_OK(cudaMemsetAsync(s.Hp, 0, (size_t)N * Lp * d * sizeof(float), st));
+  } else if (p.dqh == 16 && (dvh == 16 || dvh == 32 || dvh == 64) && p.H <= 32) {
     BWD_OK(simt_project(p, items, lengths, cands, Wq, Wk, Wv, ws, st));
-    if (dvh == 16) BWD_OK(launch_sta_fwd32<16, 16>(p, Qf, Kf, Vf, lengths, cand_offsets, s.Hp, st));
-    else BWD_OK(launch_sta_fwd32<16, 32>(p, Qf, Kf, Vf, lengths, cand_offsets, s.Hp, st));
+    BWD_OK(simt_attend_f32(p, lengths, cand_offsets, s.Hp, ws, st));
   } else {
     BWD_OK(simt_sta_f32(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, s.Hp, ws, st));
   }
@@ -1167,8 +1080,8 @@ int backward_t(const Plan& p, const T* items, const int32_t* lengths, const T* c
   auto attn_bwd = H % 4 == 0 ? (v4 ? gsta_attn_bwd_kernel<4, 4> : gsta_attn_bwd_kernel<1, 4>)
                   : H % 2 == 0 ? (v4 ? gsta_attn_bwd_kernel<4, 2> : gsta_attn_bwd_kernel<1, 2>)
                                : (v4 ? gsta_attn_bwd_kernel<4, 1> : gsta_attn_bwd_kernel<1, 1>);
-  LASER_CUDA_OK(cudaFuncSetAttribute(attn_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)attn_smem_f));
-  LASER_CUDA_OK(cudaFuncSetAttribute(attn_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)attn_smem_b));
+  LASER_CUDA_OK(allow_smem(attn_fwd, attn_smem_f));
+  LASER_CUDA_OK(allow_smem(attn_bwd, attn_smem_b));
   for (int l = 0; l < M; ++l) {
     const T *Wql = Wg + (size_t)(l * 3) * d * d, *Wkl = Wql + (size_t)d * d, *Wvl = Wkl + (size_t)d * d;
     float *Tl = s.T + l * Nd, *Tn = Tl + Nd, *Ql = s.Q + l * Nd, *Qtl = s.Qt + l * NHd, *Al = s.A + (size_t)l * N * H * Lp,
@@ -1239,7 +1152,7 @@ int backward_t(const Plan& p, const T* items, const int32_t* lengths, const T* c
                         sizeof(float);
     if (smem > 200 * 1024 || (long long)Lp * cps > 0x7fffffffLL || U > 65535 || H > 32) return LASER_ERR_UNSUPPORTED;
     auto kernel = variant == 2 ? sta_bwd_kernel<16, 32> : variant == 1 ? sta_bwd_kernel<16, 16> : sta_bwd_kernel<0, 0>;
-    LASER_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    LASER_CUDA_OK(allow_smem(kernel, smem));
     LaunchScope ls("bwd_sta", st);
     kernel<<<dim3(Lp * cps, U), 32 * H, smem, st>>>(Qf, Kf, Vf, s.dHp, lengths, cand_offsets, s.dQf, s.dK, s.dV, L, d, dqk,
                                                     H, p.S, Lp, N, cps);

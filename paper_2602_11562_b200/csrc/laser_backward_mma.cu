@@ -755,7 +755,7 @@ template <int MT, int DQ16, int DV16>
 int launch_mma(const BwdMmaParams& P, int U, cudaStream_t st) {
   constexpr int smem = kBwdWarps * 2 * 16 * ((2 * 16 * DQ16 + 16) + (2 * 16 * DV16 + 16));
   auto kernel = sta_bwd_mma_kernel<MT, DQ16, DV16>;
-  LASER_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  LASER_CUDA_OK(allow_smem(kernel, smem));
   LaunchScope ls("bwd_sta_mma", st);
   kernel<<<dim3((P.jobs + kBwdWarps - 1) / kBwdWarps, U), kBwdWarps * 32, smem, st>>>(P);
   LASER_CUDA_OK(cudaGetLastError());
@@ -771,7 +771,7 @@ size_t fwd_smem(const Plan& p) {
 template <int DQ16, int DV16>
 int launch_fwd(const FwdMmaParams& P, int U, size_t smem, cudaStream_t st) {
   auto kernel = sta_fwd_mma_kernel<DQ16, DV16>;
-  LASER_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  LASER_CUDA_OK(allow_smem(kernel, smem));
   LaunchScope ls("bwd_sta_fwd_mma", st);
   kernel<<<dim3(P.Lp * P.H, U), kBwdWarps * 32, smem, st>>>(P);
   LASER_CUDA_OK(cudaGetLastError());
@@ -849,7 +849,7 @@ int launch_attn_fwd(const AttnFwdParams& P, cudaStream_t st) {
   constexpr size_t smem = (size_t)kAttnWarps * 40 * (2 * 16 * D16 + 16);
   const int nch = (P.Lp + 31) / 32;
   auto kernel = nch <= 1 ? gsta_attn_fwd_mma_kernel<D16, 1> : nch <= 2 ? gsta_attn_fwd_mma_kernel<D16, 2> : gsta_attn_fwd_mma_kernel<D16, 4>;
-  LASER_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  LASER_CUDA_OK(allow_smem(kernel, smem));
   LaunchScope ls("bwd_attn_fwd_mma", st);
   kernel<<<(P.N + kAttnWarps - 1) / kAttnWarps, kAttnWarps * 32, smem, st>>>(P);
   LASER_CUDA_OK(cudaGetLastError());
@@ -873,7 +873,7 @@ int launch_attn_bwd(const AttnBwdParams& P, cudaStream_t st) {
   constexpr size_t smem = (size_t)kAttnWarps * 48 * (2 * 16 * D16 + 16);
   const int nch = (P.Lp + 31) / 32;
   auto kernel = nch <= 1 ? gsta_attn_bwd_mma_kernel<D16, 1> : nch <= 2 ? gsta_attn_bwd_mma_kernel<D16, 2> : gsta_attn_bwd_mma_kernel<D16, 4>;
-  LASER_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  LASER_CUDA_OK(allow_smem(kernel, smem));
   LaunchScope ls("bwd_attn_bwd_mma", st);
   kernel<<<(P.N + kAttnWarps - 1) / kAttnWarps, kAttnWarps * 32, smem, st>>>(P);
   LASER_CUDA_OK(cudaGetLastError());

@@ -533,13 +533,6 @@ __global__ void __launch_bounds__(256) bs_wv_kernel(BsParams P, int KR) {
       atomicAdd(P.dWv + (size_t)(mtile * 16 + g + (e >> 1) * 8) * d + j * 8 + 2 * t + (e & 1), acc[j][e]);
 }
 
-int sms_of_device() {
-  int dev = 0, n = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return 148;
-  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) return 148;
-  return n;
-}
-
 size_t ring_bytes(int d, int H, bool with_y) { return (size_t)kBRows * (2 * d + 16) + (with_y ? (size_t)H * d * 4 : 0); }
 int slot_steps(int H) { return (6 * H + 15) / 16; }
 size_t bwd_warp_bytes(int d, int H) {
@@ -551,7 +544,7 @@ int wv_rows(int d, int H) {                                 // rows per step tha
 }
 // Blocks per user: enough that a batch of few users still fills the GPU, at most one per kBW segments.
 int user_parts(const Plan& p) {
-  const int want = (4 * sms_of_device() + p.U - 1) / p.U, most = (p.Lp + kBW - 1) / kBW;
+  const int want = (4 * device_sms() + p.U - 1) / p.U, most = (p.Lp + kBW - 1) / kBW;
   return std::max(1, std::min(std::min(want, most), 65535));
 }
 
@@ -594,33 +587,33 @@ template <int D16>
 int bs_forward_t(const Plan& p, BsParams P, cudaStream_t st) {
   {
     const size_t smem = kBW * kBStages * ring_bytes(p.d, p.H, false);
-    LASER_CUDA_OK(cudaFuncSetAttribute(bs_fwd_kernel<D16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    LASER_CUDA_OK(allow_smem(bs_fwd_kernel<D16>, smem));
     LaunchScope ls("bs_fwd", st);
     bs_fwd_kernel<D16><<<dim3(p.U, user_parts(p)), kBThreads, smem, st>>>(P);
   }
   const size_t smem = (size_t)p.d * (2 * p.d + 16);
-  LASER_CUDA_OK(cudaFuncSetAttribute(bs_rows_kernel<D16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  LASER_CUDA_OK(allow_smem(bs_rows_kernel<D16>, smem));
   const long long jobs = (long long)p.U * ((p.Lp + 15) / 16);
   LaunchScope ls("bs_rows_s", st);
-  bs_rows_kernel<D16><<<(int)std::min<long long>((jobs + 7) / 8, 3 * sms_of_device()), 256, smem, st>>>(P, 0);
+  bs_rows_kernel<D16><<<(int)std::min<long long>((jobs + 7) / 8, 3 * device_sms()), 256, smem, st>>>(P, 0);
   LASER_CUDA_OK(cudaGetLastError());
   return LASER_OK;
 }
 
 template <int D16>
 int bs_backward_t(const Plan& p, BsParams P, cudaStream_t st) {
-  const int sms = sms_of_device(), parts = user_parts(p);
+  const int sms = device_sms(), parts = user_parts(p);
   const long long jobs = (long long)p.U * ((p.Lp + 15) / 16);
   {
     const size_t smem = (size_t)p.d * (2 * p.d + 16);
-    LASER_CUDA_OK(cudaFuncSetAttribute(bs_rows_kernel<D16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    LASER_CUDA_OK(allow_smem(bs_rows_kernel<D16>, smem));
     LaunchScope ls("bs_rows_y", st);
     bs_rows_kernel<D16><<<(int)std::min<long long>((jobs + 7) / 8, 3 * sms), 256, smem, st>>>(P, 1);
   }
   {
     const int warp_bytes = (int)bwd_warp_bytes(p.d, p.H);
     const size_t smem = (size_t)kBW * warp_bytes;
-    LASER_CUDA_OK(cudaFuncSetAttribute(bs_bwd_kernel<D16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    LASER_CUDA_OK(allow_smem(bs_bwd_kernel<D16>, smem));
     LASER_CUDA_OK(cudaMemsetAsync(P.p, 0, (size_t)p.N * p.H * p.d * sizeof(float), st));
     LaunchScope ls("bs_bwd", st);
     bs_bwd_kernel<D16><<<dim3(p.U, parts), kBThreads, smem, st>>>(P, slot_steps(p.H), warp_bytes);
@@ -628,7 +621,7 @@ int bs_backward_t(const Plan& p, BsParams P, cudaStream_t st) {
   {
     const int KR = wv_rows(p.d, p.H);
     const size_t smem = 2 * (size_t)KR * ((size_t)p.H * p.d + p.d + 16) * sizeof(float);
-    LASER_CUDA_OK(cudaFuncSetAttribute(bs_wv_kernel<D16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    LASER_CUDA_OK(allow_smem(bs_wv_kernel<D16>, smem));
     LaunchScope ls("bs_wv", st);
     bs_wv_kernel<D16><<<std::min(p.U, 2 * sms), 256, smem, st>>>(P, KR);
   }

@@ -71,9 +71,12 @@ int simt_sta_softmax(const Plan& p, const void* items, const int32_t* lengths, c
                      cudaStream_t st);
 int simt_gsta(const Plan& p, const void* Hprime, const int32_t* lengths, const int32_t* cand_offsets, const void* cands,
               const void* Wg, void* z, char* ws, cudaStream_t st);
-// Eq. 8-9 on the FP32 ALUs: leaves fp32 Q / gamma, K, V at off_q, off_k, off_v.
+// Eq. 8-9 on the FP32 ALUs (fp32 Q / gamma, K, V at off_q, off_k, off_v), and the segment sums alone, from fp32 Q / gamma, K, V at off_q, off_k, off_v (16-wide query heads, 16-, 32- or 64-wide value
+// heads; else LASER_ERR_UNSUPPORTED).
 int simt_project(const Plan& p, const void* items, const int32_t* lengths, const void* cands, const void* Wq,
                  const void* Wk, const void* Wv, char* ws, cudaStream_t st);
+int simt_attend_f32(const Plan& p, const int32_t* lengths, const int32_t* cand_offsets, float* Hprime32, char* ws,
+                    cudaStream_t st);
 // STA on the FP32 ALUs with an fp32 H' whatever the I/O dtype; leaves fp32 Q / gamma, K, V at off_q, off_k, off_v.
 int simt_sta_f32(const Plan& p, const void* items, const int32_t* lengths, const void* cands, const int32_t* cand_offsets,
                  const void* Wq, const void* Wk, const void* Wv, float* Hprime32, char* ws, cudaStream_t st);
@@ -182,6 +185,9 @@ template <typename T> __device__ __forceinline__ T from_f32(float v);
 template <> __device__ __forceinline__ float from_f32<float>(float v) { return v; }
 template <> __device__ __forceinline__ __nv_bfloat16 from_f32<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
 
+// The first kernel of a call sets the status word (this, from one thread, after its chain_wait); only later kernels of
+// the call report into it, or the same block after a block-wide barrier.
+__device__ __forceinline__ void set_status(int* status, int code) { *reinterpret_cast<volatile int*>(status) = code; }
 __device__ __forceinline__ void report_status(int* status, int code) { atomicCAS(status, 0, code); }
 
 // Programmatic dependent launch.  Kernels launched with launch_chained may start (block scheduling, shared-memory and
@@ -205,6 +211,16 @@ inline cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 bloc
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
+// SM count of the current device, asked of the driver once per device.
+int device_sms();
+// Lets `kernel` use `bytes` of dynamic shared memory on the current device.  The attribute is set on the first call with
+// a larger size only: the driver call would otherwise be a good part of what a small call costs on the host.
+cudaError_t allow_smem_ptr(const void* kernel, int bytes);
+template <typename... KArgs>
+inline cudaError_t allow_smem(void (*kernel)(KArgs...), size_t bytes) {
+  return allow_smem_ptr(reinterpret_cast<const void*>(kernel), (int)bytes);
 }
 
 #define LASER_CUDA_OK(expr)                          \

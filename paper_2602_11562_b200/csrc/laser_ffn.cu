@@ -637,16 +637,6 @@ __global__ void __launch_bounds__(256) ffn_simt_kernel(FfnSimtParams<T> P) {
   }
 }
 
-int ffn_sm_count() {
-  static int n = 0;
-  if (n == 0) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 148;
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 148;
-  }
-  return n;
-}
-
 size_t ffn_tc_smem(int d, int hid) {
   return (size_t)4 * kRows * d * 2 + (size_t)kWStages * kChunk * d * 2 + (size_t)3 * d * sizeof(float) + (size_t)hid * 2;
 }
@@ -678,9 +668,9 @@ int ffn_simt(const Plan& p, const laser_ffn_params* f, void* H, const int32_t* l
     LASER_CUDA_OK(launch_chained(ffn_simt_prep_kernel<T>, dim3(1), dim3(1024), 0, st, P));
   }
   {
-    LASER_CUDA_OK(cudaFuncSetAttribute(ffn_simt_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    LASER_CUDA_OK(allow_smem(ffn_simt_kernel<T>, smem));
     const long long blocks_needed = ((long long)p.N * p.Lp + kSimtRows - 1) / kSimtRows;
-    const int grid = (int)(blocks_needed < 8LL * ffn_sm_count() ? (blocks_needed > 0 ? blocks_needed : 1) : 8LL * ffn_sm_count());
+    const int grid = (int)(blocks_needed < 8LL * device_sms() ? (blocks_needed > 0 ? blocks_needed : 1) : 8LL * device_sms());
     LaunchScope ls("ffn_simt", st);
     LASER_CUDA_OK(launch_chained(ffn_simt_kernel<T>, dim3(grid), dim3(256), smem, st, P));
   }
@@ -732,15 +722,15 @@ int ffn_forward(const Plan& p, const laser_ffn_params* f, void* H, const int32_t
   }
   {
     const long long rows_max = (long long)p.N * p.Lp;
-    const int grid = (int)(rows_max < 256LL * 4 * ffn_sm_count() ? (rows_max + 255) / 256 : 4 * ffn_sm_count());
+    const int grid = (int)(rows_max < 256LL * 4 * device_sms() ? (rows_max + 255) / 256 : 4 * device_sms());
     LaunchScope ls("ffn_map", st);
     LASER_CUDA_OK(launch_chained(ffn_map_kernel, dim3(grid > 0 ? grid : 1), dim3(256), 0, st, P));
   }
   {
     const size_t smem = ffn_tc_smem(p.d, hid);
-    LASER_CUDA_OK(cudaFuncSetAttribute(ffn_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    LASER_CUDA_OK(allow_smem(ffn_tc_kernel, smem));
     const long long pairs_max = ((long long)p.N * p.Lp + kPairRows - 1) / kPairRows;
-    const int sms = ffn_sm_count();
+    const int sms = device_sms();
     const int grid = (int)(pairs_max < sms ? (pairs_max > 0 ? pairs_max : 1) : sms);
     LaunchScope ls("ffn_tc", st);
     LASER_CUDA_OK(launch_chained(ffn_tc_kernel, dim3(grid), dim3(kFfnThreads), smem, st, P));

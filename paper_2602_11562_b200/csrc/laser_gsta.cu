@@ -368,11 +368,10 @@ int launch_gsta(const GstaParams& P, cudaStream_t st) {
   constexpr int d = D16 * 16, RS = 2 * d + 16, TS = d + 8;
   const size_t smem = (size_t)kGT * TS * 4 + (size_t)kGT * RS + (size_t)kGT * P.H * RS + RS + kGT * sizeof(int) +
                       (size_t)kGW * 2 * kChunk * RS;
-  int dev = 0, sms = 148;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int sms = device_sms();
   const int blocks = (P.N + P.cpb - 1) / P.cpb;
   auto kernel = (D16 <= 4 && blocks > 2 * sms) ? gsta_mma_kernel<D16, (D16 <= 4 ? 3 : 2)> : gsta_mma_kernel<D16, 2>;
-  LASER_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  LASER_CUDA_OK(allow_smem(kernel, smem));
   LaunchScope ls("gsta_mma", st);
   LASER_CUDA_OK(launch_chained(kernel, dim3(blocks), dim3(kGThreads), smem, st, P));
   return LASER_OK;
@@ -396,15 +395,13 @@ size_t gsta_mma_image_bytes(const Plan& p) {       // the order table and its so
 // Small batches: 8 candidates per block (every warp then has one candidate instead of two, which halves the
 // per-candidate part of a block's latency) as long as all blocks still run at once.
 int gsta_candidates_per_block(const Plan& p) {
-  int dev = 0, sms = 148;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int sms = device_sms();
   return (p.N + 7) / 8 <= 2 * sms ? 8 : kGT;
 }
 
 // Sorting the blocks pays only when the grid runs in more than one wave.
 bool gsta_wants_order(const Plan& p) {
-  int dev = 0, sms = 148;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int sms = device_sms();
   const int cpb = gsta_candidates_per_block(p);
   return p.M > 0 && (p.N + cpb - 1) / cpb > 2 * sms;
 }

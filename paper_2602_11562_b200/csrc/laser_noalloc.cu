@@ -72,10 +72,11 @@ extern "C" int laser_sta_forward_static(const laser_config* cfg, const void* ite
   char* scratch = nullptr;
   if ((rc = static_scratch_for_current_device(&scratch)) != LASER_OK) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  // The array keeps whatever the previous call left in it.  Only the status word must start at zero: Q, K and
-  // V are fully rewritten for every row that is read afterwards.
-  LASER_CUDA_OK(cudaMemsetAsync(scratch + p.off_status, 0, kStatusWords * sizeof(int), st));
-  if (p.N > 0) {
+  // The array keeps whatever the previous call left in it.  Only the status word must start at zero (the first
+  // kernel clears it): Q, K and V are fully rewritten for every row that is read afterwards.
+  if (p.N == 0) {
+    LASER_CUDA_OK(cudaMemsetAsync(scratch + p.off_status, 0, sizeof(int), st));
+  } else {
     rc = simt_sta(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, Hprime, scratch, st);
     if (rc != LASER_OK) return rc;
   }

@@ -56,12 +56,12 @@ struct StreamParams {
 };
 
 // Candidate of user u, or -1 when it has none (or its offsets / length are invalid).
-__device__ __forceinline__ int user_candidate(const StreamParams& P, int u, int* len_out) {
+__device__ __forceinline__ int user_candidate(const StreamParams& P, int u, int* len_out, bool report = true) {
   const int c0 = P.cand_offsets[u], c1 = P.cand_offsets[u + 1], len = P.lengths[u];
   bool bad = c0 < 0 || c1 < c0 || c1 > P.N || c1 - c0 > 1 || len < 0 || len > P.L;
   if (!bad && P.item_off) bad = P.item_off[u] < 0 || P.item_off[u] > P.item_off[P.U] - len;
   if (bad) {
-    report_status(P.status, LASER_ERR_BAD_INPUT);
+    if (report) report_status(P.status, LASER_ERR_BAD_INPUT);
     return -1;
   }
   *len_out = len;
@@ -76,6 +76,7 @@ __global__ void __launch_bounds__(kPreWarps * 32) stream_pre_kernel(StreamParams
   const int dqk = P.dqk, H = P.H, dqh = dqk / H;
   chain_wait();
   chain_release();
+  if (blockIdx.x == 0 && threadIdx.x == 0) set_status(P.status, 0);   // (the attention kernel checks every user and reports)
   if (P.order && blockIdx.x == gridDim.x - 1) {
     // the last block sorts the users by length, longest first: the attention kernel's grid runs in several waves of
     // blocks whose time is proportional to the user's length, and its last wave should be made of the shortest
@@ -108,8 +109,8 @@ __global__ void __launch_bounds__(kPreWarps * 32) stream_pre_kernel(StreamParams
   // users 16 wg + g (MMA rows g) and 16 wg + g + 8 (rows g + 8); a user without a candidate is a zero row
   const int uA = wg * 16 + g, uB = uA + 8;
   int lenA = 0, lenB = 0;
-  const int cA = uA < P.U ? user_candidate(P, uA, &lenA) : -1;
-  const int cB = uB < P.U ? user_candidate(P, uB, &lenB) : -1;
+  const int cA = uA < P.U ? user_candidate(P, uA, &lenA, false) : -1;
+  const int cB = uB < P.U ? user_candidate(P, uB, &lenB, false) : -1;
   if (P.Wg && t == 0) {                                  // segment counts of these users' candidates for the GSTA kernel
     if (cA >= 0) P.gnseg[cA] = min((lenA + P.S - 1) / P.S, P.Lp);
     if (cB >= 0) P.gnseg[cB] = min((lenB + P.S - 1) / P.S, P.Lp);
@@ -367,7 +368,7 @@ size_t stream_smem_bytes(int d, int H, int Lp) {
 template <int D16>
 int launch_stream(const StreamParams& P, cudaStream_t st) {
   const size_t smem = stream_smem_bytes(P.d, P.H, P.Lp);
-  LASER_CUDA_OK(cudaFuncSetAttribute(stream_sta_kernel<D16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  LASER_CUDA_OK(allow_smem(stream_sta_kernel<D16>, smem));
   LaunchScope ls("stream_sta", st);
   LASER_CUDA_OK(launch_chained(stream_sta_kernel<D16>, dim3(P.U), dim3(kSThreads), smem, st, P));
   return LASER_OK;
@@ -411,8 +412,7 @@ size_t stream_scratch_bytes(const Plan& p) {   // u, the W_v image, the launch o
 
 // Sorting the users pays only when the attention grid runs in more than one wave (four blocks per SM).
 static bool stream_wants_order(const Plan& p) {
-  int dev = 0, sms = 148;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int sms = device_sms();
   return p.U > 4 * sms;
 }
 

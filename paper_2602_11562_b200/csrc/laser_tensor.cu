@@ -120,7 +120,9 @@ __global__ void __launch_bounds__(1024) tc_prep_kernel(TcParams P) {
       b += s.ctiles * s.nseg;
       c += proj_units_of(P, s);
     }
-    if (bad) report_status(P.status, LASER_ERR_BAD_INPUT);
+    if (tid == 0 && P.Wg && P.N > 0) bad |= P.cand_offsets[0] != 0 || P.cand_offsets[P.U] < P.N;   // (GSTA follows: every candidate has a user)
+    bad = __syncthreads_or(bad);
+    if (tid == 0) set_status(P.status, bad ? LASER_ERR_BAD_INPUT : 0);
     sa[tid] = a;
     sb[tid] = b;
     sc[tid] = c;
@@ -206,7 +208,7 @@ __global__ void __launch_bounds__(1024) tc_prep_kernel(TcParams P) {
   }
   if (P.Wg) {
     gsta_build_images(P.Wg, P.gimg, P.d, P.M, g, nthreads);
-    gsta_build_nseg(P.lengths, P.cand_offsets, P.U, P.N, P.L, P.S, P.Lp, P.status, P.gnseg, g >> 5, nthreads >> 5, tid & 31);
+    gsta_build_nseg(P.lengths, P.cand_offsets, P.U, P.N, P.L, P.S, P.Lp, nullptr, P.gnseg, g >> 5, nthreads >> 5, tid & 31);
   }
 }
 
@@ -1105,13 +1107,6 @@ __global__ void __launch_bounds__(128) tc_wait_selftest_kernel(int* status, uint
   if (tid == 0 && s_abort) report_status(status, LASER_ERR_TIMEOUT);
 }
 
-int sm_count() {                         // of the current device (a process may drive several)
-  int dev = 0, n = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return 148;
-  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) return 148;
-  return n;
-}
-
 TcParams make_params(const Plan& p, const void* items, const int32_t* lengths, const void* cands,
                      const int32_t* cand_offsets, const void* Wq, const void* Wk, const void* Wv, void* Hp, char* ws) {
   TcParams P = {};
@@ -1138,8 +1133,8 @@ TcParams make_params(const Plan& p, const void* items, const int32_t* lengths, c
   P.sta_begin = reinterpret_cast<int4*>(ws + p.off_tcount + 64 * sizeof(int));
   P.proj_begin = P.sta_begin + 1024;
   P.ctile = reinterpret_cast<int4*>(ws + p.off_tctile);
-  P.sta_grid = sm_count() < 1024 ? sm_count() : 1024;
-  P.proj_grid = 2 * sm_count() < 1024 ? 2 * sm_count() : 1024;
+  P.sta_grid = device_sms() < 1024 ? device_sms() : 1024;
+  P.proj_grid = 2 * device_sms() < 1024 ? 2 * device_sms() : 1024;
   P.imgK = (bf16*)(ws + p.off_timg);
   P.imgQ = P.imgK + (size_t)p.dqk * p.d;
   P.imgV = P.imgQ + (size_t)p.dqk * p.d;
@@ -1217,14 +1212,13 @@ int tensor_sta(const Plan& p, const void* items, const int32_t* lengths, const v
     P.gorder_keys = P.gorder + (p.N + 7) / 8;
     P.gcpb = gsta_candidates_per_block(p);
   }
-  const int sms = sm_count();
   {
     LaunchScope ls("tc_prep", st);
     LASER_CUDA_OK(launch_chained(tc_prep_kernel, dim3(1 + 32 + (P.gorder ? 1 : 0)), dim3(1024), 0, st, P));
   }
   {
     const size_t smem = ((size_t)p.dqk * p.d + 3 * (size_t)kCandTile * p.d) * 2;   // W_k^T | W_q^T, W_v^T, two staging buffers
-    LASER_CUDA_OK(cudaFuncSetAttribute(tc_proj_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    LASER_CUDA_OK(allow_smem(tc_proj_kernel, smem));
     LaunchScope ls("tc_proj", st);
     alignas(64) CUtensorMap item_map;
     memset(&item_map, 0, sizeof(item_map));
@@ -1240,7 +1234,7 @@ int tensor_sta(const Plan& p, const void* items, const int32_t* lengths, const v
     const size_t smem = sta_smem_bytes(p, P.IT, softmax);
     if (smem > 220 * 1024) return LASER_ERR_UNSUPPORTED;
     auto kernel = softmax ? tc_sta_kernel<true> : tc_sta_kernel<false>;
-    LASER_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    LASER_CUDA_OK(allow_smem(kernel, smem));
     LaunchScope ls(softmax ? "sta_tc_softmax" : "sta_tc", st);
     LASER_CUDA_OK(launch_chained(kernel, dim3(P.sta_grid), dim3(kStaThreads), smem, st, P));
   }
