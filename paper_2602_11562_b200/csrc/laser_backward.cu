@@ -18,6 +18,7 @@
 //   Qt_h = Q_h W_k[:, h]^T / tau  =>  dQ_h = dQt_h W_k[:, h] / tau,  dW_k[:, h] += dQt_h^T Q_h / tau
 // Sums over candidates that end in one weight matrix are split over blocks and finished with floating-point atomics, so
 // the last bits of the weight gradients and of d_cands' STA part depend on the order in which blocks finish.
+#include "laser_backward.cuh"
 #include "laser_common.cuh"
 #include "laser_mma.cuh"
 
@@ -820,12 +821,13 @@ gsta_attn_bwd_kernel(const float* __restrict__ Hp, const float* __restrict__ Qt,
 }
 
 // One block per (user, 32 consecutive items of one segment), thread (item n, head h); the block walks the user's
-// candidates, kCandsPerStep at a time between two block-wide barriers.  Qf holds q / gamma, so the score is Qf_h . k_n
+// candidates, `step` at a time between two block-wide barriers.  Qf holds q / gamma, so the score is Qf_h . k_n
 // and dQf is the gradient with respect to q / gamma.  dK, dV rows of this chunk are written once (no other block touches
 // them); dQf is summed over the chunks atomically: the per-item terms de_n of a step go through shared memory and thread
 // (candidate, head, component) adds up its 32 items while the next step's rows are loaded.
 constexpr int kChunk = 32;
-constexpr int kCandsPerStep = 4;
+constexpr int kCandsPerStep = 16, kCandsPerStepMin = 4;      // the smaller one where shared memory is short
+// `parts` warps share a (32 items, head): part k takes candidates k, k + parts, ... of a step (register variant only).
 // DQH, DVH > 0: the head widths are compile-time constants and thread (item, head) keeps its key / value slices and
 // their gradient accumulators in registers (shared memory then holds only the keys for the query-side sums and the
 // step's candidate rows); 0, 0: any widths, everything in shared memory.
@@ -834,7 +836,7 @@ __global__ void sta_bwd_kernel(const float* __restrict__ Qf, const float* __rest
                                const float* __restrict__ dHp, const int* __restrict__ lengths,
                                const int* __restrict__ cand_offsets, float* __restrict__ dQf, float* __restrict__ dKf,
                                float* __restrict__ dVf, int L, int d, int dqk, int H, int S, int Lp, int N,
-                               int chunks_per_seg) {
+                               int chunks_per_seg, int step, int parts) {
   constexpr bool kRegs = DQH > 0;
   constexpr int kR = kRegs ? DQH : 1, kV = kRegs ? DVH : 1;
   extern __shared__ __align__(16) float sm[];
@@ -849,10 +851,11 @@ __global__ void sta_bwd_kernel(const float* __restrict__ Qf, const float* __rest
   float* Vs = Ks + kChunk * kld;                                   // [32][d + 1]      (shared-memory variant only)
   float* dKs = Vs + (kRegs ? 0 : kChunk * vld);                    // [32][dqk + 1]    (shared-memory variant only)
   float* dVs = dKs + (kRegs ? 0 : kChunk * kld);                   // [32][d + 1]      (shared-memory variant only)
-  float* qs = dVs + (kRegs ? 0 : kChunk * vld);                    // [kCandsPerStep][dqk]
-  float* ds = qs + kCandsPerStep * dqk;                            // [kCandsPerStep][d]
-  float* des = ds + kCandsPerStep * d;                             // [kCandsPerStep][H][33]: de of (candidate, head, item)
-  const int tid = threadIdx.x, nt = blockDim.x, n = tid & 31, h = tid >> 5;
+  float* qs = dVs + (kRegs ? 0 : kChunk * vld);                    // [step][dqk]
+  float* ds = qs + step * dqk;                            // [step][d]
+  float* des = ds + step * d;                             // [step][H][33]: de of (candidate, head, item)
+  const int tid = threadIdx.x, nt = blockDim.x, n = tid & 31, h = (tid >> 5) % H, part = (tid >> 5) / H;
+  float* red = des + step * H * 33;                                // [H][DQH + DVH][33]: one part's sums (parts > 1)
   for (int i = tid; i < kChunk * dqk; i += nt) {
     const int r = i / dqk, a = i - r * dqk;
     Ks[r * kld + a] = r < cnt ? Kf[((size_t)u * L + n0 + r) * dqk + a] : 0.f;
@@ -867,7 +870,7 @@ __global__ void sta_bwd_kernel(const float* __restrict__ Qf, const float* __rest
   }
   float kreg[kR], vreg[kV], dk[kR], dv[kV];
   if (kRegs) {
-    const bool live = h < H && n < cnt;
+    const bool live = n < cnt;
     const float4* kp = reinterpret_cast<const float4*>(Kf + ((size_t)u * L + n0 + n) * dqk + h * dqh);
     const float4* vp = reinterpret_cast<const float4*>(Vf + ((size_t)u * L + n0 + n) * d + h * dvh);
 #pragma unroll
@@ -897,8 +900,8 @@ __global__ void sta_bwd_kernel(const float* __restrict__ Qf, const float* __rest
     }
   };
   int prev_lo = 0, prev_n = 0;
-  for (int c = off0; c < off1; c += kCandsPerStep) {
-    const int n_c = min(kCandsPerStep, off1 - c);
+  for (int c = off0; c < off1; c += step) {
+    const int n_c = min(step, off1 - c);
     __syncthreads();                       // the previous step's de terms are complete; its q and ds rows are free
     if (prev_n > 0) reduce_dq(prev_lo, prev_n);
     for (int i = tid; i < n_c * dqk; i += nt) qs[i] = Qf[(size_t)c * dqk + i];
@@ -907,8 +910,8 @@ __global__ void sta_bwd_kernel(const float* __restrict__ Qf, const float* __rest
       ds[i] = dHp[((size_t)(c + cc) * Lp + seg) * d + x];
     }
     __syncthreads();                       // (also: the previous step's sums have been read out of `des`)
-    if (h < H) {
-      for (int cc = 0; cc < n_c; ++cc) {
+    {
+      for (int cc = part; cc < n_c; cc += parts) {
         const float* q = qs + cc * dqk + h * dqh;
         const float* g_out = ds + cc * d + h * dvh;
         float e = 0.f, dg = 0.f;
@@ -952,7 +955,24 @@ __global__ void sta_bwd_kernel(const float* __restrict__ Qf, const float* __rest
   __syncthreads();
   if (prev_n > 0) reduce_dq(prev_lo, prev_n);
   if (kRegs) {
-    if (h < H && n < cnt) {
+    for (int k = 1; k < parts; ++k) {      // part 0 collects the other parts' sums, one after the other
+      float* mine = red + (size_t)h * (kR + kV) * 33 + n;
+      __syncthreads();
+      if (part == k) {
+#pragma unroll
+        for (int a = 0; a < kR; ++a) mine[a * 33] = dk[a];
+#pragma unroll
+        for (int v = 0; v < kV; ++v) mine[(kR + v) * 33] = dv[v];
+      }
+      __syncthreads();
+      if (part == 0) {
+#pragma unroll
+        for (int a = 0; a < kR; ++a) dk[a] += mine[a * 33];
+#pragma unroll
+        for (int v = 0; v < kV; ++v) dv[v] += mine[(kR + v) * 33];
+      }
+    }
+    if (part == 0 && n < cnt) {
       float4* kp = reinterpret_cast<float4*>(dKf + ((size_t)u * L + n0 + n) * dqk + h * dqh);
       float4* vp = reinterpret_cast<float4*>(dVf + ((size_t)u * L + n0 + n) * d + h * dvh);
 #pragma unroll
@@ -994,15 +1014,135 @@ BwdScratch carve_scratch(const Plan& p, char* base) {
   s.Qt = take(M * N * H * d);
   s.A = take(M * N * H * Lp);
   s.Mh = take(M * N * H * d);
-  s.dT = take(N * d);
+  s.dT = take((M + 1) * N * d);
   s.dM = take(N * H * d);
-  s.dQt = take(N * H * d);
-  s.dQ = take(N * d);
+  s.dQt = take(std::max<size_t>(M, 1) * N * H * d);
+  s.dQ = take(std::max<size_t>(M, 1) * N * d);
   s.dQf = take(N * p.dqk);
   s.dK = take(UL * p.dqk);
   s.dV = take(UL * d);
   s.total = off;
   return s;
+}
+
+// The gate kernel of the FP32 ALUs: dK, dV rows of valid items, adds to dQf (all of them zeroed before).
+int launch_sta_bwd(const Plan& p, const float* Qf, const float* Kf, const float* Vf, const float* dHp, const int32_t* lengths,
+                   const int32_t* cand_offsets, float* dQf, float* dK, float* dV, cudaStream_t st) {
+  const int L = p.L, d = p.d, H = p.H, dqk = p.dqk, dvh = p.dvh, Lp = p.Lp, N = p.N, U = p.U;
+  const int cps = (min(p.S, L) + kChunk - 1) / kChunk;
+  const int dqh = dqk / H;
+  const int variant = (dqh == 16 && dvh == 32) ? 2 : (dqh == 16 && dvh == 16) ? 1 : 0;   // register-resident head slices
+  // up to four warps per (32 items, head): small batches run about one block per SM and are bound by a warp's serial walk
+  int parts = 1;
+  while (variant && parts < 4 && 2 * parts * H <= 16 && p.maxC >= 4 * parts) parts *= 2;
+  auto smem_of = [&](int step) {
+    return ((parts > 1 ? (size_t)H * (dqh + dvh) * 33 : 0) + (variant ? (size_t)kChunk * (dqk + 1) : 2 * (size_t)kChunk * (dqk + 1 + d + 1)) +
+            (size_t)step * (dqk + d + H * 33)) * sizeof(float);
+  };
+  // (a step costs two barriers and a round trip to L2 whatever it holds: 6 users x 23 candidates 40 -> 22 us with 16)
+  const int step = smem_of(kCandsPerStep) <= 72 * 1024 ? kCandsPerStep : kCandsPerStepMin;
+  const size_t smem = smem_of(step);
+  if (smem > 200 * 1024 || (long long)Lp * cps > 0x7fffffffLL || U > 65535 || H > 32) return LASER_ERR_UNSUPPORTED;
+  auto kernel = variant == 2 ? sta_bwd_kernel<16, 32> : variant == 1 ? sta_bwd_kernel<16, 16> : sta_bwd_kernel<0, 0>;
+  LASER_CUDA_OK(allow_smem(kernel, smem));
+  LaunchScope ls("bwd_sta", st);
+  kernel<<<dim3(Lp * cps, U), 32 * H * parts, smem, st>>>(Qf, Kf, Vf, dHp, lengths, cand_offsets, dQf, dK, dV, L, d, dqk,
+                                                  H, p.S, Lp, N, cps, step, parts);
+  LASER_CUDA_OK(cudaGetLastError());
+  return LASER_OK;
+}
+
+// Several arrays set to zero by one launch.
+struct ZeroList {
+  float* p[8];
+  unsigned long long n[8];
+  int count;
+  void add(float* q, size_t len) {
+    if (len) { p[count] = q; n[count++] = len; }
+  }
+};
+__global__ void __launch_bounds__(256) zero_kernel(const __grid_constant__ ZeroList Z) {
+  for (int a = 0; a < Z.count; ++a) {
+    float4* q = reinterpret_cast<float4*>(Z.p[a]);           // (16-byte aligned arrays)
+    const unsigned long long n4 = Z.n[a] / 4, i0 = (unsigned long long)blockIdx.x * 256 + threadIdx.x;
+    for (unsigned long long i = i0; i < n4; i += (unsigned long long)gridDim.x * 256) q[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (i0 < (Z.n[a] & 3)) Z.p[a][n4 * 4 + i0] = 0.f;
+  }
+}
+int zero_arrays(const ZeroList& Z, cudaStream_t st) {
+  unsigned long long total = 0;
+  for (int i = 0; i < Z.count; ++i) total += Z.n[i];
+  if (total == 0) return LASER_OK;
+  LaunchScope ls("bwd_zero", st);
+  zero_kernel<<<(int)std::min<unsigned long long>((total / 4 + 255) / 256 + 1, 8ull * device_sms()), 256, 0, st>>>(Z);
+  LASER_CUDA_OK(cudaGetLastError());
+  return LASER_OK;
+}
+
+// FP32 ALUs throughout, M > 0: projections, segment sums, all layers of the stacked attention forward and backward, the
+// gates, and every dense product of the gradients in one launch.
+template <typename T>
+int backward_simt(const Plan& p, const T* items, const int32_t* lengths, const T* cands, const int32_t* cand_offsets,
+                  const T* Wq, const T* Wk, const T* Wv, const T* Wg, const float* dz, float* d_items, float* d_cands,
+                  float* dWq, float* dWk, float* dWv, float* dWg, char* ws, cudaStream_t st) {
+  const int N = p.N, d = p.d, H = p.H, M = p.M, dqk = p.dqk, dvh = p.dvh, UL = p.U * p.L;
+  const BwdScratch s = carve_scratch(p, ws + p.total);
+  float* Qf = reinterpret_cast<float*>(ws + p.off_q);
+  float* Kf = reinterpret_cast<float*>(ws + p.off_k);
+  float* Vf = reinterpret_cast<float*>(ws + p.off_v);
+  int rc;
+#define BWD_OK(...) do { rc = (__VA_ARGS__); if (rc != LASER_OK) return rc; } while (0)
+  ZeroList Z = {};
+  Z.add(dWq, (size_t)d * dqk); Z.add(dWk, (size_t)d * dqk); Z.add(dWv, (size_t)d * d); Z.add(dWg, (size_t)M * 3 * d * d);
+  Z.add(s.dQf, (size_t)N * dqk); Z.add(s.dK, (size_t)UL * dqk); Z.add(s.dV, (size_t)UL * d);
+  BWD_OK(zero_arrays(Z, st));
+  if (p.dqh == 16 && (dvh == 16 || dvh == 32 || dvh == 64) && H <= 32) {
+    BWD_OK(simt_project(p, items, lengths, cands, Wq, Wk, Wv, ws, st));
+    BWD_OK(simt_attend_f32(p, lengths, cand_offsets, s.Hp, ws, st));
+  } else {
+    BWD_OK(simt_sta_f32(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, s.Hp, ws, st));
+  }
+  const size_t Nd = (size_t)N * d, dd = (size_t)d * d;
+  const GstaTrain G = {s.T, s.Q, s.dT, s.dQ, s.Mh, s.dQt, s.dT + M * Nd};
+  BWD_OK(gsta_train_simt(p, s.Hp, lengths, cand_offsets, cands, Wg, dz, G, s.dHp, st));
+  BWD_OK(launch_sta_bwd(p, Qf, Kf, Vf, s.dHp, lengths, cand_offsets, s.dQf, s.dK, s.dV, st));
+#undef BWD_OK
+  constexpr bool w16 = sizeof(T) == 2;
+  Product list[kMaxProducts];
+  int n = 0;
+  auto flush = [&]() {
+    const int r = run_products(list, n, st);
+    n = 0;
+    return r;
+  };
+  auto rows_sum = [&](const void* A, int lda, bool a16, const float* B, int ldb, float* C, int ldc, int cols, int rows,
+                      float alpha, int batch, int sa, int sb) {      // C[d x cols] += alpha A^T B over the rows
+    Product P = {};
+    P.A = A; P.lda = lda; P.ta = true; P.a16 = a16; P.B = B; P.ldb = ldb; P.C = C; P.ldc = ldc;
+    P.M = d; P.N = cols; P.K = rows; P.alpha = alpha; P.atomic = true; P.batch = batch; P.sa = sa; P.sb = sb; P.sc = sb;
+    list[n++] = P;
+  };
+  {
+    Product P = {};                                                  // d_items = dK W_k^T + dV W_v^T
+    P.A = s.dK; P.lda = dqk; P.B = Wk; P.ldb = dqk; P.K = dqk; P.A2 = s.dV; P.lda2 = d; P.B2 = Wv; P.ldb2 = d; P.K2 = d;
+    P.tb = true; P.b16 = w16; P.C = d_items; P.ldc = d; P.M = UL; P.N = d; P.alpha = 1.f; P.batch = 1;
+    list[n++] = P;
+    P = Product{};                                                   // d_cands = dt_0 + dQf W_q^T / gamma
+    P.A = s.dQf; P.lda = dqk; P.B = Wq; P.ldb = dqk; P.K = dqk; P.tb = true; P.b16 = w16; P.D = G.dT0; P.C = d_cands; P.ldc = d;
+    P.M = N; P.N = d; P.alpha = p.inv_gamma; P.batch = 1;
+    list[n++] = P;
+  }
+  rows_sum(items, d, w16, s.dK, dqk, dWk, dqk, dqk, UL, 1.f, 1, 0, 0);
+  rows_sum(items, d, w16, s.dV, d, dWv, d, d, UL, 1.f, 1, 0, 0);
+  rows_sum(cands, d, w16, s.dQf, dqk, dWq, dqk, dqk, N, p.inv_gamma, 1, 0, 0);
+  for (int l = 0; l < M; ++l) {
+    float *gWq = dWg + (size_t)(l * 3) * dd, *gWk = gWq + dd, *gWv = gWk + dd;
+    if (n + 3 > kMaxProducts && (rc = flush()) != LASER_OK) return rc;
+    rows_sum(G.Mh + l * Nd * H, H * d, false, G.dT + l * Nd, d, gWv, d, dvh, N, 1.f, H, d, dvh);
+    rows_sum(G.dQt + l * Nd * H, H * d, false, G.Q + l * Nd, d, gWk, d, dvh, N, p.inv_tau, H, d, dvh);
+    rows_sum(G.T + l * Nd, d, false, G.dQ + l * Nd, d, gWq, d, d, N, 1.f, 1, 0, 0);
+  }
+  return flush();
 }
 
 template <typename T>
@@ -1011,6 +1151,8 @@ int backward_t(const Plan& p, const T* items, const int32_t* lengths, const T* c
                float* dWq, float* dWk, float* dWv, float* dWg, char* ws, cudaStream_t st, bool tensor) {
   const int N = p.N, d = p.d, H = p.H, Lp = p.Lp, M = p.M, dqk = p.dqk, dvh = p.dvh, U = p.U, L = p.L;
   const size_t UL = (size_t)U * L;
+  if (!tensor && N > 0 && U > 0 && gsta_train_simt_supported(p))
+    return backward_simt<T>(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, Wg, dz, d_items, d_cands, dWq, dWk, dWv, dWg, ws, st);
   // (d_items: with candidates present its first matrix product writes every row, padding included)
   if (N == 0 || U == 0) LASER_CUDA_OK(cudaMemsetAsync(d_items, 0, UL * d * sizeof(float), st));
   LASER_CUDA_OK(cudaMemsetAsync(dWq, 0, (size_t)d * dqk * sizeof(float), st));
@@ -1144,19 +1286,7 @@ int backward_t(const Plan& p, const T* items, const int32_t* lengths, const T* c
     // (with the attention on the MMAs and at least one layer, dH' has arrived in bf16 already)
     BWD_OK(sta_bwd_mma(p, attn_mma && M > 0 ? nullptr : s.dHp, lengths, cand_offsets, s.dQf, s.dK, s.dV, mma_scratch, st));
   } else {
-    const int cps = (min(p.S, L) + kChunk - 1) / kChunk;
-    const int dqh = dqk / H;
-    const int variant = (dqh == 16 && dvh == 32) ? 2 : (dqh == 16 && dvh == 16) ? 1 : 0;   // register-resident head slices
-    const size_t step_floats = (size_t)kCandsPerStep * (dqk + d + H * 33);
-    const size_t smem = ((variant ? (size_t)kChunk * (dqk + 1) : 2 * (size_t)kChunk * (dqk + 1 + d + 1)) + step_floats) *
-                        sizeof(float);
-    if (smem > 200 * 1024 || (long long)Lp * cps > 0x7fffffffLL || U > 65535 || H > 32) return LASER_ERR_UNSUPPORTED;
-    auto kernel = variant == 2 ? sta_bwd_kernel<16, 32> : variant == 1 ? sta_bwd_kernel<16, 16> : sta_bwd_kernel<0, 0>;
-    LASER_CUDA_OK(allow_smem(kernel, smem));
-    LaunchScope ls("bwd_sta", st);
-    kernel<<<dim3(Lp * cps, U), 32 * H, smem, st>>>(Qf, Kf, Vf, s.dHp, lengths, cand_offsets, s.dQf, s.dK, s.dV, L, d, dqk,
-                                                    H, p.S, Lp, N, cps);
-    LASER_CUDA_OK(cudaGetLastError());
+    BWD_OK(launch_sta_bwd(p, Qf, Kf, Vf, s.dHp, lengths, cand_offsets, s.dQf, s.dK, s.dV, st));
   }
 
   // ---- backward through the projections (Qf = T W_q / gamma)

@@ -1,0 +1,36 @@
+// Interfaces between the source files of the backward pass.
+#pragma once
+
+#include "laser_common.cuh"
+
+namespace laser {
+
+// What the stacked-attention kernels leave for the weight gradients, per layer (l = 0 .. M - 1): the targets t_l, q, m_h,
+// and the gradients of t_{l+1}, q, qt_h; and, in dT0, the gradient of t_0.
+struct GstaTrain {
+  float *T, *Q, *dT, *dQ;         // [M, N, d]
+  float *Mh, *dQt;                // [M, N, H, d]
+  float* dT0;                     // [N, d]
+};
+
+// FP32 ALUs (laser_backward_simt.cu): recomputes the layers from the fp32 H' and runs them backward; writes every row of dHp.
+bool gsta_train_simt_supported(const Plan& p);
+int gsta_train_simt(const Plan& p, const float* Hp, const int32_t* lengths, const int32_t* cand_offsets, const void* cands,
+                    const void* Wg, const float* dz, const GstaTrain& G, float* dHp, cudaStream_t st);
+
+// A dense product on the FP32 ALUs: C[m][n] = D[m][n] + alpha (sum_k A(m, k) B(k, n) + sum_k A2(m, k) B2(k, n)), or, with
+// atomic, C += alpha A B in slices of the contraction.  A(m, k) = ta ? A[k lda + m] : A[m lda + k], B(k, n) = tb ?
+// B[n ldb + k] : B[k ldb + n] (A2, B2 alike); a16 / b16: bf16 operands.  `batch` products sa, sb, sc elements apart.
+struct Product {
+  const void *A, *B, *A2, *B2;
+  const float* D;
+  float* C;
+  int lda, ldb, lda2, ldb2, ldc, M, N, K, K2, batch, sa, sb, sc, k_per;
+  float alpha;
+  bool ta, tb, a16, b16, atomic;
+};
+constexpr int kMaxProducts = 24;
+// Independent products in as few launches as possible (k_per is filled in).
+int run_products(Product* list, int n, cudaStream_t st);
+
+}  // namespace laser

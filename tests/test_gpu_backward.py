@@ -22,6 +22,9 @@ CASES = [
     dict(U=2, C=9, L=40, d=32, H=2, S=8, M=0, dtype="f32", lengths=[40, 13]),              # no GSTA layer: z = t
     dict(U=3, C=130, L=512, d=64, H=4, S=64, M=2, dtype="bf16", lengths=[512, 300, 77]),   # serving-like, more rows
     dict(U=2, C=5, L=40, d=18, H=3, S=8, M=2, dtype="f32", lengths=[40, 21], d_qh=4),      # a width that is no multiple of 4
+    dict(U=3, C=399, L=48, d=32, H=2, S=16, M=2, dtype="f32", lengths=[48, 17, 33]),       # four candidates per attention block, a partial one
+    dict(U=1, C=6, L=30, d=64, H=4, S=7, M=7, dtype="f32", lengths=[30]),                  # more products than one launch takes
+    dict(U=2, C=3, L=33, d=256, H=4, S=16, M=1, dtype="f32", lengths=[33, 32], d_qh=16),   # as many columns as threads
 ]
 
 
