@@ -1079,6 +1079,65 @@ int zero_arrays(const ZeroList& Z, cudaStream_t st) {
   return LASER_OK;
 }
 
+// Products collected for as few launches as possible.
+template <typename T>
+struct ProductBatch {
+  static constexpr bool w16 = sizeof(T) == 2;
+  const Plan& p;
+  cudaStream_t st;
+  Product list[kMaxProducts];
+  int n = 0, rc = LASER_OK;
+  ProductBatch(const Plan& plan, cudaStream_t stream) : p(plan), st(stream) {}
+  int flush() {
+    if (rc == LASER_OK && n > 0) rc = run_products(list, n, st);
+    n = 0;
+    return rc;
+  }
+  void add(const Product& P) {
+    if (n == kMaxProducts) flush();
+    list[n++] = P;
+  }
+  // C[d x cols] += alpha A^T B over `rows` rows
+  void add_rows_sum(const void* A, int lda, bool a16, const float* B, int ldb, float* C, int ldc, int cols, int rows,
+                    float alpha, int batch, int sa, int sb) {
+    Product P = {};
+    P.A = A; P.lda = lda; P.ta = true; P.a16 = a16; P.B = B; P.ldb = ldb; P.C = C; P.ldc = ldc;
+    P.M = p.d; P.N = cols; P.K = rows; P.alpha = alpha; P.atomic = true; P.batch = batch; P.sa = sa; P.sb = sb; P.sc = sb;
+    add(P);
+  }
+  // d_items = dK W_k^T + dV W_v^T,  dW_k += X^T dK,  dW_v += X^T dV
+  void add_item_products(const T* items, const T* Wk, const T* Wv, const float* dK, const float* dV, float* d_items, float* dWk,
+                         float* dWv) {
+    const int d = p.d, dqk = p.dqk, UL = p.U * p.L;
+    Product P = {};
+    P.A = dK; P.lda = dqk; P.B = Wk; P.ldb = dqk; P.K = dqk; P.A2 = dV; P.lda2 = d; P.B2 = Wv; P.ldb2 = d; P.K2 = d;
+    P.tb = true; P.b16 = w16; P.C = d_items; P.ldc = d; P.M = UL; P.N = d; P.alpha = 1.f; P.batch = 1;
+    add(P);
+    add_rows_sum(items, d, w16, dK, dqk, dWk, dqk, dqk, UL, 1.f, 1, 0, 0);
+    add_rows_sum(items, d, w16, dV, d, dWv, d, d, UL, 1.f, 1, 0, 0);
+  }
+  // d_cands = dt_0 + dQf W_q^T / gamma,  dW_q += T^T dQf / gamma
+  void add_query_products(const T* cands, const T* Wq, const float* dQf, const float* dT0, float* d_cands, float* dWq) {
+    Product P = {};
+    P.A = dQf; P.lda = p.dqk; P.B = Wq; P.ldb = p.dqk; P.K = p.dqk; P.tb = true; P.b16 = w16; P.D = dT0; P.C = d_cands; P.ldc = p.d;
+    P.M = p.N; P.N = p.d; P.alpha = p.inv_gamma; P.batch = 1;
+    add(P);
+    add_rows_sum(cands, p.d, w16, dQf, p.dqk, dWq, p.dqk, p.dqk, p.N, p.inv_gamma, 1, 0, 0);
+  }
+  // the stacked attention's weight gradients, and the last launch
+  int finish(const GstaTrain& G, float* dWg) {
+    const int N = p.N, d = p.d, H = p.H, dvh = p.dvh;
+    const size_t Nd = (size_t)N * d, dd = (size_t)d * d;
+    for (int l = 0; l < p.M; ++l) {
+      float *gWq = dWg + (size_t)(l * 3) * dd, *gWk = gWq + dd, *gWv = gWk + dd;
+      add_rows_sum(G.Mh + l * Nd * H, H * d, false, G.dT + l * Nd, d, gWv, d, dvh, N, 1.f, H, d, dvh);
+      add_rows_sum(G.dQt + l * Nd * H, H * d, false, G.Q + l * Nd, d, gWk, d, dvh, N, p.inv_tau, H, d, dvh);
+      add_rows_sum(G.T + l * Nd, d, false, G.dQ + l * Nd, d, gWq, d, d, N, 1.f, 1, 0, 0);
+    }
+    return flush();
+  }
+};
+
 // FP32 ALUs throughout, M > 0: projections, segment sums, all layers of the stacked attention forward and backward, the
 // gates, and every dense product of the gradients in one launch.
 template <typename T>
@@ -1102,47 +1161,54 @@ int backward_simt(const Plan& p, const T* items, const int32_t* lengths, const T
   } else {
     BWD_OK(simt_sta_f32(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, s.Hp, ws, st));
   }
-  const size_t Nd = (size_t)N * d, dd = (size_t)d * d;
-  const GstaTrain G = {s.T, s.Q, s.dT, s.dQ, s.Mh, s.dQt, s.dT + M * Nd};
+  const GstaTrain G = {s.T, s.Q, s.dT, s.dQ, s.Mh, s.dQt, s.dT + M * (size_t)N * d};
   BWD_OK(gsta_train_simt(p, s.Hp, lengths, cand_offsets, cands, Wg, dz, G, s.dHp, st));
   BWD_OK(launch_sta_bwd(p, Qf, Kf, Vf, s.dHp, lengths, cand_offsets, s.dQf, s.dK, s.dV, st));
 #undef BWD_OK
-  constexpr bool w16 = sizeof(T) == 2;
-  Product list[kMaxProducts];
-  int n = 0;
-  auto flush = [&]() {
-    const int r = run_products(list, n, st);
-    n = 0;
-    return r;
-  };
-  auto rows_sum = [&](const void* A, int lda, bool a16, const float* B, int ldb, float* C, int ldc, int cols, int rows,
-                      float alpha, int batch, int sa, int sb) {      // C[d x cols] += alpha A^T B over the rows
-    Product P = {};
-    P.A = A; P.lda = lda; P.ta = true; P.a16 = a16; P.B = B; P.ldb = ldb; P.C = C; P.ldc = ldc;
-    P.M = d; P.N = cols; P.K = rows; P.alpha = alpha; P.atomic = true; P.batch = batch; P.sa = sa; P.sb = sb; P.sc = sb;
-    list[n++] = P;
-  };
+  ProductBatch<T> list(p, st);
+  list.add_item_products(items, Wk, Wv, s.dK, s.dV, d_items, dWk, dWv);
+  list.add_query_products(cands, Wq, s.dQf, G.dT0, d_cands, dWq);
+  return list.finish(G, dWg);
+}
+
+// One candidate per user (laser_backward_stream.cu), M > 0, the stacked attention on the tensor cores.
+template <typename T>
+int backward_stream_all(const Plan& p, const T* items, const int32_t* lengths, const T* cands, const int32_t* cand_offsets,
+                        const T* Wq, const T* Wk, const T* Wv, const T* Wg, const float* dz, float* d_items, float* d_cands,
+                        float* dWq, float* dWk, float* dWv, float* dWg, char* ws, cudaStream_t st) {
+  const int N = p.N, d = p.d, H = p.H, M = p.M, dqk = p.dqk, dqh = p.dqh;
+  const BwdScratch s = carve_scratch(p, ws + p.total);
+  char *stream_scratch = ws + p.total + s.total, *train_scratch = stream_scratch + backward_stream_scratch_bytes(p);
+  float* Qf = reinterpret_cast<float*>(ws + p.off_q);
+  int rc;
+#define BWD_OK(...) do { rc = (__VA_ARGS__); if (rc != LASER_OK) return rc; } while (0)
+  ZeroList Z = {};
+  Z.add(dWq, (size_t)d * dqk); Z.add(dWk, (size_t)d * dqk); Z.add(dWv, (size_t)d * d); Z.add(dWg, (size_t)M * 3 * d * d);
+  BWD_OK(zero_arrays(Z, st));
+  bf16 *Hhi = reinterpret_cast<bf16*>(s.Hp), *Hlo = Hhi + (size_t)N * p.Lp * d;
+  BWD_OK(backward_stream_forward(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, nullptr, Hhi, Hlo, ws, stream_scratch, st));
+  const GstaTrain G = {s.T, s.Q, s.dT, s.dQ, s.Mh, s.dQt, s.dT + M * (size_t)N * d};
+  BWD_OK(gsta_train(p, 2, Hhi, Hlo, lengths, cand_offsets, cands, Wg, dz, G, s.dHp, train_scratch, st));
+  const float* p_sums = nullptr;
+  BWD_OK(backward_stream(p, items, lengths, cand_offsets, Wv, s.dHp, d_items, dWv, &p_sums, ws, stream_scratch, st));
+#undef BWD_OK
+  // q / gamma, and d(q_h / gamma) = p_h W_k[:, h]; then everything that needs them
+  ProductBatch<T> first(p, st), list(p, st);
   {
-    Product P = {};                                                  // d_items = dK W_k^T + dV W_v^T
-    P.A = s.dK; P.lda = dqk; P.B = Wk; P.ldb = dqk; P.K = dqk; P.A2 = s.dV; P.lda2 = d; P.B2 = Wv; P.ldb2 = d; P.K2 = d;
-    P.tb = true; P.b16 = w16; P.C = d_items; P.ldc = d; P.M = UL; P.N = d; P.alpha = 1.f; P.batch = 1;
-    list[n++] = P;
-    P = Product{};                                                   // d_cands = dt_0 + dQf W_q^T / gamma
-    P.A = s.dQf; P.lda = dqk; P.B = Wq; P.ldb = dqk; P.K = dqk; P.tb = true; P.b16 = w16; P.D = G.dT0; P.C = d_cands; P.ldc = d;
-    P.M = N; P.N = d; P.alpha = p.inv_gamma; P.batch = 1;
-    list[n++] = P;
+    Product P = {};
+    P.A = cands; P.lda = d; P.a16 = sizeof(T) == 2; P.B = Wq; P.ldb = dqk; P.b16 = sizeof(T) == 2; P.C = Qf; P.ldc = dqk;
+    P.M = N; P.N = dqk; P.K = d; P.alpha = p.inv_gamma; P.batch = 1;
+    first.add(P);
+    P = Product{};
+    P.A = p_sums; P.lda = H * d; P.sa = d; P.B = Wk; P.ldb = dqk; P.sb = dqh; P.b16 = sizeof(T) == 2; P.C = s.dQf; P.ldc = dqk;
+    P.sc = dqh; P.M = N; P.N = dqh; P.K = d; P.alpha = 1.f; P.batch = H;
+    first.add(P);
   }
-  rows_sum(items, d, w16, s.dK, dqk, dWk, dqk, dqk, UL, 1.f, 1, 0, 0);
-  rows_sum(items, d, w16, s.dV, d, dWv, d, d, UL, 1.f, 1, 0, 0);
-  rows_sum(cands, d, w16, s.dQf, dqk, dWq, dqk, dqk, N, p.inv_gamma, 1, 0, 0);
-  for (int l = 0; l < M; ++l) {
-    float *gWq = dWg + (size_t)(l * 3) * dd, *gWk = gWq + dd, *gWv = gWk + dd;
-    if (n + 3 > kMaxProducts && (rc = flush()) != LASER_OK) return rc;
-    rows_sum(G.Mh + l * Nd * H, H * d, false, G.dT + l * Nd, d, gWv, d, dvh, N, 1.f, H, d, dvh);
-    rows_sum(G.dQt + l * Nd * H, H * d, false, G.Q + l * Nd, d, gWk, d, dvh, N, p.inv_tau, H, d, dvh);
-    rows_sum(G.T + l * Nd, d, false, G.dQ + l * Nd, d, gWq, d, d, N, 1.f, 1, 0, 0);
-  }
-  return flush();
+  if ((rc = first.flush()) != LASER_OK) return rc;
+  list.add_rows_sum(p_sums, H * d, false, Qf, dqk, dWk, dqk, dqh, N, 1.f, H, d, dqh);      // dW_k[:, h] += p_h^T q_h / gamma
+  list.add_query_products(cands, Wq, s.dQf, G.dT0, d_cands, dWq);
+  if ((rc = list.flush()) != LASER_OK) return rc;
+  return gsta_weight_sums(p, G, dWg, st);
 }
 
 template <typename T>
@@ -1153,6 +1219,8 @@ int backward_t(const Plan& p, const T* items, const int32_t* lengths, const T* c
   const size_t UL = (size_t)U * L;
   if (!tensor && N > 0 && U > 0 && gsta_train_simt_supported(p))
     return backward_simt<T>(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, Wg, dz, d_items, d_cands, dWq, dWk, dWv, dWg, ws, st);
+  if (tensor && N > 0 && U > 0 && backward_stream_supported(p) && gsta_train_supported(p, 2))
+    return backward_stream_all<T>(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, Wg, dz, d_items, d_cands, dWq, dWk, dWv, dWg, ws, st);
   // (d_items: with candidates present its first matrix product writes every row, padding included)
   if (N == 0 || U == 0) LASER_CUDA_OK(cudaMemsetAsync(d_items, 0, UL * d * sizeof(float), st));
   LASER_CUDA_OK(cudaMemsetAsync(dWq, 0, (size_t)d * dqk * sizeof(float), st));
@@ -1172,10 +1240,11 @@ int backward_t(const Plan& p, const T* items, const int32_t* lengths, const T* c
   char* mma_scratch = ws + p.total + s.total;
   const bool mma = tensor && sta_bwd_mma_supported(p);     // (users with very few candidates keep the FP32 gate kernels)
   const bool stream = tensor && backward_stream_supported(p);   // one candidate per user: no keys or values of the items
-  const bool attn_mma = mma && gsta_attn_mma_supported(p); // the recomputed GSTA attention on the MMAs as well
+  const bool train = mma && sta_fwd_mma_supported(p) && gsta_train_supported(p, 1);   // the stacked attention as well
+  char* train_scratch = mma_scratch + sta_bwd_mma_scratch_bytes(p);
   if (stream) {
     BWD_OK(gemm<T, T>(gx, N, dqk, d, cands, d, false, Wq, dqk, false, Qf, dqk, p.inv_gamma, false, false));
-    BWD_OK(backward_stream_forward(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, s.Hp, ws, mma_scratch, st));
+    BWD_OK(backward_stream_forward(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, s.Hp, nullptr, nullptr, ws, mma_scratch, st));
   } else if (tensor) {
     // (sta_fwd_mma writes every row of H' that is read later: all candidates of every non-empty segment)
     if (!(mma && sta_fwd_mma_supported(p))) LASER_CUDA_OK(cudaMemsetAsync(s.Hp, 0, (size_t)N * Lp * d * sizeof(float), st));
@@ -1196,7 +1265,7 @@ int backward_t(const Plan& p, const T* items, const int32_t* lengths, const T* c
       BWD_OK(gemm<T, T>(gx, (int)UL, d, d, items, d, false, Wv, d, false, Vf, d, 1.f, false, false));
     }
     if (mma) BWD_OK(sta_mma_operands(p, Qf, kv_ready ? nullptr : Kf, kv_ready ? nullptr : Vf, mma_scratch, st));
-    if (mma && sta_fwd_mma_supported(p)) BWD_OK(sta_fwd_mma(p, lengths, cand_offsets, attn_mma ? nullptr : s.Hp, attn_mma, mma_scratch, st));
+    if (mma && sta_fwd_mma_supported(p)) BWD_OK(sta_fwd_mma(p, lengths, cand_offsets, train ? nullptr : s.Hp, train, mma_scratch, st));
     else if (p.dqh == 16 && (dvh == 16 || dvh == 32 || dvh == 64) && p.H <= 32) BWD_OK(simt_attend_f32(p, lengths, cand_offsets, s.Hp, ws, st));
     else BWD_OK(simt_sta_f32(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, s.Hp, ws, st));
   } else if (p.dqh == 16 && (dvh == 16 || dvh == 32 || dvh == 64) && p.H <= 32) {
@@ -1206,66 +1275,72 @@ int backward_t(const Plan& p, const T* items, const int32_t* lengths, const T* c
     BWD_OK(simt_sta_f32(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, s.Hp, ws, st));
   }
   const size_t Nd = (size_t)N * d, NHd = Nd * H;
-  {
-    LaunchScope ls("bwd_to_f32", st);
-    to_f32_kernel<T><<<296, 256, 0, st>>>(cands, s.T, Nd);
-  }
-  constexpr int attn_warps = kAttnThreads / 32;
-  const size_t attn_smem_f = ((size_t)(1 + attn_warps) * H * d + (size_t)H * Lp) * sizeof(float);
-  const size_t attn_smem_b = ((size_t)(2 + attn_warps) * H * d + 2 * (size_t)H * Lp) * sizeof(float);
-  if (attn_smem_b > 200 * 1024) return LASER_ERR_UNSUPPORTED;
-  // 16-byte accesses when rows allow; heads in groups of four, two or one, whichever divides H
-  const bool v4 = d % 4 == 0;
-  auto attn_fwd = H % 4 == 0 ? (v4 ? gsta_attn_fwd_kernel<4, 4> : gsta_attn_fwd_kernel<1, 4>)
-                  : H % 2 == 0 ? (v4 ? gsta_attn_fwd_kernel<4, 2> : gsta_attn_fwd_kernel<1, 2>)
-                               : (v4 ? gsta_attn_fwd_kernel<4, 1> : gsta_attn_fwd_kernel<1, 1>);
-  auto attn_bwd = H % 4 == 0 ? (v4 ? gsta_attn_bwd_kernel<4, 4> : gsta_attn_bwd_kernel<1, 4>)
-                  : H % 2 == 0 ? (v4 ? gsta_attn_bwd_kernel<4, 2> : gsta_attn_bwd_kernel<1, 2>)
-                               : (v4 ? gsta_attn_bwd_kernel<4, 1> : gsta_attn_bwd_kernel<1, 1>);
-  LASER_CUDA_OK(allow_smem(attn_fwd, attn_smem_f));
-  LASER_CUDA_OK(allow_smem(attn_bwd, attn_smem_b));
-  for (int l = 0; l < M; ++l) {
-    const T *Wql = Wg + (size_t)(l * 3) * d * d, *Wkl = Wql + (size_t)d * d, *Wvl = Wkl + (size_t)d * d;
-    float *Tl = s.T + l * Nd, *Tn = Tl + Nd, *Ql = s.Q + l * Nd, *Qtl = s.Qt + l * NHd, *Al = s.A + (size_t)l * N * H * Lp,
-          *Ml = s.Mh + l * NHd;
-    BWD_OK(gemm<float, T>(gx, N, d, d, Tl, d, false, Wql, d, false, Ql, d, 1.f, false, false));
-    // Qt_h = Q_h W_k[:, h]^T / tau, every head
-    BWD_OK(gemm<float, T>(gx, N, d, dvh, Ql, d, false, Wkl, d, true, Qtl, H * d, p.inv_tau, false, false, H, dvh, dvh, d));
-    if (attn_mma) {
-      BWD_OK(gsta_attn_fwd_mma(p, Qtl, lengths, cand_offsets, Al, Ml, mma_scratch, st));
-    } else {
-      LaunchScope ls("bwd_attn_fwd", st);
-      attn_fwd<<<N, kAttnThreads, attn_smem_f, st>>>(s.Hp, Qtl, lengths, cand_offsets, Al, Ml, U, L, p.S, Lp,
-                                                                 H, d);
+  float* dT0 = s.dT;
+  if (train) {
+    bf16 *Hb, *dSb;
+    sta_mma_segment_arrays(p, mma_scratch, &Hb, &dSb);
+    const GstaTrain G = {s.T, s.Q, s.dT, s.dQ, s.Mh, s.dQt, s.dT + M * Nd};
+    dT0 = G.dT0;
+    BWD_OK(gsta_train(p, 1, Hb, nullptr, lengths, cand_offsets, cands, Wg, dz, G, dSb, train_scratch, st));
+    BWD_OK(gsta_weight_sums(p, G, dWg, st));
+  } else {
+    {
+      LaunchScope ls("bwd_to_f32", st);
+      to_f32_kernel<T><<<296, 256, 0, st>>>(cands, s.T, Nd);
     }
-    LASER_CUDA_OK(cudaMemcpyAsync(Tn, Tl, Nd * sizeof(float), cudaMemcpyDeviceToDevice, st));
-    // t += o,  o_h = m_h W_v[:, h], every head
-    BWD_OK(gemm<float, T>(gx, N, dvh, d, Ml, H * d, false, Wvl, d, false, Tn, d, 1.f, true, false, H, d, dvh, dvh));
-  }
+    constexpr int attn_warps = kAttnThreads / 32;
+    const size_t attn_smem_f = ((size_t)(1 + attn_warps) * H * d + (size_t)H * Lp) * sizeof(float);
+    const size_t attn_smem_b = ((size_t)(2 + attn_warps) * H * d + 2 * (size_t)H * Lp) * sizeof(float);
+    if (attn_smem_b > 200 * 1024) return LASER_ERR_UNSUPPORTED;
+    // 16-byte accesses when rows allow; heads in groups of four, two or one, whichever divides H
+    const bool v4 = d % 4 == 0;
+    auto attn_fwd = H % 4 == 0 ? (v4 ? gsta_attn_fwd_kernel<4, 4> : gsta_attn_fwd_kernel<1, 4>)
+                    : H % 2 == 0 ? (v4 ? gsta_attn_fwd_kernel<4, 2> : gsta_attn_fwd_kernel<1, 2>)
+                                 : (v4 ? gsta_attn_fwd_kernel<4, 1> : gsta_attn_fwd_kernel<1, 1>);
+    auto attn_bwd = H % 4 == 0 ? (v4 ? gsta_attn_bwd_kernel<4, 4> : gsta_attn_bwd_kernel<1, 4>)
+                    : H % 2 == 0 ? (v4 ? gsta_attn_bwd_kernel<4, 2> : gsta_attn_bwd_kernel<1, 2>)
+                                 : (v4 ? gsta_attn_bwd_kernel<4, 1> : gsta_attn_bwd_kernel<1, 1>);
+    LASER_CUDA_OK(allow_smem(attn_fwd, attn_smem_f));
+    LASER_CUDA_OK(allow_smem(attn_bwd, attn_smem_b));
+    for (int l = 0; l < M; ++l) {
+      const T *Wql = Wg + (size_t)(l * 3) * d * d, *Wkl = Wql + (size_t)d * d, *Wvl = Wkl + (size_t)d * d;
+      float *Tl = s.T + l * Nd, *Tn = Tl + Nd, *Ql = s.Q + l * Nd, *Qtl = s.Qt + l * NHd, *Al = s.A + (size_t)l * N * H * Lp,
+            *Ml = s.Mh + l * NHd;
+      BWD_OK(gemm<float, T>(gx, N, d, d, Tl, d, false, Wql, d, false, Ql, d, 1.f, false, false));
+      // Qt_h = Q_h W_k[:, h]^T / tau, every head
+      BWD_OK(gemm<float, T>(gx, N, d, dvh, Ql, d, false, Wkl, d, true, Qtl, H * d, p.inv_tau, false, false, H, dvh, dvh, d));
+      {
+        LaunchScope ls("bwd_attn_fwd", st);
+        attn_fwd<<<N, kAttnThreads, attn_smem_f, st>>>(s.Hp, Qtl, lengths, cand_offsets, Al, Ml, U, L, p.S, Lp,
+                                                                   H, d);
+      }
+      LASER_CUDA_OK(cudaMemcpyAsync(Tn, Tl, Nd * sizeof(float), cudaMemcpyDeviceToDevice, st));
+      // t += o,  o_h = m_h W_v[:, h], every head
+      BWD_OK(gemm<float, T>(gx, N, dvh, d, Ml, H * d, false, Wvl, d, false, Tn, d, 1.f, true, false, H, d, dvh, dvh));
+    }
 
-  // ---- backward through the GSTA layers
-  LASER_CUDA_OK(cudaMemcpyAsync(s.dT, dz, Nd * sizeof(float), cudaMemcpyDeviceToDevice, st));
-  if (M == 0) LASER_CUDA_OK(cudaMemsetAsync(s.dHp, 0, (size_t)N * Lp * d * sizeof(float), st));
-  for (int l = M - 1; l >= 0; --l) {
-    const T *Wql = Wg + (size_t)(l * 3) * d * d, *Wkl = Wql + (size_t)d * d, *Wvl = Wkl + (size_t)d * d;
-    float *Tl = s.T + l * Nd, *Ql = s.Q + l * Nd, *Qtl = s.Qt + l * NHd, *Al = s.A + (size_t)l * N * H * Lp,
-          *Ml = s.Mh + l * NHd;
-    float *gWq = dWg + (size_t)(l * 3) * d * d, *gWk = gWq + (size_t)d * d, *gWv = gWk + (size_t)d * d;
-    // dW_v[:, h] += m_h^T do_h;  dm_h = do_h W_v[:, h]^T, every head
-    BWD_OK(gemm<float, float>(gx, d, dvh, N, Ml, H * d, true, s.dT, d, false, gWv, d, 1.f, true, true, H, d, dvh, dvh));
-    BWD_OK(gemm<float, T>(gx, N, d, dvh, s.dT, d, false, Wvl, d, true, s.dM, H * d, 1.f, false, false, H, dvh, dvh, d));
-    if (attn_mma) {
-      BWD_OK(gsta_attn_bwd_mma(p, Qtl, Al, s.dM, lengths, cand_offsets, s.dQt, s.dHp, l == M - 1, l == 0, mma_scratch, st));
-    } else {
-      LaunchScope ls("bwd_attn_bwd", st);
-      attn_bwd<<<N, kAttnThreads, attn_smem_b, st>>>(s.Hp, Qtl, Al, s.dM, lengths, cand_offsets, s.dQt, s.dHp,
-                                                                 U, L, p.S, Lp, H, d, l == M - 1 ? 1 : 0);
+    // ---- backward through the GSTA layers
+    LASER_CUDA_OK(cudaMemcpyAsync(s.dT, dz, Nd * sizeof(float), cudaMemcpyDeviceToDevice, st));
+    if (M == 0) LASER_CUDA_OK(cudaMemsetAsync(s.dHp, 0, (size_t)N * Lp * d * sizeof(float), st));
+    for (int l = M - 1; l >= 0; --l) {
+      const T *Wql = Wg + (size_t)(l * 3) * d * d, *Wkl = Wql + (size_t)d * d, *Wvl = Wkl + (size_t)d * d;
+      float *Tl = s.T + l * Nd, *Ql = s.Q + l * Nd, *Qtl = s.Qt + l * NHd, *Al = s.A + (size_t)l * N * H * Lp,
+            *Ml = s.Mh + l * NHd;
+      float *gWq = dWg + (size_t)(l * 3) * d * d, *gWk = gWq + (size_t)d * d, *gWv = gWk + (size_t)d * d;
+      // dW_v[:, h] += m_h^T do_h;  dm_h = do_h W_v[:, h]^T, every head
+      BWD_OK(gemm<float, float>(gx, d, dvh, N, Ml, H * d, true, s.dT, d, false, gWv, d, 1.f, true, true, H, d, dvh, dvh));
+      BWD_OK(gemm<float, T>(gx, N, d, dvh, s.dT, d, false, Wvl, d, true, s.dM, H * d, 1.f, false, false, H, dvh, dvh, d));
+      {
+        LaunchScope ls("bwd_attn_bwd", st);
+        attn_bwd<<<N, kAttnThreads, attn_smem_b, st>>>(s.Hp, Qtl, Al, s.dM, lengths, cand_offsets, s.dQt, s.dHp,
+                                                                   U, L, p.S, Lp, H, d, l == M - 1 ? 1 : 0);
+      }
+      // dQ_h = dQt_h W_k[:, h] / tau;  dW_k[:, h] += dQt_h^T Q_h / tau, every head
+      BWD_OK(gemm<float, T>(gx, N, dvh, d, s.dQt, H * d, false, Wkl, d, false, s.dQ, d, p.inv_tau, false, false, H, d, dvh, dvh));
+      BWD_OK(gemm<float, float>(gx, d, dvh, N, s.dQt, H * d, true, Ql, d, false, gWk, d, p.inv_tau, true, true, H, d, dvh, dvh));
+      BWD_OK(gemm<float, float>(gx, d, d, N, Tl, d, true, s.dQ, d, false, gWq, d, 1.f, true, true));        // dW_q += T^T dQ
+      BWD_OK(gemm<float, T>(gx, N, d, d, s.dQ, d, false, Wql, d, true, s.dT, d, 1.f, true, false));            // dT += dQ W_q^T
     }
-    // dQ_h = dQt_h W_k[:, h] / tau;  dW_k[:, h] += dQt_h^T Q_h / tau, every head
-    BWD_OK(gemm<float, T>(gx, N, dvh, d, s.dQt, H * d, false, Wkl, d, false, s.dQ, d, p.inv_tau, false, false, H, d, dvh, dvh));
-    BWD_OK(gemm<float, float>(gx, d, dvh, N, s.dQt, H * d, true, Ql, d, false, gWk, d, p.inv_tau, true, true, H, d, dvh, dvh));
-    BWD_OK(gemm<float, float>(gx, d, d, N, Tl, d, true, s.dQ, d, false, gWq, d, 1.f, true, true));        // dW_q += T^T dQ
-    BWD_OK(gemm<float, T>(gx, N, d, d, s.dQ, d, false, Wql, d, true, s.dT, d, 1.f, true, false));            // dT += dQ W_q^T
   }
 
   // ---- backward through the segment aggregation and the gates
@@ -1283,22 +1358,21 @@ int backward_t(const Plan& p, const T* items, const int32_t* lengths, const T* c
   }
   if (stream) {
   } else if (mma) {
-    // (with the attention on the MMAs and at least one layer, dH' has arrived in bf16 already)
-    BWD_OK(sta_bwd_mma(p, attn_mma && M > 0 ? nullptr : s.dHp, lengths, cand_offsets, s.dQf, s.dK, s.dV, mma_scratch, st));
+    BWD_OK(sta_bwd_mma(p, train ? nullptr : s.dHp, lengths, cand_offsets, s.dQf, s.dK, s.dV, mma_scratch, st));
   } else {
     BWD_OK(launch_sta_bwd(p, Qf, Kf, Vf, s.dHp, lengths, cand_offsets, s.dQf, s.dK, s.dV, st));
   }
 
   // ---- backward through the projections (Qf = T W_q / gamma)
   BWD_OK(gemm<T, float>(gx, d, dqk, N, cands, d, true, s.dQf, dqk, false, dWq, dqk, p.inv_gamma, true, true));
-  BWD_OK(gemm<float, T>(gx, N, d, dqk, s.dQf, dqk, false, Wq, dqk, true, s.dT, d, p.inv_gamma, true, false));
+  BWD_OK(gemm<float, T>(gx, N, d, dqk, s.dQf, dqk, false, Wq, dqk, true, dT0, d, p.inv_gamma, true, false));
   if (!stream) {
     BWD_OK(gemm<T, float>(gx, d, dqk, (int)UL, items, d, true, s.dK, dqk, false, dWk, dqk, 1.f, true, true));
     BWD_OK(gemm<T, float>(gx, d, d, (int)UL, items, d, true, s.dV, d, false, dWv, d, 1.f, true, true));
     BWD_OK(gemm<float, T>(gx, (int)UL, d, dqk, s.dK, dqk, false, Wk, dqk, true, d_items, d, 1.f, false, false));
     BWD_OK(gemm<float, T>(gx, (int)UL, d, d, s.dV, d, false, Wv, d, true, d_items, d, 1.f, true, false));
   }
-  LASER_CUDA_OK(cudaMemcpyAsync(d_cands, s.dT, Nd * sizeof(float), cudaMemcpyDeviceToDevice, st));
+  LASER_CUDA_OK(cudaMemcpyAsync(d_cands, dT0, Nd * sizeof(float), cudaMemcpyDeviceToDevice, st));
 #undef BWD_OK
   LASER_CUDA_OK(cudaGetLastError());
   return LASER_OK;
@@ -1306,7 +1380,10 @@ int backward_t(const Plan& p, const T* items, const int32_t* lengths, const T* c
 
 }  // namespace
 
-size_t backward_scratch_bytes(const Plan& p) { return carve_scratch(p, nullptr).total + sta_bwd_mma_scratch_bytes(p) + backward_stream_scratch_bytes(p); }
+size_t backward_scratch_bytes(const Plan& p) {
+  return carve_scratch(p, nullptr).total + sta_bwd_mma_scratch_bytes(p) + backward_stream_scratch_bytes(p) +
+         std::max(gsta_train_scratch_bytes(p, 1), gsta_train_scratch_bytes(p, 2));
+}
 
 bool backward_tensor_supported(const Plan& p) { return p.dtype == LASER_BF16; }
 

@@ -18,6 +18,15 @@ bool gsta_train_simt_supported(const Plan& p);
 int gsta_train_simt(const Plan& p, const float* Hp, const int32_t* lengths, const int32_t* cand_offsets, const void* cands,
                     const void* Wg, const float* dz, const GstaTrain& G, float* dHp, cudaStream_t st);
 
+// Tensor cores (laser_backward_gsta.cu), bf16 inputs: np = 1: segment vectors S0 in bf16, dS [N, Lp, d] leaves as bf16;
+// np = 2: segment vectors S0 + S1 (bf16 high and low parts of fp32 values), dS leaves as fp32.  Rows of empty segments are
+// neither read nor written.  gsta_weight_sums adds the layers' weight gradients from what gsta_train left in G.
+bool gsta_train_supported(const Plan& p, int np);
+size_t gsta_train_scratch_bytes(const Plan& p, int np);
+int gsta_train(const Plan& p, int np, const void* S0, const void* S1, const int32_t* lengths, const int32_t* cand_offsets,
+               const void* cands, const void* Wg, const float* dz, const GstaTrain& G, void* dS, char* scratch, cudaStream_t st);
+int gsta_weight_sums(const Plan& p, const GstaTrain& G, float* dWg, cudaStream_t st);
+
 // A dense product on the FP32 ALUs: C[m][n] = D[m][n] + alpha (sum_k A(m, k) B(k, n) + sum_k A2(m, k) B2(k, n)), or, with
 // atomic, C += alpha A B in slices of the contraction.  A(m, k) = ta ? A[k lda + m] : A[m lda + k], B(k, n) = tb ?
 // B[n ldb + k] : B[k ldb + n] (A2, B2 alike); a16 / b16: bf16 operands.  `batch` products sa, sb, sc elements apart.

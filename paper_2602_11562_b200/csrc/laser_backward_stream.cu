@@ -44,7 +44,8 @@ struct BsParams {
   const bf16 *items, *Wv;
   const int *lengths, *cand_offsets, *order;
   const float* u;                  // [U, H, d]
-  float *r, *s, *y, *p;            // [N, Lp, H, d], [N, Lp, d], [N, Lp, H, d], [N, H, d]
+  float *r, *s, *y, *p;            // [N, Lp, H, d], [N, Lp, d] (null: s_hi, s_lo), [N, Lp, H, d], [N, H, d]
+  bf16 *s_hi, *s_lo;               // H' as bf16 high and low parts, [N, Lp, d] each, instead of s
   const float* ds;                 // [N, Lp, d]
   float *d_items, *dWv;
   int* status;
@@ -253,6 +254,17 @@ __global__ void __launch_bounds__(256) bs_rows_kernel(BsParams P, int to_y) {
 #pragma unroll
       for (int j = 0; j < 2 * D16; ++j) {
         if (j >= 2 * NP) break;
+        if (!to_y && !P.s) {
+#pragma unroll
+          for (int hf = 0; hf < 2; ++hf)
+            if (g + 8 * hf < rows) {
+              const size_t at = (row0 + g + 8 * hf) * d + h * dvh + j * 8 + 2 * t;
+              const uint32_t hi = pack2(acc[j][2 * hf], acc[j][2 * hf + 1]);
+              *reinterpret_cast<uint32_t*>(P.s_hi + at) = hi;
+              *reinterpret_cast<uint32_t*>(P.s_lo + at) = pack2(acc[j][2 * hf] - bf16_lo(hi), acc[j][2 * hf + 1] - bf16_hi(hi));
+            }
+          continue;
+        }
         if (g < rows) *reinterpret_cast<float2*>(C + g * ldc + j * 8 + 2 * t) = make_float2(acc[j][0], acc[j][1]);
         if (g + 8 < rows) *reinterpret_cast<float2*>(C + (g + 8) * ldc + j * 8 + 2 * t) = make_float2(acc[j][2], acc[j][3]);
       }
@@ -651,13 +663,13 @@ size_t backward_stream_scratch_bytes(const Plan& p) { return backward_stream_sup
   }
 
 int backward_stream_forward(const Plan& p, const void* items, const int32_t* lengths, const void* cands,
-                            const int32_t* cand_offsets, const void* Wq, const void* Wk, const void* Wv, float* Hp, char* ws,
-                            char* scratch, cudaStream_t st) {
+                            const int32_t* cand_offsets, const void* Wq, const void* Wk, const void* Wv, float* Hp,
+                            __nv_bfloat16* Hp_hi, __nv_bfloat16* Hp_lo, char* ws, char* scratch, cudaStream_t st) {
   const BsScratch s = carve_bs(p, scratch);
   const int rc = stream_fold(p, lengths, cands, cand_offsets, Wq, Wk, Wv, s.u, s.fold, reinterpret_cast<int*>(ws + p.off_status), st);
   if (rc != LASER_OK) return rc;
   BsParams P = bs_params(p, s, items, lengths, cand_offsets, Wv, ws);
-  P.s = Hp;
+  P.s = Hp; P.s_hi = Hp_hi; P.s_lo = Hp_lo;
   LASER_BS_DISPATCH(bs_forward_t, p, P, st)
 }
 

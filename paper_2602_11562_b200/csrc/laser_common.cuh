@@ -100,19 +100,10 @@ int sta_mma_operands(const Plan& p, const float* Qf, const float* Kf, const floa
 // The bf16 K [U L, d_qk] and V [U L, d] arrays inside `scratch`, for a producer that writes them directly (it then passes
 // Kf = Vf = null to sta_mma_operands).
 void sta_mma_operand_arrays(const Plan& p, char* scratch, __nv_bfloat16** Kb, __nv_bfloat16** Vb);
+// The bf16 H' that sta_fwd_mma leaves (bf16_copy) and the bf16 dH' that sta_bwd_mma reads, [N, L', d] each.
+void sta_mma_segment_arrays(const Plan& p, char* scratch, __nv_bfloat16** Hb, __nv_bfloat16** dSb);
 int sta_fwd_mma(const Plan& p, const int32_t* lengths, const int32_t* cand_offsets, float* Hp, bool bf16_copy, char* scratch,
                 cudaStream_t st);
-// The attention of a recomputed GSTA layer on the bf16 copy of H' that sta_fwd_mma keeps (bf16_copy): writes the weights
-// Aw [N, H, Lp] and the weighted sums Mh [N, H, d] (fp32) from Qt [N, H, d].
-bool gsta_attn_mma_supported(const Plan& p);
-int gsta_attn_fwd_mma(const Plan& p, const float* Qt, const int32_t* lengths, const int32_t* cand_offsets, float* Aw,
-                      float* Mh, char* scratch, cudaStream_t st);
-// Its backward: dQt [N, H, d] from Qt, Aw and dM [N, H, d]; dHp [N, Lp, d] written (overwrite) or added to; for the
-// layer processed last the sum leaves as the bf16 array sta_bwd_mma reads (which then takes dHp = null) and dHp stays
-// as it was.
-int gsta_attn_bwd_mma(const Plan& p, const float* Qt, const float* Aw, const float* dM, const int32_t* lengths,
-                      const int32_t* cand_offsets, float* dQt, float* dHp, bool overwrite, bool last, char* scratch,
-                      cudaStream_t st);
 int sta_bwd_mma(const Plan& p, const float* dHp, const int32_t* lengths, const int32_t* cand_offsets, float* dQf,
                 float* dK, float* dV, char* scratch, cudaStream_t st);
 
@@ -154,14 +145,14 @@ const int* stream_fold_order(const Plan& p, const char* scratch);   // null: ind
 int stream_fold(const Plan& p, const int32_t* lengths, const void* cands, const int32_t* cand_offsets, const void* Wq,
                 const void* Wk, const void* Wv, float* u, char* scratch, int* status, cudaStream_t st);
 
-// Backward pass of batches with at most one candidate per user (laser_backward_stream.cu).  _forward recomputes H' (fp32,
-// rows of non-empty segments only); the other writes every row of d_items, adds to dWv and leaves
+// Backward pass of batches with at most one candidate per user (laser_backward_stream.cu).  _forward recomputes H' (fp32, or,
+// with Hp null, its bf16 high and low parts; rows of non-empty segments only); the other writes every row of d_items, adds to dWv and leaves
 // p_h = sum_n de_{n,h} x_n, from which the gradients of the query side and of W_k follow, in *p_sums [N, H, d].
 bool backward_stream_supported(const Plan& p);
 size_t backward_stream_scratch_bytes(const Plan& p);
 int backward_stream_forward(const Plan& p, const void* items, const int32_t* lengths, const void* cands,
-                            const int32_t* cand_offsets, const void* Wq, const void* Wk, const void* Wv, float* Hp, char* ws,
-                            char* scratch, cudaStream_t st);
+                            const int32_t* cand_offsets, const void* Wq, const void* Wk, const void* Wv, float* Hp,
+                            __nv_bfloat16* Hp_hi, __nv_bfloat16* Hp_lo, char* ws, char* scratch, cudaStream_t st);
 int backward_stream(const Plan& p, const void* items, const int32_t* lengths, const int32_t* cand_offsets, const void* Wv,
                     const float* dHp, float* d_items, float* dWv, const float** p_sums, char* ws, char* scratch,
                     cudaStream_t st);

@@ -93,6 +93,8 @@ TENSOR_CASES = [
     dict(U=1, C=70, L=96, d=16, H=1, S=96, M=3, dtype="bf16", lengths=[90]),               # one head, one segment
     dict(U=3, C=9, L=64, d=64, H=2, S=16, M=1, dtype="bf16", lengths=[64, 1, 0], d_qh=32), # d_qh = 32, fewer than 16 candidates
     dict(U=2, C=300, L=128, d=128, H=8, S=32, M=2, dtype="bf16", lengths=[128, 100]),      # eight heads, many candidate tiles
+    dict(U=2, C=21, L=170, d=96, H=6, S=10, M=3, dtype="bf16", lengths=[170, 161]),        # 36 slots in the attention kernel, 17 segments
+    dict(U=3, C=800, L=60, d=32, H=2, S=20, M=1, dtype="bf16", lengths=[60, 19, 0]),       # 16 candidates per attention block, an empty user
 ]
 
 
@@ -173,6 +175,8 @@ STREAM_CASES = [
     dict(U=3, C=1, L=1100, d=128, H=8, S=17, M=1, dtype="bf16", lengths=[1100, 1099, 16]),
     dict(U=2, C=1, L=400, d=96, H=3, S=10, M=2, dtype="bf16", lengths=[400, 211]),
     dict(U=640, C=1, L=40, d=64, H=2, S=10, M=2, dtype="bf16"),
+    dict(U=7, C=1, L=330, d=128, H=8, S=10, M=3, dtype="bf16"),                              # 48 slots, three staging buffers
+    dict(U=3000, C=1, L=24, d=32, H=1, S=8, M=1, dtype="bf16"),                              # 16 candidates per attention block
 ]
 
 
