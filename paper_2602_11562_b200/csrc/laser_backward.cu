@@ -1211,6 +1211,39 @@ int backward_stream_all(const Plan& p, const T* items, const int32_t* lengths, c
   return gsta_weight_sums(p, G, dWg, st);
 }
 
+// Candidate lists, bf16, M > 0: gates, stacked attention and every product over the item rows on the MMAs.
+bool backward_lists_supported(const Plan& p) {
+  return sta_bwd_mma_supported(p) && sta_fwd_mma_supported(p) && gsta_train_supported(p, 1) && rows_mma_supported(p);
+}
+int backward_lists(const Plan& p, const bf16* items, const int32_t* lengths, const bf16* cands, const int32_t* cand_offsets,
+                   const bf16* Wq, const bf16* Wk, const bf16* Wv, const bf16* Wg, const float* dz, float* d_items,
+                   float* d_cands, float* dWq, float* dWk, float* dWv, float* dWg, char* ws, cudaStream_t st) {
+  const size_t N = p.N, d = p.d, M = p.M, dqk = p.dqk, UL = (size_t)p.U * p.L;
+  const BwdScratch s = carve_scratch(p, ws + p.total);
+  char *mma_scratch = ws + p.total + s.total, *train_scratch = mma_scratch + sta_bwd_mma_scratch_bytes(p);
+  bf16 *Qb, *Kb, *Vb, *Hb, *dSb;
+  sta_mma_operand_arrays(p, mma_scratch, &Qb, &Kb, &Vb);
+  sta_mma_segment_arrays(p, mma_scratch, &Hb, &dSb);
+  bf16 *dKh = reinterpret_cast<bf16*>(s.dK), *dKl = dKh + UL * dqk, *dVh = reinterpret_cast<bf16*>(s.dV), *dVl = dVh + UL * d;
+  const GstaTrain G = {s.T, s.Q, s.dT, s.dQ, s.Mh, s.dQt, s.dT + M * N * d};
+  int rc;
+#define BWD_OK(...) do { rc = (__VA_ARGS__); if (rc != LASER_OK) return rc; } while (0)
+  ZeroList Z = {};
+  Z.add(dWq, d * dqk); Z.add(dWk, d * dqk); Z.add(dWv, d * d); Z.add(dWg, M * 3 * d * d); Z.add(s.dQf, N * dqk);
+  BWD_OK(zero_arrays(Z, st));
+  BWD_OK(rows_project_cands(p, cands, Wq, 0.5f * p.inv_gamma, Qb, st));
+  BWD_OK(rows_project_items(p, items, lengths, cand_offsets, Wk, Wv, Kb, Vb, st));
+  BWD_OK(sta_fwd_mma(p, lengths, cand_offsets, nullptr, true, mma_scratch, st));
+  BWD_OK(gsta_train(p, 1, Hb, nullptr, lengths, cand_offsets, cands, Wg, dz, G, dSb, train_scratch, st));
+  BWD_OK(gsta_weight_sums(p, G, dWg, st));
+  BWD_OK(sta_bwd_mma_split(p, lengths, cand_offsets, s.dQf, dKh, dKl, dVh, dVl, mma_scratch, st));
+  BWD_OK(rows_gradients(p, items, lengths, cand_offsets, Wk, Wv, dKh, dKl, dVh, dVl, d_items, dWk, dWv, st));
+#undef BWD_OK
+  ProductBatch<bf16> list(p, st);
+  list.add_query_products(cands, Wq, s.dQf, G.dT0, d_cands, dWq);
+  return list.flush();
+}
+
 template <typename T>
 int backward_t(const Plan& p, const T* items, const int32_t* lengths, const T* cands, const int32_t* cand_offsets,
                const T* Wq, const T* Wk, const T* Wv, const T* Wg, const float* dz, float* d_items, float* d_cands,
@@ -1221,6 +1254,10 @@ int backward_t(const Plan& p, const T* items, const int32_t* lengths, const T* c
     return backward_simt<T>(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, Wg, dz, d_items, d_cands, dWq, dWk, dWv, dWg, ws, st);
   if (tensor && N > 0 && U > 0 && backward_stream_supported(p) && gsta_train_supported(p, 2))
     return backward_stream_all<T>(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, Wg, dz, d_items, d_cands, dWq, dWk, dWv, dWg, ws, st);
+  if constexpr (sizeof(T) == 2) {
+    if (tensor && N > 0 && U > 0 && backward_lists_supported(p))
+      return backward_lists(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, Wg, dz, d_items, d_cands, dWq, dWk, dWv, dWg, ws, st);
+  }
   // (d_items: with candidates present its first matrix product writes every row, padding included)
   if (N == 0 || U == 0) LASER_CUDA_OK(cudaMemsetAsync(d_items, 0, UL * d * sizeof(float), st));
   LASER_CUDA_OK(cudaMemsetAsync(dWq, 0, (size_t)d * dqk * sizeof(float), st));
@@ -1253,8 +1290,8 @@ int backward_t(const Plan& p, const T* items, const int32_t* lengths, const T* c
     // K and V: as bf16 straight into the MMA kernels' operand arrays when nothing reads them in fp32
     bool kv_ready = false;
     if (mma && sta_fwd_mma_supported(p)) {
-      bf16 *Kb, *Vb;
-      sta_mma_operand_arrays(p, mma_scratch, &Kb, &Vb);
+      bf16 *Qb, *Kb, *Vb;
+      sta_mma_operand_arrays(p, mma_scratch, &Qb, &Kb, &Vb);
       const int r1 = gemm_rows_bf16<T, T>(gx, (int)UL, dqk, d, items, d, Wk, dqk, Kb, dqk);
       const int r2 = r1 == LASER_OK ? gemm_rows_bf16<T, T>(gx, (int)UL, d, d, items, d, Wv, d, Vb, d) : r1;
       if (r2 != LASER_OK && r2 != LASER_ERR_UNSUPPORTED) return r2;

@@ -27,6 +27,17 @@ int gsta_train(const Plan& p, int np, const void* S0, const void* S1, const int3
                const void* cands, const void* Wg, const float* dz, const GstaTrain& G, void* dS, char* scratch, cudaStream_t st);
 int gsta_weight_sums(const Plan& p, const GstaTrain& G, float* dWg, cudaStream_t st);
 
+// Products over the item rows on the tensor cores (laser_backward_rows.cu), users' valid rows only, bf16 inputs: K and V (or
+// scale Q of the candidates) as bf16; every row of d_items (zeros for padding) and the sums into dWk, dWv from dK and dV
+// given as bf16 high and low parts.
+bool rows_mma_supported(const Plan& p);
+int rows_project_items(const Plan& p, const void* items, const int32_t* lengths, const int32_t* cand_offsets, const void* Wk,
+                       const void* Wv, __nv_bfloat16* Kb, __nv_bfloat16* Vb, cudaStream_t st);
+int rows_project_cands(const Plan& p, const void* cands, const void* Wq, float scale, __nv_bfloat16* Qb, cudaStream_t st);
+int rows_gradients(const Plan& p, const void* items, const int32_t* lengths, const int32_t* cand_offsets, const void* Wk,
+                   const void* Wv, const __nv_bfloat16* dK_hi, const __nv_bfloat16* dK_lo, const __nv_bfloat16* dV_hi,
+                   const __nv_bfloat16* dV_lo, float* d_items, float* dWk, float* dWv, cudaStream_t st);
+
 // A dense product on the FP32 ALUs: C[m][n] = D[m][n] + alpha (sum_k A(m, k) B(k, n) + sum_k A2(m, k) B2(k, n)), or, with
 // atomic, C += alpha A B in slices of the contraction.  A(m, k) = ta ? A[k lda + m] : A[m lda + k], B(k, n) = tb ?
 // B[n ldb + k] : B[k ldb + n] (A2, B2 alike); a16 / b16: bf16 operands.  `batch` products sa, sb, sc elements apart.

@@ -51,6 +51,7 @@ struct BwdMmaParams {
   const bf16 *Qb, *Kb, *Vb, *dSb;
   const int32_t *lengths, *cand_offsets;
   float *dQf, *dK, *dV;
+  bf16 *dKh, *dKl, *dVh, *dVl;                   // non-null: dK and dV leave as bf16 high and low parts instead
   int L, d, dqk, H, S, Lp, N, R, jobs;           // R item tiles per segment, jobs = Lp R H per user
 };
 
@@ -264,23 +265,31 @@ __global__ void __launch_bounds__(kBwdWarps * 32, 2) sta_bwd_mma_kernel(const Bw
     __syncwarp();                        // every lane is done with this buffer before the next request overwrites it
   }
 
-  // ---- this job's rows of dK and dV (valid rows only; the others keep the zeros the caller put there)
-  float* dKr = P.dK + ((size_t)u * P.L + n0) * dqk + h * DQH;
-  float* dVr = P.dV + ((size_t)u * P.L + n0) * d + h * DVH;
+  // ---- this job's rows of dK and dV (valid rows only; the others keep what the caller put there)
+  const size_t k_at = ((size_t)u * P.L + n0) * dqk + h * DQH, v_at = ((size_t)u * P.L + n0) * d + h * DVH;
+  auto put = [&](float* f, bf16* hi, bf16* lo, size_t at, float x0, float x1) {
+    if (hi) {
+      const uint32_t a = pack2(x0, x1);
+      *reinterpret_cast<uint32_t*>(hi + at) = a;
+      *reinterpret_cast<uint32_t*>(lo + at) = pack2(x0 - bf16_lo(a), x1 - bf16_hi(a));
+    } else {
+      *reinterpret_cast<float2*>(f + at) = make_float2(x0, x1);
+    }
+  };
 #pragma unroll
   for (int mt = 0; mt < MT; ++mt) {
     const int r0 = mt * 16 + g, r1 = r0 + 8;
 #pragma unroll
     for (int j = 0; j < 2 * DQ16; ++j) {
       const int c = j * 8 + 2 * t;
-      if (r0 < cnt) *reinterpret_cast<float2*>(dKr + (size_t)r0 * dqk + c) = make_float2(0.5f * dKacc[mt][j][0], 0.5f * dKacc[mt][j][1]);
-      if (r1 < cnt) *reinterpret_cast<float2*>(dKr + (size_t)r1 * dqk + c) = make_float2(0.5f * dKacc[mt][j][2], 0.5f * dKacc[mt][j][3]);
+      if (r0 < cnt) put(P.dK, P.dKh, P.dKl, k_at + (size_t)r0 * dqk + c, 0.5f * dKacc[mt][j][0], 0.5f * dKacc[mt][j][1]);
+      if (r1 < cnt) put(P.dK, P.dKh, P.dKl, k_at + (size_t)r1 * dqk + c, 0.5f * dKacc[mt][j][2], 0.5f * dKacc[mt][j][3]);
     }
 #pragma unroll
     for (int j = 0; j < 2 * DV16; ++j) {
       const int c = j * 8 + 2 * t;
-      if (r0 < cnt) *reinterpret_cast<float2*>(dVr + (size_t)r0 * d + c) = make_float2(dVacc[mt][j][0], dVacc[mt][j][1]);
-      if (r1 < cnt) *reinterpret_cast<float2*>(dVr + (size_t)r1 * d + c) = make_float2(dVacc[mt][j][2], dVacc[mt][j][3]);
+      if (r0 < cnt) put(P.dV, P.dVh, P.dVl, v_at + (size_t)r0 * d + c, dVacc[mt][j][0], dVacc[mt][j][1]);
+      if (r1 < cnt) put(P.dV, P.dVh, P.dVl, v_at + (size_t)r1 * d + c, dVacc[mt][j][2], dVacc[mt][j][3]);
     }
   }
 }
@@ -479,8 +488,9 @@ int sta_mma_operands(const Plan& p, const float* Qf, const float* Kf, const floa
   return Vf ? cast(Vf, s.Vb, UL * p.d, 1.f, st) : (int)LASER_OK;
 }
 
-void sta_mma_operand_arrays(const Plan& p, char* scratch, __nv_bfloat16** Kb, __nv_bfloat16** Vb) {
+void sta_mma_operand_arrays(const Plan& p, char* scratch, __nv_bfloat16** Qb, __nv_bfloat16** Kb, __nv_bfloat16** Vb) {
   const MmaScratch s = carve_mma(p, scratch);
+  *Qb = s.Qb;
   *Kb = s.Kb;
   *Vb = s.Vb;
 }
@@ -516,17 +526,14 @@ int sta_fwd_mma(const Plan& p, const int32_t* lengths, const int32_t* cand_offse
   return LASER_ERR_UNSUPPORTED;
 }
 
-int sta_bwd_mma(const Plan& p, const float* dHp, const int32_t* lengths, const int32_t* cand_offsets, float* dQf,
-                float* dK, float* dV, char* scratch, cudaStream_t st) {
+static int run_bwd_mma(const Plan& p, BwdMmaParams P, const int32_t* lengths, const int32_t* cand_offsets, float* dQf,
+                       char* scratch, cudaStream_t st) {
   MmaShape sh;
   if (!mma_shape(p, &sh)) return LASER_ERR_UNSUPPORTED;
   const MmaScratch s = carve_mma(p, scratch);
-  int rc;
-  if (dHp && (rc = cast(dHp, s.dSb, (size_t)p.N * p.Lp * p.d, 1.f, st)) != LASER_OK) return rc;
-  BwdMmaParams P;
   P.Qb = s.Qb; P.Kb = s.Kb; P.Vb = s.Vb; P.dSb = s.dSb;
   P.lengths = lengths; P.cand_offsets = cand_offsets;
-  P.dQf = dQf; P.dK = dK; P.dV = dV;
+  P.dQf = dQf;
   P.L = p.L; P.d = p.d; P.dqk = p.dqk; P.H = p.H; P.S = p.S; P.Lp = p.Lp; P.N = p.N;
   P.R = (std::min(p.S, p.L) + 16 * sh.mt - 1) / (16 * sh.mt);
   P.jobs = p.Lp * P.R * p.H;
@@ -538,6 +545,22 @@ int sta_bwd_mma(const Plan& p, const float* dHp, const int32_t* lengths, const i
   LASER_MMA_CASE(2, 2, 1) LASER_MMA_CASE(2, 2, 2)
 #undef LASER_MMA_CASE
   return LASER_ERR_UNSUPPORTED;
+}
+
+int sta_bwd_mma(const Plan& p, const float* dHp, const int32_t* lengths, const int32_t* cand_offsets, float* dQf,
+                float* dK, float* dV, char* scratch, cudaStream_t st) {
+  int rc;
+  if (dHp && (rc = cast(dHp, carve_mma(p, scratch).dSb, (size_t)p.N * p.Lp * p.d, 1.f, st)) != LASER_OK) return rc;
+  BwdMmaParams P = {};
+  P.dK = dK; P.dV = dV;
+  return run_bwd_mma(p, P, lengths, cand_offsets, dQf, scratch, st);
+}
+
+int sta_bwd_mma_split(const Plan& p, const int32_t* lengths, const int32_t* cand_offsets, float* dQf, __nv_bfloat16* dK_hi,
+                      __nv_bfloat16* dK_lo, __nv_bfloat16* dV_hi, __nv_bfloat16* dV_lo, char* scratch, cudaStream_t st) {
+  BwdMmaParams P = {};
+  P.dKh = dK_hi; P.dKl = dK_lo; P.dVh = dV_hi; P.dVl = dV_lo;
+  return run_bwd_mma(p, P, lengths, cand_offsets, dQf, scratch, st);
 }
 
 }  // namespace laser

@@ -1,0 +1,367 @@
+// The dense products of the backward pass over the item rows (bf16 inputs, warp-level MMAs), in two kernels that touch only
+// the users' valid rows:
+//
+//   rows_project_kernel   Y = scale X [W_a | W_b] as bf16: K and V of the recomputed forward (X read once for both), or Q
+//   rows_grad_kernel      d_items = dK W_k^T + dV W_v^T (zero rows for padding), dW_k += X^T dK, dW_v += X^T dV, all from one
+//                         read of X, dK and dV
+//
+// dK and dV arrive as bf16 high and low parts (16 bits; TF32 operands, 11 bits, before), so every operand tile is copied to
+// shared memory as it is and read with ldmatrix; the weights stay in shared memory for the block's lifetime, the weight
+// gradients in its registers until one atomic add per element at the end.
+// Bound by HBM: 0.64 and 1.5 KB per valid row at d = 128, d_qk = 64.  Six kernels over all rows, padding included, and two
+// memsets before: 470 us at 64 users of 512 .. 4096 of 4096 rows.
+#include <algorithm>
+
+#include "laser_backward.cuh"
+#include "laser_common.cuh"
+#include "laser_mma.cuh"
+
+namespace laser {
+namespace {
+
+using bf16 = __nv_bfloat16;
+using namespace mma;
+
+constexpr int kRT = 64;                 // rows per tile
+constexpr int kRThreads = 512;          // 16 warps: 4 row tiles x 4 column parts
+
+struct RowsParams {
+  int groups, rows_per_group, tiles_per_group;       // users x L, or one group of N rows
+  int na, nb;                                        // columns of W_a and W_b (nb may be 0)
+  const bf16 *X, *Wa, *Wb;                           // X [groups, rows_per_group, d], W_a [d, na], W_b [d, nb]
+  const int *lengths, *cand_offsets;                 // null: every row is valid
+  int N;
+  // projection
+  bf16 *Ya, *Yb;
+  float scale;
+  // gradients
+  const bf16 *Ahi, *Alo, *Bhi, *Blo;                 // dK [.., na], dV [.., nb]: high and low parts
+  float *dX, *dWa, *dWb;
+};
+
+// Rows of a group that take part (a user without candidates, or with invalid inputs, has none).
+__device__ __forceinline__ int valid_rows(const RowsParams& P, int u) {
+  if (!P.lengths) return P.rows_per_group;
+  const int len = P.lengths[u], o0 = P.cand_offsets[u], o1 = P.cand_offsets[u + 1];
+  return len <= 0 || len > P.rows_per_group || o0 < 0 || o1 <= o0 || o1 > P.N ? 0 : len;
+}
+
+template <int D16>
+__global__ void __launch_bounds__(kRThreads) rows_project_kernel(const RowsParams P) {
+  constexpr int d = 16 * D16, XS = 2 * d + 16;
+  extern __shared__ __align__(128) uint8_t smem[];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+  const int n = P.na + P.nb, WS = 2 * n + 16;                        // bytes per row of [W_a | W_b] and of the output tile
+  uint8_t* Ws = smem;                                                // [d][WS]
+  uint8_t* Xs = Ws + (size_t)d * WS;                                 // [2][64][XS]
+  uint8_t* Ys = Xs + 2 * kRT * XS;                                   // [64][WS]
+  for (int i = tid; i < d * (n / 8); i += kRThreads) {
+    const int k = i / (n / 8), c = (i - k * (n / 8)) * 8;
+    cp16(smem_addr(Ws) + k * WS + c * 2, c < P.na ? P.Wa + (size_t)k * P.na + c : P.Wb + (size_t)k * P.nb + c - P.na, 16u);
+  }
+  const int jobs = P.groups * P.tiles_per_group;
+  // job j = (tile j / groups, group j mod groups): the tiles that only long users have come last, spread over the blocks
+  auto rows_of = [&](int j) { return j < jobs ? valid_rows(P, j % P.groups) - j / P.groups * kRT : 0; };
+  auto next_job = [&](int j) {
+    while (j < jobs && rows_of(j) <= 0) j += gridDim.x;
+    return j;
+  };
+  auto stage = [&](int j, int b) {
+    const int rows = rows_of(j);
+    const bf16* src = P.X + ((size_t)(j % P.groups) * P.rows_per_group + j / P.groups * kRT) * d;
+    for (int i = tid; i < kRT * 2 * D16; i += kRThreads) {
+      const int r = i / (2 * D16), q = i - r * (2 * D16);
+      cp16(smem_addr(Xs) + b * kRT * XS + r * XS + q * 16, r < rows ? src + (size_t)r * d + q * 8 : P.X, r < rows ? 16u : 0u);
+    }
+  };
+  int job = next_job(blockIdx.x);
+  if (job < jobs) stage(job, 0);
+  cp_commit();
+  const int m0 = (warp >> 2) * 16, part = warp & 3, pairs = n >> 4;  // column tiles in pairs: part, part + 4, ...
+  const uint32_t a_row = ((lane & 7) + ((lane >> 3) & 1) * 8 + m0) * XS + (lane >> 4) * 16;
+  const uint32_t b_row = ((lane & 7) + ((lane >> 3) & 1) * 8) * WS + (lane >> 4) * 16;
+  int b = 0;
+  while (job < jobs) {
+    const int nxt = next_job(job + gridDim.x);
+    if (nxt < jobs) stage(nxt, b ^ 1);
+    cp_commit();
+    cp_wait<1>();
+    __syncthreads();
+    float acc[4][2][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) acc[i][0][e] = acc[i][1][e] = 0.f;
+    const uint32_t xa = smem_addr(Xs) + b * kRT * XS + a_row, wa = smem_addr(Ws) + b_row;
+#pragma unroll
+    for (int kt = 0; kt < D16; ++kt) {
+      uint32_t a[4];
+      ldsm_x4(a, xa + kt * 32);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int p = part + 4 * i;
+        if (p < pairs) {
+          uint32_t w[4];
+          ldsm_x4_t(w, wa + kt * 16 * WS + p * 32);
+          mma16816(acc[i][0], a[0], a[1], a[2], a[3], w[0], w[1]);
+          mma16816(acc[i][1], a[0], a[1], a[2], a[3], w[2], w[3]);
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int p = part + 4 * i;
+      if (p < pairs) {
+        uint8_t* y = Ys + (m0 + g) * WS + p * 32 + 4 * t;
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt) {
+          *reinterpret_cast<uint32_t*>(y + nt * 16) = pack2(acc[i][nt][0] * P.scale, acc[i][nt][1] * P.scale);
+          *reinterpret_cast<uint32_t*>(y + 8 * WS + nt * 16) = pack2(acc[i][nt][2] * P.scale, acc[i][nt][3] * P.scale);
+        }
+      }
+    }
+    __syncthreads();
+    {
+      const int rows = min(rows_of(job), kRT);
+      const size_t row0 = (size_t)(job % P.groups) * P.rows_per_group + job / P.groups * kRT;
+      for (int i = tid; i < rows * (n / 8); i += kRThreads) {
+        const int r = i / (n / 8), c = (i - r * (n / 8)) * 8;
+        const uint4 v = *reinterpret_cast<const uint4*>(Ys + r * WS + c * 2);
+        if (c < P.na) *reinterpret_cast<uint4*>(P.Ya + (row0 + r) * P.na + c) = v;
+        else *reinterpret_cast<uint4*>(P.Yb + (row0 + r) * P.nb + c - P.na) = v;
+      }
+    }
+    job = nxt;
+    b ^= 1;
+  }
+  cp_wait<0>();
+}
+
+template <int D16>
+__global__ void __launch_bounds__(kRThreads) rows_grad_kernel(const RowsParams P, int nbuf) {
+  constexpr int d = 16 * D16, XS = 2 * d + 16, kParts = 16 / D16, kMaxPairs = (16 + kParts - 1) / kParts;
+  extern __shared__ __align__(128) uint8_t smem[];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+  const int n = P.na + P.nb, WS = 2 * n + 16, pairs = n >> 4;
+  uint8_t* Ws = smem;                                                // [d][WS]  [W_k | W_v]
+  uint8_t* Xs = Ws + (size_t)d * WS;                                 // [nbuf][64][XS]
+  uint8_t* Gs = Xs + (size_t)nbuf * kRT * XS;                        // [nbuf][2][64][WS]  [dK | dV], high and low parts
+  for (int i = tid; i < d * (n / 8); i += kRThreads) {
+    const int k = i / (n / 8), c = (i - k * (n / 8)) * 8;
+    cp16(smem_addr(Ws) + k * WS + c * 2, c < P.na ? P.Wa + (size_t)k * P.na + c : P.Wb + (size_t)k * P.nb + c - P.na, 16u);
+  }
+  const int jobs = P.groups * P.tiles_per_group;
+  auto rows_of = [&](int j) { return j < jobs ? valid_rows(P, j % P.groups) - j / P.groups * kRT : 0; };
+  auto next_job = [&](int j) {
+    while (j < jobs && rows_of(j) <= 0) j += gridDim.x;
+    return j;
+  };
+  auto stage = [&](int j, int b) {
+    const int rows = rows_of(j);
+    const size_t row0 = (size_t)(j % P.groups) * P.rows_per_group + j / P.groups * kRT;
+    for (int i = tid; i < kRT * 2 * D16; i += kRThreads) {
+      const int r = i / (2 * D16), q = i - r * (2 * D16);
+      cp16(smem_addr(Xs) + b * kRT * XS + r * XS + q * 16, r < rows ? P.X + (row0 + r) * d + q * 8 : P.X, r < rows ? 16u : 0u);
+    }
+    for (int i = tid; i < kRT * (n / 8); i += kRThreads) {
+      const int r = i / (n / 8), c = (i - r * (n / 8)) * 8;
+      const uint32_t dst = smem_addr(Gs) + b * 2 * kRT * WS + r * WS + c * 2, bytes = r < rows ? 16u : 0u;
+      const size_t at = r < rows ? (c < P.na ? (row0 + r) * P.na + c : (row0 + r) * P.nb + c - P.na) : 0;
+      cp16(dst, (c < P.na ? P.Ahi : P.Bhi) + at, bytes);
+      cp16(dst + kRT * WS, (c < P.na ? P.Alo : P.Blo) + at, bytes);
+    }
+  };
+  int job = next_job(blockIdx.x);
+  if (job < jobs) stage(job, 0);
+  cp_commit();
+  // rows that receive no gradient
+  for (int j = blockIdx.x; j < jobs; j += gridDim.x) {
+    const int first = max(0, min(kRT, rows_of(j))), last = min(kRT, P.rows_per_group - j / P.groups * kRT);
+    float4* out = reinterpret_cast<float4*>(P.dX + ((size_t)(j % P.groups) * P.rows_per_group + j / P.groups * kRT) * d);
+    for (int i = first * (d / 4) + tid; i < last * (d / 4); i += kRThreads) out[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  const int m0 = (warp >> 2) * 16, part = warp & 3;                  // d_items: 16 rows, feature pairs part, part + 4
+  const int mw = warp % D16, wpart = warp / D16;                     // weight gradients: 16 features, column pairs wpart, ...
+  const int mi = lane >> 3, lr = lane & 7;
+  const uint32_t a_row = ((mi & 1) * 8 + lr + m0) * WS + (mi >> 1) * 16;            // [dK | dV] as A (rows, columns)
+  const uint32_t w_row = ((mi >> 1) * 8 + lr) * WS + (mi & 1) * 16;                 // W^T as B: W rows are its columns
+  const uint32_t xt_row = ((mi >> 1) * 8 + lr) * XS + mw * 32 + (mi & 1) * 16;      // X^T as A
+  const uint32_t g_row = ((mi & 1) * 8 + lr) * WS + (mi >> 1) * 16;                 // [dK | dV] as B
+  float wacc[kMaxPairs][2][4];
+#pragma unroll
+  for (int i = 0; i < kMaxPairs; ++i)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) wacc[i][0][e] = wacc[i][1][e] = 0.f;
+  int b = 0;
+  while (job < jobs) {
+    const int nxt = next_job(job + gridDim.x);
+    if (nbuf == 2) {
+      if (nxt < jobs) stage(nxt, b ^ 1);
+      cp_commit();
+      cp_wait<1>();
+    } else {
+      cp_wait<0>();
+    }
+    __syncthreads();
+    const uint32_t xs = smem_addr(Xs) + b * kRT * XS, hi = smem_addr(Gs) + b * 2 * kRT * WS, lo = hi + kRT * WS;
+    float acc[2][2][4];
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) acc[i][0][e] = acc[i][1][e] = 0.f;
+#pragma unroll 2
+    for (int kt = 0; kt < pairs; ++kt) {
+      uint32_t ah[4], al[4];
+      ldsm_x4(ah, hi + a_row + kt * 32);
+      ldsm_x4(al, lo + a_row + kt * 32);
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const int p = part + 4 * i;
+        if (p < D16) {
+          uint32_t w[4];
+          ldsm_x4(w, smem_addr(Ws) + w_row + p * 16 * WS + kt * 32);
+          mma16816(acc[i][0], ah[0], ah[1], ah[2], ah[3], w[0], w[1]);
+          mma16816(acc[i][1], ah[0], ah[1], ah[2], ah[3], w[2], w[3]);
+          mma16816(acc[i][0], al[0], al[1], al[2], al[3], w[0], w[1]);
+          mma16816(acc[i][1], al[0], al[1], al[2], al[3], w[2], w[3]);
+        }
+      }
+    }
+    {
+      const int rows = rows_of(job);
+      float* out = P.dX + ((size_t)(job % P.groups) * P.rows_per_group + job / P.groups * kRT + m0 + g) * d + 2 * t;
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const int p = part + 4 * i;
+        if (p < D16) {
+#pragma unroll
+          for (int nt = 0; nt < 2; ++nt) {
+            if (m0 + g < rows) *reinterpret_cast<float2*>(out + p * 16 + nt * 8) = make_float2(acc[i][nt][0], acc[i][nt][1]);
+            if (m0 + g + 8 < rows) *reinterpret_cast<float2*>(out + 8 * d + p * 16 + nt * 8) = make_float2(acc[i][nt][2], acc[i][nt][3]);
+          }
+        }
+      }
+    }
+    if (wpart < kParts) {
+#pragma unroll
+      for (int kt = 0; kt < kRT / 16; ++kt) {
+        uint32_t a[4];
+        ldsm_x4_t(a, xs + xt_row + kt * 16 * XS);
+#pragma unroll
+        for (int i = 0; i < kMaxPairs; ++i) {
+          const int p = wpart + kParts * i;
+          if (p < pairs) {
+            uint32_t bh[4], bl[4];
+            ldsm_x4_t(bh, hi + g_row + kt * 16 * WS + p * 32);
+            ldsm_x4_t(bl, lo + g_row + kt * 16 * WS + p * 32);
+            mma16816(wacc[i][0], a[0], a[1], a[2], a[3], bh[0], bh[1]);
+            mma16816(wacc[i][1], a[0], a[1], a[2], a[3], bh[2], bh[3]);
+            mma16816(wacc[i][0], a[0], a[1], a[2], a[3], bl[0], bl[1]);
+            mma16816(wacc[i][1], a[0], a[1], a[2], a[3], bl[2], bl[3]);
+          }
+        }
+      }
+    }
+    __syncthreads();                       // the tile just read may be overwritten
+    if (nbuf == 2) {
+      b ^= 1;
+    } else if (nxt < jobs) {
+      stage(nxt, 0);
+      cp_commit();
+    }
+    job = nxt;
+  }
+  cp_wait<0>();
+  if (wpart >= kParts) return;
+#pragma unroll
+  for (int i = 0; i < kMaxPairs; ++i) {
+    const int p = wpart + kParts * i;
+    if (p < pairs) {
+#pragma unroll
+      for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int m = mw * 16 + g + (e >> 1) * 8, c = p * 16 + nt * 8 + 2 * t + (e & 1);
+          if (c < P.na) atomicAdd(P.dWa + (size_t)m * P.na + c, wacc[i][nt][e]);
+          else atomicAdd(P.dWb + (size_t)m * P.nb + c - P.na, wacc[i][nt][e]);
+        }
+    }
+  }
+}
+
+size_t project_smem(int d, int n) { return (size_t)d * (2 * n + 16) + 2 * kRT * (2 * (size_t)d + 16) + (size_t)kRT * (2 * n + 16); }
+size_t grad_smem(int d, int n, int nbuf) {
+  return (size_t)d * (2 * n + 16) + nbuf * (kRT * (2 * (size_t)d + 16) + 2 * kRT * (2 * (size_t)n + 16));
+}
+constexpr size_t kRowsSmemMax = 226 * 1024;
+
+template <int D16>
+int launch_project(const RowsParams& P, cudaStream_t st) {
+  const size_t smem = project_smem(16 * D16, P.na + P.nb);
+  LASER_CUDA_OK(allow_smem(rows_project_kernel<D16>, smem));
+  const long long jobs = (long long)P.groups * P.tiles_per_group;
+  const int per_sm = smem <= 112 * 1024 ? 2 : 1;
+  LaunchScope ls("bwd_rows_project", st);
+  rows_project_kernel<D16><<<(int)std::min<long long>(jobs, (long long)per_sm * device_sms()), kRThreads, smem, st>>>(P);
+  LASER_CUDA_OK(cudaGetLastError());
+  return LASER_OK;
+}
+template <int D16>
+int launch_grad(const RowsParams& P, cudaStream_t st) {
+  const int n = P.na + P.nb, nbuf = grad_smem(16 * D16, n, 2) <= kRowsSmemMax ? 2 : 1;
+  const size_t smem = grad_smem(16 * D16, n, nbuf);
+  LASER_CUDA_OK(allow_smem(rows_grad_kernel<D16>, smem));
+  const long long jobs = (long long)P.groups * P.tiles_per_group;
+  LaunchScope ls("bwd_rows_grad", st);
+  rows_grad_kernel<D16><<<(int)std::min<long long>(jobs, device_sms()), kRThreads, smem, st>>>(P, nbuf);
+  LASER_CUDA_OK(cudaGetLastError());
+  return LASER_OK;
+}
+
+#define LASER_ROWS_DISPATCH(fn)               \
+  switch (p.d / 16) {                         \
+    case 1: return fn<1>(P, st);              \
+    case 2: return fn<2>(P, st);              \
+    case 3: return fn<3>(P, st);              \
+    case 4: return fn<4>(P, st);              \
+    case 5: return fn<5>(P, st);              \
+    case 6: return fn<6>(P, st);              \
+    case 7: return fn<7>(P, st);              \
+    case 8: return fn<8>(P, st);              \
+    default: return LASER_ERR_UNSUPPORTED;    \
+  }
+
+}  // namespace
+
+bool rows_mma_supported(const Plan& p) {
+  return p.dtype == LASER_BF16 && p.d % 16 == 0 && p.d <= 128 && p.dqk % 16 == 0 && p.dqk <= 128 &&
+         grad_smem(p.d, p.dqk + p.d, 1) <= kRowsSmemMax && (long long)p.U * ((p.L + kRT - 1) / kRT) < (1ll << 30);
+}
+
+int rows_project_items(const Plan& p, const void* items, const int32_t* lengths, const int32_t* cand_offsets, const void* Wk,
+                       const void* Wv, __nv_bfloat16* Kb, __nv_bfloat16* Vb, cudaStream_t st) {
+  RowsParams P = {};
+  P.groups = p.U; P.rows_per_group = p.L; P.tiles_per_group = (p.L + kRT - 1) / kRT; P.na = p.dqk; P.nb = p.d;
+  P.X = (const bf16*)items; P.Wa = (const bf16*)Wk; P.Wb = (const bf16*)Wv; P.lengths = lengths; P.cand_offsets = cand_offsets;
+  P.N = p.N; P.Ya = Kb; P.Yb = Vb; P.scale = 1.f;
+  LASER_ROWS_DISPATCH(launch_project)
+}
+
+int rows_project_cands(const Plan& p, const void* cands, const void* Wq, float scale, __nv_bfloat16* Qb, cudaStream_t st) {
+  RowsParams P = {};
+  P.groups = 1; P.rows_per_group = p.N; P.tiles_per_group = (p.N + kRT - 1) / kRT; P.na = p.dqk;
+  P.X = (const bf16*)cands; P.Wa = P.Wb = (const bf16*)Wq; P.N = p.N; P.Ya = Qb; P.scale = scale;
+  LASER_ROWS_DISPATCH(launch_project)
+}
+
+int rows_gradients(const Plan& p, const void* items, const int32_t* lengths, const int32_t* cand_offsets, const void* Wk,
+                   const void* Wv, const __nv_bfloat16* dK_hi, const __nv_bfloat16* dK_lo, const __nv_bfloat16* dV_hi,
+                   const __nv_bfloat16* dV_lo, float* d_items, float* dWk, float* dWv, cudaStream_t st) {
+  RowsParams P = {};
+  P.groups = p.U; P.rows_per_group = p.L; P.tiles_per_group = (p.L + kRT - 1) / kRT; P.na = p.dqk; P.nb = p.d;
+  P.X = (const bf16*)items; P.Wa = (const bf16*)Wk; P.Wb = (const bf16*)Wv; P.lengths = lengths; P.cand_offsets = cand_offsets;
+  P.N = p.N; P.Ahi = dK_hi; P.Alo = dK_lo; P.Bhi = dV_hi; P.Blo = dV_lo; P.dX = d_items; P.dWa = dWk; P.dWb = dWv;
+  LASER_ROWS_DISPATCH(launch_grad)
+}
+
+}  // namespace laser

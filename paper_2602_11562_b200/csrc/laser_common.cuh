@@ -97,15 +97,18 @@ bool sta_bwd_mma_supported(const Plan& p);
 bool sta_fwd_mma_supported(const Plan& p);
 size_t sta_bwd_mma_scratch_bytes(const Plan& p);
 int sta_mma_operands(const Plan& p, const float* Qf, const float* Kf, const float* Vf, char* scratch, cudaStream_t st);
-// The bf16 K [U L, d_qk] and V [U L, d] arrays inside `scratch`, for a producer that writes them directly (it then passes
+// The bf16 Q / (2 gamma) [N, d_qk], K [U L, d_qk] and V [U L, d] arrays inside `scratch`, for a producer that writes them directly (it then passes
 // Kf = Vf = null to sta_mma_operands).
-void sta_mma_operand_arrays(const Plan& p, char* scratch, __nv_bfloat16** Kb, __nv_bfloat16** Vb);
+void sta_mma_operand_arrays(const Plan& p, char* scratch, __nv_bfloat16** Qb, __nv_bfloat16** Kb, __nv_bfloat16** Vb);
 // The bf16 H' that sta_fwd_mma leaves (bf16_copy) and the bf16 dH' that sta_bwd_mma reads, [N, L', d] each.
 void sta_mma_segment_arrays(const Plan& p, char* scratch, __nv_bfloat16** Hb, __nv_bfloat16** dSb);
 int sta_fwd_mma(const Plan& p, const int32_t* lengths, const int32_t* cand_offsets, float* Hp, bool bf16_copy, char* scratch,
                 cudaStream_t st);
 int sta_bwd_mma(const Plan& p, const float* dHp, const int32_t* lengths, const int32_t* cand_offsets, float* dQf,
                 float* dK, float* dV, char* scratch, cudaStream_t st);
+// The same with dK and dV as bf16 high and low parts.
+int sta_bwd_mma_split(const Plan& p, const int32_t* lengths, const int32_t* cand_offsets, float* dQf, __nv_bfloat16* dK_hi,
+                      __nv_bfloat16* dK_lo, __nv_bfloat16* dV_hi, __nv_bfloat16* dV_lo, char* scratch, cudaStream_t st);
 
 bool tensor_supported(const Plan& p);
 void tensor_geometry(const Plan& p, TensorGeom* g);
