@@ -1052,6 +1052,12 @@ int launch_sta_bwd(const Plan& p, const float* Qf, const float* Kf, const float*
   return LASER_OK;
 }
 
+// Where the tensor-core attention kernel leaves its rows: the fp32 arrays' memory, two bf16 parts each.
+GstaPlanes train_planes(const Plan& p, const BwdScratch& s) {
+  auto h = [](float* q) { return reinterpret_cast<bf16*>(q); };
+  return {h(s.T), h(s.Q), h(s.dT), h(s.dQ), h(s.Mh), h(s.dQt), s.dT + p.M * (size_t)p.N * p.d};
+}
+
 // Several arrays set to zero by one launch.
 struct ZeroList {
   float* p[8];
@@ -1187,7 +1193,7 @@ int backward_stream_all(const Plan& p, const T* items, const int32_t* lengths, c
   BWD_OK(zero_arrays(Z, st));
   bf16 *Hhi = reinterpret_cast<bf16*>(s.Hp), *Hlo = Hhi + (size_t)N * p.Lp * d;
   BWD_OK(backward_stream_forward(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, nullptr, Hhi, Hlo, ws, stream_scratch, st));
-  const GstaTrain G = {s.T, s.Q, s.dT, s.dQ, s.Mh, s.dQt, s.dT + M * (size_t)N * d};
+  const GstaPlanes G = train_planes(p, s);
   BWD_OK(gsta_train(p, 2, Hhi, Hlo, lengths, cand_offsets, cands, Wg, dz, G, s.dHp, train_scratch, st));
   const float* p_sums = nullptr;
   BWD_OK(backward_stream(p, items, lengths, cand_offsets, Wv, s.dHp, d_items, dWv, &p_sums, ws, stream_scratch, st));
@@ -1225,7 +1231,7 @@ int backward_lists(const Plan& p, const bf16* items, const int32_t* lengths, con
   sta_mma_operand_arrays(p, mma_scratch, &Qb, &Kb, &Vb);
   sta_mma_segment_arrays(p, mma_scratch, &Hb, &dSb);
   bf16 *dKh = reinterpret_cast<bf16*>(s.dK), *dKl = dKh + UL * dqk, *dVh = reinterpret_cast<bf16*>(s.dV), *dVl = dVh + UL * d;
-  const GstaTrain G = {s.T, s.Q, s.dT, s.dQ, s.Mh, s.dQt, s.dT + M * N * d};
+  const GstaPlanes G = train_planes(p, s);
   int rc;
 #define BWD_OK(...) do { rc = (__VA_ARGS__); if (rc != LASER_OK) return rc; } while (0)
   ZeroList Z = {};
@@ -1316,7 +1322,7 @@ int backward_t(const Plan& p, const T* items, const int32_t* lengths, const T* c
   if (train) {
     bf16 *Hb, *dSb;
     sta_mma_segment_arrays(p, mma_scratch, &Hb, &dSb);
-    const GstaTrain G = {s.T, s.Q, s.dT, s.dQ, s.Mh, s.dQt, s.dT + M * Nd};
+    const GstaPlanes G = train_planes(p, s);
     dT0 = G.dT0;
     BWD_OK(gsta_train(p, 1, Hb, nullptr, lengths, cand_offsets, cands, Wg, dz, G, dSb, train_scratch, st));
     BWD_OK(gsta_weight_sums(p, G, dWg, st));

@@ -18,14 +18,20 @@ bool gsta_train_simt_supported(const Plan& p);
 int gsta_train_simt(const Plan& p, const float* Hp, const int32_t* lengths, const int32_t* cand_offsets, const void* cands,
                     const void* Wg, const float* dz, const GstaTrain& G, float* dHp, cudaStream_t st);
 
+// The same for the tensor-core kernel, as bf16 high and low parts: arrays of [2][M, N, d] and [2][M, N, H, d].
+struct GstaPlanes {
+  __nv_bfloat16 *T, *Q, *dT, *dQ, *Mh, *dQt;
+  float* dT0;
+};
+
 // Tensor cores (laser_backward_gsta.cu), bf16 inputs: np = 1: segment vectors S0 in bf16, dS [N, Lp, d] leaves as bf16;
 // np = 2: segment vectors S0 + S1 (bf16 high and low parts of fp32 values), dS leaves as fp32.  Rows of empty segments are
 // neither read nor written.  gsta_weight_sums adds the layers' weight gradients from what gsta_train left in G.
 bool gsta_train_supported(const Plan& p, int np);
 size_t gsta_train_scratch_bytes(const Plan& p, int np);
 int gsta_train(const Plan& p, int np, const void* S0, const void* S1, const int32_t* lengths, const int32_t* cand_offsets,
-               const void* cands, const void* Wg, const float* dz, const GstaTrain& G, void* dS, char* scratch, cudaStream_t st);
-int gsta_weight_sums(const Plan& p, const GstaTrain& G, float* dWg, cudaStream_t st);
+               const void* cands, const void* Wg, const float* dz, const GstaPlanes& G, void* dS, char* scratch, cudaStream_t st);
+int gsta_weight_sums(const Plan& p, const GstaPlanes& G, float* dWg, cudaStream_t st);
 
 // Products over the item rows on the tensor cores (laser_backward_rows.cu), users' valid rows only, bf16 inputs: K and V (or
 // scale Q of the candidates) as bf16; every row of d_items (zeros for padding) and the sums into dWk, dWv from dK and dV

@@ -39,10 +39,11 @@ struct TrainParams {
   const float* dz;
   const uint4* img;                               // [M][3][2][d/16][d/16][32]: W_q, W_k, W_v as stored and transposed
   const int *nseg, *order;
-  GstaTrain G;
+  GstaPlanes G;
   float* stat;                                    // [M, N, H, 2] softmax maximum and 1 / sum
   bf16 *rows0, *rows1;                            // [N, slots, d] qt and dm per slot (high, low)
-  float* ad;                                      // [N, Lp, slots] de and a per slot
+  float* ad32;                                    // [N, Lp, slots] de and a per slot (NP = 2)
+  bf16* ad16;                                     // the same as the bf16 operand it becomes (NP = 1)
   bf16* dS16;                                     // [N, Lp, d] out (NP = 1)
   float* dS32;                                    // [N, Lp, d] out (NP = 2)
 };
@@ -87,22 +88,23 @@ __device__ __forceinline__ void split2(float x0, float x1, uint32_t& hi, uint32_
 
 template <int D16, int NP>
 struct TrainSmem {
-  static constexpr int d = 16 * D16, RS = 2 * d + 16, TS = d + 8;
+  static constexpr int d = 16 * D16, RS = 2 * d + 16;
   static __host__ __device__ constexpr size_t plane(int H) { return (size_t)kTRows * H * RS; }
   static size_t bytes(int H, int nb) {
-    return (size_t)kTRows * TS * 4 + 2 * NP * plane(H) + RS + kTRows * sizeof(int) + 48 + (size_t)kTW * nb * kTRows * RS * NP;
+    return 2 * (size_t)kTRows * RS + 2 * NP * plane(H) + RS + kTRows * sizeof(int) + 48 + (size_t)kTW * nb * kTRows * RS * NP;
   }
 };
 
 template <int D16, int NP>
 __global__ void __launch_bounds__(kTThreads, 2) gsta_train_kernel(const __grid_constant__ TrainParams P) {
   using SM = TrainSmem<D16, NP>;
-  constexpr int d = SM::d, RS = SM::RS, TS = SM::TS;
+  constexpr int d = SM::d, RS = SM::RS;
   extern __shared__ __align__(128) uint8_t smem[];
   const int H = P.H, Lp = P.Lp, dvh = d / H, KH = dvh >> 4;
   const uint32_t plane = (uint32_t)SM::plane(H);
-  float* Ts = reinterpret_cast<float*>(smem);                        // [16][TS]  t, later dt
-  uint8_t* Qt = smem + kTRows * TS * 4;                              // [NP][16][H] rows: qt; m or dqt (high) later
+  uint8_t* Thi = smem;                                               // [16] rows: t, later dt, high and low parts (the fp32
+  uint8_t* Tlo = Thi + kTRows * RS;                                  // values live in the registers of the columns' warp)
+  uint8_t* Qt = smem + 2 * kTRows * RS;                              // [NP][16][H] rows: qt; m or dqt (high) later
   uint8_t* Dm = Qt + NP * plane;                                     // [NP][16][H] rows: dm; NP = 1: also m or dqt (low)
   uint8_t* Xlo = NP == 1 ? Dm : Qt + plane;                          // low parts of m / dqt (their high parts: Qt)
   uint8_t* zrow = Dm + NP * plane;
@@ -123,28 +125,12 @@ __global__ void __launch_bounds__(kTThreads, 2) gsta_train_kernel(const __grid_c
   const int wcol = warp * 16;                                        // this warp's 16 columns of the dense phases
   constexpr int kImg = D16 * D16 * 32;
   if (tid < kTRows) nv_s[tid] = c_base + tid < c_end ? min(max(P.nseg[c_base + tid], 0), Lp) : 0;
-  for (int i = tid; i < kTRows * (d / 8); i += kTThreads) {
-    const int r = i / (d / 8), c8 = (i - r * (d / 8)) * 8;
-    uint4 v = make_uint4(0, 0, 0, 0);
-    if (c_base + r < c_end) v = *reinterpret_cast<const uint4*>(P.cands + (size_t)(c_base + r) * d + c8);
-    float* dst = Ts + r * TS + c8;
-    dst[0] = bf16_lo(v.x); dst[1] = bf16_hi(v.x); dst[2] = bf16_lo(v.y); dst[3] = bf16_hi(v.y);
-    dst[4] = bf16_lo(v.z); dst[5] = bf16_hi(v.z); dst[6] = bf16_lo(v.w); dst[7] = bf16_hi(v.w);
-  }
   for (int i = tid; i < RS / 4; i += kTThreads) reinterpret_cast<uint32_t*>(zrow)[i] = 0u;
   for (uint32_t i = tid * 4; i < 2 * NP * plane; i += kTThreads * 4) *reinterpret_cast<uint32_t*>(Qt + i) = 0u;   // (rows of absent candidates)
   __syncthreads();
 
   // ---- dense building blocks.  Weight fragments of k-tile kt for this warp's columns: image entry (kt, warp).
   auto weights = [&](int l, int m, int trans) { return P.img + (size_t)((l * 3 + m) * 2 + trans) * kImg + (size_t)warp * 32 + lane; };
-  // high / low A fragments of k-tile kt of the fp32 rows in Ts
-  auto ts_frag = [&](int kt, uint32_t (&hi)[4], uint32_t (&lo)[4]) {
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const float2 x = *reinterpret_cast<const float2*>(Ts + (g + (e & 1) * 8) * TS + kt * 16 + 2 * t + (e >> 1) * 8);
-      split2(x.x, x.y, hi[e], lo[e]);
-    }
-  };
   auto mma_pair = [&](float (&acc)[2][4], const uint32_t (&a)[4], const uint4& b) {
     mma16816(acc[0], a[0], a[1], a[2], a[3], b.x, b.y);
     mma16816(acc[1], a[0], a[1], a[2], a[3], b.z, b.w);
@@ -164,42 +150,77 @@ __global__ void __launch_bounds__(kTThreads, 2) gsta_train_kernel(const __grid_c
       mma_pair(acc, lo, b);
     }
   };
-  // rows of a [16][d] result: fp32 to global memory (dst, N rows of d) and as high / low rows for the next product
-  auto put_rows = [&](const float (&acc)[2][4], float scale, float* dst, bool split) {
+  // this warp's columns of a [16][d] result as high / low rows: to shared memory (hi, lo; the next product's operand) and
+  // to global memory (dst: N rows of d, the low parts `lo_at` elements behind)
+  auto put_rows = [&](const float (&v)[2][4], float scale, uint8_t* hi, uint8_t* lo, bf16* dst, size_t lo_at) {
 #pragma unroll
     for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
       for (int hf = 0; hf < 2; ++hf) {
         const int r = g + hf * 8, col = wcol + nt * 8 + 2 * t;
-        const float x0 = acc[nt][2 * hf] * scale, x1 = acc[nt][2 * hf + 1] * scale;
-        if (c_base + r < c_end) *reinterpret_cast<float2*>(dst + (size_t)(c_base + r) * d + col) = make_float2(x0, x1);
-        if (split) {
-          uint32_t hi, lo;
-          split2(x0, x1, hi, lo);
-          *reinterpret_cast<uint32_t*>(Qhi + r * RS + col * 2) = hi;
-          *reinterpret_cast<uint32_t*>(Qlo + r * RS + col * 2) = lo;
+        uint32_t h, l;
+        split2(v[nt][2 * hf] * scale, v[nt][2 * hf + 1] * scale, h, l);
+        *reinterpret_cast<uint32_t*>(hi + r * RS + col * 2) = h;
+        *reinterpret_cast<uint32_t*>(lo + r * RS + col * 2) = l;
+        if (dst && c_base + r < c_end) {
+          const size_t at = (size_t)(c_base + r) * d + col;
+          *reinterpret_cast<uint32_t*>(dst + at) = h;
+          *reinterpret_cast<uint32_t*>(dst + lo_at + at) = l;
         }
       }
   };
-  auto save_rows = [&](float* dst) {                                 // the block's rows of Ts to global memory
-    for (int i = tid; i < kTRows * (d / 4); i += kTThreads) {
-      const int r = i / (d / 4), c4 = (i - r * (d / 4)) * 4;
-      if (c_base + r < c_end)
-        *reinterpret_cast<float4*>(dst + (size_t)(c_base + r) * d + c4) = *reinterpret_cast<const float4*>(Ts + r * TS + c4);
+  // acc += x W with x the 16 high / low rows at hi, lo
+  auto from_rows = [&](float (&acc)[2][4], const uint8_t* hi, const uint8_t* lo, const uint4* w) {
+    const uint32_t ah = smem_addr(hi + ldsm_row * RS) + ldsm_kc * 16, al = smem_addr(lo + ldsm_row * RS) + ldsm_kc * 16;
+#pragma unroll
+    for (int kt = 0; kt < D16; ++kt) {
+      const uint4 b = __ldg(w + kt * D16 * 32);
+      uint32_t x[4];
+      ldsm_x4(x, ah + kt * 32);
+      mma_pair(acc, x, b);
+      ldsm_x4(x, al + kt * 32);
+      mma_pair(acc, x, b);
     }
   };
-  auto add_rows = [&](const float (&acc)[2][4]) {                    // Ts += this warp's columns
+  // the same head by head (k-tiles of head h only), each result as head rows of the planes at dst (low parts: NP = 2)
+  auto fold_heads = [&](const uint8_t* hi, const uint8_t* lo, const uint4* w, float scale, uint8_t* dst) {
+    const uint32_t ah = smem_addr(hi + ldsm_row * RS) + ldsm_kc * 16, al = smem_addr(lo + ldsm_row * RS) + ldsm_kc * 16;
+    float acc[2][4] = {};
 #pragma unroll
-    for (int nt = 0; nt < 2; ++nt) {
-      const int col = wcol + nt * 8 + 2 * t;
-      float2* r0 = reinterpret_cast<float2*>(Ts + g * TS + col);
-      float2* r1 = reinterpret_cast<float2*>(Ts + (g + 8) * TS + col);
-      float2 v0 = *r0, v1 = *r1;
-      v0.x += acc[nt][0]; v0.y += acc[nt][1];
-      v1.x += acc[nt][2]; v1.y += acc[nt][3];
-      *r0 = v0;
-      *r1 = v1;
+    for (int kt = 0; kt < D16; ++kt) {
+      const uint4 b = __ldg(w + kt * D16 * 32);
+      uint32_t x[4];
+      ldsm_x4(x, ah + kt * 32);
+      mma_pair(acc, x, b);
+      ldsm_x4(x, al + kt * 32);
+      mma_pair(acc, x, b);
+      if ((kt + 1) % KH == 0) {                                      // last k-tile of head kt / KH
+        const int h = kt / KH;
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+          for (int hf = 0; hf < 2; ++hf) {
+            uint32_t vh, vl;
+            split2(acc[nt][2 * hf] * scale, acc[nt][2 * hf + 1] * scale, vh, vl);
+            const uint32_t o = ((g + hf * 8) * H + h) * RS + (wcol + nt * 8 + 2 * t) * 2;
+            *reinterpret_cast<uint32_t*>(dst + o) = vh;
+            if (NP == 2) *reinterpret_cast<uint32_t*>(dst + plane + o) = vl;
+            acc[nt][2 * hf] = acc[nt][2 * hf + 1] = 0.f;
+          }
+      }
     }
+  };
+  float tr[2][4] = {};                                               // t, later dt: this warp's columns, rows g and g + 8
+  auto load_rows = [&](auto at) {
+#pragma unroll
+    for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+      for (int hf = 0; hf < 2; ++hf) {
+        float2 v = make_float2(0.f, 0.f);
+        if (c_base + g + hf * 8 < c_end) v = at((size_t)(c_base + g + hf * 8) * d + wcol + nt * 8 + 2 * t);
+        tr[nt][2 * hf] = v.x;
+        tr[nt][2 * hf + 1] = v.y;
+      }
   };
 
   // ---- staging of a candidate's segment vectors, 16 rows per buffer (rows past its segments: zeros)
@@ -224,8 +245,7 @@ __global__ void __launch_bounds__(kTThreads, 2) gsta_train_kernel(const __grid_c
     return smem_addr(((lane & 7) < H ? base + (c * H + (lane & 7)) * RS : zrow) + ((lane >> 3) & 1) * 16);
   };
   // e += S x^T for one staged chunk, x = head rows at b0 (and b1: low parts)
-  auto dot_tile = [&](uint32_t sb, int kt, const uint32_t (&a0)[4], const uint32_t (&a1)[4], uint32_t b0, uint32_t b1, float (&e)[4]) {
-    (void)sb;
+  auto dot_tile = [&](int kt, const uint32_t (&a0)[4], const uint32_t (&a1)[4], uint32_t b0, uint32_t b1, float (&e)[4]) {
     uint32_t b[2];
     ldsm_x2(b, b0 + kt * 32);
     mma16816(e, a0[0], a0[1], a0[2], a0[3], b[0], b[1]);
@@ -254,19 +274,13 @@ __global__ void __launch_bounds__(kTThreads, 2) gsta_train_kernel(const __grid_c
       }
     }
   };
-  // rows [head][feature] of candidate c from x^T (scaled per head): high parts to Qt, low parts to Xlo, fp32 to dst [H, d]
-  auto put_heads = [&](int c, const float (&x)[D16][4], float f0, float f1, float* dst) {
-    const int h0 = 2 * t, h1 = 2 * t + 1;
+  // rows [head][feature] of candidate c from x^T (scaled per head): high parts to Qt, low parts to Xlo
+  auto put_heads = [&](int c, const float (&x)[D16][4], float f0, float f1) {
 #pragma unroll
     for (int jt = 0; jt < D16; ++jt) {
-      const float v0 = x[jt][0] * f0, v1 = x[jt][1] * f1, v2 = x[jt][2] * f0, v3 = x[jt][3] * f1;
-      if (dst) {
-        if (h0 < H) { dst[h0 * d + jt * 16 + g] = v0; dst[h0 * d + jt * 16 + g + 8] = v2; }
-        if (h1 < H) { dst[h1 * d + jt * 16 + g] = v1; dst[h1 * d + jt * 16 + g + 8] = v3; }
-      }
       uint32_t ha, la, hb, lb;
-      split2(v0, v1, ha, la);
-      split2(v2, v3, hb, lb);
+      split2(x[jt][0] * f0, x[jt][1] * f1, ha, la);
+      split2(x[jt][2] * f0, x[jt][3] * f1, hb, lb);
       ha = movmatrix_t(ha); hb = movmatrix_t(hb); la = movmatrix_t(la); lb = movmatrix_t(lb);   // (head g, features 2t, 2t + 1)
       if (g < H) {
         const uint32_t o = (c * H + g) * RS + jt * 32 + 4 * t;
@@ -277,70 +291,63 @@ __global__ void __launch_bounds__(kTThreads, 2) gsta_train_kernel(const __grid_c
       }
     }
   };
+  // 16-byte pieces of a candidate's head rows, lanes over (head, piece): f(head, piece, offset in a plane)
+  auto pieces = [&](int c, auto f) {
+    for (int i = lane; i < H * 2 * D16; i += 32) {
+      const int h = i / (2 * D16), q = i - h * (2 * D16);
+      f(h, q, (uint32_t)((c * H + h) * RS + q * 16));
+    }
+  };
+  auto ld16 = [](const void* p) { return *reinterpret_cast<const uint4*>(p); };
+  auto unpack = [](float (&v)[8], const uint4& x) {
+    v[0] = bf16_lo(x.x); v[1] = bf16_hi(x.x); v[2] = bf16_lo(x.y); v[3] = bf16_hi(x.y);
+    v[4] = bf16_lo(x.z); v[5] = bf16_hi(x.z); v[6] = bf16_lo(x.w); v[7] = bf16_hi(x.w);
+  };
+  auto add_lo = [](float (&v)[8], const uint4& x) {
+    v[0] += bf16_lo(x.x); v[1] += bf16_hi(x.x); v[2] += bf16_lo(x.y); v[3] += bf16_hi(x.y);
+    v[4] += bf16_lo(x.z); v[5] += bf16_hi(x.z); v[6] += bf16_lo(x.w); v[7] += bf16_hi(x.w);
+  };
+  auto split8 = [](const float (&v)[8], uint4& hi, uint4& lo) {
+    split2(v[0], v[1], hi.x, lo.x); split2(v[2], v[3], hi.y, lo.y); split2(v[4], v[5], hi.z, lo.z); split2(v[6], v[7], hi.w, lo.w);
+  };
+  const size_t lo_d = (size_t)P.M * Nd, lo_h = (size_t)P.M * NHd;    // distance of the low-part planes in global memory
 
   // =============================================================================================== forward
+  if (dense) {
+    load_rows([&](size_t at) {
+      const uint32_t v = *reinterpret_cast<const uint32_t*>(P.cands + at);
+      return make_float2(bf16_lo(v), bf16_hi(v));
+    });
+    put_rows(tr, 1.f, Thi, Tlo, P.G.T, lo_d);
+  }
+  __syncthreads();
   for (int l = 0; l < P.M; ++l) {
-    save_rows(P.G.T + l * Nd);
     if (dense) {                                                     // q = t W_q
       float acc[2][4] = {};
-      const uint4* w = weights(l, 0, 0);
-#pragma unroll
-      for (int kt = 0; kt < D16; ++kt) {
-        const uint4 b = __ldg(w + kt * D16 * 32);
-        uint32_t hi[4], lo[4];
-        ts_frag(kt, hi, lo);
-        mma_pair(acc, hi, b);
-        mma_pair(acc, lo, b);
-      }
-      put_rows(acc, 1.f, P.G.Q + l * Nd, true);
+      from_rows(acc, Thi, Tlo, weights(l, 0, 0));
+      put_rows(acc, 1.f, Qhi, Qlo, P.G.Q + l * Nd, lo_d);
     }
     __syncthreads();
-    if (dense) {                                                     // qt_h = q_h W_k[:, h]^T / tau
-      float acc[2][4] = {};
-      const uint4* w = weights(l, 1, 1);
-#pragma unroll
-      for (int kt = 0; kt < D16; ++kt) {
-        const uint4 b = __ldg(w + kt * D16 * 32);
-        uint32_t hi[4], lo[4];
-        ldsm_x4(hi, smem_addr(Qhi + ldsm_row * RS + (kt * 2 + ldsm_kc) * 16));
-        ldsm_x4(lo, smem_addr(Qlo + ldsm_row * RS + (kt * 2 + ldsm_kc) * 16));
-        mma_pair(acc, hi, b);
-        mma_pair(acc, lo, b);
-        if ((kt + 1) % KH == 0) {                                    // last k-tile of head kt / KH
-          const int h = kt / KH;
-#pragma unroll
-          for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-            for (int hf = 0; hf < 2; ++hf) {
-              uint32_t hi2, lo2;
-              split2(acc[nt][2 * hf] * P.inv_tau, acc[nt][2 * hf + 1] * P.inv_tau, hi2, lo2);
-              const uint32_t o = ((g + hf * 8) * H + h) * RS + (wcol + nt * 8 + 2 * t) * 2;
-              *reinterpret_cast<uint32_t*>(Qt + o) = hi2;
-              if (NP == 2) *reinterpret_cast<uint32_t*>(Qt + plane + o) = lo2;
-              acc[nt][2 * hf] = acc[nt][2 * hf + 1] = 0.f;
-            }
-        }
-      }
-    }
+    if (dense) fold_heads(Qhi, Qlo, weights(l, 1, 1), P.inv_tau, Qt);   // qt_h = q_h W_k[:, h]^T / tau
     __syncthreads();
 #pragma unroll 1
     for (int sl = 0; sl < n_slots; ++sl) {                           // attention, one candidate of this warp after the other
       const int c = warp + kTW * sl, cand = c_base + c, nv = nv_s[c];
       if (cand >= c_end) continue;
-      // the slot rows (qt of this layer): kept for the backward part
-      for (int i = lane; i < H * 2 * D16; i += 32) {
-        const int h = i / (2 * D16), q = i - h * (2 * D16);
-        const size_t at = ((size_t)cand * P.slots + l * 2 * H + h) * d + q * 8;
-        *reinterpret_cast<uint4*>(P.rows0 + at) = *reinterpret_cast<const uint4*>(Qt + (c * H + h) * RS + q * 16);
-        if (NP == 2) *reinterpret_cast<uint4*>(P.rows1 + at) = *reinterpret_cast<const uint4*>(Qt + plane + (c * H + h) * RS + q * 16);
+      const int nch = (nv + kTRows - 1) / kTRows;
+      if (nch > 0) stage_chunk(cand, 0, nv, 0);
+      {                                                              // the slot rows of qt, for the backward part
+        bf16 *r0 = P.rows0 + ((size_t)cand * P.slots + l * 2 * H) * d, *r1 = P.rows1 + ((size_t)cand * P.slots + l * 2 * H) * d;
+        pieces(c, [&](int h, int q, uint32_t o) {
+          *reinterpret_cast<uint4*>(r0 + h * d + q * 8) = ld16(Qt + o);
+          if (NP == 2) *reinterpret_cast<uint4*>(r1 + h * d + q * 8) = ld16(Qt + plane + o);
+        });
       }
       float x[D16][4];
 #pragma unroll
       for (int jt = 0; jt < D16; ++jt) x[jt][0] = x[jt][1] = x[jt][2] = x[jt][3] = 0.f;
       float rm0 = -INFINITY, rm1 = -INFINITY, rs0 = 0.f, rs1 = 0.f;
       const uint32_t q0 = head_rows(Qt, c), q1 = head_rows(Qt + plane, c);
-      const int nch = (nv + kTRows - 1) / kTRows;
-      if (nch > 0) stage_chunk(cand, 0, nv, 0);
       int b = 0;
       for (int ch = 0; ch < nch; ++ch) {
         if (P.nb > 1 && ch + 1 < nch) {
@@ -357,7 +364,7 @@ __global__ void __launch_bounds__(kTThreads, 2) gsta_train_kernel(const __grid_c
           uint32_t a0[4], a1[4];
           ldsm_x4(a0, sb + a_off + kt * 32);
           if (NP == 2) ldsm_x4(a1, sb + kTRows * RS + a_off + kt * 32);
-          dot_tile(sb, kt, a0, a1, q0, q1, e);
+          dot_tile(kt, a0, a1, q0, q1, e);
         }
         const int rows = nv - ch * kTRows;
         if (g >= rows) e[0] = e[1] = -INFINITY;
@@ -366,7 +373,7 @@ __global__ void __launch_bounds__(kTThreads, 2) gsta_train_kernel(const __grid_c
         const float sc0 = __expf(rm0 - nm0), sc1 = __expf(rm1 - nm1);
         rm0 = nm0;
         rm1 = nm1;
-        float w0 = __expf(e[0] - nm0), w1 = __expf(e[1] - nm1), w2 = __expf(e[2] - nm0), w3 = __expf(e[3] - nm1);
+        const float w0 = __expf(e[0] - nm0), w1 = __expf(e[1] - nm1), w2 = __expf(e[2] - nm0), w3 = __expf(e[3] - nm1);
         rs0 = rs0 * sc0 + w0 + w2;
         rs1 = rs1 * sc1 + w1 + w3;
         if (ch > 0) {
@@ -381,57 +388,35 @@ __global__ void __launch_bounds__(kTThreads, 2) gsta_train_kernel(const __grid_c
       const float s0 = group_sum(rs0), s1 = group_sum(rs1);
       const float i0 = s0 > 0.f ? 1.f / s0 : 0.f, i1 = s1 > 0.f ? 1.f / s1 : 0.f;
       __syncwarp();
-      put_heads(c, x, i0, i1, P.G.Mh + l * NHd + (size_t)cand * H * d);
+      put_heads(c, x, i0, i1);
       if (g == 0) {
         float* st = P.stat + ((size_t)(l * P.N + cand) * H) * 2;
         if (2 * t < H) *reinterpret_cast<float2*>(st + 4 * t) = make_float2(rm0, i0);
         if (2 * t + 1 < H) *reinterpret_cast<float2*>(st + 4 * t + 2) = make_float2(rm1, i1);
       }
+      __syncwarp();
+      bf16* mg = P.G.Mh + l * NHd + (size_t)cand * H * d;
+      pieces(c, [&](int h, int q, uint32_t o) {
+        *reinterpret_cast<uint4*>(mg + h * d + q * 8) = ld16(Qt + o);
+        *reinterpret_cast<uint4*>(mg + lo_h + h * d + q * 8) = ld16(Xlo + o);
+      });
     }
     __syncthreads();
     if (dense && l + 1 < P.M) {                                      // t += m_h W_v[:, h]  (the last layer's t is not needed)
-      float acc[2][4] = {};
-      from_heads(acc, weights(l, 2, 0));
-      add_rows(acc);
+      from_heads(tr, weights(l, 2, 0));
+      put_rows(tr, 1.f, Thi, Tlo, P.G.T + (l + 1) * Nd, lo_d);
     }
     __syncthreads();
   }
 
   // =============================================================================================== backward
-  for (int i = tid; i < kTRows * (d / 4); i += kTThreads) {          // dt of the last target
-    const int r = i / (d / 4), c4 = (i - r * (d / 4)) * 4;
-    *reinterpret_cast<float4*>(Ts + r * TS + c4) =
-        c_base + r < c_end ? *reinterpret_cast<const float4*>(P.dz + (size_t)(c_base + r) * d + c4) : make_float4(0.f, 0.f, 0.f, 0.f);
+  if (dense) {                                                       // dt of the last target
+    load_rows([&](size_t at) { return *reinterpret_cast<const float2*>(P.dz + at); });
+    put_rows(tr, 1.f, Thi, Tlo, P.G.dT + (P.M - 1) * Nd, lo_d);
   }
   __syncthreads();
   for (int l = P.M - 1; l >= 0; --l) {
-    save_rows(P.G.dT + l * Nd);
-    if (dense) {                                                     // dm_h = dt_h W_v[:, h]^T
-      float acc[2][4] = {};
-      const uint4* w = weights(l, 2, 1);
-#pragma unroll
-      for (int kt = 0; kt < D16; ++kt) {
-        const uint4 b = __ldg(w + kt * D16 * 32);
-        uint32_t hi[4], lo[4];
-        ts_frag(kt, hi, lo);
-        mma_pair(acc, hi, b);
-        mma_pair(acc, lo, b);
-        if ((kt + 1) % KH == 0) {
-          const int h = kt / KH;
-#pragma unroll
-          for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-            for (int hf = 0; hf < 2; ++hf) {
-              uint32_t hi2, lo2;
-              split2(acc[nt][2 * hf], acc[nt][2 * hf + 1], hi2, lo2);
-              const uint32_t o = ((g + hf * 8) * H + h) * RS + (wcol + nt * 8 + 2 * t) * 2;
-              *reinterpret_cast<uint32_t*>(Dm + o) = hi2;
-              if (NP == 2) *reinterpret_cast<uint32_t*>(Dm + plane + o) = lo2;
-              acc[nt][2 * hf] = acc[nt][2 * hf + 1] = 0.f;
-            }
-        }
-      }
-    }
+    if (dense) fold_heads(Thi, Tlo, weights(l, 2, 1), 1.f, Dm);      // dm_h = dt_h W_v[:, h]^T
     __syncthreads();
 #pragma unroll 1
     for (int sl = 0; sl < n_slots; ++sl) {
@@ -439,27 +424,40 @@ __global__ void __launch_bounds__(kTThreads, 2) gsta_train_kernel(const __grid_c
       if (cand >= c_end) continue;
       const int nch = (nv + kTRows - 1) / kTRows;
       if (nch > 0) stage_chunk(cand, 0, nv, 0);
-      // this layer's qt rows back from the slot rows; m . dm per head (lanes split the features)
-      const float* mg = P.G.Mh + l * NHd + (size_t)cand * H * d;
+      const bf16* mg = P.G.Mh + l * NHd + (size_t)cand * H * d;
+      bf16 *r0 = P.rows0 + ((size_t)cand * P.slots + l * 2 * H) * d, *r1 = P.rows1 + ((size_t)cand * P.slots + l * 2 * H) * d;
+      // this layer's qt rows back from the slot rows, and m . dm per head
       float dot0 = 0.f, dot1 = 0.f;                                  // heads 2t, 2t + 1
-      for (int h = 0; h < H; ++h) {
-        float v = 0.f;
-        for (int q = lane; q < 2 * D16; q += 32) {
-          const size_t at = ((size_t)cand * P.slots + l * 2 * H + h) * d + q * 8;
-          const uint32_t o = (c * H + h) * RS + q * 16;
-          *reinterpret_cast<uint4*>(Qt + o) = *reinterpret_cast<const uint4*>(P.rows0 + at);
-          if (NP == 2) *reinterpret_cast<uint4*>(Qt + plane + o) = *reinterpret_cast<const uint4*>(P.rows1 + at);
-          const float4 m0 = *reinterpret_cast<const float4*>(mg + h * d + q * 8), m1 = *reinterpret_cast<const float4*>(mg + h * d + q * 8 + 4);
+      auto piece_dot = [&](int h, int q, uint32_t o) {
+        *reinterpret_cast<uint4*>(Qt + o) = ld16(r0 + h * d + q * 8);
+        if (NP == 2) *reinterpret_cast<uint4*>(Qt + plane + o) = ld16(r1 + h * d + q * 8);
+        float m[8], y[8], v = 0.f;
+        unpack(m, ld16(mg + h * d + q * 8));
+        add_lo(m, ld16(mg + lo_h + h * d + q * 8));
+        unpack(y, ld16(Dm + o));
+        if (NP == 2) add_lo(y, ld16(Dm + plane + o));
 #pragma unroll
-          for (int pl = 0; pl < NP; ++pl) {
-            const uint4 x = *reinterpret_cast<const uint4*>(Dm + pl * plane + o);
-            v += m0.x * bf16_lo(x.x) + m0.y * bf16_hi(x.x) + m0.z * bf16_lo(x.y) + m0.w * bf16_hi(x.y) + m1.x * bf16_lo(x.z) +
-                 m1.y * bf16_hi(x.z) + m1.z * bf16_lo(x.w) + m1.w * bf16_hi(x.w);
-          }
+        for (int e = 0; e < 8; ++e) v = fmaf(m[e], y[e], v);
+        return v;
+      };
+      if constexpr ((D16 & (D16 - 1)) == 0) {                        // whole heads per step: sums over 2 D16 lanes
+        for (int i0 = 0; i0 < H * 2 * D16; i0 += 32) {
+          const int i = i0 + lane, h = i / (2 * D16), q = i % (2 * D16);
+          float v = h < H ? piece_dot(h, q, (uint32_t)((c * H + h) * RS + q * 16)) : 0.f;
+#pragma unroll
+          for (int o = 1; o < 2 * D16; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+          const int h0 = i0 / (2 * D16), per = 32 / (2 * D16);       // heads h0 .. h0 + per - 1 sit in lanes 0, 2 D16, ...
+          const float v0 = __shfl_sync(0xffffffffu, v, ((2 * t - h0) * 2 * D16) & 31), v1 = __shfl_sync(0xffffffffu, v, ((2 * t + 1 - h0) * 2 * D16) & 31);
+          if (2 * t >= h0 && 2 * t < h0 + per) dot0 = v0;
+          if (2 * t + 1 >= h0 && 2 * t + 1 < h0 + per) dot1 = v1;
         }
-        v = group_sum(quad_sum(v));
-        if (h == 2 * t) dot0 = v;
-        if (h == 2 * t + 1) dot1 = v;
+      } else {
+        for (int h = 0; h < H; ++h) {
+          float v = lane < 2 * D16 ? piece_dot(h, lane, (uint32_t)((c * H + h) * RS + lane * 16)) : 0.f;
+          v = group_sum(quad_sum(v));
+          if (h == 2 * t) dot0 = v;
+          if (h == 2 * t + 1) dot1 = v;
+        }
       }
       __syncwarp();
       float mx0 = 0.f, iv0 = 0.f, mx1 = 0.f, iv1 = 0.f;
@@ -489,8 +487,8 @@ __global__ void __launch_bounds__(kTThreads, 2) gsta_train_kernel(const __grid_c
           uint32_t a0[4], a1[4];
           ldsm_x4(a0, sb + a_off + kt * 32);
           if (NP == 2) ldsm_x4(a1, sb + kTRows * RS + a_off + kt * 32);
-          dot_tile(sb, kt, a0, a1, q0, q1, e);
-          dot_tile(sb, kt, a0, a1, d0, d1, da);
+          dot_tile(kt, a0, a1, q0, q1, e);
+          dot_tile(kt, a0, a1, d0, d1, da);
         }
         float a[4], de[4];
 #pragma unroll
@@ -505,9 +503,21 @@ __global__ void __launch_bounds__(kTThreads, 2) gsta_train_kernel(const __grid_c
         for (int hf = 0; hf < 2; ++hf) {
           const int j = ch * kTRows + g + hf * 8;
           if (j < nv) {
-            float* o = P.ad + ((size_t)cand * Lp + j) * P.slots + l * 2 * H;
-            if (2 * t < H) { o[2 * t] = de[2 * hf]; o[H + 2 * t] = a[2 * hf]; }
-            if (2 * t + 1 < H) { o[2 * t + 1] = de[2 * hf + 1]; o[H + 2 * t + 1] = a[2 * hf + 1]; }
+            const size_t at = ((size_t)cand * Lp + j) * P.slots + l * 2 * H + 2 * t;
+            if constexpr (NP == 1) {
+              if (H % 2 == 0) {                                      // (slot pairs of two heads: aligned)
+                if (2 * t < H) {
+                  *reinterpret_cast<uint32_t*>(P.ad16 + at) = pack2(de[2 * hf], de[2 * hf + 1]);
+                  *reinterpret_cast<uint32_t*>(P.ad16 + at + H) = pack2(a[2 * hf], a[2 * hf + 1]);
+                }
+              } else {
+                if (2 * t < H) { P.ad16[at] = __float2bfloat16_rn(de[2 * hf]); P.ad16[at + H] = __float2bfloat16_rn(a[2 * hf]); }
+                if (2 * t + 1 < H) { P.ad16[at + 1] = __float2bfloat16_rn(de[2 * hf + 1]); P.ad16[at + H + 1] = __float2bfloat16_rn(a[2 * hf + 1]); }
+              }
+            } else {
+              if (2 * t < H) { P.ad32[at] = de[2 * hf]; P.ad32[at + H] = a[2 * hf]; }
+              if (2 * t + 1 < H) { P.ad32[at + 1] = de[2 * hf + 1]; P.ad32[at + H + 1] = a[2 * hf + 1]; }
+            }
           }
         }
         weigh_chunk(sb, x, de[0], de[1], de[2], de[3]);
@@ -518,58 +528,73 @@ __global__ void __launch_bounds__(kTThreads, 2) gsta_train_kernel(const __grid_c
       // what the rounding of m leaves of sum_j de: taken out of every de_j (rho a_j), i.e. of dqt (rho m) and of the dm rows
       rho0 = group_sum(rho0);
       rho1 = group_sum(rho1);
+      auto rho_of = [&](int h) {                                     // (called by all lanes)
+        const float a0 = __shfl_sync(0xffffffffu, rho0, (h >> 1) & 3), a1 = __shfl_sync(0xffffffffu, rho1, (h >> 1) & 3);
+        return (h & 1) ? a1 : a0;
+      };
+      const int n_pieces = H * 2 * D16;
+      for (int i0 = 0; i0 < n_pieces; i0 += 32) {                    // dm rows
+        const int i = min(i0 + lane, n_pieces - 1), h = i / (2 * D16), q = i - h * (2 * D16);
+        const uint32_t o = (c * H + h) * RS + q * 16;
+        const float rho = rho_of(h);
+        float m[8], y[8];
+        unpack(m, ld16(Qt + o));
+        unpack(y, ld16(Dm + o));
+        if (NP == 2) { add_lo(m, ld16(Qt + plane + o)); add_lo(y, ld16(Dm + plane + o)); }
 #pragma unroll
-      for (int jt = 0; jt < D16; ++jt) {
-        const float* mp = mg + jt * 16 + g;
-        if (2 * t < H) { x[jt][0] -= rho0 * mp[2 * t * d]; x[jt][2] -= rho0 * mp[2 * t * d + 8]; }
-        if (2 * t + 1 < H) { x[jt][1] -= rho1 * mp[(2 * t + 1) * d]; x[jt][3] -= rho1 * mp[(2 * t + 1) * d + 8]; }
-      }
-      for (int h = 0; h < H; ++h) {
-        const float r0 = __shfl_sync(0xffffffffu, rho0, (h >> 1) & 3), r1 = __shfl_sync(0xffffffffu, rho1, (h >> 1) & 3);
-        const float rho = (h & 1) ? r1 : r0;
-        for (int q = lane; q < d / 2; q += 32) {
-          const uint32_t o = (c * H + h) * RS + q * 4;
-          const size_t at = ((size_t)cand * P.slots + l * 2 * H + H + h) * d + q * 2;
-          float2 q2 = make_float2(0.f, 0.f), m2 = make_float2(0.f, 0.f);
-#pragma unroll
-          for (int pl = 0; pl < NP; ++pl) {
-            const uint32_t qv = *reinterpret_cast<const uint32_t*>(Qt + pl * plane + o), mv = *reinterpret_cast<const uint32_t*>(Dm + pl * plane + o);
-            q2.x += bf16_lo(qv); q2.y += bf16_hi(qv);
-            m2.x += bf16_lo(mv); m2.y += bf16_hi(mv);
-          }
-          uint32_t hi, lo;
-          split2(m2.x - rho * q2.x, m2.y - rho * q2.y, hi, lo);
-          *reinterpret_cast<uint32_t*>(P.rows0 + at) = hi;
-          if (NP == 2) *reinterpret_cast<uint32_t*>(P.rows1 + at) = lo;
-        }
+        for (int e = 0; e < 8; ++e) y[e] = fmaf(-rho, m[e], y[e]);
+        uint4 hi, lo;
+        split8(y, hi, lo);
+        *reinterpret_cast<uint4*>(r0 + (H + h) * d + q * 8) = hi;
+        if (NP == 2) *reinterpret_cast<uint4*>(r1 + (H + h) * d + q * 8) = lo;
       }
       __syncwarp();
-      put_heads(c, x, 1.f, 1.f, P.G.dQt + l * NHd + (size_t)cand * H * d);
+      put_heads(c, x, 1.f, 1.f);
+      __syncwarp();
+      bf16* dg = P.G.dQt + l * NHd + (size_t)cand * H * d;
+      for (int i0 = 0; i0 < n_pieces; i0 += 32) {                    // dqt rows
+        const int i = i0 + lane, h = min(i / (2 * D16), H - 1), q = i % (2 * D16);
+        const float rho = rho_of(h);
+        if (i < n_pieces) {
+          const uint32_t o = (c * H + h) * RS + q * 16;
+          float m[8], y[8];
+          unpack(m, ld16(mg + h * d + q * 8));
+          add_lo(m, ld16(mg + lo_h + h * d + q * 8));
+          unpack(y, ld16(Qt + o));
+          add_lo(y, ld16(Xlo + o));
+#pragma unroll
+          for (int e = 0; e < 8; ++e) y[e] = fmaf(-rho, m[e], y[e]);
+          uint4 hi, lo;
+          split8(y, hi, lo);
+          *reinterpret_cast<uint4*>(Qt + o) = hi;
+          *reinterpret_cast<uint4*>(Xlo + o) = lo;
+          *reinterpret_cast<uint4*>(dg + h * d + q * 8) = hi;
+          *reinterpret_cast<uint4*>(dg + lo_h + h * d + q * 8) = lo;
+        }
+      }
     }
     __syncthreads();
     if (dense) {                                                     // dq_h = dqt_h W_k[:, h] / tau
       float acc[2][4] = {};
       from_heads(acc, weights(l, 1, 0));
-      put_rows(acc, P.inv_tau, P.G.dQ + l * Nd, true);
+      put_rows(acc, P.inv_tau, Qhi, Qlo, P.G.dQ + l * Nd, lo_d);
     }
     __syncthreads();
     if (dense) {                                                     // dt += dq W_q^T
-      float acc[2][4] = {};
-      const uint4* w = weights(l, 0, 1);
-#pragma unroll
-      for (int kt = 0; kt < D16; ++kt) {
-        const uint4 b = __ldg(w + kt * D16 * 32);
-        uint32_t hi[4], lo[4];
-        ldsm_x4(hi, smem_addr(Qhi + ldsm_row * RS + (kt * 2 + ldsm_kc) * 16));
-        ldsm_x4(lo, smem_addr(Qlo + ldsm_row * RS + (kt * 2 + ldsm_kc) * 16));
-        mma_pair(acc, hi, b);
-        mma_pair(acc, lo, b);
-      }
-      add_rows(acc);
+      from_rows(tr, Qhi, Qlo, weights(l, 0, 1));
+      if (l > 0) put_rows(tr, 1.f, Thi, Tlo, P.G.dT + (l - 1) * Nd, lo_d);
     }
     __syncthreads();
   }
-  save_rows(P.G.dT0);
+  if (dense) {
+#pragma unroll
+    for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+      for (int hf = 0; hf < 2; ++hf)
+        if (c_base + g + hf * 8 < c_end)
+          *reinterpret_cast<float2*>(P.G.dT0 + (size_t)(c_base + g + hf * 8) * d + wcol + nt * 8 + 2 * t) =
+              make_float2(tr[nt][2 * hf], tr[nt][2 * hf + 1]);
+  }
 
   // =============================================================================================== dH'
   // rows = segments, k = slots: A from the de / a array, B = the candidate's slot rows (staged once: slots <= 64)
@@ -592,14 +617,21 @@ __global__ void __launch_bounds__(kTThreads, 2) gsta_train_kernel(const __grid_c
     for (int j0 = 0; j0 < nv; j0 += kTRows) {
       uint32_t ah[4][4], al[4][4];
 #pragma unroll
-      for (int ks = 0; ks < 4; ++ks)
+      for (int ks = 0; ks < 4; ++ks) {
+        if (ks >= KS) break;
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
           const int j = j0 + g + (e & 1) * 8, s = ks * 16 + 2 * t + (e >> 1) * 8;
-          float2 v = make_float2(0.f, 0.f);
-          if (ks < KS && j < nv && s < P.slots) v = *reinterpret_cast<const float2*>(P.ad + ((size_t)cand * Lp + j) * P.slots + s);
-          split2(v.x, v.y, ah[ks][e], al[ks][e]);
+          const bool in = j < nv && s < P.slots;
+          const size_t at = ((size_t)cand * Lp + j) * P.slots + s;
+          if constexpr (NP == 1) {
+            ah[ks][e] = in ? *reinterpret_cast<const uint32_t*>(P.ad16 + at) : 0u;
+          } else {
+            const float2 v = in ? *reinterpret_cast<const float2*>(P.ad32 + at) : make_float2(0.f, 0.f);
+            split2(v.x, v.y, ah[ks][e], al[ks][e]);
+          }
         }
+      }
 #pragma unroll
       for (int jp = 0; jp < D16; ++jp) {
         float c0[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f};
@@ -610,7 +642,7 @@ __global__ void __launch_bounds__(kTThreads, 2) gsta_train_kernel(const __grid_c
           ldsm_x4_t(b, mine_a + ks * 16 * RS + s_trans + jp * 32);
           mma16816(c0, ah[ks][0], ah[ks][1], ah[ks][2], ah[ks][3], b[0], b[1]);
           mma16816(c1, ah[ks][0], ah[ks][1], ah[ks][2], ah[ks][3], b[2], b[3]);
-          if (NP == 2) {
+          if constexpr (NP == 2) {
             mma16816(c0, al[ks][0], al[ks][1], al[ks][2], al[ks][3], b[0], b[1]);
             mma16816(c1, al[ks][0], al[ks][1], al[ks][2], al[ks][3], b[2], b[3]);
             ldsm_x4_t(b, mine_a + (16 * KS + ks * 16) * RS + s_trans + jp * 32);
@@ -623,7 +655,7 @@ __global__ void __launch_bounds__(kTThreads, 2) gsta_train_kernel(const __grid_c
           const int j = j0 + g + hf * 8;
           if (j >= nv) continue;
           const size_t at = ((size_t)cand * Lp + j) * d + jp * 16 + 2 * t;
-          if (NP == 1) {
+          if constexpr (NP == 1) {
             *reinterpret_cast<uint32_t*>(P.dS16 + at) = pack2(c0[2 * hf], c0[2 * hf + 1]);
             *reinterpret_cast<uint32_t*>(P.dS16 + at + 8) = pack2(c1[2 * hf], c1[2 * hf + 1]);
           } else {
@@ -636,53 +668,61 @@ __global__ void __launch_bounds__(kTThreads, 2) gsta_train_kernel(const __grid_c
   }
 }
 
-// Weight gradients: C[m][n] += alpha sum_r A_h[r][m] B[r][n], h = the head of column n (A: [rows, heads, d], B: [rows, d]),
-// for up to 3 M arrays in one launch.  TF32 MMAs (operands rounded to nearest), fp32 sums of the whole d x d matrix in a
-// block's registers over its slice of the rows, one atomic add per element and block.
+// Weight gradients: C[m][n] += alpha sum_r A_h[r][m] B[r][n], h = the head of column n (A: [rows, heads, d], B: [rows, d],
+// both as bf16 high and low parts: three products per term), for up to kMaxSums arrays in one launch.  A block takes a slice
+// of the rows, KR at a time through two shared-memory buffers, and keeps the whole d x d sum in its registers: one atomic
+// add per element and block at the end.
 constexpr int kMaxSums = 24;
 struct SumList {
-  const float *A[kMaxSums], *B[kMaxSums];
+  const bf16 *A[kMaxSums], *B[kMaxSums];
+  size_t a_lo[kMaxSums], b_lo[kMaxSums];            // distance of the low parts, in elements
   float* C[kMaxSums];
   float alpha[kMaxSums];
   int heads[kMaxSums];
 };
-__device__ __forceinline__ uint32_t to_tf32(float v) {
-  uint32_t r;
-  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(v));
-  return r;
-}
 template <int D16>
 __global__ void __launch_bounds__(256, 2) weight_sums_kernel(const __grid_constant__ SumList L, int R, int rows_per_block, int KR,
                                                              int dvh) {
-  constexpr int d = 16 * D16, kParts = 8 / D16 > 0 ? 8 / D16 : 1;    // warps that share a row tile split the rows
+  constexpr int d = 16 * D16, kParts = 8 / D16 > 0 ? 8 / D16 : 1, kPairs = (D16 + kParts - 1) / kParts;
   extern __shared__ __align__(128) uint8_t smem[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
-  const float *A = L.A[blockIdx.y], *B = L.B[blockIdx.y];
-  const int heads = L.heads[blockIdx.y], lda = heads * d, pa = lda + 8, pb = d + 8;
+  const bf16 *A = L.A[blockIdx.y], *B = L.B[blockIdx.y];
+  const size_t a_lo = L.a_lo[blockIdx.y], b_lo = L.b_lo[blockIdx.y];
+  const int heads = L.heads[blockIdx.y], lda = heads * d, AS = 2 * lda + 16, BS = 2 * d + 16;
   const int hw = heads == 1 ? d : dvh;                               // columns of a head
-  float* buf0 = reinterpret_cast<float*>(smem);
-  const int buf_words = KR * (pa + pb);
-  const int mtile = warp % D16, part = warp / D16;
+  const uint32_t a_plane = KR * AS, b_plane = KR * BS, buf_bytes = 2 * (a_plane + b_plane);
+  const uint32_t base = smem_addr(smem);
+  const int mtile = warp % D16, part = warp / D16;                   // 16 rows of C; column pairs part, part + kParts, ...
   const bool active = part < kParts;
-  float acc[2 * D16][4];
+  float acc[kPairs][2][4];
 #pragma unroll
-  for (int j = 0; j < 2 * D16; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
+  for (int j = 0; j < kPairs; ++j)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) acc[j][0][e] = acc[j][1][e] = 0.f;
   const int r_lo = blockIdx.x * rows_per_block, r_hi = min(R, r_lo + rows_per_block);
+  if (r_lo >= r_hi) return;
   auto stage = [&](int r0, int b) {
-    float* As = buf0 + b * buf_words;
-    float* Bs = As + KR * pa;
-    const int ca = lda / 4, cb = d / 4;
+    const uint32_t dst = base + b * buf_bytes;
+    const int ca = lda / 8, cb = d / 8;
     for (int i = tid; i < KR * ca; i += 256) {
       const int rr = i / ca, c = i - rr * ca;
-      cp16(smem_addr(As + rr * pa + c * 4), A + (size_t)min(r0 + rr, r_hi - 1) * lda + c * 4, r0 + rr < r_hi ? 16u : 0u);
+      const uint32_t n = r0 + rr < r_hi ? 16u : 0u;
+      const bf16* src = A + (size_t)min(r0 + rr, r_hi - 1) * lda + c * 8;
+      cp16(dst + rr * AS + c * 16, src, n);
+      cp16(dst + a_plane + rr * AS + c * 16, src + a_lo, n);
     }
     for (int i = tid; i < KR * cb; i += 256) {
       const int rr = i / cb, c = i - rr * cb;
-      cp16(smem_addr(Bs + rr * pb + c * 4), B + (size_t)min(r0 + rr, r_hi - 1) * d + c * 4, r0 + rr < r_hi ? 16u : 0u);
+      const uint32_t n = r0 + rr < r_hi ? 16u : 0u;
+      const bf16* src = B + (size_t)min(r0 + rr, r_hi - 1) * d + c * 8;
+      cp16(dst + 2 * a_plane + rr * BS + c * 16, src, n);
+      cp16(dst + 2 * a_plane + b_plane + rr * BS + c * 16, src + b_lo, n);
     }
     cp_commit();
   };
-  if (r_lo >= r_hi) return;
+  const int mi = lane >> 3, lr = lane & 7;
+  const uint32_t a_off = ((mi >> 1) * 8 + lr) * AS + mtile * 32 + (mi & 1) * 16;      // A^T: rows = columns of A
+  const uint32_t b_off = ((mi & 1) * 8 + lr) * BS + (mi >> 1) * 16;
   stage(r_lo, 0);
   int b = 0;
   for (int r0 = r_lo; r0 < r_hi; r0 += KR, b ^= 1) {
@@ -693,25 +733,31 @@ __global__ void __launch_bounds__(256, 2) weight_sums_kernel(const __grid_consta
       cp_wait<0>();
     }
     __syncthreads();
-    const float* As = buf0 + b * buf_words;
-    const float* Bs = As + KR * pa;
+    const uint32_t as = base + b * buf_bytes + a_off, bs = base + b * buf_bytes + 2 * a_plane + b_off;
     if (active)
-      for (int k = part * 8; k < KR; k += kParts * 8) {
-        const float* ap = As + (k + t) * pa + mtile * 16 + g;
-        const float* bp = Bs + (k + t) * pb + g;
-        uint32_t a[4];
+      for (int k = 0; k < KR; k += 16) {
+        uint32_t ah[4], al[4];
+        int head = -1;
 #pragma unroll
-        for (int j = 0; j < 2 * D16; ++j) {
-          if ((j * 8) % hw == 0) {                                   // first column tile of a head
-            const float* q = ap + (j * 8) / hw * d;
-            a[0] = to_tf32(q[0]); a[1] = to_tf32(q[8]);
-            a[2] = to_tf32(q[4 * pa]); a[3] = to_tf32(q[4 * pa + 8]);
+        for (int j = 0; j < kPairs; ++j) {
+          const int p = part + kParts * j;
+          if (p < D16) {
+            const int h = p * 16 / hw;
+            if (h != head) {
+              head = h;
+              ldsm_x4_t(ah, as + k * AS + h * (2 * d));
+              ldsm_x4_t(al, as + a_plane + k * AS + h * (2 * d));
+            }
+            uint32_t bh[4], bl[4];
+            ldsm_x4_t(bh, bs + k * BS + p * 32);
+            ldsm_x4_t(bl, bs + b_plane + k * BS + p * 32);
+            mma16816(acc[j][0], ah[0], ah[1], ah[2], ah[3], bh[0], bh[1]);
+            mma16816(acc[j][1], ah[0], ah[1], ah[2], ah[3], bh[2], bh[3]);
+            mma16816(acc[j][0], al[0], al[1], al[2], al[3], bh[0], bh[1]);
+            mma16816(acc[j][1], al[0], al[1], al[2], al[3], bh[2], bh[3]);
+            mma16816(acc[j][0], ah[0], ah[1], ah[2], ah[3], bl[0], bl[1]);
+            mma16816(acc[j][1], ah[0], ah[1], ah[2], ah[3], bl[2], bl[3]);
           }
-          const uint32_t b0 = to_tf32(bp[j * 8]), b1 = to_tf32(bp[j * 8 + 4 * pb]);
-          asm volatile(
-              "mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-              : "+f"(acc[j][0]), "+f"(acc[j][1]), "+f"(acc[j][2]), "+f"(acc[j][3])
-              : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
         }
       }
     __syncthreads();
@@ -720,16 +766,23 @@ __global__ void __launch_bounds__(256, 2) weight_sums_kernel(const __grid_consta
   float* C = L.C[blockIdx.y];
   const float alpha = L.alpha[blockIdx.y];
 #pragma unroll
-  for (int j = 0; j < 2 * D16; ++j)
+  for (int j = 0; j < kPairs; ++j) {
+    const int p = part + kParts * j;
+    if (p < D16) {
 #pragma unroll
-    for (int e = 0; e < 4; ++e)
-      atomicAdd(C + (size_t)(mtile * 16 + g + (e >> 1) * 8) * d + j * 8 + 2 * t + (e & 1), alpha * acc[j][e]);
+      for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          atomicAdd(C + (size_t)(mtile * 16 + g + (e >> 1) * 8) * d + p * 16 + nt * 8 + 2 * t + (e & 1), alpha * acc[j][nt][e]);
+    }
+  }
 }
 
 struct TrainScratch {
   uint4* img;
   int *nseg, *order, *keys;
-  float *stat, *ad;
+  float *stat, *ad32;
+  bf16* ad16;
   bf16 *rows0, *rows1;
   size_t total;
 };
@@ -747,7 +800,8 @@ TrainScratch carve_train(const Plan& p, int np, char* base) {
   s.order = (int*)take(blocks * sizeof(int));
   s.keys = (int*)take(blocks * sizeof(int));
   s.stat = (float*)take((size_t)p.M * N * p.H * 2 * sizeof(float));
-  s.ad = (float*)take(N * p.Lp * slots * sizeof(float));
+  s.ad16 = np == 1 ? (bf16*)take(N * p.Lp * slots * sizeof(bf16)) : nullptr;
+  s.ad32 = np == 2 ? (float*)take(N * p.Lp * slots * sizeof(float)) : nullptr;
   s.rows0 = (bf16*)take(N * slots * p.d * sizeof(bf16));
   s.rows1 = np == 2 ? (bf16*)take(N * slots * p.d * sizeof(bf16)) : nullptr;
   s.total = off;
@@ -781,10 +835,10 @@ int launch_train(TrainParams P, const Plan& p, const TrainScratch& s, const void
 }
 
 template <int D16>
-int launch_sums(const Plan& p, const GstaTrain& G, float* dWg, cudaStream_t st) {
-  const size_t Nd = (size_t)p.N * p.d, dd = (size_t)p.d * p.d;
-  const size_t row = 2 * ((size_t)p.H * p.d + p.d + 16) * sizeof(float);
-  const int KR = row * 32 <= 110 * 1024 ? 32 : row * 16 <= 110 * 1024 ? 16 : 8;
+int launch_sums(const Plan& p, const GstaPlanes& G, float* dWg, cudaStream_t st) {
+  const size_t Nd = (size_t)p.N * p.d, dd = (size_t)p.d * p.d, lo_d = (size_t)p.M * Nd, lo_h = lo_d * p.H;
+  const size_t row = 2 * 2 * (2 * ((size_t)p.H * p.d + p.d) + 32);    // bytes per row in two buffers of two parts
+  const int KR = row * 32 <= 110 * 1024 ? 32 : 16;
   const size_t smem = row * KR;
   LASER_CUDA_OK(allow_smem(weight_sums_kernel<D16>, smem));
   for (int l0 = 0; l0 < p.M; l0 += kMaxSums / 3) {
@@ -792,13 +846,13 @@ int launch_sums(const Plan& p, const GstaTrain& G, float* dWg, cudaStream_t st) 
     int n = 0;
     for (int l = l0; l < p.M && n + 3 <= kMaxSums; ++l) {
       float *gWq = dWg + (size_t)(l * 3) * dd, *gWk = gWq + dd, *gWv = gWk + dd;
-      auto add = [&](const float* A, int heads, const float* B, float* C, float alpha) {
-        L.A[n] = A; L.B[n] = B; L.C[n] = C; L.alpha[n] = alpha; L.heads[n] = heads;
+      auto add = [&](const bf16* A, size_t a_lo, int heads, const bf16* B, float* C, float alpha) {
+        L.A[n] = A; L.a_lo[n] = a_lo; L.B[n] = B; L.b_lo[n] = lo_d; L.C[n] = C; L.alpha[n] = alpha; L.heads[n] = heads;
         ++n;
       };
-      add(G.Mh + l * Nd * p.H, p.H, G.dT + l * Nd, gWv, 1.f);
-      add(G.dQt + l * Nd * p.H, p.H, G.Q + l * Nd, gWk, p.inv_tau);
-      add(G.T + l * Nd, 1, G.dQ + l * Nd, gWq, 1.f);
+      add(G.Mh + l * Nd * p.H, lo_h, p.H, G.dT + l * Nd, gWv, 1.f);
+      add(G.dQt + l * Nd * p.H, lo_h, p.H, G.Q + l * Nd, gWk, p.inv_tau);
+      add(G.T + l * Nd, lo_d, 1, G.dQ + l * Nd, gWq, 1.f);
     }
     // about one wave of two blocks per SM over all sums
     const int want = std::max(1, 2 * device_sms() / n);
@@ -812,7 +866,7 @@ int launch_sums(const Plan& p, const GstaTrain& G, float* dWg, cudaStream_t st) 
 
 size_t train_smem(const Plan& p, int np) {
   const size_t RS = 2 * p.d + 16;
-  return (size_t)kTRows * (p.d + 8) * 4 + 2 * np * (size_t)kTRows * p.H * RS + RS + kTRows * sizeof(int) + 48 +
+  return 2 * (size_t)kTRows * RS + 2 * np * (size_t)kTRows * p.H * RS + RS + kTRows * sizeof(int) + 48 +
          (size_t)kTW * train_buffers(p, np) * kTRows * RS * np;
 }
 
@@ -838,20 +892,20 @@ size_t gsta_train_scratch_bytes(const Plan& p, int np) { return gsta_train_suppo
   }
 
 int gsta_train(const Plan& p, int np, const void* S0, const void* S1, const int32_t* lengths, const int32_t* cand_offsets,
-               const void* cands, const void* Wg, const float* dz, const GstaTrain& G, void* dS, char* scratch, cudaStream_t st) {
+               const void* cands, const void* Wg, const float* dz, const GstaPlanes& G, void* dS, char* scratch, cudaStream_t st) {
   const TrainScratch s = carve_train(p, np, scratch);
   TrainParams P = {};
   P.N = p.N; P.U = p.U; P.L = p.L; P.S = p.S; P.Lp = p.Lp; P.H = p.H; P.M = p.M; P.slots = 2 * p.M * p.H; P.nb = train_buffers(p, np);
   P.inv_tau = p.inv_tau;
   P.S0 = (const bf16*)S0; P.S1 = (const bf16*)S1; P.cands = (const bf16*)cands; P.dz = dz;
-  P.img = s.img; P.nseg = s.nseg; P.G = G; P.stat = s.stat; P.rows0 = s.rows0; P.rows1 = s.rows1; P.ad = s.ad;
+  P.img = s.img; P.nseg = s.nseg; P.G = G; P.stat = s.stat; P.rows0 = s.rows0; P.rows1 = s.rows1; P.ad16 = s.ad16; P.ad32 = s.ad32;
   P.dS16 = (bf16*)dS; P.dS32 = (float*)dS;
 #define LASER_TRAIN_CALL(D) (np == 1 ? launch_train<D, 1>(P, p, s, Wg, lengths, cand_offsets, st) : launch_train<D, 2>(P, p, s, Wg, lengths, cand_offsets, st))
   LASER_TRAIN_DISPATCH(LASER_TRAIN_CALL)
 #undef LASER_TRAIN_CALL
 }
 
-int gsta_weight_sums(const Plan& p, const GstaTrain& G, float* dWg, cudaStream_t st) {
+int gsta_weight_sums(const Plan& p, const GstaPlanes& G, float* dWg, cudaStream_t st) {
 #define LASER_TRAIN_CALL(D) launch_sums<D>(p, G, dWg, st)
   LASER_TRAIN_DISPATCH(LASER_TRAIN_CALL)
 #undef LASER_TRAIN_CALL
