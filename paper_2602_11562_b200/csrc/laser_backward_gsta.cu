@@ -89,7 +89,10 @@ __device__ __forceinline__ void split2(float x0, float x1, uint32_t& hi, uint32_
 template <int D16, int NP>
 struct TrainSmem {
   static constexpr int d = 16 * D16, RS = 2 * d + 16;
-  static __host__ __device__ constexpr size_t plane(int H) { return (size_t)kTRows * H * RS; }
+  // Bytes from one candidate's head rows to the next's: with an even number of heads 16 bytes more than the rows take, so that
+  // the same head of eight candidates (an operand of the dense products) lies in eight different 16-byte bank groups.
+  static __host__ __device__ constexpr uint32_t cand_pitch(int H) { return (uint32_t)(H * RS + (H % 2 ? 0 : 16)); }
+  static __host__ __device__ constexpr size_t plane(int H) { return (size_t)kTRows * cand_pitch(H); }
   static size_t bytes(int H, int nb) {
     return 2 * (size_t)kTRows * RS + 2 * NP * plane(H) + RS + kTRows * sizeof(int) + 48 + (size_t)kTW * nb * kTRows * RS * NP;
   }
@@ -101,11 +104,11 @@ __global__ void __launch_bounds__(kTThreads, 2) gsta_train_kernel(const __grid_c
   constexpr int d = SM::d, RS = SM::RS;
   extern __shared__ __align__(128) uint8_t smem[];
   const int H = P.H, Lp = P.Lp, dvh = d / H, KH = dvh >> 4;
-  const uint32_t plane = (uint32_t)SM::plane(H);
+  const uint32_t plane = (uint32_t)SM::plane(H), CP = SM::cand_pitch(H);
   uint8_t* Thi = smem;                                               // [16] rows: t, later dt, high and low parts (the fp32
   uint8_t* Tlo = Thi + kTRows * RS;                                  // values live in the registers of the columns' warp)
-  uint8_t* Qt = smem + 2 * kTRows * RS;                              // [NP][16][H] rows: qt; m or dqt (high) later
-  uint8_t* Dm = Qt + NP * plane;                                     // [NP][16][H] rows: dm; NP = 1: also m or dqt (low)
+  uint8_t* Qt = smem + 2 * kTRows * RS;                              // [NP][16] candidates' H rows: qt; m or dqt (high) later
+  uint8_t* Dm = Qt + NP * plane;                                     // [NP][16] candidates' H rows: dm; NP = 1: also m or dqt (low)
   uint8_t* Xlo = NP == 1 ? Dm : Qt + plane;                          // low parts of m / dqt (their high parts: Qt)
   uint8_t* zrow = Dm + NP * plane;
   int* nv_s = reinterpret_cast<int*>(zrow + RS);
@@ -136,9 +139,9 @@ __global__ void __launch_bounds__(kTThreads, 2) gsta_train_kernel(const __grid_c
     mma16816(acc[1], a[0], a[1], a[2], a[3], b.z, b.w);
   };
   const uint32_t ldsm_row = (lane & 7) + ((lane >> 3) & 1) * 8, ldsm_kc = lane >> 4;
-  // acc = x_h W with x rows (row r H + h of the planes hi, lo), h = the head of this warp's columns
+  // acc = x_h W with x rows (head rows of the planes), h = the head of this warp's columns
   auto from_heads = [&](float (&acc)[2][4], const uint4* w) {
-    const uint32_t o = (ldsm_row * H + wcol / dvh) * RS + ldsm_kc * 16;
+    const uint32_t o = ldsm_row * CP + wcol / dvh * RS + ldsm_kc * 16;
     const uint32_t ah = smem_addr(Qt) + o, al = smem_addr(Xlo) + o;
 #pragma unroll
     for (int kt = 0; kt < D16; ++kt) {
@@ -202,7 +205,7 @@ __global__ void __launch_bounds__(kTThreads, 2) gsta_train_kernel(const __grid_c
           for (int hf = 0; hf < 2; ++hf) {
             uint32_t vh, vl;
             split2(acc[nt][2 * hf] * scale, acc[nt][2 * hf + 1] * scale, vh, vl);
-            const uint32_t o = ((g + hf * 8) * H + h) * RS + (wcol + nt * 8 + 2 * t) * 2;
+            const uint32_t o = (g + hf * 8) * CP + h * RS + (wcol + nt * 8 + 2 * t) * 2;
             *reinterpret_cast<uint32_t*>(dst + o) = vh;
             if (NP == 2) *reinterpret_cast<uint32_t*>(dst + plane + o) = vl;
             acc[nt][2 * hf] = acc[nt][2 * hf + 1] = 0.f;
@@ -242,7 +245,7 @@ __global__ void __launch_bounds__(kTThreads, 2) gsta_train_kernel(const __grid_c
   const uint32_t t_off = ((lane & 7) + (lane >> 4) * 8) * RS + ((lane >> 3) & 1) * 16;       // S^T as [feature][segment]
   // B fragments of 8 head rows (row c H + h of a plane; heads past H read zeros)
   auto head_rows = [&](const uint8_t* base, int c) {
-    return smem_addr(((lane & 7) < H ? base + (c * H + (lane & 7)) * RS : zrow) + ((lane >> 3) & 1) * 16);
+    return smem_addr(((lane & 7) < H ? base + c * CP + (lane & 7) * RS : zrow) + ((lane >> 3) & 1) * 16);
   };
   // e += S x^T for one staged chunk, x = head rows at b0 (and b1: low parts)
   auto dot_tile = [&](int kt, const uint32_t (&a0)[4], const uint32_t (&a1)[4], uint32_t b0, uint32_t b1, float (&e)[4]) {
@@ -283,7 +286,7 @@ __global__ void __launch_bounds__(kTThreads, 2) gsta_train_kernel(const __grid_c
       split2(x[jt][2] * f0, x[jt][3] * f1, hb, lb);
       ha = movmatrix_t(ha); hb = movmatrix_t(hb); la = movmatrix_t(la); lb = movmatrix_t(lb);   // (head g, features 2t, 2t + 1)
       if (g < H) {
-        const uint32_t o = (c * H + g) * RS + jt * 32 + 4 * t;
+        const uint32_t o = c * CP + g * RS + jt * 32 + 4 * t;
         *reinterpret_cast<uint32_t*>(Qt + o) = ha;
         *reinterpret_cast<uint32_t*>(Qt + o + 16) = hb;
         *reinterpret_cast<uint32_t*>(Xlo + o) = la;
@@ -295,7 +298,7 @@ __global__ void __launch_bounds__(kTThreads, 2) gsta_train_kernel(const __grid_c
   auto pieces = [&](int c, auto f) {
     for (int i = lane; i < H * 2 * D16; i += 32) {
       const int h = i / (2 * D16), q = i - h * (2 * D16);
-      f(h, q, (uint32_t)((c * H + h) * RS + q * 16));
+      f(h, q, (uint32_t)(c * CP + h * RS + q * 16));
     }
   };
   auto ld16 = [](const void* p) { return *reinterpret_cast<const uint4*>(p); };
@@ -443,7 +446,7 @@ __global__ void __launch_bounds__(kTThreads, 2) gsta_train_kernel(const __grid_c
       if constexpr ((D16 & (D16 - 1)) == 0) {                        // whole heads per step: sums over 2 D16 lanes
         for (int i0 = 0; i0 < H * 2 * D16; i0 += 32) {
           const int i = i0 + lane, h = i / (2 * D16), q = i % (2 * D16);
-          float v = h < H ? piece_dot(h, q, (uint32_t)((c * H + h) * RS + q * 16)) : 0.f;
+          float v = h < H ? piece_dot(h, q, (uint32_t)(c * CP + h * RS + q * 16)) : 0.f;
 #pragma unroll
           for (int o = 1; o < 2 * D16; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
           const int h0 = i0 / (2 * D16), per = 32 / (2 * D16);       // heads h0 .. h0 + per - 1 sit in lanes 0, 2 D16, ...
@@ -453,7 +456,7 @@ __global__ void __launch_bounds__(kTThreads, 2) gsta_train_kernel(const __grid_c
         }
       } else {
         for (int h = 0; h < H; ++h) {
-          float v = lane < 2 * D16 ? piece_dot(h, lane, (uint32_t)((c * H + h) * RS + lane * 16)) : 0.f;
+          float v = lane < 2 * D16 ? piece_dot(h, lane, (uint32_t)(c * CP + h * RS + lane * 16)) : 0.f;
           v = group_sum(quad_sum(v));
           if (h == 2 * t) dot0 = v;
           if (h == 2 * t + 1) dot1 = v;
@@ -535,7 +538,7 @@ __global__ void __launch_bounds__(kTThreads, 2) gsta_train_kernel(const __grid_c
       const int n_pieces = H * 2 * D16;
       for (int i0 = 0; i0 < n_pieces; i0 += 32) {                    // dm rows
         const int i = min(i0 + lane, n_pieces - 1), h = i / (2 * D16), q = i - h * (2 * D16);
-        const uint32_t o = (c * H + h) * RS + q * 16;
+        const uint32_t o = c * CP + h * RS + q * 16;
         const float rho = rho_of(h);
         float m[8], y[8];
         unpack(m, ld16(Qt + o));
@@ -556,7 +559,7 @@ __global__ void __launch_bounds__(kTThreads, 2) gsta_train_kernel(const __grid_c
         const int i = i0 + lane, h = min(i / (2 * D16), H - 1), q = i % (2 * D16);
         const float rho = rho_of(h);
         if (i < n_pieces) {
-          const uint32_t o = (c * H + h) * RS + q * 16;
+          const uint32_t o = c * CP + h * RS + q * 16;
           float m[8], y[8];
           unpack(m, ld16(mg + h * d + q * 8));
           add_lo(m, ld16(mg + lo_h + h * d + q * 8));
@@ -599,6 +602,7 @@ __global__ void __launch_bounds__(kTThreads, 2) gsta_train_kernel(const __grid_c
   // =============================================================================================== dH'
   // rows = segments, k = slots: A from the de / a array, B = the candidate's slot rows (staged once: slots <= 64)
   const int KS = (P.slots + 15) >> 4;
+  const bool staged = P.nb > KS;                                     // 16 staging rows are left beside the slot rows
   const int mi = lane >> 3, lr = lane & 7;
   const uint32_t s_trans = ((mi & 1) * 8 + lr) * RS + (mi >> 1) * 16;
 #pragma unroll 1
@@ -650,6 +654,14 @@ __global__ void __launch_bounds__(kTThreads, 2) gsta_train_kernel(const __grid_c
             mma16816(c1, ah[ks][0], ah[ks][1], ah[ks][2], ah[ks][3], b[2], b[3]);
           }
         }
+        if (NP == 1 && staged) {                                     // through shared memory: whole rows leave in 16-byte pieces
+          uint8_t* o = mine + 16 * KS * RS + g * RS + jp * 32 + 4 * t;
+          *reinterpret_cast<uint32_t*>(o) = pack2(c0[0], c0[1]);
+          *reinterpret_cast<uint32_t*>(o + 16) = pack2(c1[0], c1[1]);
+          *reinterpret_cast<uint32_t*>(o + 8 * RS) = pack2(c0[2], c0[3]);
+          *reinterpret_cast<uint32_t*>(o + 8 * RS + 16) = pack2(c1[2], c1[3]);
+          continue;
+        }
 #pragma unroll
         for (int hf = 0; hf < 2; ++hf) {
           const int j = j0 + g + hf * 8;
@@ -663,6 +675,16 @@ __global__ void __launch_bounds__(kTThreads, 2) gsta_train_kernel(const __grid_c
             *reinterpret_cast<float2*>(P.dS32 + at + 8) = make_float2(c1[2 * hf], c1[2 * hf + 1]);
           }
         }
+      }
+      if (NP == 1 && staged) {
+        __syncwarp();
+        bf16* out = P.dS16 + ((size_t)cand * Lp + j0) * d;
+#pragma unroll
+        for (int i = 0; i < D16; ++i) {
+          const int piece = i * 32 + lane, r = piece / (2 * D16), q = piece - r * (2 * D16);
+          if (j0 + r < nv) *reinterpret_cast<uint4*>(out + r * d + q * 8) = ld16(mine + (16 * KS + r) * RS + q * 16);
+        }
+        __syncwarp();
       }
     }
   }
@@ -866,7 +888,7 @@ int launch_sums(const Plan& p, const GstaPlanes& G, float* dWg, cudaStream_t st)
 
 size_t train_smem(const Plan& p, int np) {
   const size_t RS = 2 * p.d + 16;
-  return 2 * (size_t)kTRows * RS + 2 * np * (size_t)kTRows * p.H * RS + RS + kTRows * sizeof(int) + 48 +
+  return 2 * (size_t)kTRows * RS + 2 * np * (size_t)kTRows * (p.H * RS + (p.H % 2 ? 0 : 16)) + RS + kTRows * sizeof(int) + 48 +
          (size_t)kTW * train_buffers(p, np) * kTRows * RS * np;
 }
 

@@ -74,7 +74,10 @@ __global__ void __launch_bounds__(kGThreads, BPS) gsta_mma_kernel(GstaParams P) 
   float* Ts = reinterpret_cast<float*>(smem);                       // [16][TS]
   uint8_t* Qs = smem + kGT * TS * 4;                                // [16] rows: Q (bf16)
   uint8_t* Qt = Qs + kGT * RS;                                      // [16][H] rows: Qt, later m
-  uint8_t* zrow = Qt + kGT * H * RS;                                // one row of zeros
+  // Bytes from one candidate's head rows to the next's: with an even number of heads 16 more than the rows take, so that the
+  // same head of eight candidates (phase D's operand) lies in eight different 16-byte bank groups (4-way conflicts before).
+  const uint32_t CP = H * RS + (H % 2 ? 0 : 16);
+  uint8_t* zrow = Qt + kGT * CP;                                // one row of zeros
   int* nv_s = reinterpret_cast<int*>(zrow + RS);                    // [16] non-empty segments per candidate
   uint8_t* stage = reinterpret_cast<uint8_t*>(nv_s + kGT);          // [kGW][2][kChunk] rows
 
@@ -227,9 +230,9 @@ __global__ void __launch_bounds__(kGThreads, BPS) gsta_mma_kernel(GstaParams P) 
 #pragma unroll
             for (int nt = 0; nt < 2; ++nt) {
               const int col = p * 16 + nt * 8 + 2 * t;
-              *reinterpret_cast<uint32_t*>(Qt + (g * H + h) * RS + col * 2) =
+              *reinterpret_cast<uint32_t*>(Qt + g * CP + h * RS + col * 2) =
                   pack2(acc[nt][0] * P.inv_tau, acc[nt][1] * P.inv_tau);
-              *reinterpret_cast<uint32_t*>(Qt + ((g + 8) * H + h) * RS + col * 2) =
+              *reinterpret_cast<uint32_t*>(Qt + (g + 8) * CP + h * RS + col * 2) =
                   pack2(acc[nt][2] * P.inv_tau, acc[nt][3] * P.inv_tau);
               acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
             }
@@ -255,7 +258,7 @@ __global__ void __launch_bounds__(kGThreads, BPS) gsta_mma_kernel(GstaParams P) 
         uint32_t qb[D16][2];
         {
           const int h = lane & 7;
-          const uint8_t* qrow = (h < H ? Qt + (c * H + h) * RS : zrow) + ((lane >> 3) & 1) * 16;
+          const uint8_t* qrow = (h < H ? Qt + c * CP + h * RS : zrow) + ((lane >> 3) & 1) * 16;
 #pragma unroll
           for (int kt = 0; kt < D16; ++kt) ldsm_x2(qb[kt], smem_addr(qrow + kt * 32));
         }
@@ -305,7 +308,7 @@ __global__ void __launch_bounds__(kGThreads, BPS) gsta_mma_kernel(GstaParams P) 
         // m_h = (sum_j p_j s_j) / (sum_j p_j), stored as rows [head][feature] of the candidate's block
         const float s0 = group_sum(rs0), s1 = group_sum(rs1);
         const float i0 = s0 > 0.f ? 1.f / s0 : 0.f, i1 = s1 > 0.f ? 1.f / s1 : 0.f;   // no segment: m = 0 (o_l = 0)
-        uint8_t* dst = Qt + (c * H + g) * RS + 4 * t;
+        uint8_t* dst = Qt + c * CP + g * RS + 4 * t;
 #pragma unroll
         for (int jt = 0; jt < D16; ++jt) {
           const uint32_t lo = movmatrix_t(pack2(macc[jt][0] * i0, macc[jt][1] * i1));   // (head g, features 16 jt + 2t..)
@@ -329,7 +332,7 @@ __global__ void __launch_bounds__(kGThreads, BPS) gsta_mma_kernel(GstaParams P) 
 #pragma unroll
       for (int kt = 0; kt < D16; ++kt) {
         uint32_t a[4];
-        ldsm_x4(a, smem_addr(Qt + ((int)ldsm_row * H + h) * RS + (kt * 2 + ldsm_kc) * 16));
+        ldsm_x4(a, smem_addr(Qt + ldsm_row * CP + h * RS + (kt * 2 + ldsm_kc) * 16));
         mma16816(acc[0], a[0], a[1], a[2], a[3], wpre[kt].x, wpre[kt].y);
         mma16816(acc[1], a[0], a[1], a[2], a[3], wpre[kt].z, wpre[kt].w);
       }
@@ -366,7 +369,7 @@ __global__ void __launch_bounds__(kGThreads, BPS) gsta_mma_kernel(GstaParams P) 
 template <int D16>
 int launch_gsta(const GstaParams& P, cudaStream_t st) {
   constexpr int d = D16 * 16, RS = 2 * d + 16, TS = d + 8;
-  const size_t smem = (size_t)kGT * TS * 4 + (size_t)kGT * RS + (size_t)kGT * P.H * RS + RS + kGT * sizeof(int) +
+  const size_t smem = (size_t)kGT * TS * 4 + (size_t)kGT * RS + (size_t)kGT * (P.H * RS + (P.H % 2 ? 0 : 16)) + RS + kGT * sizeof(int) +
                       (size_t)kGW * 2 * kChunk * RS;
   const int sms = device_sms();
   const int blocks = (P.N + P.cpb - 1) / P.cpb;
