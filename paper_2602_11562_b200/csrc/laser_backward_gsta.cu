@@ -726,25 +726,26 @@ __global__ void __launch_bounds__(256, 2) weight_sums_kernel(const __grid_consta
   auto stage = [&](int r0, int b) {
     const uint32_t dst = base + b * buf_bytes;
     const int ca = lda / 8, cb = d / 8;
-    for (int i = tid; i < KR * ca; i += 256) {
-      const int rr = i / ca, c = i - rr * ca;
+    for (int rr = warp; rr < KR; rr += 8) {                          // a warp per row: no divisions by the run-time row width
       const uint32_t n = r0 + rr < r_hi ? 16u : 0u;
-      const bf16* src = A + (size_t)min(r0 + rr, r_hi - 1) * lda + c * 8;
-      cp16(dst + rr * AS + c * 16, src, n);
-      cp16(dst + a_plane + rr * AS + c * 16, src + a_lo, n);
-    }
-    for (int i = tid; i < KR * cb; i += 256) {
-      const int rr = i / cb, c = i - rr * cb;
-      const uint32_t n = r0 + rr < r_hi ? 16u : 0u;
-      const bf16* src = B + (size_t)min(r0 + rr, r_hi - 1) * d + c * 8;
-      cp16(dst + 2 * a_plane + rr * BS + c * 16, src, n);
-      cp16(dst + 2 * a_plane + b_plane + rr * BS + c * 16, src + b_lo, n);
+      const bf16 *sa = A + (size_t)min(r0 + rr, r_hi - 1) * lda, *sb = B + (size_t)min(r0 + rr, r_hi - 1) * d;
+      for (int c = lane; c < ca; c += 32) {
+        cp16(dst + rr * AS + c * 16, sa + c * 8, n);
+        cp16(dst + a_plane + rr * AS + c * 16, sa + a_lo + c * 8, n);
+      }
+      for (int c = lane; c < cb; c += 32) {
+        cp16(dst + 2 * a_plane + rr * BS + c * 16, sb + c * 8, n);
+        cp16(dst + 2 * a_plane + b_plane + rr * BS + c * 16, sb + b_lo + c * 8, n);
+      }
     }
     cp_commit();
   };
   const int mi = lane >> 3, lr = lane & 7;
   const uint32_t a_off = ((mi >> 1) * 8 + lr) * AS + mtile * 32 + (mi & 1) * 16;      // A^T: rows = columns of A
   const uint32_t b_off = ((mi & 1) * 8 + lr) * BS + (mi >> 1) * 16;
+  uint32_t head_at[kPairs];                                          // byte offset of each column pair's head in a row of A
+#pragma unroll
+  for (int j = 0; j < kPairs; ++j) head_at[j] = (uint32_t)min((part + kParts * j) * 16 / hw, heads - 1) * (2 * d);
   stage(r_lo, 0);
   int b = 0;
   for (int r0 = r_lo; r0 < r_hi; r0 += KR, b ^= 1) {
@@ -759,16 +760,13 @@ __global__ void __launch_bounds__(256, 2) weight_sums_kernel(const __grid_consta
     if (active)
       for (int k = 0; k < KR; k += 16) {
         uint32_t ah[4], al[4];
-        int head = -1;
 #pragma unroll
         for (int j = 0; j < kPairs; ++j) {
           const int p = part + kParts * j;
           if (p < D16) {
-            const int h = p * 16 / hw;
-            if (h != head) {
-              head = h;
-              ldsm_x4_t(ah, as + k * AS + h * (2 * d));
-              ldsm_x4_t(al, as + a_plane + k * AS + h * (2 * d));
+            if (j == 0 || head_at[j] != head_at[j > 0 ? j - 1 : 0]) {
+              ldsm_x4_t(ah, as + k * AS + head_at[j]);
+              ldsm_x4_t(al, as + a_plane + k * AS + head_at[j]);
             }
             uint32_t bh[4], bl[4];
             ldsm_x4_t(bh, bs + k * BS + p * 32);

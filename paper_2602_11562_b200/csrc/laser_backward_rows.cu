@@ -47,7 +47,7 @@ __device__ __forceinline__ int valid_rows(const RowsParams& P, int u) {
 }
 
 template <int D16>
-__global__ void __launch_bounds__(kRThreads) rows_project_kernel(const RowsParams P) {
+__global__ void __launch_bounds__(kRThreads, 2) rows_project_kernel(const RowsParams P) {
   constexpr int d = 16 * D16, XS = 2 * d + 16;
   extern __shared__ __align__(128) uint8_t smem[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
@@ -163,12 +163,14 @@ __global__ void __launch_bounds__(kRThreads) rows_grad_kernel(const RowsParams P
       const int r = i / (2 * D16), q = i - r * (2 * D16);
       cp16(smem_addr(Xs) + b * kRT * XS + r * XS + q * 16, r < rows ? P.X + (row0 + r) * d + q * 8 : P.X, r < rows ? 16u : 0u);
     }
-    for (int i = tid; i < kRT * (n / 8); i += kRThreads) {
-      const int r = i / (n / 8), c = (i - r * (n / 8)) * 8;
-      const uint32_t dst = smem_addr(Gs) + b * 2 * kRT * WS + r * WS + c * 2, bytes = r < rows ? 16u : 0u;
-      const size_t at = r < rows ? (c < P.na ? (row0 + r) * P.na + c : (row0 + r) * P.nb + c - P.na) : 0;
-      cp16(dst, (c < P.na ? P.Ahi : P.Bhi) + at, bytes);
-      cp16(dst + kRT * WS, (c < P.na ? P.Alo : P.Blo) + at, bytes);
+    for (int r = warp; r < kRT; r += kRThreads / 32) {               // a warp per row: no divisions by the run-time width
+      const uint32_t bytes = r < rows ? 16u : 0u, dst = smem_addr(Gs) + b * 2 * kRT * WS + r * WS;
+      const size_t row = r < rows ? row0 + r : 0;
+      for (int c = lane * 8; c < n; c += 256) {
+        const size_t at = c < P.na ? row * P.na + c : row * P.nb + c - P.na;
+        cp16(dst + c * 2, (c < P.na ? P.Ahi : P.Bhi) + at, bytes);
+        cp16(dst + kRT * WS + c * 2, (c < P.na ? P.Alo : P.Blo) + at, bytes);
+      }
     }
   };
   int job = next_job(blockIdx.x);

@@ -195,9 +195,10 @@ __global__ void __launch_bounds__(kBThreads) bs_fwd_kernel(BsParams P) {
 }
 
 // One product per (segment row, head) with a slice of W_v (staged once per block): to_y = 0: s[h] = r_h W_v[:, h]
-// (K = d, d / H columns); to_y = 1: y_h = ds[h] W_v[:, h]^T (K = d / H, d columns).  A warp takes 16 segments of a user.
+// (K = d, d / H columns); to_y = 1: y_h = ds[h] W_v[:, h]^T (K = d / H, d columns).  A warp takes one head of 16
+// segments of a user.
 template <int D16>
-__global__ void __launch_bounds__(256) bs_rows_kernel(BsParams P, int to_y) {
+__global__ void __launch_bounds__(256, 2) bs_rows_kernel(BsParams P, int to_y) {
   constexpr int d = 16 * D16, WS = 2 * d + 16;
   extern __shared__ __align__(128) uint8_t smem[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3, H = P.H, dvh = d / H;
@@ -209,17 +210,17 @@ __global__ void __launch_bounds__(256) bs_rows_kernel(BsParams P, int to_y) {
   cp_wait<0>();
   __syncthreads();
   const int tiles = (P.Lp + 15) >> 4;
-  const long long jobs = (long long)P.U * tiles;
+  const long long jobs = (long long)P.U * tiles * H;
   const uint32_t w = smem_addr(smem);
   const int mi = lane >> 3, lr = lane & 7;
   for (long long job = (long long)blockIdx.x * 8 + warp; job < jobs; job += (long long)gridDim.x * 8) {
-    const int u = (int)(job / tiles), i0 = (int)(job - (long long)u * tiles) * 16;
+    const int h = (int)(job % H), u = (int)(job / H / tiles), i0 = (int)(job / H - (long long)u * tiles) * 16;
     int len = 0;
     const int cand = one_candidate(P, u, &len);
     const int rows = (len + P.S - 1) / P.S - i0;
     if (cand < 0 || rows <= 0) continue;
     const size_t row0 = (size_t)cand * P.Lp + i0;
-    for (int h = 0; h < H; ++h) {
+    {
       const float* A = to_y ? P.ds + row0 * d + h * dvh : P.r + (row0 * H + h) * d;
       float* C = to_y ? P.y + (row0 * H + h) * d : P.s + row0 * d + h * dvh;
       const size_t lda = to_y ? d : (size_t)H * d, ldc = to_y ? (size_t)H * d : d;
@@ -227,28 +228,42 @@ __global__ void __launch_bounds__(256) bs_rows_kernel(BsParams P, int to_y) {
       float acc[2 * D16][4];
 #pragma unroll
       for (int j = 0; j < 2 * D16; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
+      // A four k-tiles at a time, all of their loads in flight together (one tile at a time, each with its own round trip to
+      // memory, took 107 us for r -> s and 80 us for ds -> y at 2048 users of 61 segments, d = 128)
+      constexpr int kAhead = D16 < 4 ? D16 : 4;
+#pragma unroll 1
+      for (int k0 = 0; k0 < KT; k0 += kAhead) {
+        float2 x[kAhead][4];
 #pragma unroll
-      for (int kt = 0; kt < D16; ++kt) {
-        if (kt >= KT) break;
-        uint32_t hi[4], lo[4];
+        for (int k = 0; k < kAhead; ++k)
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const int rr = g + (e & 1) * 8;
-          const float2 x = rr < rows ? *reinterpret_cast<const float2*>(A + rr * lda + kt * 16 + (e >> 1) * 8 + 2 * t)
-                                     : make_float2(0.f, 0.f);
-          hi[e] = pack2(x.x, x.y);
-          lo[e] = pack2(x.x - bf16_lo(hi[e]), x.y - bf16_hi(hi[e]));
-        }
+          for (int e = 0; e < 4; ++e) {
+            const int rr = g + (e & 1) * 8;
+            x[k][e] = rr < rows && k0 + k < KT
+                          ? *reinterpret_cast<const float2*>(A + rr * lda + (k0 + k) * 16 + (e >> 1) * 8 + 2 * t)
+                          : make_float2(0.f, 0.f);
+          }
 #pragma unroll
-        for (int np = 0; np < D16; ++np) {
-          if (np >= NP) break;
-          uint32_t b[4];
-          if (to_y) ldsm_x4(b, w + (np * 16 + (mi >> 1) * 8 + lr) * WS + (h * dvh + kt * 16 + (mi & 1) * 8) * 2);
-          else ldsm_x4_t(b, w + (kt * 16 + (mi & 1) * 8 + lr) * WS + (h * dvh + np * 16 + (mi >> 1) * 8) * 2);
-          mma16816(acc[2 * np], hi[0], hi[1], hi[2], hi[3], b[0], b[1]);
-          mma16816(acc[2 * np], lo[0], lo[1], lo[2], lo[3], b[0], b[1]);
-          mma16816(acc[2 * np + 1], hi[0], hi[1], hi[2], hi[3], b[2], b[3]);
-          mma16816(acc[2 * np + 1], lo[0], lo[1], lo[2], lo[3], b[2], b[3]);
+        for (int k = 0; k < kAhead; ++k) {
+          if (k0 + k >= KT) break;
+          const int kt = k0 + k;
+          uint32_t hi[4], lo[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            hi[e] = pack2(x[k][e].x, x[k][e].y);
+            lo[e] = pack2(x[k][e].x - bf16_lo(hi[e]), x[k][e].y - bf16_hi(hi[e]));
+          }
+#pragma unroll
+          for (int np = 0; np < D16; ++np) {
+            if (np >= NP) break;
+            uint32_t b[4];
+            if (to_y) ldsm_x4(b, w + (np * 16 + (mi >> 1) * 8 + lr) * WS + (h * dvh + kt * 16 + (mi & 1) * 8) * 2);
+            else ldsm_x4_t(b, w + (kt * 16 + (mi & 1) * 8 + lr) * WS + (h * dvh + np * 16 + (mi >> 1) * 8) * 2);
+            mma16816(acc[2 * np], hi[0], hi[1], hi[2], hi[3], b[0], b[1]);
+            mma16816(acc[2 * np], lo[0], lo[1], lo[2], lo[3], b[0], b[1]);
+            mma16816(acc[2 * np + 1], hi[0], hi[1], hi[2], hi[3], b[2], b[3]);
+            mma16816(acc[2 * np + 1], lo[0], lo[1], lo[2], lo[3], b[2], b[3]);
+          }
         }
       }
 #pragma unroll
@@ -472,6 +487,8 @@ __global__ void __launch_bounds__(256) bs_wv_kernel(BsParams P, int KR) {
   const int buf_words = KR * (pa + pb);
   const int mtile = warp % D16, part = warp / D16;
   const bool active = part < kParts;
+  uint32_t starts = 0;                                      // column tiles that open a head (no divisions in the loop)
+  for (int h = 0; h < H; ++h) starts |= 1u << (h * (dvh >> 3));
   float acc[2 * D16][4];
 #pragma unroll
   for (int j = 0; j < 2 * D16; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
@@ -494,13 +511,11 @@ __global__ void __launch_bounds__(256) bs_wv_kernel(BsParams P, int KR) {
     float* B = A + KR * pa;
     const size_t row0 = (size_t)cand * P.Lp + i0;
     const int rows = nv - i0, ca = H * d / 4, cb = d / 4;
-    for (int i = tid; i < KR * ca; i += 256) {
-      const int rr = i / ca, c = i - rr * ca;
-      cp16(smem_addr(A + rr * pa + c * 4), P.r + (row0 + min(rr, rows - 1)) * H * d + c * 4, rr < rows ? 16u : 0u);
-    }
-    for (int i = tid; i < KR * cb; i += 256) {
-      const int rr = i / cb, c = i - rr * cb;
-      cp16(smem_addr(B + rr * pb + c * 4), P.ds + (row0 + min(rr, rows - 1)) * d + c * 4, rr < rows ? 16u : 0u);
+    for (int rr = warp; rr < KR; rr += 8) {                 // a warp per row: no divisions by the run-time row width
+      const uint32_t n = rr < rows ? 16u : 0u;
+      const size_t at = row0 + min(rr, rows - 1);
+      for (int c = lane; c < ca; c += 32) cp16(smem_addr(A + rr * pa + c * 4), P.r + at * H * d + c * 4, n);
+      for (int c = lane; c < cb; c += 32) cp16(smem_addr(B + rr * pb + c * 4), P.ds + at * d + c * 4, n);
     }
   };
   bool have = next();
@@ -513,21 +528,31 @@ __global__ void __launch_bounds__(256) bs_wv_kernel(BsParams P, int KR) {
     cp_commit();
     cp_wait<1>();
     __syncthreads();
-    const float* A = buf0 + b * buf_words;
-    const float* B = A + KR * pa;
+    // every element is rounded to TF32 once, in place (eight warps read each of them: rounding at every read was half of
+    // the kernel's instructions)
+    {
+      uint4* q = reinterpret_cast<uint4*>(buf0 + b * buf_words);
+      for (int i = tid; i < buf_words / 4; i += 256) {
+        const uint4 v = q[i];
+        q[i] = make_uint4(tf32_bits(__uint_as_float(v.x)), tf32_bits(__uint_as_float(v.y)), tf32_bits(__uint_as_float(v.z)),
+                          tf32_bits(__uint_as_float(v.w)));
+      }
+      __syncthreads();
+    }
+    const uint32_t* A = reinterpret_cast<const uint32_t*>(buf0 + b * buf_words);
+    const uint32_t* B = A + KR * pa;
     if (active)
       for (int k = part * 8; k < KR; k += kParts * 8) {
-        const float* ap = A + (k + t) * pa + mtile * 16 + g;
-        const float* bp = B + (k + t) * pb + g;
+        const uint32_t* ap = A + (k + t) * pa + mtile * 16 + g;
+        const uint32_t* bp = B + (k + t) * pb + g;
         uint32_t a[4];
 #pragma unroll
         for (int j = 0; j < 2 * D16; ++j) {
-          if ((j * 8) % dvh == 0) {                         // first column tile of head h
-            const float* q = ap + (j * 8) / dvh * d;
-            a[0] = tf32_bits(q[0]); a[1] = tf32_bits(q[8]);
-            a[2] = tf32_bits(q[4 * pa]); a[3] = tf32_bits(q[4 * pa + 8]);
+          if (starts >> j & 1u) {                           // first column tile of the next head
+            a[0] = ap[0]; a[1] = ap[8]; a[2] = ap[4 * pa]; a[3] = ap[4 * pa + 8];
+            ap += d;
           }
-          const uint32_t b0 = tf32_bits(bp[j * 8]), b1 = tf32_bits(bp[j * 8 + 4 * pb]);
+          const uint32_t b0 = bp[j * 8], b1 = bp[j * 8 + 4 * pb];
           asm volatile(
               "mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
               : "+f"(acc[j][0]), "+f"(acc[j][1]), "+f"(acc[j][2]), "+f"(acc[j][3])
@@ -605,9 +630,9 @@ int bs_forward_t(const Plan& p, BsParams P, cudaStream_t st) {
   }
   const size_t smem = (size_t)p.d * (2 * p.d + 16);
   LASER_CUDA_OK(allow_smem(bs_rows_kernel<D16>, smem));
-  const long long jobs = (long long)p.U * ((p.Lp + 15) / 16);
+  const long long jobs = (long long)p.U * ((p.Lp + 15) / 16) * p.H;
   LaunchScope ls("bs_rows_s", st);
-  bs_rows_kernel<D16><<<(int)std::min<long long>((jobs + 7) / 8, 3 * device_sms()), 256, smem, st>>>(P, 0);
+  bs_rows_kernel<D16><<<(int)std::min<long long>((jobs + 7) / 8, 2 * device_sms()), 256, smem, st>>>(P, 0);
   LASER_CUDA_OK(cudaGetLastError());
   return LASER_OK;
 }
@@ -615,12 +640,12 @@ int bs_forward_t(const Plan& p, BsParams P, cudaStream_t st) {
 template <int D16>
 int bs_backward_t(const Plan& p, BsParams P, cudaStream_t st) {
   const int sms = device_sms(), parts = user_parts(p);
-  const long long jobs = (long long)p.U * ((p.Lp + 15) / 16);
+  const long long jobs = (long long)p.U * ((p.Lp + 15) / 16) * p.H;
   {
     const size_t smem = (size_t)p.d * (2 * p.d + 16);
     LASER_CUDA_OK(allow_smem(bs_rows_kernel<D16>, smem));
     LaunchScope ls("bs_rows_y", st);
-    bs_rows_kernel<D16><<<(int)std::min<long long>((jobs + 7) / 8, 3 * sms), 256, smem, st>>>(P, 1);
+    bs_rows_kernel<D16><<<(int)std::min<long long>((jobs + 7) / 8, 2 * sms), 256, smem, st>>>(P, 1);
   }
   {
     const int warp_bytes = (int)bwd_warp_bytes(p.d, p.H);
