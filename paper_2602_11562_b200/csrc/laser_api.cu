@@ -441,6 +441,7 @@ int laser_forward_ffn(const laser_config* cfg, const void* items, const int32_t*
   if (p.N == 0) return clear_status(p, ws, st);
   void* Hp = Hprime ? Hprime : (void*)(ws + p.off_hp);
   const bool side_images = p.M > 0 && p.path != LASER_PATH_SIMT && gsta_mma_supported(p);
+  p.zero_in_ffn = Hprime && p.path == LASER_PATH_TENSOR && ffn_on_tensor_cores(p, ffn->d_hidden);
   rc = run_sta(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, Hp, ws, st, side_images ? Wgsta : nullptr);
   if (rc != LASER_OK) return rc;
   rc = ffn_forward(p, ffn, Hp, lengths, cand_offsets, ws, ws + p.total, st);

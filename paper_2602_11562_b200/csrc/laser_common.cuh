@@ -28,6 +28,7 @@ struct Plan {
   int Lp, dqh, dvh;
   float inv_gamma, inv_tau;
   size_t esize;
+  bool zero_in_ffn;                // the FFN kernel writes the zero rows of empty segments, STA's extra kernel does not
   const int32_t* item_offsets;     // packed item layout: first row of every user ([U + 1]); null = padded [U, L, d]
   // workspace byte offsets
   size_t off_status;
@@ -166,6 +167,7 @@ int fusion_forward(const Plan& p, const void* Hprime, const void* z, const int32
 
 // Feed-forward refinement of H' (laser_ffn.cu); needs ffn_scratch_bytes(p, d_hidden) of scratch of its own.
 bool ffn_supported(const Plan& p, int hid);
+bool ffn_on_tensor_cores(const Plan& p, int hid);
 size_t ffn_scratch_bytes(const Plan& p, int hid);
 int ffn_forward(const Plan& p, const laser_ffn_params* f, void* H, const int32_t* lengths, const int32_t* cand_offsets,
                 char* ws, char* scratch, cudaStream_t st);

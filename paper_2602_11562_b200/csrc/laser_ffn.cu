@@ -30,8 +30,9 @@ using namespace ptx;
 constexpr int kRows = 128;            // rows per tile = MMA M = TMEM lanes
 constexpr int kChunk = 128;           // hidden units per step
 constexpr int kPairRows = 2 * kRows;  // two tiles share every weight chunk
-constexpr int kFfnThreads = 576;      // warp 0 weight producer + TMEM, warp 1 MMA issuer, warps 2-5 / 6-9 hidden-
-                                      // activation warpgroups of tile 0 / 1, warps 10-13 / 14-17 layer-norm warpgroups
+constexpr int kFfnThreads = 608;      // warp 0 weight producer + TMEM, warp 1 MMA issuer, warps 2-5 / 6-9 hidden-
+                                      // activation warpgroups of tile 0 / 1, warps 10-13 / 14-17 layer-norm warpgroups,
+                                      // warp 18 zero rows of empty segments (when the caller wants them)
 constexpr int kWStages = 3;
 constexpr int kFfnTmemCols = 512;     // acc2[t] at 128 t; acc1[t], then the hidden activations, at 256 + 128 t
 constexpr int kSimtRows = 8;
@@ -48,6 +49,7 @@ struct FfnParams {
   float* lnv;                                 // [3][d] fp32 copies of b_2, the layer norm's gain and its shift
   int* rowmap;                                // [N * Lp] compact row -> row of H' (first counters[0] entries valid)
   int* status;
+  int zero_empty;                             // also write the zero rows of empty segments
 };
 
 struct RowUser {
@@ -255,6 +257,18 @@ __global__ void __launch_bounds__(kFfnThreads, 1) ffn_tc_kernel(FfnParams P) {
     return __all_sync(0xffffffffu, done) != 0;
   };
 
+  if (warp == 18 && P.zero_empty) {
+    // Rows of H' of empty segments, candidates dealt over the blocks: this kernel is bound by its MMAs, so the stores ride
+    // along (64 x 256 candidates, 39 of 100 segments empty, d = 128: 25 us of a call as a kernel of its own).
+    for (int u = 0; u < P.U; ++u) {
+      const RowUser s = row_user(P, u);
+      const int n = (P.Lp - s.nseg) * (d >> 3);
+      for (int c = (bidx + G - s.c0 % G) % G; c < s.nc && n > 0; c += G) {
+        uint4* out = reinterpret_cast<uint4*>(P.H + ((size_t)(s.c0 + c) * P.Lp + s.nseg) * d);
+        for (int i = lane; i < n; i += 32) out[i] = make_uint4(0, 0, 0, 0);
+      }
+    }
+  }
   if (my_pairs > 0) {
     if (warp == 0) {
       // ------------------------------------------------------------------ weight chunks: L2 -> ring
@@ -418,7 +432,7 @@ __global__ void __launch_bounds__(kFfnThreads, 1) ffn_tc_kernel(FfnParams P) {
         if (it + 1 < my_pairs) publish_x();                // the next pair's rows are staged
       }
       cp_async_wait_all();
-    } else {
+    } else if (warp < 18) {
       // ------------------------------------------------------------------ layer-norm warp: rows 32 quad .. + 31 of tile t
       const int t = (warp - 10) >> 2, quad = warp & 3;
       const int r = quad * 32 + lane;                      // my row of the tile = my TMEM lane
@@ -685,10 +699,12 @@ size_t ffn_scratch_bytes(const Plan& p, int hid) {
          align_up((size_t)3 * p.d * sizeof(float)) + align_up((size_t)p.N * p.Lp * sizeof(int));
 }
 
+bool ffn_on_tensor_cores(const Plan& p, int hid) { return ffn_tc_supported(p, hid) && p.path != LASER_PATH_SIMT; }
+
 bool ffn_supported(const Plan& p, int hid) {
   if (hid < 1) return false;
   if ((long long)p.N * p.Lp >= (1ll << 31) - kPairRows) return false;
-  if (ffn_tc_supported(p, hid) && p.path != LASER_PATH_SIMT) return true;
+  if (ffn_on_tensor_cores(p, hid)) return true;
   if ((p.d * p.esize) % 16) return false;
   return ((size_t)2 * kSimtRows * p.d + (size_t)kSimtRows * hid) * sizeof(float) <= 200 * 1024;
 }
@@ -698,7 +714,7 @@ int ffn_forward(const Plan& p, const laser_ffn_params* f, void* H, const int32_t
   if (p.N == 0 || p.U == 0) return LASER_OK;
   const int hid = f->d_hidden;
   if (!ffn_supported(p, hid)) return LASER_ERR_UNSUPPORTED;
-  if (!(ffn_tc_supported(p, hid) && p.path != LASER_PATH_SIMT)) {
+  if (!ffn_on_tensor_cores(p, hid)) {
     if (p.dtype == LASER_F32) return ffn_simt<float>(p, f, H, lengths, cand_offsets, ws, scratch, st);
     return ffn_simt<bf16>(p, f, H, lengths, cand_offsets, ws, scratch, st);
   }
@@ -716,6 +732,7 @@ int ffn_forward(const Plan& p, const laser_ffn_params* f, void* H, const int32_t
   P.lnv = (float*)((char*)P.img2 + align_up((size_t)p.d * hid * 2));
   P.rowmap = (int*)((char*)P.lnv + align_up((size_t)3 * p.d * sizeof(float)));
   P.status = (int*)(ws + p.off_status);
+  P.zero_empty = p.zero_in_ffn ? 1 : 0;
   {
     LaunchScope ls("ffn_prep", st);
     LASER_CUDA_OK(launch_chained(ffn_prep_kernel, dim3(1 + 16), dim3(1024), 0, st, P, 1));

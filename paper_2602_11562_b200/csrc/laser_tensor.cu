@@ -1226,7 +1226,7 @@ int tensor_sta(const Plan& p, const void* items, const int32_t* lengths, const v
     const int use_tma = !P.item_off && P.IT >= 32 && encode_item_map(p, P.IT, items, &item_map) ? 1 : 0;
     LASER_CUDA_OK(launch_chained(tc_proj_kernel, dim3(P.proj_grid), dim3(kProjThreads), smem, st, P, item_map, use_tma));
   }
-  if (user_wants_hp) {
+  if (user_wants_hp && !p.zero_in_ffn) {
     LaunchScope ls("tc_zero_empty", st);
     LASER_CUDA_OK(launch_chained(tc_zero_empty_kernel, dim3(p.Lp, p.U), dim3(256), 0, st, P));
   }

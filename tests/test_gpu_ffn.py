@@ -165,3 +165,20 @@ def test_ffn_many_users_and_no_rows_at_all():
     P.laser_ffn_forward(b0.cfg, _ffn_dev(fw, torch.bfloat16), H0, b0.lengths, b0.cand_offsets, workspace=ws0)
     assert P.laser_check_status(ws0) == 0
     assert bool((H0 == SENTINEL).all())
+
+
+@pytest.mark.parametrize("U,C", [(3, 5), (2, 300)])
+def test_full_stack_writes_zero_rows_of_empty_segments(U, C):
+    """The FFN kernel writes them (fewer and more candidates than blocks; an empty and a full user)."""
+    lengths = [0, 64, 17][:U] if U == 3 else [33, 64]
+    w = make_custom(U=U, C=C, L=64, d=64, H=2, S=8, M=1, dtype="bf16", seed=4400 + C, lengths=lengths)
+    fw = make_ffn_weights(64, 4, "bf16", seed=4)
+    b = P.DeviceBatch.from_workload(w, path=P.PATH_TENSOR)
+    fdev = {k: torch.from_numpy(v).to(torch.bfloat16).cuda() for k, v in fw.items()}
+    Hp = torch.full((w.N, 8, 64), 3.0, dtype=torch.bfloat16, device="cuda")
+    P.laser_forward_ffn(b.cfg, *b.args(), b.Wg, fdev, Hprime=Hp)
+    for u in range(U):
+        rows = Hp[u * C:(u + 1) * C]
+        n = -(-int(w.lengths[u]) // 8)
+        assert not rows[:, n:].any()
+        assert (rows[:, :n].float().abs().amax(dim=-1) > 0).all()
