@@ -46,10 +46,19 @@ __device__ __forceinline__ int valid_rows(const RowsParams& P, int u) {
   return len <= 0 || len > P.rows_per_group || o0 < 0 || o1 <= o0 || o1 > P.N ? 0 : len;
 }
 
+// The same from a table in shared memory, when the groups fit (the walks below ask for every tile they pass).
+constexpr int kTableGroups = 256;
+__device__ __forceinline__ void fill_table(const RowsParams& P, int* table, int tid) {
+  if (P.groups <= kTableGroups)
+    for (int u = tid; u < P.groups; u += kRThreads) table[u] = valid_rows(P, u);
+  __syncthreads();
+}
+
 template <int D16>
 __global__ void __launch_bounds__(kRThreads, 2) rows_project_kernel(const RowsParams P) {
   constexpr int d = 16 * D16, XS = 2 * d + 16;
   extern __shared__ __align__(128) uint8_t smem[];
+  __shared__ int table[kTableGroups];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
   const int n = P.na + P.nb, WS = 2 * n + 16;                        // bytes per row of [W_a | W_b] and of the output tile
   uint8_t* Ws = smem;                                                // [d][WS]
@@ -59,9 +68,14 @@ __global__ void __launch_bounds__(kRThreads, 2) rows_project_kernel(const RowsPa
     const int k = i / (n / 8), c = (i - k * (n / 8)) * 8;
     cp16(smem_addr(Ws) + k * WS + c * 2, c < P.na ? P.Wa + (size_t)k * P.na + c : P.Wb + (size_t)k * P.nb + c - P.na, 16u);
   }
+  fill_table(P, table, tid);
   const int jobs = P.groups * P.tiles_per_group;
   // job j = (tile j / groups, group j mod groups): the tiles that only long users have come last, spread over the blocks
-  auto rows_of = [&](int j) { return j < jobs ? valid_rows(P, j % P.groups) - j / P.groups * kRT : 0; };
+  auto rows_of = [&](int j) {
+    if (j >= jobs) return 0;
+    const int tile = j / P.groups, u = j - tile * P.groups;
+    return (P.groups <= kTableGroups ? table[u] : valid_rows(P, u)) - tile * kRT;
+  };
   auto next_job = [&](int j) {
     while (j < jobs && rows_of(j) <= 0) j += gridDim.x;
     return j;
@@ -141,6 +155,7 @@ template <int D16>
 __global__ void __launch_bounds__(kRThreads) rows_grad_kernel(const RowsParams P, int nbuf) {
   constexpr int d = 16 * D16, XS = 2 * d + 16, kParts = 16 / D16, kMaxPairs = (16 + kParts - 1) / kParts;
   extern __shared__ __align__(128) uint8_t smem[];
+  __shared__ int table[kTableGroups];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
   const int n = P.na + P.nb, WS = 2 * n + 16, pairs = n >> 4;
   uint8_t* Ws = smem;                                                // [d][WS]  [W_k | W_v]
@@ -150,8 +165,13 @@ __global__ void __launch_bounds__(kRThreads) rows_grad_kernel(const RowsParams P
     const int k = i / (n / 8), c = (i - k * (n / 8)) * 8;
     cp16(smem_addr(Ws) + k * WS + c * 2, c < P.na ? P.Wa + (size_t)k * P.na + c : P.Wb + (size_t)k * P.nb + c - P.na, 16u);
   }
+  fill_table(P, table, tid);
   const int jobs = P.groups * P.tiles_per_group;
-  auto rows_of = [&](int j) { return j < jobs ? valid_rows(P, j % P.groups) - j / P.groups * kRT : 0; };
+  auto rows_of = [&](int j) {
+    if (j >= jobs) return 0;
+    const int tile = j / P.groups, u = j - tile * P.groups;
+    return (P.groups <= kTableGroups ? table[u] : valid_rows(P, u)) - tile * kRT;
+  };
   auto next_job = [&](int j) {
     while (j < jobs && rows_of(j) <= 0) j += gridDim.x;
     return j;

@@ -317,8 +317,9 @@ __global__ void __launch_bounds__(kBThreads, 3) bs_bwd_kernel(BsParams P, int KS
   ring.y_bytes = H * d * 4;
   ring.len = len; ring.S = P.S; ring.nv = nv; ring.seg = blockIdx.y * kBW + warp; ring.stride = kBW * gridDim.y;
   ring.grp = 0; ring.lane = lane; ring.live = ring.seg < nv;
-  uint8_t* rows = mine + kBStages * ring.stage_bytes;       // u high [H], y high [H], u low [H], y low [H], one zero row
-  uint8_t* tile = rows + (4 * H + 1) * RS;                  // [16 KS] slots of 16 items
+  uint8_t* rows = mine + kBStages * ring.stage_bytes;       // u high [H], y high [H], u low [H], y low [H]
+  uint8_t* tile = rows + 4 * H * RS;                        // [16 KS] slots of 16 items
+  uint8_t* zero = smem + (size_t)kBW * warp_bytes;          // a zero row, one per block (two heads at d = 128: a third block fits)
   const int seg0 = ring.seg, stride = ring.stride;
 #pragma unroll
   for (int s = 0; s < kBStages - 1; ++s) ring.issue(s, P.items);
@@ -336,7 +337,7 @@ __global__ void __launch_bounds__(kBThreads, 3) bs_bwd_kernel(BsParams P, int KS
       *reinterpret_cast<uint32_t*>(dst + 2 * H * RS + 16) = ua[kt][3];
     }
   }
-  for (int i = lane; i < RS / 4; i += 32) reinterpret_cast<uint32_t*>(rows + 4 * H * RS)[i] = 0u;
+  for (int i = lane; i < RS / 4; i += 32) reinterpret_cast<uint32_t*>(zero)[i] = 0u;      // (every warp: the same zeros)
   for (int i = lane; i < 16 * KS * kSlotPitch / 4; i += 32) reinterpret_cast<uint32_t*>(tile)[i] = 0u;
   __syncwarp();
 
@@ -345,12 +346,13 @@ __global__ void __launch_bounds__(kBThreads, 3) bs_bwd_kernel(BsParams P, int KS
   const uint32_t off1 = ((lane & 7) + ((lane >> 4) & 1) * 8) * RS + ((lane >> 3) & 1) * 16;   // [item][k] operand
   const uint32_t off2 = ((lane & 7) + ((lane >> 3) & 1) * 8) * RS + (lane >> 4) * 16;         // [item][col], transposed
   // y as an A operand: rows 0-7 high parts, rows 8-15 low parts, heads past H read the zero row
-  const uint32_t y_row = rows_a + (lr < H ? ((mi & 1) ? 3 * H : H) + lr : 4 * H) * RS + (mi >> 1) * 16;
+  const uint32_t zero_a = smem_addr(zero);
+  const uint32_t y_row = (lr < H ? rows_a + (((mi & 1) ? 3 * H : H) + lr) * RS : zero_a) + (mi >> 1) * 16;
   uint32_t slot_row[3];                                     // this lane's row of the slot operand, per 16-slot step
 #pragma unroll
   for (int ks = 0; ks < 3; ++ks) {
     const int s = ks * 16 + (mi & 1) * 8 + lr;
-    slot_row[ks] = rows_a + (s >= 6 * H ? 4 * H : s < 2 * H ? s : s - 2 * H) * RS + (mi >> 1) * 16;
+    slot_row[ks] = (s >= 6 * H ? zero_a : rows_a + (s < 2 * H ? s : s - 2 * H) * RS) + (mi >> 1) * 16;
   }
   const uint32_t tile_ld = tile_a + ((mi >> 1) * 8 + lr) * kSlotPitch + (mi & 1) * 16;
   uint8_t* tile_st = tile + g * kSlotPitch + 4 * t;
@@ -573,7 +575,7 @@ __global__ void __launch_bounds__(256) bs_wv_kernel(BsParams P, int KR) {
 size_t ring_bytes(int d, int H, bool with_y) { return (size_t)kBRows * (2 * d + 16) + (with_y ? (size_t)H * d * 4 : 0); }
 int slot_steps(int H) { return (6 * H + 15) / 16; }
 size_t bwd_warp_bytes(int d, int H) {
-  return (kBStages * ring_bytes(d, H, true) + (size_t)(4 * H + 1) * (2 * d + 16) + (size_t)16 * slot_steps(H) * kSlotPitch + 127) / 128 * 128;
+  return (kBStages * ring_bytes(d, H, true) + (size_t)4 * H * (2 * d + 16) + (size_t)16 * slot_steps(H) * kSlotPitch + 127) / 128 * 128;
 }
 int wv_rows(int d, int H) {                                 // rows per step that keep two buffers within about 100 KB
   const size_t row = 2 * ((size_t)H * d + d + 16) * sizeof(float);
@@ -649,7 +651,7 @@ int bs_backward_t(const Plan& p, BsParams P, cudaStream_t st) {
   }
   {
     const int warp_bytes = (int)bwd_warp_bytes(p.d, p.H);
-    const size_t smem = (size_t)kBW * warp_bytes;
+    const size_t smem = (size_t)kBW * warp_bytes + 2 * p.d + 16;
     LASER_CUDA_OK(allow_smem(bs_bwd_kernel<D16>, smem));
     LASER_CUDA_OK(cudaMemsetAsync(P.p, 0, (size_t)p.N * p.H * p.d * sizeof(float), st));
     LaunchScope ls("bs_bwd", st);
@@ -670,7 +672,7 @@ int bs_backward_t(const Plan& p, BsParams P, cudaStream_t st) {
 
 bool backward_stream_supported(const Plan& p) {
   return p.dtype == LASER_BF16 && p.maxC <= 1 && p.d % 16 == 0 && p.d >= 16 && p.d <= 128 && p.H <= 8 && p.dvh % 16 == 0 &&
-         p.dqh % 16 == 0 && kBW * bwd_warp_bytes(p.d, p.H) <= 220 * 1024;
+         p.dqh % 16 == 0 && kBW * bwd_warp_bytes(p.d, p.H) + 2 * p.d + 16 <= 220 * 1024;
 }
 size_t backward_stream_scratch_bytes(const Plan& p) { return backward_stream_supported(p) ? carve_bs(p, nullptr).total : 0; }
 
