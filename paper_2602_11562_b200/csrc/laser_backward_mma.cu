@@ -390,10 +390,22 @@ __global__ void __launch_bounds__(kBwdWarps * 32) sta_fwd_mma_kernel(const FwdMm
         if (r0 < C) *reinterpret_cast<float2*>(P.Hp + at + (size_t)r0 * row + c) = make_float2(acc[j][0], acc[j][1]);
         if (r1 < C) *reinterpret_cast<float2*>(P.Hp + at + (size_t)r1 * row + c) = make_float2(acc[j][2], acc[j][3]);
       }
-      if (P.Hb) {
-        if (r0 < C) *reinterpret_cast<uint32_t*>(P.Hb + at + (size_t)r0 * row + c) = pack2(acc[j][0], acc[j][1]);
-        if (r1 < C) *reinterpret_cast<uint32_t*>(P.Hb + at + (size_t)r1 * row + c) = pack2(acc[j][2], acc[j][3]);
+      if (P.Hb) {                                                  // through shared memory: 16-byte pieces of a candidate's row
+        unsigned char* o = smem + P.rows * (KS + VS) + warp * 16 * VS + g * VS + c * 2;
+        *reinterpret_cast<uint32_t*>(o) = pack2(acc[j][0], acc[j][1]);
+        *reinterpret_cast<uint32_t*>(o + 8 * VS) = pack2(acc[j][2], acc[j][3]);
       }
+    }
+    if (P.Hb) {
+      __syncwarp();
+#pragma unroll
+      for (int i = 0; i < DV16; ++i) {
+        const int piece = i * 32 + lane, r = piece / (2 * DV16), q = piece - r * (2 * DV16);
+        if (c0 + r < C)
+          *reinterpret_cast<uint4*>(P.Hb + at + (size_t)(c0 + r) * row + q * 8) =
+              *reinterpret_cast<const uint4*>(smem + P.rows * (KS + VS) + warp * 16 * VS + r * VS + q * 16);
+      }
+      __syncwarp();
     }
   }
 }
@@ -423,7 +435,7 @@ int launch_mma(const BwdMmaParams& P, int U, cudaStream_t st) {
 constexpr size_t kFwdSmemMax = 160 * 1024;
 size_t fwd_smem(const Plan& p) {
   const size_t rows = (size_t)(std::min(p.S, p.L) + 15) / 16 * 16;
-  return rows * (2 * p.dqh + 16 + 2 * p.dvh + 16);
+  return rows * (2 * p.dqh + 16 + 2 * p.dvh + 16) + (size_t)kBwdWarps * 16 * (2 * p.dvh + 16);    // K and V rows, output tiles
 }
 
 template <int DQ16, int DV16>
