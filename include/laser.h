@@ -215,14 +215,15 @@ LASER_API int laser_sta_softmax_forward(const laser_config* cfg, const void* ite
  * cfg->dtype; the inputs are read in cfg->dtype.  The forward is recomputed and every intermediate kept in the workspace;
  * padded item layout only.  Two versions, chosen by cfg->path:
  *   LASER_PATH_SIMT                 FP32 ALUs throughout, either dtype: every gradient within 1e-4 of its largest entry.
- *   LASER_PATH_AUTO / _STREAM       fp32 batches as above.  bf16 batches on the tensor cores: every batched matrix product
- *                                   with TF32 operands and fp32 accumulation, and, when max_cands_per_user >= 8 and the head
- *                                   widths d_qk / H and d / H are multiples of 16 (d_qk / H at most 32, d / H at most 64), the
- *                                   five contractions through the gates, the recomputed H' and (d in {32, 64, 128}, at most 8
- *                                   heads and 128 segments) the GSTA attention with bf16 operands, as the forward's
- *                                   tensor-core path rounds them: every gradient within 2e-2 of its largest entry while the
- *                                   attention logits stay within a few nats (at tens of nats the bf16 rounding of a
- *                                   segment vector alone moves a softmax weight by several per cent: ask for the FP32 ALUs).
+ *   LASER_PATH_AUTO / _STREAM       fp32 batches as above.  bf16 batches on the tensor cores, fp32 accumulation throughout.
+ *                                   Candidate lists (max_cands_per_user >= 8, d_qk / H in {16, 32}, d / H in {16, 32, 64}): the
+ *                                   contractions through the gates, the recomputed H' and the attention itself with bf16
+ *                                   operands, as the forward's tensor-core path rounds them, the dense products with 16-bit
+ *                                   (bf16 pairs) or TF32 operands: every gradient within 2e-2 of its largest entry while the
+ *                                   attention logits stay within a few nats (at tens of nats the bf16 rounding of a segment
+ *                                   vector alone moves a softmax weight by several per cent: ask for the FP32 ALUs).  One
+ *                                   candidate per user: 16-bit or TF32 operands everywhere (2e-3).  Fewer than 8 candidates, or
+ *                                   other widths: FP32 gates and attention, TF32 products.
  *   LASER_PATH_TENSOR               as LASER_PATH_AUTO for bf16 batches; LASER_ERR_UNSUPPORTED for fp32 batches.
  *   dz          [N, d] fp32            IN
  *   d_items     [U, L, d] fp32         OUT (rows of padding are zero)
