@@ -216,7 +216,7 @@ KERNEL_SOURCE = {"sta_tc": "laser_tensor.cu", "tc_proj": "laser_tensor.cu", "gst
                  "stream_sta": "laser_stream.cu", "ffn_tc": "laser_ffn.cu"}
 OTHER_WORKLOADS = ("cfg1", "cfg2", "cfg2x32", "cfg3", "cfg4", "cfg5", "prod")      # entries of the `configs` array
 MAIN_KERNELS = ("sta_tc", "tc_proj", "gsta_mma", "stream_sta",      # kernels of the timed step (roofline candidates)
-                "proj_simt_q", "proj_simt_kv", "sta_simt", "gsta_simt")
+                "proj_simt", "sta_simt", "gsta_simt")
 
 
 def _source_digest(fname):
@@ -243,11 +243,11 @@ def kernel_roofline(w, name, ms, peaks):
     sec = ms * 1e-3
     src = "of measured" if peaks["_source"] == "measured" else "of fallback"
     traffic = ncu_traffic(name, w.spec.name)
-    if name.endswith("_simt") or "_simt_" in name:
+    if name.endswith("_simt"):
         # FP32-ALU path (the fp32 configuration): plain FMA arithmetic.  Peak = 148 SMs x 128 FP32 lanes x 2 flops x the
         # maximum SM clock (1965 MHz) = 74.4 TFLOP/s, derived from the unit counts, not measured.
         s = w.spec
-        flops = {"proj_simt_q": 2 * w.N * s.d * s.d_qk, "proj_simt_kv": work["proj_flops"], "sta_simt": work["attn_flops"],
+        flops = {"proj_simt": 2 * w.N * s.d * s.d_qk + work["proj_flops"], "sta_simt": work["attn_flops"],
                  "gsta_simt": work["gsta_flops"]}.get(name, 0)
         peak = 148 * 128 * 2 * 1.965e9 / 1e12
         achieved = flops / sec / 1e12
@@ -468,8 +468,8 @@ def backward_row(P, w, b, flush, stream, steps, peaks, dev):
     finally:
         P.laser_profile_enable(False)
     assert P.laser_check_status(bws) == 0
-    tensor = "bwd_gemm_tf32" in kernels
-    gates_tensor = "bwd_sta_mma" in kernels
+    tensor = bool({"bwd_gemm_tf32", "bwd_rows_grad", "bs_bwd"} & kernels.keys())
+    gates_tensor = bool({"bwd_sta_mma", "bs_bwd"} & kernels.keys())
     users = [u for u in range(s.U) if w.cand_offsets[u + 1] > w.cand_offsets[u]][:2]
     ref = backward_oracle.backward(w.items, w.lengths, w.cands, w.cand_offsets, w.Wq, w.Wk, w.Wv, w.Wg, s.S, s.H,
                                    dz.astype(np.float64), w.gamma, w.tau, users=users)
@@ -498,7 +498,7 @@ def backward_row(P, w, b, flush, stream, steps, peaks, dev):
     work = algorithmic_work(w)
     # forward recomputed once, then about two products per forward product: three times the forward's flops
     flops = 3.0 * (work["proj_flops"] + 2 * w.N * s.d * s.d_qk + work["attn_flops"] + work["gsta_flops"])
-    if tensor:      # matrix products in TF32, gate contractions in bf16: against the TF32 figure (the smaller of the two)
+    if tensor:      # matrix products of 16-bit or TF32 operands, gate contractions in bf16: against the TF32 figure
         peak = peaks["bf16_tflops"] * 1.1 / 2.25
         bound, source = "tensor", f"{peaks['_source']} bf16 GEMM peak x nominal tf32 : bf16 ratio (1.1 : 2.25)"
     else:
@@ -509,8 +509,8 @@ def backward_row(P, w, b, flush, stream, steps, peaks, dev):
             "bound": bound, "flops": flops, "achieved": ach, "peak": peak, "achieved_unit": "TFLOP/s", "frac": ach / peak,
             "peak_source": source,
             "parity": {"err_over_max": err, "tol": tol, "users_checked": len(users), "scores_checked": checked},
-            "matrix_products": "tensor cores (mma.sync, TF32 operands)" if tensor else "FP32 ALUs",
-            "gate_contractions": "tensor cores (mma.sync, bf16 operands)" if gates_tensor else "FP32 ALUs",
+            "matrix_products": "tensor cores (mma.sync, bf16 pairs or TF32 operands)" if tensor else "FP32 ALUs",
+            "gate_contractions": "tensor cores (mma.sync, bf16 operands or pairs)" if gates_tensor else "FP32 ALUs",
             "kernel_ms_first_call": {k: round(v, 4) for k, v in sorted(kernels.items())},
             "workspace_bytes": need}
 
