@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(kBwdWarps * 32, 2) sta_bwd_mma_kernel(const Bw
         mma16816(dKacc[mt][2 * k + 1], eA[mt][0], eA[mt][1], eA[mt][2], eA[mt][3], b[2], b[3]);
       }
     }
-    // dQf^T [key components] x [candidates] = K_h^T (dG w)^T: the B operand is the transposed 8 x 8 blocks of eA
+    // dQf [candidates] x [key components] = (dG w) K_h: A = the transposed 8 x 8 blocks of eA, B = the fragments of K_h^T
     float dQ[DQ16][2][4];
 #pragma unroll
     for (int q = 0; q < DQ16; ++q)
@@ -241,25 +241,29 @@ __global__ void __launch_bounds__(kBwdWarps * 32, 2) sta_bwd_mma_kernel(const Bw
 #pragma unroll
         for (int e = 0; e < 4; ++e) dQ[q][nt][e] = 0.f;
 #pragma unroll
-    for (int mt = 0; mt < MT; ++mt)
+    for (int mt = 0; mt < MT; ++mt) {
+      const uint32_t a0 = movmatrix_t(eA[mt][0]), a1 = movmatrix_t(eA[mt][2]), a2 = movmatrix_t(eA[mt][1]),
+                     a3 = movmatrix_t(eA[mt][3]);
 #pragma unroll
-      for (int nt = 0; nt < 2; ++nt) {
-        const uint32_t b0 = movmatrix_t(eA[mt][2 * nt]), b1 = movmatrix_t(eA[mt][2 * nt + 1]);
+      for (int q = 0; q < DQ16; ++q)
 #pragma unroll
-        for (int q = 0; q < DQ16; ++q) mma16816(dQ[q][nt], Kt[q][mt][0], Kt[q][mt][1], Kt[q][mt][2], Kt[q][mt][3], b0, b1);
-      }
+        for (int nt = 0; nt < 2; ++nt) mma16816(dQ[q][nt], a0, a1, a2, a3, Kt[q][mt][nt], Kt[q][mt][2 + nt]);
+    }
+    // Every segment adds into the same rows.  Neighbouring lanes trade halves, so that a lane owns four components of one
+    // candidate and adds them with one 16-byte reduction.
+    const int c = c0 + g + (t & 1) * 8;
 #pragma unroll
     for (int q = 0; q < DQ16; ++q)
 #pragma unroll
       for (int nt = 0; nt < 2; ++nt) {
-        const int c = c0 + nt * 8 + 2 * t, kq = q * 16 + g;
+        const float* v = dQ[q][nt];
+        const float o0 = __shfl_xor_sync(0xffffffffu, t & 1 ? v[0] : v[2], 1);
+        const float o1 = __shfl_xor_sync(0xffffffffu, t & 1 ? v[1] : v[3], 1);
         if (c < C) {
-          atomicAdd(dQg + (size_t)c * dqk + kq, 0.25f * dQ[q][nt][0]);
-          atomicAdd(dQg + (size_t)c * dqk + kq + 8, 0.25f * dQ[q][nt][2]);
-        }
-        if (c + 1 < C) {
-          atomicAdd(dQg + (size_t)(c + 1) * dqk + kq, 0.25f * dQ[q][nt][1]);
-          atomicAdd(dQg + (size_t)(c + 1) * dqk + kq + 8, 0.25f * dQ[q][nt][3]);
+          float* at = dQg + (size_t)c * dqk + q * 16 + nt * 8 + (t >> 1) * 4;
+          const bool odd = t & 1;
+          red_add4(at, 0.25f * (odd ? o0 : v[0]), 0.25f * (odd ? o1 : v[1]), 0.25f * (odd ? v[2] : o0),
+                   0.25f * (odd ? v[3] : o1));
         }
       }
     __syncwarp();                        // every lane is done with this buffer before the next request overwrites it

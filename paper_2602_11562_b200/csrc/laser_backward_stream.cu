@@ -52,14 +52,16 @@ struct BsParams {
 };
 
 // Candidate of user u (-1: none, or invalid inputs, which are reported) and the user's valid items.
-__device__ __forceinline__ int one_candidate(const BsParams& P, int u, int* len_out) {
-  const int c0 = P.cand_offsets[u], c1 = P.cand_offsets[u + 1], len = P.lengths[u];
+__device__ __forceinline__ int one_candidate(const BsParams& P, int c0, int c1, int len, int* len_out) {
   if (c0 < 0 || c1 < c0 || c1 > P.N || c1 - c0 > 1 || len < 0 || len > P.L) {
     report_status(P.status, LASER_ERR_BAD_INPUT);
     return -1;
   }
   *len_out = len;
   return c1 > c0 ? c0 : -1;
+}
+__device__ __forceinline__ int one_candidate(const BsParams& P, int u, int* len_out) {
+  return one_candidate(P, P.cand_offsets[u], P.cand_offsets[u + 1], P.lengths[u], len_out);
 }
 
 __device__ __forceinline__ float gate_of(float x) {
@@ -197,28 +199,47 @@ __global__ void __launch_bounds__(kBThreads) bs_fwd_kernel(BsParams P) {
 // One product per (segment row, head) with a slice of W_v (staged once per block): to_y = 0: s[h] = r_h W_v[:, h]
 // (K = d, d / H columns); to_y = 1: y_h = ds[h] W_v[:, h]^T (K = d / H, d columns).  A warp takes one head of 16
 // segments of a user.
+//
+// A job is (16-segment tile, user, head), tiles slowest and users in the launch order (longest first): the tiles that exist
+// are the first ones of each tile index, so the warps' shares are equal to within a job.  Candidate and segment count of a
+// user come from a table that the block fills once: looked up per job they were two dependent round trips to memory in front
+// of the rows' own.
+constexpr int kBsTable = 2048;
+
 template <int D16>
 __global__ void __launch_bounds__(256, 2) bs_rows_kernel(BsParams P, int to_y) {
   constexpr int d = 16 * D16, WS = 2 * d + 16;
   extern __shared__ __align__(128) uint8_t smem[];
+  __shared__ int2 table[kBsTable];                          // (candidate, segments) by launch position
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3, H = P.H, dvh = d / H;
   for (int i = tid; i < d * 2 * D16; i += 256) {
     const int row = i / (2 * D16), q = i - row * (2 * D16);
     cp16(smem_addr(smem) + row * WS + q * 16, P.Wv + (size_t)row * d + q * 8, 16u);
   }
   cp_commit();
+  auto look_up = [&](int pos) {
+    int len = 0;
+    const int cand = one_candidate(P, P.order ? min(max(P.order[pos], 0), P.U - 1) : pos, &len);
+    return make_int2(cand, cand >= 0 ? (len + P.S - 1) / P.S : 0);
+  };
+  const bool tabled = P.U <= kBsTable;
+  if (tabled)
+    for (int i = tid; i < P.U; i += 256) table[i] = look_up(i);
   cp_wait<0>();
   __syncthreads();
-  const int tiles = (P.Lp + 15) >> 4;
-  const long long jobs = (long long)P.U * tiles * H;
+  const int tiles = (P.Lp + 15) >> 4, stride = gridDim.x * 8;
   const uint32_t w = smem_addr(smem);
   const int mi = lane >> 3, lr = lane & 7;
-  for (long long job = (long long)blockIdx.x * 8 + warp; job < jobs; job += (long long)gridDim.x * 8) {
-    const int h = (int)(job % H), u = (int)(job / H / tiles), i0 = (int)(job / H - (long long)u * tiles) * 16;
-    int len = 0;
-    const int cand = one_candidate(P, u, &len);
-    const int rows = (len + P.S - 1) / P.S - i0;
-    if (cand < 0 || rows <= 0) continue;
+  // cursor (tile, position, head) instead of a job number: no divisions
+  const int step_h = stride % H, step_pos = stride / H;
+  int tile = 0, pos = (blockIdx.x * 8 + warp) / H, h = (blockIdx.x * 8 + warp) % H;
+  for (;; h += step_h, pos += step_pos + (h >= H), h -= h >= H ? H : 0) {
+    while (pos >= P.U) pos -= P.U, ++tile;
+    if (tile >= tiles) break;
+    const int i0 = tile * 16;
+    const int2 user = tabled ? table[pos] : look_up(pos);
+    const int cand = user.x, rows = user.y - i0;
+    if (rows <= 0) continue;
     const size_t row0 = (size_t)cand * P.Lp + i0;
     {
       const float* A = to_y ? P.ds + row0 * d + h * dvh : P.r + (row0 * H + h) * d;
@@ -473,7 +494,7 @@ __global__ void __launch_bounds__(kBThreads, 3) bs_bwd_kernel(BsParams P, int KS
 
 // dW_v[:, h] += sum over the non-empty segments of r_h^T ds[h]: TF32 MMAs (operands rounded to nearest), fp32 partial sums
 // of the whole d x d matrix in a block's registers, one atomic add per element and block.  The rows of a user's segments
-// arrive KR at a time by cp.async in two buffers (r: all heads; ds), zero rows past the user's last segment.
+// arrive KR at a time by cp.async in two buffers (r: all heads; ds), zero rows past the user's last segment up to a whole step.
 __device__ __forceinline__ uint32_t tf32_bits(float v) {
   uint32_t r;
   asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(v));
@@ -494,17 +515,30 @@ __global__ void __launch_bounds__(256) bs_wv_kernel(BsParams P, int KR) {
   float acc[2 * D16][4];
 #pragma unroll
   for (int j = 0; j < 2 * D16; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
-  // cursor over (user, chunk of KR segments)
-  int u = (int)blockIdx.x - (int)gridDim.x, i0 = 0, nv = 0, cand = -1;
+  // cursor over (user, chunk of KR segments).  Users in the launch order (longest first), dealt to the blocks there and back:
+  // every block gets about the same number of segments (in index order the busiest of 296 blocks had 1.4 times the mean).
+  // What the next user needs is requested while this one's segments are summed.
+  int round = 0, i0 = 0, nv = 0, cand = -1;
+  auto user_at = [&](int k) {                               // the k-th user of this block, -1 past the last
+    const long long pos = (long long)k * gridDim.x + (k & 1 ? gridDim.x - 1 - blockIdx.x : blockIdx.x);
+    return pos >= P.U ? -1 : P.order ? min(max(P.order[pos], 0), P.U - 1) : (int)pos;
+  };
+  int u1 = user_at(0), u2 = user_at(1), c0 = 0, c1 = 0, len1 = 0;     // the next user with its words, and the one after it
+  auto request = [&]() {
+    if (u1 >= 0) c0 = P.cand_offsets[u1], c1 = P.cand_offsets[u1 + 1], len1 = P.lengths[u1];
+  };
+  request();
   auto next = [&]() -> bool {                               // to the next chunk with rows; false past the last
     i0 += KR;
     while (i0 >= nv) {
-      u += gridDim.x;
-      if (u >= P.U) return false;
+      if (u1 < 0) return false;
       int len = 0;
-      cand = one_candidate(P, u, &len);
+      cand = one_candidate(P, c0, c1, len1, &len);
       nv = cand >= 0 ? (len + P.S - 1) / P.S : 0;
       i0 = 0;
+      u1 = u2;
+      request();
+      u2 = user_at(++round + 1);
     }
     return true;
   };
@@ -512,8 +546,8 @@ __global__ void __launch_bounds__(256) bs_wv_kernel(BsParams P, int KR) {
     float* A = buf0 + b * buf_words;
     float* B = A + KR * pa;
     const size_t row0 = (size_t)cand * P.Lp + i0;
-    const int rows = nv - i0, ca = H * d / 4, cb = d / 4;
-    for (int rr = warp; rr < KR; rr += 8) {                 // a warp per row: no divisions by the run-time row width
+    const int rows = nv - i0, ca = H * d / 4, cb = d / 4, used = min(KR, (rows + 7) & ~7);
+    for (int rr = warp; rr < used; rr += 8) {               // a warp per row: no divisions by the run-time row width
       const uint32_t n = rr < rows ? 16u : 0u;
       const size_t at = row0 + min(rr, rows - 1);
       for (int c = lane; c < ca; c += 32) cp16(smem_addr(A + rr * pa + c * 4), P.r + at * H * d + c * 4, n);
@@ -525,6 +559,7 @@ __global__ void __launch_bounds__(256) bs_wv_kernel(BsParams P, int KR) {
   cp_commit();
   int b = 0;
   while (have) {
+    const int used = min(KR, (nv - i0 + 7) & ~7);           // rows of this chunk in whole MMA steps
     have = next();
     if (have) stage(b ^ 1);
     cp_commit();
@@ -533,18 +568,22 @@ __global__ void __launch_bounds__(256) bs_wv_kernel(BsParams P, int KR) {
     // every element is rounded to TF32 once, in place (eight warps read each of them: rounding at every read was half of
     // the kernel's instructions)
     {
-      uint4* q = reinterpret_cast<uint4*>(buf0 + b * buf_words);
-      for (int i = tid; i < buf_words / 4; i += 256) {
-        const uint4 v = q[i];
-        q[i] = make_uint4(tf32_bits(__uint_as_float(v.x)), tf32_bits(__uint_as_float(v.y)), tf32_bits(__uint_as_float(v.z)),
-                          tf32_bits(__uint_as_float(v.w)));
-      }
+      auto round_rows = [&](float* rows, int words) {
+        uint4* q = reinterpret_cast<uint4*>(rows);
+        for (int i = tid; i < words / 4; i += 256) {
+          const uint4 v = q[i];
+          q[i] = make_uint4(tf32_bits(__uint_as_float(v.x)), tf32_bits(__uint_as_float(v.y)), tf32_bits(__uint_as_float(v.z)),
+                            tf32_bits(__uint_as_float(v.w)));
+        }
+      };
+      round_rows(buf0 + b * buf_words, used * pa);
+      round_rows(buf0 + b * buf_words + KR * pa, used * pb);
       __syncthreads();
     }
     const uint32_t* A = reinterpret_cast<const uint32_t*>(buf0 + b * buf_words);
     const uint32_t* B = A + KR * pa;
     if (active)
-      for (int k = part * 8; k < KR; k += kParts * 8) {
+      for (int k = part * 8; k < used; k += kParts * 8) {
         const uint32_t* ap = A + (k + t) * pa + mtile * 16 + g;
         const uint32_t* bp = B + (k + t) * pb + g;
         uint32_t a[4];

@@ -51,6 +51,11 @@ __device__ __forceinline__ uint32_t movmatrix_t(uint32_t a) {
   return d;
 }
 
+// Adds four floats to a 16-byte aligned place in global memory with one reduction.
+__device__ __forceinline__ void red_add4(float* at, float x, float y, float z, float w) {
+  asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(at), "f"(x), "f"(y), "f"(z), "f"(w) : "memory");
+}
+
 // 16-byte asynchronous global -> shared copy; src_bytes = 0 zero-fills the destination.
 __device__ __forceinline__ void cp16(uint32_t dst, const void* src, uint32_t src_bytes) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");

@@ -177,6 +177,7 @@ STREAM_CASES = [
     dict(U=640, C=1, L=40, d=64, H=2, S=10, M=2, dtype="bf16"),
     dict(U=7, C=1, L=330, d=128, H=8, S=10, M=3, dtype="bf16"),                              # 48 slots, three staging buffers
     dict(U=3000, C=1, L=24, d=32, H=1, S=8, M=1, dtype="bf16"),                              # 16 candidates per attention block
+    dict(U=2100, C=1, L=36, d=32, H=2, S=2, M=1, dtype="bf16"),                              # two row tiles, no table of users
 ]
 
 
