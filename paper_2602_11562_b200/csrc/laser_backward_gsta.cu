@@ -790,10 +790,7 @@ __global__ void __launch_bounds__(256, 2) weight_sums_kernel(const __grid_consta
     const int p = part + kParts * j;
     if (p < D16) {
 #pragma unroll
-      for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-          atomicAdd(C + (size_t)(mtile * 16 + g + (e >> 1) * 8) * d + p * 16 + nt * 8 + 2 * t + (e & 1), alpha * acc[j][nt][e]);
+      for (int nt = 0; nt < 2; ++nt) red_tile(C + (size_t)mtile * 16 * d + p * 16 + nt * 8, d, acc[j][nt], alpha, lane);
     }
   }
 }

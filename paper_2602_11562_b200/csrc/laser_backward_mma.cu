@@ -249,23 +249,11 @@ __global__ void __launch_bounds__(kBwdWarps * 32, 2) sta_bwd_mma_kernel(const Bw
 #pragma unroll
         for (int nt = 0; nt < 2; ++nt) mma16816(dQ[q][nt], a0, a1, a2, a3, Kt[q][mt][nt], Kt[q][mt][2 + nt]);
     }
-    // Every segment adds into the same rows.  Neighbouring lanes trade halves, so that a lane owns four components of one
-    // candidate and adds them with one 16-byte reduction.
-    const int c = c0 + g + (t & 1) * 8;
+    // every segment adds into the same rows
 #pragma unroll
     for (int q = 0; q < DQ16; ++q)
 #pragma unroll
-      for (int nt = 0; nt < 2; ++nt) {
-        const float* v = dQ[q][nt];
-        const float o0 = __shfl_xor_sync(0xffffffffu, t & 1 ? v[0] : v[2], 1);
-        const float o1 = __shfl_xor_sync(0xffffffffu, t & 1 ? v[1] : v[3], 1);
-        if (c < C) {
-          float* at = dQg + (size_t)c * dqk + q * 16 + nt * 8 + (t >> 1) * 4;
-          const bool odd = t & 1;
-          red_add4(at, 0.25f * (odd ? o0 : v[0]), 0.25f * (odd ? o1 : v[1]), 0.25f * (odd ? v[2] : o0),
-                   0.25f * (odd ? v[3] : o1));
-        }
-      }
+      for (int nt = 0; nt < 2; ++nt) red_tile(dQg + (size_t)c0 * dqk + q * 16 + nt * 8, dqk, dQ[q][nt], 0.25f, lane, C - c0);
     __syncwarp();                        // every lane is done with this buffer before the next request overwrites it
   }
 

@@ -300,13 +300,11 @@ __global__ void __launch_bounds__(kRThreads) rows_grad_kernel(const RowsParams P
     const int p = wpart + kParts * i;
     if (p < pairs) {
 #pragma unroll
-      for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const int m = mw * 16 + g + (e >> 1) * 8, c = p * 16 + nt * 8 + 2 * t + (e & 1);
-          if (c < P.na) atomicAdd(P.dWa + (size_t)m * P.na + c, wacc[i][nt][e]);
-          else atomicAdd(P.dWb + (size_t)m * P.nb + c - P.na, wacc[i][nt][e]);
-        }
+      for (int nt = 0; nt < 2; ++nt) {
+        const int c = p * 16 + nt * 8;
+        if (c < P.na) red_tile(P.dWa + (size_t)mw * 16 * P.na + c, P.na, wacc[i][nt], 1.f, lane);
+        else red_tile(P.dWb + (size_t)mw * 16 * P.nb + c - P.na, P.nb, wacc[i][nt], 1.f, lane);
+      }
     }
   }
 }

@@ -206,8 +206,10 @@ __global__ void __launch_bounds__(kBThreads) bs_fwd_kernel(BsParams P) {
 // of the rows' own.
 constexpr int kBsTable = 2048;
 
-template <int D16>
-__global__ void __launch_bounds__(256, 2) bs_rows_kernel(BsParams P, int to_y) {
+// (NPC: the most column pairs a head has; KA: k-tiles requested together.  Half a matrix of columns at most leaves the
+// registers for all of a row tile's k-tiles: r -> s 68 -> 58 us, with the high and low products interleaved.)
+template <int D16, int NPC, int KA, bool to_y>
+__global__ void __launch_bounds__(256, 2) bs_rows_kernel(BsParams P) {
   constexpr int d = 16 * D16, WS = 2 * d + 16;
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ int2 table[kBsTable];                          // (candidate, segments) by launch position
@@ -246,12 +248,12 @@ __global__ void __launch_bounds__(256, 2) bs_rows_kernel(BsParams P, int to_y) {
       float* C = to_y ? P.y + (row0 * H + h) * d : P.s + row0 * d + h * dvh;
       const size_t lda = to_y ? d : (size_t)H * d, ldc = to_y ? (size_t)H * d : d;
       const int KT = to_y ? dvh >> 4 : D16, NP = to_y ? D16 : dvh >> 4;      // 16-wide steps of K, pairs of column tiles
-      float acc[2 * D16][4];
+      float acc[2 * NPC][4];
 #pragma unroll
-      for (int j = 0; j < 2 * D16; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
-      // A four k-tiles at a time, all of their loads in flight together (one tile at a time, each with its own round trip to
+      for (int j = 0; j < 2 * NPC; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
+      // A several k-tiles at a time, all of their loads in flight together (one tile at a time, each with its own round trip to
       // memory, took 107 us for r -> s and 80 us for ds -> y at 2048 users of 61 segments, d = 128)
-      constexpr int kAhead = D16 < 4 ? D16 : 4;
+      constexpr int kAhead = D16 < KA ? D16 : KA;
 #pragma unroll 1
       for (int k0 = 0; k0 < KT; k0 += kAhead) {
         float2 x[kAhead][4];
@@ -275,20 +277,20 @@ __global__ void __launch_bounds__(256, 2) bs_rows_kernel(BsParams P, int to_y) {
             lo[e] = pack2(x[k][e].x - bf16_lo(hi[e]), x[k][e].y - bf16_hi(hi[e]));
           }
 #pragma unroll
-          for (int np = 0; np < D16; ++np) {
+          for (int np = 0; np < NPC; ++np) {
             if (np >= NP) break;
             uint32_t b[4];
             if (to_y) ldsm_x4(b, w + (np * 16 + (mi >> 1) * 8 + lr) * WS + (h * dvh + kt * 16 + (mi & 1) * 8) * 2);
             else ldsm_x4_t(b, w + (kt * 16 + (mi & 1) * 8 + lr) * WS + (h * dvh + np * 16 + (mi >> 1) * 8) * 2);
             mma16816(acc[2 * np], hi[0], hi[1], hi[2], hi[3], b[0], b[1]);
-            mma16816(acc[2 * np], lo[0], lo[1], lo[2], lo[3], b[0], b[1]);
             mma16816(acc[2 * np + 1], hi[0], hi[1], hi[2], hi[3], b[2], b[3]);
+            mma16816(acc[2 * np], lo[0], lo[1], lo[2], lo[3], b[0], b[1]);
             mma16816(acc[2 * np + 1], lo[0], lo[1], lo[2], lo[3], b[2], b[3]);
           }
         }
       }
 #pragma unroll
-      for (int j = 0; j < 2 * D16; ++j) {
+      for (int j = 0; j < 2 * NPC; ++j) {
         if (j >= 2 * NP) break;
         if (!to_y && !P.s) {
 #pragma unroll
@@ -493,8 +495,11 @@ __global__ void __launch_bounds__(kBThreads, 3) bs_bwd_kernel(BsParams P, int KS
 }
 
 // dW_v[:, h] += sum over the non-empty segments of r_h^T ds[h]: TF32 MMAs (operands rounded to nearest), fp32 partial sums
-// of the whole d x d matrix in a block's registers, one atomic add per element and block.  The rows of a user's segments
+// of the whole d x d matrix in a block's registers, one reduction per four elements and block.  The rows of a user's segments
 // arrive KR at a time by cp.async in two buffers (r: all heads; ds), zero rows past the user's last segment up to a whole step.
+// Bound by shared-memory reads: a warp takes two row tiles x half of the column tiles where their number is even (24 words per
+// lane and step for 16 MMAs, rounded as they are read; one row tile x all columns took 40 words and, with a pass that rounded
+// the buffers in place, 97 us instead of 68 at 2048 users of 61 segments, d = 128).
 __device__ __forceinline__ uint32_t tf32_bits(float v) {
   uint32_t r;
   asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(v));
@@ -508,13 +513,17 @@ __global__ void __launch_bounds__(256) bs_wv_kernel(BsParams P, int KR) {
   const int pa = H * d + 8, pb = d + 8;                     // row pitches in words (conflict-free fragment reads)
   float* buf0 = reinterpret_cast<float*>(smem);
   const int buf_words = KR * (pa + pb);
-  const int mtile = warp % D16, part = warp / D16;
+  constexpr int kM = D16 % 2 == 0 ? 2 : 1, kN = 2 * D16 / kM;        // row tiles and column tiles of a warp
+  const int mtile = warp % (D16 / kM) * kM, n0 = warp % D16 / (D16 / kM) * kN, part = warp / D16;
   const bool active = part < kParts;
   uint32_t starts = 0;                                      // column tiles that open a head (no divisions in the loop)
   for (int h = 0; h < H; ++h) starts |= 1u << (h * (dvh >> 3));
-  float acc[2 * D16][4];
+  const int h0 = n0 * 8 / dvh;
+  float acc[kM][kN][4];
 #pragma unroll
-  for (int j = 0; j < 2 * D16; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
+  for (int m = 0; m < kM; ++m)
+#pragma unroll
+    for (int j = 0; j < kN; ++j) acc[m][j][0] = acc[m][j][1] = acc[m][j][2] = acc[m][j][3] = 0.f;
   // cursor over (user, chunk of KR segments).  Users in the launch order (longest first), dealt to the blocks there and back:
   // every block gets about the same number of segments (in index order the busiest of 296 blocks had 1.4 times the mean).
   // What the next user needs is requested while this one's segments are summed.
@@ -565,39 +574,29 @@ __global__ void __launch_bounds__(256) bs_wv_kernel(BsParams P, int KR) {
     cp_commit();
     cp_wait<1>();
     __syncthreads();
-    // every element is rounded to TF32 once, in place (eight warps read each of them: rounding at every read was half of
-    // the kernel's instructions)
-    {
-      auto round_rows = [&](float* rows, int words) {
-        uint4* q = reinterpret_cast<uint4*>(rows);
-        for (int i = tid; i < words / 4; i += 256) {
-          const uint4 v = q[i];
-          q[i] = make_uint4(tf32_bits(__uint_as_float(v.x)), tf32_bits(__uint_as_float(v.y)), tf32_bits(__uint_as_float(v.z)),
-                            tf32_bits(__uint_as_float(v.w)));
-        }
-      };
-      round_rows(buf0 + b * buf_words, used * pa);
-      round_rows(buf0 + b * buf_words + KR * pa, used * pb);
-      __syncthreads();
-    }
-    const uint32_t* A = reinterpret_cast<const uint32_t*>(buf0 + b * buf_words);
-    const uint32_t* B = A + KR * pa;
+    const float* A = buf0 + b * buf_words;
+    const float* B = A + KR * pa;
     if (active)
       for (int k = part * 8; k < used; k += kParts * 8) {
-        const uint32_t* ap = A + (k + t) * pa + mtile * 16 + g;
-        const uint32_t* bp = B + (k + t) * pb + g;
-        uint32_t a[4];
+        const float* ap = A + (k + t) * pa + h0 * d + mtile * 16 + g;
+        const float* bp = B + (k + t) * pb + n0 * 8 + g;
+        uint32_t a[kM][4];
 #pragma unroll
-        for (int j = 0; j < 2 * D16; ++j) {
-          if (starts >> j & 1u) {                           // first column tile of the next head
-            a[0] = ap[0]; a[1] = ap[8]; a[2] = ap[4 * pa]; a[3] = ap[4 * pa + 8];
-            ap += d;
-          }
-          const uint32_t b0 = bp[j * 8], b1 = bp[j * 8 + 4 * pb];
-          asm volatile(
-              "mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-              : "+f"(acc[j][0]), "+f"(acc[j][1]), "+f"(acc[j][2]), "+f"(acc[j][3])
-              : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+        for (int j = 0; j < kN; ++j) {
+          const bool opens = j > 0 && (starts >> (n0 + j) & 1u);      // first column tile of the next head
+          if (opens) ap += d;
+          if (j == 0 || opens)
+#pragma unroll
+            for (int m = 0; m < kM; ++m)
+#pragma unroll
+              for (int e = 0; e < 4; ++e) a[m][e] = tf32_bits(ap[(e >> 1) * 4 * pa + m * 16 + (e & 1) * 8]);
+          const uint32_t b0 = tf32_bits(bp[j * 8]), b1 = tf32_bits(bp[j * 8 + 4 * pb]);
+#pragma unroll
+          for (int m = 0; m < kM; ++m)
+            asm volatile(
+                "mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                : "+f"(acc[m][j][0]), "+f"(acc[m][j][1]), "+f"(acc[m][j][2]), "+f"(acc[m][j][3])
+                : "r"(a[m][0]), "r"(a[m][1]), "r"(a[m][2]), "r"(a[m][3]), "r"(b0), "r"(b1));
         }
       }
     __syncthreads();
@@ -605,10 +604,9 @@ __global__ void __launch_bounds__(256) bs_wv_kernel(BsParams P, int KR) {
   }
   if (!active) return;
 #pragma unroll
-  for (int j = 0; j < 2 * D16; ++j)
+  for (int m = 0; m < kM; ++m)
 #pragma unroll
-    for (int e = 0; e < 4; ++e)
-      atomicAdd(P.dWv + (size_t)(mtile * 16 + g + (e >> 1) * 8) * d + j * 8 + 2 * t + (e & 1), acc[j][e]);
+    for (int j = 0; j < kN; ++j) red_tile(P.dWv + (size_t)(mtile + m) * 16 * d + (n0 + j) * 8, d, acc[m][j], 1.f, lane);
 }
 
 size_t ring_bytes(int d, int H, bool with_y) { return (size_t)kBRows * (2 * d + 16) + (with_y ? (size_t)H * d * 4 : 0); }
@@ -661,6 +659,17 @@ BsParams bs_params(const Plan& p, const BsScratch& s, const void* items, const i
   return P;
 }
 
+template <int D16, int NPC, int KA, bool to_y>
+int launch_rows(const Plan& p, const BsParams& P, cudaStream_t st) {
+  const size_t smem = (size_t)p.d * (2 * p.d + 16);
+  const long long jobs = (long long)p.U * ((p.Lp + 15) / 16) * p.H;
+  auto kernel = bs_rows_kernel<D16, NPC, KA, to_y>;
+  LASER_CUDA_OK(allow_smem(kernel, smem));
+  kernel<<<(int)std::min<long long>((jobs + 7) / 8, 2 * device_sms()), 256, smem, st>>>(P);
+  LASER_CUDA_OK(cudaGetLastError());
+  return LASER_OK;
+}
+
 template <int D16>
 int bs_forward_t(const Plan& p, BsParams P, cudaStream_t st) {
   {
@@ -669,24 +678,17 @@ int bs_forward_t(const Plan& p, BsParams P, cudaStream_t st) {
     LaunchScope ls("bs_fwd", st);
     bs_fwd_kernel<D16><<<dim3(p.U, user_parts(p)), kBThreads, smem, st>>>(P);
   }
-  const size_t smem = (size_t)p.d * (2 * p.d + 16);
-  LASER_CUDA_OK(allow_smem(bs_rows_kernel<D16>, smem));
-  const long long jobs = (long long)p.U * ((p.Lp + 15) / 16) * p.H;
   LaunchScope ls("bs_rows_s", st);
-  bs_rows_kernel<D16><<<(int)std::min<long long>((jobs + 7) / 8, 2 * device_sms()), 256, smem, st>>>(P, 0);
-  LASER_CUDA_OK(cudaGetLastError());
-  return LASER_OK;
+  return p.H > 1 ? launch_rows<D16, (D16 + 1) / 2, 8, false>(p, P, st) : launch_rows<D16, D16, 4, false>(p, P, st);
 }
 
 template <int D16>
 int bs_backward_t(const Plan& p, BsParams P, cudaStream_t st) {
   const int sms = device_sms(), parts = user_parts(p);
-  const long long jobs = (long long)p.U * ((p.Lp + 15) / 16) * p.H;
   {
-    const size_t smem = (size_t)p.d * (2 * p.d + 16);
-    LASER_CUDA_OK(allow_smem(bs_rows_kernel<D16>, smem));
     LaunchScope ls("bs_rows_y", st);
-    bs_rows_kernel<D16><<<(int)std::min<long long>((jobs + 7) / 8, 2 * sms), 256, smem, st>>>(P, 1);
+    const int rc = launch_rows<D16, D16, 4, true>(p, P, st);
+    if (rc != LASER_OK) return rc;
   }
   {
     const int warp_bytes = (int)bwd_warp_bytes(p.d, p.H);

@@ -56,6 +56,18 @@ __device__ __forceinline__ void red_add4(float* at, float x, float y, float z, f
   asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(at), "f"(x), "f"(y), "f"(z), "f"(w) : "memory");
 }
 
+// Adds scale * (a 16 x 8 accumulator tile of mma16816) to the rows of C below `rows`.  Neighbouring lanes trade halves, so that
+// a lane owns four columns of one row and adds them with one 16-byte reduction (C 16-byte aligned, ld a multiple of 4).
+__device__ __forceinline__ void red_tile(float* C, size_t ld, const float (&v)[4], float scale, int lane, int rows = 16) {
+  const int g = lane >> 2, t = lane & 3;
+  const bool odd = t & 1;
+  const float o0 = __shfl_xor_sync(0xffffffffu, odd ? v[0] : v[2], 1), o1 = __shfl_xor_sync(0xffffffffu, odd ? v[1] : v[3], 1);
+  const int row = g + (odd ? 8 : 0);
+  if (row < rows)
+    red_add4(C + (size_t)row * ld + (t >> 1) * 4, scale * (odd ? o0 : v[0]), scale * (odd ? o1 : v[1]), scale * (odd ? v[2] : o0),
+             scale * (odd ? v[3] : o1));
+}
+
 // 16-byte asynchronous global -> shared copy; src_bytes = 0 zero-fills the destination.
 __device__ __forceinline__ void cp16(uint32_t dst, const void* src, uint32_t src_bytes) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
