@@ -1190,6 +1190,7 @@ int backward_stream_all(const Plan& p, const T* items, const int32_t* lengths, c
 #define BWD_OK(...) do { rc = (__VA_ARGS__); if (rc != LASER_OK) return rc; } while (0)
   ZeroList Z = {};
   Z.add(dWq, (size_t)d * dqk); Z.add(dWk, (size_t)d * dqk); Z.add(dWv, (size_t)d * d); Z.add(dWg, (size_t)M * 3 * d * d);
+  Z.add(backward_stream_sums(p, stream_scratch), (size_t)N * H * d);
   BWD_OK(zero_arrays(Z, st));
   bf16 *Hhi = reinterpret_cast<bf16*>(s.Hp), *Hlo = Hhi + (size_t)N * p.Lp * d;
   BWD_OK(backward_stream_forward(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, nullptr, Hhi, Hlo, ws, stream_scratch, st));
@@ -1389,6 +1390,7 @@ int backward_t(const Plan& p, const T* items, const int32_t* lengths, const T* c
   // ---- backward through the segment aggregation and the gates
   const float* p_sums = nullptr;
   if (stream) {
+    LASER_CUDA_OK(cudaMemsetAsync(backward_stream_sums(p, mma_scratch), 0, (size_t)N * H * d * sizeof(float), st));
     BWD_OK(backward_stream(p, items, lengths, cand_offsets, Wv, s.dHp, d_items, dWv, &p_sums, ws, mma_scratch, st));
     // d(q_h / gamma) = p_h W_k[:, h];  dW_k[:, h] += p_h^T q_h / gamma, every head
     const int dqh = p.dqh;

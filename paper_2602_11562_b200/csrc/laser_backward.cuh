@@ -1,4 +1,6 @@
-// Interfaces between the source files of the backward pass.
+// Interfaces between the source files of the backward pass.  The kernels of the two tensor-core routes are chained (the next
+// one's blocks are placed while the last blocks of this one run: 1.2 % of a call of 0.75-0.85 ms).  Those of the FP32 route are
+// not: their grids are smaller than the GPU, and blocks placed early crowd the SMs that happen to be idle (83 -> 88 us).
 #pragma once
 
 #include "laser_common.cuh"

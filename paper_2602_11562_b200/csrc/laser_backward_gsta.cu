@@ -52,6 +52,8 @@ struct TrainParams {
 __global__ void __launch_bounds__(256) train_prep_kernel(const bf16* Wg, uint4* img, int d, int M, const int* lengths,
                                                          const int* cand_offsets, int U, int N, int L, int S, int Lp, int cpb,
                                                          int* nseg, int* order, int* keys) {
+  chain_wait();
+  chain_release();
   const int n_blocks = gridDim.x - (order ? 1 : 0);
   if ((int)blockIdx.x == n_blocks) {
     gsta_build_order(lengths, cand_offsets, U, N, L, S, Lp, cpb, order, keys);
@@ -103,6 +105,8 @@ __global__ void __launch_bounds__(kTThreads, 2) gsta_train_kernel(const __grid_c
   using SM = TrainSmem<D16, NP>;
   constexpr int d = SM::d, RS = SM::RS;
   extern __shared__ __align__(128) uint8_t smem[];
+  chain_wait();
+  chain_release();
   const int H = P.H, Lp = P.Lp, dvh = d / H, KH = dvh >> 4;
   const uint32_t plane = (uint32_t)SM::plane(H), CP = SM::cand_pitch(H);
   uint8_t* Thi = smem;                                               // [16] rows: t, later dt, high and low parts (the fp32
@@ -707,6 +711,8 @@ __global__ void __launch_bounds__(256, 2) weight_sums_kernel(const __grid_consta
                                                              int dvh) {
   constexpr int d = 16 * D16, kParts = 8 / D16 > 0 ? 8 / D16 : 1, kPairs = (D16 + kParts - 1) / kParts;
   extern __shared__ __align__(128) uint8_t smem[];
+  chain_wait();
+  chain_release();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
   const bf16 *A = L.A[blockIdx.y], *B = L.B[blockIdx.y];
   const size_t a_lo = L.a_lo[blockIdx.y], b_lo = L.b_lo[blockIdx.y];
@@ -839,15 +845,14 @@ int launch_train(TrainParams P, const Plan& p, const TrainScratch& s, const void
   {
     const int total = p.M * 6 * D16 * D16 * 32;
     LaunchScope ls("gsta_train_prep", st);
-    train_prep_kernel<<<std::min((total + 255) / 256, 4 * sms) + (P.order ? 1 : 0), 256, 0, st>>>(
-        (const bf16*)Wg, s.img, p.d, p.M, lengths, cand_offsets, p.U, p.N, p.L, p.S, p.Lp, P.cpb, s.nseg,
-        P.order ? s.order : nullptr, s.keys);
+    LASER_CUDA_OK(launch_chained(train_prep_kernel, dim3(std::min((total + 255) / 256, 4 * sms) + (P.order ? 1 : 0)), dim3(256), 0,
+                                 st, (const bf16*)Wg, s.img, p.d, p.M, lengths, cand_offsets, p.U, p.N, p.L, p.S, p.Lp, P.cpb,
+                                 s.nseg, P.order ? s.order : nullptr, s.keys));
   }
   const size_t smem = TrainSmem<D16, NP>::bytes(p.H, P.nb);
   LASER_CUDA_OK(allow_smem(gsta_train_kernel<D16, NP>, smem));
   LaunchScope ls("gsta_train", st);
-  gsta_train_kernel<D16, NP><<<blocks, kTThreads, smem, st>>>(P);
-  LASER_CUDA_OK(cudaGetLastError());
+  LASER_CUDA_OK(launch_chained(gsta_train_kernel<D16, NP>, dim3(blocks), dim3(kTThreads), smem, st, P));
   return LASER_OK;
 }
 
@@ -875,8 +880,7 @@ int launch_sums(const Plan& p, const GstaPlanes& G, float* dWg, cudaStream_t st)
     const int want = std::max(1, 2 * device_sms() / n);
     const int per = std::max(KR, ((p.N + want - 1) / want + KR - 1) / KR * KR);
     LaunchScope ls("gsta_weight_sums", st);
-    weight_sums_kernel<D16><<<dim3((p.N + per - 1) / per, n), 256, smem, st>>>(L, p.N, per, KR, p.dvh);
-    LASER_CUDA_OK(cudaGetLastError());
+    LASER_CUDA_OK(launch_chained(weight_sums_kernel<D16>, dim3((p.N + per - 1) / per, n), dim3(256), smem, st, L, p.N, per, KR, p.dvh));
   }
   return LASER_OK;
 }

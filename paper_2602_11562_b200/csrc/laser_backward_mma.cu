@@ -64,6 +64,8 @@ __global__ void __launch_bounds__(kBwdWarps * 32, 2) sta_bwd_mma_kernel(const Bw
   constexpr int QS = 2 * DQH + 16, DS = 2 * DVH + 16;          // bytes per staged row (padding: conflict-free ldmatrix)
   constexpr int kBuf = 16 * (QS + DS);                         // one staging buffer: 16 candidate rows of Qb_h and ds_i,h
   extern __shared__ __align__(16) unsigned char smem[];
+  chain_wait();
+  chain_release();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const int u = blockIdx.y, job = blockIdx.x * kBwdWarps + warp;
   if (job >= P.jobs) return;
@@ -304,6 +306,8 @@ __global__ void __launch_bounds__(kBwdWarps * 32) sta_fwd_mma_kernel(const FwdMm
   constexpr int DQH = 16 * DQ16, DVH = 16 * DV16;
   constexpr int KS = 2 * DQH + 16, VS = 2 * DVH + 16;          // bytes per staged row
   extern __shared__ __align__(16) unsigned char smem[];
+  chain_wait();
+  chain_release();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
   const int u = blockIdx.y, seg = blockIdx.x / P.H, h = blockIdx.x - seg * P.H;
   const int len = P.lengths[u], off0 = P.cand_offsets[u], off1 = P.cand_offsets[u + 1];
@@ -419,8 +423,7 @@ int launch_mma(const BwdMmaParams& P, int U, cudaStream_t st) {
   auto kernel = sta_bwd_mma_kernel<MT, DQ16, DV16>;
   LASER_CUDA_OK(allow_smem(kernel, smem));
   LaunchScope ls("bwd_sta_mma", st);
-  kernel<<<dim3((P.jobs + kBwdWarps - 1) / kBwdWarps, U), kBwdWarps * 32, smem, st>>>(P);
-  LASER_CUDA_OK(cudaGetLastError());
+  LASER_CUDA_OK(launch_chained(kernel, dim3((P.jobs + kBwdWarps - 1) / kBwdWarps, U), dim3(kBwdWarps * 32), smem, st, P));
   return LASER_OK;
 }
 
@@ -435,8 +438,7 @@ int launch_fwd(const FwdMmaParams& P, int U, size_t smem, cudaStream_t st) {
   auto kernel = sta_fwd_mma_kernel<DQ16, DV16>;
   LASER_CUDA_OK(allow_smem(kernel, smem));
   LaunchScope ls("bwd_sta_fwd_mma", st);
-  kernel<<<dim3(P.Lp * P.H, U), kBwdWarps * 32, smem, st>>>(P);
-  LASER_CUDA_OK(cudaGetLastError());
+  LASER_CUDA_OK(launch_chained(kernel, dim3(P.Lp * P.H, U), dim3(kBwdWarps * 32), smem, st, P));
   return LASER_OK;
 }
 

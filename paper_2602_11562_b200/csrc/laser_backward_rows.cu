@@ -59,6 +59,8 @@ __global__ void __launch_bounds__(kRThreads, 2) rows_project_kernel(const RowsPa
   constexpr int d = 16 * D16, XS = 2 * d + 16;
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ int table[kTableGroups];
+  chain_wait();
+  chain_release();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
   const int n = P.na + P.nb, WS = 2 * n + 16;                        // bytes per row of [W_a | W_b] and of the output tile
   uint8_t* Ws = smem;                                                // [d][WS]
@@ -156,6 +158,8 @@ __global__ void __launch_bounds__(kRThreads) rows_grad_kernel(const RowsParams P
   constexpr int d = 16 * D16, XS = 2 * d + 16, kParts = 16 / D16, kMaxPairs = (16 + kParts - 1) / kParts;
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ int table[kTableGroups];
+  chain_wait();
+  chain_release();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
   const int n = P.na + P.nb, WS = 2 * n + 16, pairs = n >> 4;
   uint8_t* Ws = smem;                                                // [d][WS]  [W_k | W_v]
@@ -322,8 +326,8 @@ int launch_project(const RowsParams& P, cudaStream_t st) {
   const long long jobs = (long long)P.groups * P.tiles_per_group;
   const int per_sm = smem <= 112 * 1024 ? 2 : 1;
   LaunchScope ls("bwd_rows_project", st);
-  rows_project_kernel<D16><<<(int)std::min<long long>(jobs, (long long)per_sm * device_sms()), kRThreads, smem, st>>>(P);
-  LASER_CUDA_OK(cudaGetLastError());
+  LASER_CUDA_OK(launch_chained(rows_project_kernel<D16>, dim3((unsigned)std::min<long long>(jobs, (long long)per_sm * device_sms())),
+                               dim3(kRThreads), smem, st, P));
   return LASER_OK;
 }
 template <int D16>
@@ -333,8 +337,8 @@ int launch_grad(const RowsParams& P, cudaStream_t st) {
   LASER_CUDA_OK(allow_smem(rows_grad_kernel<D16>, smem));
   const long long jobs = (long long)P.groups * P.tiles_per_group;
   LaunchScope ls("bwd_rows_grad", st);
-  rows_grad_kernel<D16><<<(int)std::min<long long>(jobs, device_sms()), kRThreads, smem, st>>>(P, nbuf);
-  LASER_CUDA_OK(cudaGetLastError());
+  LASER_CUDA_OK(launch_chained(rows_grad_kernel<D16>, dim3((unsigned)std::min<long long>(jobs, device_sms())), dim3(kRThreads), smem, st,
+                               P, nbuf));
   return LASER_OK;
 }
 

@@ -128,6 +128,8 @@ template <int D16>
 __global__ void __launch_bounds__(kBThreads) bs_fwd_kernel(BsParams P) {
   constexpr int d = 16 * D16, RS = RowRing<D16>::RS;
   extern __shared__ __align__(128) uint8_t smem[];
+  chain_wait();
+  chain_release();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, H = P.H;
   const int u = P.order ? min(max(P.order[blockIdx.x], 0), P.U - 1) : (int)blockIdx.x;
   int len = 0;
@@ -213,6 +215,8 @@ __global__ void __launch_bounds__(256, 2) bs_rows_kernel(BsParams P) {
   constexpr int d = 16 * D16, WS = 2 * d + 16;
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ int2 table[kBsTable];                          // (candidate, segments) by launch position
+  chain_wait();
+  chain_release();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3, H = P.H, dvh = d / H;
   for (int i = tid; i < d * 2 * D16; i += 256) {
     const int row = i / (2 * D16), q = i - row * (2 * D16);
@@ -319,6 +323,8 @@ template <int D16>
 __global__ void __launch_bounds__(kBThreads, 3) bs_bwd_kernel(BsParams P, int KS, int warp_bytes) {
   constexpr int d = 16 * D16, RS = RowRing<D16>::RS;
   extern __shared__ __align__(128) uint8_t smem[];
+  chain_wait();
+  chain_release();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3, H = P.H;
   const int u = P.order ? min(max(P.order[blockIdx.x], 0), P.U - 1) : (int)blockIdx.x;
   int len = 0;
@@ -489,7 +495,7 @@ __global__ void __launch_bounds__(kBThreads, 3) bs_bwd_kernel(BsParams P, int KS
 #pragma unroll
     for (int w = 0; w < kBW; ++w) v += red[(size_t)w * H * d + i];
     float* out = P.p + (size_t)cand * H * d + i;
-    if (gridDim.y > 1) atomicAdd(out, v);                   // (p was zeroed before)
+    if (gridDim.y > 1) atomicAdd(out, v);                   // (p is zero before)
     else *out = v;
   }
 }
@@ -509,6 +515,8 @@ template <int D16>
 __global__ void __launch_bounds__(256) bs_wv_kernel(BsParams P, int KR) {
   constexpr int d = 16 * D16, kParts = 8 / D16 > 0 ? 8 / D16 : 1;    // warps that share a row tile split the rows
   extern __shared__ __align__(128) uint8_t smem[];
+  chain_wait();
+  chain_release();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3, H = P.H, dvh = d / H;
   const int pa = H * d + 8, pb = d + 8;                     // row pitches in words (conflict-free fragment reads)
   float* buf0 = reinterpret_cast<float*>(smem);
@@ -665,8 +673,7 @@ int launch_rows(const Plan& p, const BsParams& P, cudaStream_t st) {
   const long long jobs = (long long)p.U * ((p.Lp + 15) / 16) * p.H;
   auto kernel = bs_rows_kernel<D16, NPC, KA, to_y>;
   LASER_CUDA_OK(allow_smem(kernel, smem));
-  kernel<<<(int)std::min<long long>((jobs + 7) / 8, 2 * device_sms()), 256, smem, st>>>(P);
-  LASER_CUDA_OK(cudaGetLastError());
+  LASER_CUDA_OK(launch_chained(kernel, dim3((unsigned)std::min<long long>((jobs + 7) / 8, 2 * device_sms())), dim3(256), smem, st, P));
   return LASER_OK;
 }
 
@@ -676,7 +683,7 @@ int bs_forward_t(const Plan& p, BsParams P, cudaStream_t st) {
     const size_t smem = kBW * kBStages * ring_bytes(p.d, p.H, false);
     LASER_CUDA_OK(allow_smem(bs_fwd_kernel<D16>, smem));
     LaunchScope ls("bs_fwd", st);
-    bs_fwd_kernel<D16><<<dim3(p.U, user_parts(p)), kBThreads, smem, st>>>(P);
+    LASER_CUDA_OK(launch_chained(bs_fwd_kernel<D16>, dim3(p.U, user_parts(p)), dim3(kBThreads), smem, st, P));
   }
   LaunchScope ls("bs_rows_s", st);
   return p.H > 1 ? launch_rows<D16, (D16 + 1) / 2, 8, false>(p, P, st) : launch_rows<D16, D16, 4, false>(p, P, st);
@@ -694,16 +701,15 @@ int bs_backward_t(const Plan& p, BsParams P, cudaStream_t st) {
     const int warp_bytes = (int)bwd_warp_bytes(p.d, p.H);
     const size_t smem = (size_t)kBW * warp_bytes + 2 * p.d + 16;
     LASER_CUDA_OK(allow_smem(bs_bwd_kernel<D16>, smem));
-    LASER_CUDA_OK(cudaMemsetAsync(P.p, 0, (size_t)p.N * p.H * p.d * sizeof(float), st));
     LaunchScope ls("bs_bwd", st);
-    bs_bwd_kernel<D16><<<dim3(p.U, parts), kBThreads, smem, st>>>(P, slot_steps(p.H), warp_bytes);
+    LASER_CUDA_OK(launch_chained(bs_bwd_kernel<D16>, dim3(p.U, parts), dim3(kBThreads), smem, st, P, slot_steps(p.H), warp_bytes));
   }
   {
     const int KR = wv_rows(p.d, p.H);
     const size_t smem = 2 * (size_t)KR * ((size_t)p.H * p.d + p.d + 16) * sizeof(float);
     LASER_CUDA_OK(allow_smem(bs_wv_kernel<D16>, smem));
     LaunchScope ls("bs_wv", st);
-    bs_wv_kernel<D16><<<std::min(p.U, 2 * sms), 256, smem, st>>>(P, KR);
+    LASER_CUDA_OK(launch_chained(bs_wv_kernel<D16>, dim3(std::min(p.U, 2 * sms)), dim3(256), smem, st, P, KR));
   }
   LASER_CUDA_OK(cudaGetLastError());
   return LASER_OK;
@@ -715,6 +721,7 @@ bool backward_stream_supported(const Plan& p) {
   return p.dtype == LASER_BF16 && p.maxC <= 1 && p.d % 16 == 0 && p.d >= 16 && p.d <= 128 && p.H <= 8 && p.dvh % 16 == 0 &&
          p.dqh % 16 == 0 && kBW * bwd_warp_bytes(p.d, p.H) + 2 * p.d + 16 <= 220 * 1024;
 }
+float* backward_stream_sums(const Plan& p, char* scratch) { return carve_bs(p, scratch).p; }
 size_t backward_stream_scratch_bytes(const Plan& p) { return backward_stream_supported(p) ? carve_bs(p, nullptr).total : 0; }
 
 #define LASER_BS_DISPATCH(fn, ...)                     \

@@ -154,6 +154,7 @@ int stream_fold(const Plan& p, const int32_t* lengths, const void* cands, const 
 // p_h = sum_n de_{n,h} x_n, from which the gradients of the query side and of W_k follow, in *p_sums [N, H, d].
 bool backward_stream_supported(const Plan& p);
 size_t backward_stream_scratch_bytes(const Plan& p);
+float* backward_stream_sums(const Plan& p, char* scratch);      // p of backward_stream, [N, H, d]: zeroed by the caller
 int backward_stream_forward(const Plan& p, const void* items, const int32_t* lengths, const void* cands,
                             const int32_t* cand_offsets, const void* Wq, const void* Wk, const void* Wv, float* Hp,
                             __nv_bfloat16* Hp_hi, __nv_bfloat16* Hp_lo, char* ws, char* scratch, cudaStream_t st);
