@@ -54,6 +54,40 @@ __device__ __forceinline__ void fill_table(const RowsParams& P, int* table, int 
   __syncthreads();
 }
 
+// Tile `tile` of group `u`.  A block takes every gridDim.x-th one, groups fastest: the tiles that only long users have come
+// last, spread over the blocks.  (A cursor instead of a tile number: divisions were a third of the gradient kernel's instructions.)
+struct RowTile { int tile, u; };
+struct RowWalk {
+  const RowsParams& P;
+  const int* table;
+  int dt, du;
+  __device__ __forceinline__ RowWalk(const RowsParams& params, const int* t) : P(params), table(t) {
+    dt = gridDim.x / P.groups;
+    du = gridDim.x - dt * P.groups;
+  }
+  __device__ __forceinline__ RowTile first() const {
+    const int tile = blockIdx.x / P.groups;
+    return {tile, (int)blockIdx.x - tile * P.groups};
+  }
+  __device__ __forceinline__ bool in(RowTile c) const { return c.tile < P.tiles_per_group; }
+  __device__ __forceinline__ RowTile step(RowTile c) const {
+    c.tile += dt;
+    c.u += du;
+    if (c.u >= P.groups) c.u -= P.groups, ++c.tile;
+    return c;
+  }
+  // valid rows of the tile and beyond it
+  __device__ __forceinline__ int rows(RowTile c) const {
+    return (P.groups <= kTableGroups ? table[c.u] : valid_rows(P, c.u)) - c.tile * kRT;
+  }
+  __device__ __forceinline__ size_t row0(RowTile c) const { return (size_t)c.u * P.rows_per_group + c.tile * kRT; }
+  // c, or the first tile after it with valid rows
+  __device__ __forceinline__ RowTile valid(RowTile c) const {
+    while (in(c) && rows(c) <= 0) c = step(c);
+    return c;
+  }
+};
+
 template <int D16>
 __global__ void __launch_bounds__(kRThreads, 2) rows_project_kernel(const RowsParams P) {
   constexpr int d = 16 * D16, XS = 2 * d + 16;
@@ -71,35 +105,27 @@ __global__ void __launch_bounds__(kRThreads, 2) rows_project_kernel(const RowsPa
     cp16(smem_addr(Ws) + k * WS + c * 2, c < P.na ? P.Wa + (size_t)k * P.na + c : P.Wb + (size_t)k * P.nb + c - P.na, 16u);
   }
   fill_table(P, table, tid);
-  const int jobs = P.groups * P.tiles_per_group;
-  // job j = (tile j / groups, group j mod groups): the tiles that only long users have come last, spread over the blocks
-  auto rows_of = [&](int j) {
-    if (j >= jobs) return 0;
-    const int tile = j / P.groups, u = j - tile * P.groups;
-    return (P.groups <= kTableGroups ? table[u] : valid_rows(P, u)) - tile * kRT;
-  };
-  auto next_job = [&](int j) {
-    while (j < jobs && rows_of(j) <= 0) j += gridDim.x;
-    return j;
-  };
-  auto stage = [&](int j, int b) {
-    const int rows = rows_of(j);
-    const bf16* src = P.X + ((size_t)(j % P.groups) * P.rows_per_group + j / P.groups * kRT) * d;
+  const RowWalk walk(P, table);
+  auto stage = [&](RowTile j, int b) {
+    const int rows = walk.rows(j);
+    const bf16* src = P.X + walk.row0(j) * d;
     for (int i = tid; i < kRT * 2 * D16; i += kRThreads) {
       const int r = i / (2 * D16), q = i - r * (2 * D16);
       cp16(smem_addr(Xs) + b * kRT * XS + r * XS + q * 16, r < rows ? src + (size_t)r * d + q * 8 : P.X, r < rows ? 16u : 0u);
     }
   };
-  int job = next_job(blockIdx.x);
-  if (job < jobs) stage(job, 0);
+  RowTile job = walk.valid(walk.first());
+  if (walk.in(job)) stage(job, 0);
   cp_commit();
   const int m0 = (warp >> 2) * 16, part = warp & 3, pairs = n >> 4;  // column tiles in pairs: part, part + 4, ...
   const uint32_t a_row = ((lane & 7) + ((lane >> 3) & 1) * 8 + m0) * XS + (lane >> 4) * 16;
   const uint32_t b_row = ((lane & 7) + ((lane >> 3) & 1) * 8) * WS + (lane >> 4) * 16;
   int b = 0;
-  while (job < jobs) {
-    const int nxt = next_job(job + gridDim.x);
-    if (nxt < jobs) stage(nxt, b ^ 1);
+  const int out_c = lane * 8, out_ld = out_c < P.na ? P.na : P.nb;          // this lane's 8 columns of an output row
+  bf16* out = out_c < P.na ? P.Ya + out_c : P.Yb + out_c - P.na;
+  while (walk.in(job)) {
+    const RowTile nxt = walk.valid(walk.step(job));
+    if (walk.in(nxt)) stage(nxt, b ^ 1);
     cp_commit();
     cp_wait<1>();
     __syncthreads();
@@ -138,14 +164,11 @@ __global__ void __launch_bounds__(kRThreads, 2) rows_project_kernel(const RowsPa
     }
     __syncthreads();
     {
-      const int rows = min(rows_of(job), kRT);
-      const size_t row0 = (size_t)(job % P.groups) * P.rows_per_group + job / P.groups * kRT;
-      for (int i = tid; i < rows * (n / 8); i += kRThreads) {
-        const int r = i / (n / 8), c = (i - r * (n / 8)) * 8;
-        const uint4 v = *reinterpret_cast<const uint4*>(Ys + r * WS + c * 2);
-        if (c < P.na) *reinterpret_cast<uint4*>(P.Ya + (row0 + r) * P.na + c) = v;
-        else *reinterpret_cast<uint4*>(P.Yb + (row0 + r) * P.nb + c - P.na) = v;
-      }
+      const int rows = min(walk.rows(job), kRT);
+      bf16* y = out + walk.row0(job) * out_ld;
+      if (out_c < n)
+        for (int r = warp; r < rows; r += kRThreads / 32)
+          *reinterpret_cast<uint4*>(y + r * out_ld) = *reinterpret_cast<const uint4*>(Ys + r * WS + out_c * 2);
     }
     job = nxt;
     b ^= 1;
@@ -155,7 +178,9 @@ __global__ void __launch_bounds__(kRThreads, 2) rows_project_kernel(const RowsPa
 
 template <int D16>
 __global__ void __launch_bounds__(kRThreads) rows_grad_kernel(const RowsParams P, int nbuf) {
-  constexpr int d = 16 * D16, XS = 2 * d + 16, kParts = 16 / D16, kMaxPairs = (16 + kParts - 1) / kParts;
+  constexpr int d = 16 * D16, XS = 2 * d + 16;
+  // a warp's share of the weight gradients: kM tiles of 16 features, column pairs wpart, wpart + kParts, ...
+  constexpr int kM = D16 % 2 == 0 ? 2 : 1, kParts = 16 * kM / D16, kMaxPairs = (16 + kParts - 1) / kParts;
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ int table[kTableGroups];
   chain_wait();
@@ -170,59 +195,56 @@ __global__ void __launch_bounds__(kRThreads) rows_grad_kernel(const RowsParams P
     cp16(smem_addr(Ws) + k * WS + c * 2, c < P.na ? P.Wa + (size_t)k * P.na + c : P.Wb + (size_t)k * P.nb + c - P.na, 16u);
   }
   fill_table(P, table, tid);
-  const int jobs = P.groups * P.tiles_per_group;
-  auto rows_of = [&](int j) {
-    if (j >= jobs) return 0;
-    const int tile = j / P.groups, u = j - tile * P.groups;
-    return (P.groups <= kTableGroups ? table[u] : valid_rows(P, u)) - tile * kRT;
-  };
-  auto next_job = [&](int j) {
-    while (j < jobs && rows_of(j) <= 0) j += gridDim.x;
-    return j;
-  };
-  auto stage = [&](int j, int b) {
-    const int rows = rows_of(j);
-    const size_t row0 = (size_t)(j % P.groups) * P.rows_per_group + j / P.groups * kRT;
+  const RowWalk walk(P, table);
+  const int g_c = lane * 8, g_ld = g_c < P.na ? P.na : P.nb;                 // this lane's 8 columns of [dK | dV]
+  const bf16 *g_hi = g_c < P.na ? P.Ahi + g_c : P.Bhi + g_c - P.na, *g_lo = g_c < P.na ? P.Alo + g_c : P.Blo + g_c - P.na;
+  auto stage = [&](RowTile j, int b) {
+    const int rows = walk.rows(j);
+    const size_t row0 = walk.row0(j);
+    const bf16* x = P.X + row0 * d;
     for (int i = tid; i < kRT * 2 * D16; i += kRThreads) {
       const int r = i / (2 * D16), q = i - r * (2 * D16);
-      cp16(smem_addr(Xs) + b * kRT * XS + r * XS + q * 16, r < rows ? P.X + (row0 + r) * d + q * 8 : P.X, r < rows ? 16u : 0u);
+      cp16(smem_addr(Xs) + b * kRT * XS + r * XS + q * 16, r < rows ? x + r * d + q * 8 : P.X, r < rows ? 16u : 0u);
     }
-    for (int r = warp; r < kRT; r += kRThreads / 32) {               // a warp per row: no divisions by the run-time width
-      const uint32_t bytes = r < rows ? 16u : 0u, dst = smem_addr(Gs) + b * 2 * kRT * WS + r * WS;
-      const size_t row = r < rows ? row0 + r : 0;
-      for (int c = lane * 8; c < n; c += 256) {
-        const size_t at = c < P.na ? row * P.na + c : row * P.nb + c - P.na;
-        cp16(dst + c * 2, (c < P.na ? P.Ahi : P.Bhi) + at, bytes);
-        cp16(dst + kRT * WS + c * 2, (c < P.na ? P.Alo : P.Blo) + at, bytes);
+    if (g_c < n) {                                                   // a warp per row, 8 columns per lane
+      const bf16 *hi = g_hi + row0 * g_ld, *lo = g_lo + row0 * g_ld;
+      uint32_t dst = smem_addr(Gs) + b * 2 * kRT * WS + warp * WS + g_c * 2;
+#pragma unroll
+      for (int r = warp; r < kRT; r += kRThreads / 32, dst += kRThreads / 32 * WS) {
+        const bool ok = r < rows;
+        cp16(dst, ok ? hi + r * g_ld : P.X, ok ? 16u : 0u);
+        cp16(dst + kRT * WS, ok ? lo + r * g_ld : P.X, ok ? 16u : 0u);
       }
     }
   };
-  int job = next_job(blockIdx.x);
-  if (job < jobs) stage(job, 0);
+  RowTile job = walk.valid(walk.first());
+  if (walk.in(job)) stage(job, 0);
   cp_commit();
   // rows that receive no gradient
-  for (int j = blockIdx.x; j < jobs; j += gridDim.x) {
-    const int first = max(0, min(kRT, rows_of(j))), last = min(kRT, P.rows_per_group - j / P.groups * kRT);
-    float4* out = reinterpret_cast<float4*>(P.dX + ((size_t)(j % P.groups) * P.rows_per_group + j / P.groups * kRT) * d);
+  for (RowTile j = walk.first(); walk.in(j); j = walk.step(j)) {
+    const int first = max(0, min(kRT, walk.rows(j))), last = min(kRT, P.rows_per_group - j.tile * kRT);
+    float4* out = reinterpret_cast<float4*>(P.dX + walk.row0(j) * d);
     for (int i = first * (d / 4) + tid; i < last * (d / 4); i += kRThreads) out[i] = make_float4(0.f, 0.f, 0.f, 0.f);
   }
   const int m0 = (warp >> 2) * 16, part = warp & 3;                  // d_items: 16 rows, feature pairs part, part + 4
-  const int mw = warp % D16, wpart = warp / D16;                     // weight gradients: 16 features, column pairs wpart, ...
+  const int mw = warp % (D16 / kM) * kM, wpart = warp / (D16 / kM);
   const int mi = lane >> 3, lr = lane & 7;
   const uint32_t a_row = ((mi & 1) * 8 + lr + m0) * WS + (mi >> 1) * 16;            // [dK | dV] as A (rows, columns)
   const uint32_t w_row = ((mi >> 1) * 8 + lr) * WS + (mi & 1) * 16;                 // W^T as B: W rows are its columns
   const uint32_t xt_row = ((mi >> 1) * 8 + lr) * XS + mw * 32 + (mi & 1) * 16;      // X^T as A
   const uint32_t g_row = ((mi & 1) * 8 + lr) * WS + (mi >> 1) * 16;                 // [dK | dV] as B
-  float wacc[kMaxPairs][2][4];
+  float wacc[kM][kMaxPairs][2][4];
 #pragma unroll
-  for (int i = 0; i < kMaxPairs; ++i)
+  for (int m = 0; m < kM; ++m)
 #pragma unroll
-    for (int e = 0; e < 4; ++e) wacc[i][0][e] = wacc[i][1][e] = 0.f;
+    for (int i = 0; i < kMaxPairs; ++i)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) wacc[m][i][0][e] = wacc[m][i][1][e] = 0.f;
   int b = 0;
-  while (job < jobs) {
-    const int nxt = next_job(job + gridDim.x);
+  while (walk.in(job)) {
+    const RowTile nxt = walk.valid(walk.step(job));
     if (nbuf == 2) {
-      if (nxt < jobs) stage(nxt, b ^ 1);
+      if (walk.in(nxt)) stage(nxt, b ^ 1);
       cp_commit();
       cp_wait<1>();
     } else {
@@ -230,68 +252,80 @@ __global__ void __launch_bounds__(kRThreads) rows_grad_kernel(const RowsParams P
     }
     __syncthreads();
     const uint32_t xs = smem_addr(Xs) + b * kRT * XS, hi = smem_addr(Gs) + b * 2 * kRT * WS, lo = hi + kRT * WS;
-    float acc[2][2][4];
+    // the two products of the tile are independent: half of the warps of every scheduler take them in the other order, so that
+    // one's MMAs run beside the other's stores
+#pragma unroll 1
+    for (int phase = 0; phase < 2; ++phase)
+      if (phase == (warp >> 2 & 1)) {
+        float acc[2][2][4];
 #pragma unroll
-    for (int i = 0; i < 2; ++i)
+        for (int i = 0; i < 2; ++i)
 #pragma unroll
-      for (int e = 0; e < 4; ++e) acc[i][0][e] = acc[i][1][e] = 0.f;
+          for (int e = 0; e < 4; ++e) acc[i][0][e] = acc[i][1][e] = 0.f;
 #pragma unroll 2
-    for (int kt = 0; kt < pairs; ++kt) {
-      uint32_t ah[4], al[4];
-      ldsm_x4(ah, hi + a_row + kt * 32);
-      ldsm_x4(al, lo + a_row + kt * 32);
+        for (int kt = 0; kt < pairs; ++kt) {
+          uint32_t ah[4], al[4];
+          ldsm_x4(ah, hi + a_row + kt * 32);
+          ldsm_x4(al, lo + a_row + kt * 32);
 #pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        const int p = part + 4 * i;
-        if (p < D16) {
-          uint32_t w[4];
-          ldsm_x4(w, smem_addr(Ws) + w_row + p * 16 * WS + kt * 32);
-          mma16816(acc[i][0], ah[0], ah[1], ah[2], ah[3], w[0], w[1]);
-          mma16816(acc[i][1], ah[0], ah[1], ah[2], ah[3], w[2], w[3]);
-          mma16816(acc[i][0], al[0], al[1], al[2], al[3], w[0], w[1]);
-          mma16816(acc[i][1], al[0], al[1], al[2], al[3], w[2], w[3]);
+          for (int i = 0; i < 2; ++i) {
+            const int p = part + 4 * i;
+            if (p < D16) {
+              uint32_t w[4];
+              ldsm_x4(w, smem_addr(Ws) + w_row + p * 16 * WS + kt * 32);
+              mma16816(acc[i][0], ah[0], ah[1], ah[2], ah[3], w[0], w[1]);
+              mma16816(acc[i][1], ah[0], ah[1], ah[2], ah[3], w[2], w[3]);
+              mma16816(acc[i][0], al[0], al[1], al[2], al[3], w[0], w[1]);
+              mma16816(acc[i][1], al[0], al[1], al[2], al[3], w[2], w[3]);
+            }
+          }
         }
-      }
-    }
-    {
-      const int rows = rows_of(job);
-      float* out = P.dX + ((size_t)(job % P.groups) * P.rows_per_group + job / P.groups * kRT + m0 + g) * d + 2 * t;
+        {
+          const int rows = walk.rows(job);
+          float* out = P.dX + (walk.row0(job) + m0 + g) * d + 2 * t;
 #pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        const int p = part + 4 * i;
-        if (p < D16) {
+          for (int i = 0; i < 2; ++i) {
+            const int p = part + 4 * i;
+            if (p < D16) {
 #pragma unroll
-          for (int nt = 0; nt < 2; ++nt) {
-            if (m0 + g < rows) *reinterpret_cast<float2*>(out + p * 16 + nt * 8) = make_float2(acc[i][nt][0], acc[i][nt][1]);
-            if (m0 + g + 8 < rows) *reinterpret_cast<float2*>(out + 8 * d + p * 16 + nt * 8) = make_float2(acc[i][nt][2], acc[i][nt][3]);
+              for (int nt = 0; nt < 2; ++nt) {
+                if (m0 + g < rows) *reinterpret_cast<float2*>(out + p * 16 + nt * 8) = make_float2(acc[i][nt][0], acc[i][nt][1]);
+                if (m0 + g + 8 < rows) *reinterpret_cast<float2*>(out + 8 * d + p * 16 + nt * 8) = make_float2(acc[i][nt][2], acc[i][nt][3]);
+              }
+            }
+          }
+        }
+      } else if (wpart < kParts) {
+#pragma unroll
+        for (int kt = 0; kt < kRT / 16; ++kt) {
+          uint32_t a[kM][4];
+#pragma unroll
+          for (int m = 0; m < kM; ++m) ldsm_x4_t(a[m], xs + xt_row + kt * 16 * XS + m * 32);
+#pragma unroll
+          for (int i = 0; i < kMaxPairs; ++i) {
+            const int p = wpart + kParts * i;
+            if (p < pairs) {
+              uint32_t bh[4], bl[4];
+              ldsm_x4_t(bh, hi + g_row + kt * 16 * WS + p * 32);
+              ldsm_x4_t(bl, lo + g_row + kt * 16 * WS + p * 32);
+#pragma unroll
+              for (int m = 0; m < kM; ++m) {
+                mma16816(wacc[m][i][0], a[m][0], a[m][1], a[m][2], a[m][3], bh[0], bh[1]);
+                mma16816(wacc[m][i][1], a[m][0], a[m][1], a[m][2], a[m][3], bh[2], bh[3]);
+              }
+#pragma unroll
+              for (int m = 0; m < kM; ++m) {
+                mma16816(wacc[m][i][0], a[m][0], a[m][1], a[m][2], a[m][3], bl[0], bl[1]);
+                mma16816(wacc[m][i][1], a[m][0], a[m][1], a[m][2], a[m][3], bl[2], bl[3]);
+              }
+            }
           }
         }
       }
-    }
-    if (wpart < kParts) {
-#pragma unroll
-      for (int kt = 0; kt < kRT / 16; ++kt) {
-        uint32_t a[4];
-        ldsm_x4_t(a, xs + xt_row + kt * 16 * XS);
-#pragma unroll
-        for (int i = 0; i < kMaxPairs; ++i) {
-          const int p = wpart + kParts * i;
-          if (p < pairs) {
-            uint32_t bh[4], bl[4];
-            ldsm_x4_t(bh, hi + g_row + kt * 16 * WS + p * 32);
-            ldsm_x4_t(bl, lo + g_row + kt * 16 * WS + p * 32);
-            mma16816(wacc[i][0], a[0], a[1], a[2], a[3], bh[0], bh[1]);
-            mma16816(wacc[i][1], a[0], a[1], a[2], a[3], bh[2], bh[3]);
-            mma16816(wacc[i][0], a[0], a[1], a[2], a[3], bl[0], bl[1]);
-            mma16816(wacc[i][1], a[0], a[1], a[2], a[3], bl[2], bl[3]);
-          }
-        }
-      }
-    }
     __syncthreads();                       // the tile just read may be overwritten
     if (nbuf == 2) {
       b ^= 1;
-    } else if (nxt < jobs) {
+    } else if (walk.in(nxt)) {
       stage(nxt, 0);
       cp_commit();
     }
@@ -300,17 +334,19 @@ __global__ void __launch_bounds__(kRThreads) rows_grad_kernel(const RowsParams P
   cp_wait<0>();
   if (wpart >= kParts) return;
 #pragma unroll
-  for (int i = 0; i < kMaxPairs; ++i) {
-    const int p = wpart + kParts * i;
-    if (p < pairs) {
+  for (int m = 0; m < kM; ++m)
 #pragma unroll
-      for (int nt = 0; nt < 2; ++nt) {
-        const int c = p * 16 + nt * 8;
-        if (c < P.na) red_tile(P.dWa + (size_t)mw * 16 * P.na + c, P.na, wacc[i][nt], 1.f, lane);
-        else red_tile(P.dWb + (size_t)mw * 16 * P.nb + c - P.na, P.nb, wacc[i][nt], 1.f, lane);
+    for (int i = 0; i < kMaxPairs; ++i) {
+      const int p = wpart + kParts * i;
+      if (p < pairs) {
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt) {
+          const int c = p * 16 + nt * 8;
+          if (c < P.na) red_tile(P.dWa + (size_t)(mw + m) * 16 * P.na + c, P.na, wacc[m][i][nt], 1.f, lane);
+          else red_tile(P.dWb + (size_t)(mw + m) * 16 * P.nb + c - P.na, P.nb, wacc[m][i][nt], 1.f, lane);
+        }
       }
     }
-  }
 }
 
 size_t project_smem(int d, int n) { return (size_t)d * (2 * n + 16) + 2 * kRT * (2 * (size_t)d + 16) + (size_t)kRT * (2 * n + 16); }
