@@ -1245,10 +1245,10 @@ int backward_lists(const Plan& p, const bf16* items, const int32_t* lengths, con
   BWD_OK(gsta_weight_sums(p, G, dWg, st));
   BWD_OK(sta_bwd_mma_split(p, lengths, cand_offsets, s.dQf, dKh, dKl, dVh, dVl, mma_scratch, st));
   BWD_OK(rows_gradients(p, items, lengths, cand_offsets, Wk, Wv, dKh, dKl, dVh, dVl, d_items, dWk, dWv, st));
+  // (Qt and dM are not used on this route; each holds N rows of H d floats, and d_qk <= 2 H d)
+  BWD_OK(rows_gradients_cands(p, cands, Wq, s.dQf, reinterpret_cast<bf16*>(s.Qt), reinterpret_cast<bf16*>(s.dM), G.dT0, d_cands, dWq, st));
 #undef BWD_OK
-  ProductBatch<bf16> list(p, st);
-  list.add_query_products(cands, Wq, s.dQf, G.dT0, d_cands, dWq);
-  return list.flush();
+  return LASER_OK;
 }
 
 template <typename T>

@@ -45,6 +45,9 @@ int rows_project_cands(const Plan& p, const void* cands, const void* Wq, float s
 int rows_gradients(const Plan& p, const void* items, const int32_t* lengths, const int32_t* cand_offsets, const void* Wk,
                    const void* Wv, const __nv_bfloat16* dK_hi, const __nv_bfloat16* dK_lo, const __nv_bfloat16* dV_hi,
                    const __nv_bfloat16* dV_lo, float* d_items, float* dWk, float* dWv, cudaStream_t st);
+// d_cands = dT0 + dQf W_q^T / gamma and dWq += T^T dQf / gamma; hi, lo: room for N rows of d_qk bf16 each.
+int rows_gradients_cands(const Plan& p, const void* cands, const void* Wq, const float* dQf, __nv_bfloat16* hi, __nv_bfloat16* lo,
+                         const float* dT0, float* d_cands, float* dWq, cudaStream_t st);
 
 // A dense product on the FP32 ALUs: C[m][n] = D[m][n] + alpha (sum_k A(m, k) B(k, n) + sum_k A2(m, k) B2(k, n)), or, with
 // atomic, C += alpha A B in slices of the contraction.  A(m, k) = ta ? A[k lda + m] : A[m lda + k], B(k, n) = tb ?

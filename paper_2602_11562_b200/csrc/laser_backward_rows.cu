@@ -3,7 +3,8 @@
 //
 //   rows_project_kernel   Y = scale X [W_a | W_b] as bf16: K and V of the recomputed forward (X read once for both), or Q
 //   rows_grad_kernel      d_items = dK W_k^T + dV W_v^T (zero rows for padding), dW_k += X^T dK, dW_v += X^T dV, all from one
-//                         read of X, dK and dV
+//                         read of X, dK and dV; or d_cands = dt_0 + dQ W_q^T, dW_q += T^T dQ (16384 candidates: 37 us as two
+//                         products on the FP32 ALUs)
 //
 // dK and dV arrive as bf16 high and low parts (16 bits; TF32 operands, 11 bits, before), so every operand tile is copied to
 // shared memory as it is and read with ldmatrix; the weights stay in shared memory for the block's lifetime, the weight
@@ -36,6 +37,7 @@ struct RowsParams {
   float scale;
   // gradients
   const bf16 *Ahi, *Alo, *Bhi, *Blo;                 // dK [.., na], dV [.., nb]: high and low parts
+  const float* add;                                  // not null: dX = add + the products
   float *dX, *dWa, *dWb;
 };
 
@@ -240,6 +242,14 @@ __global__ void __launch_bounds__(kRThreads) rows_grad_kernel(const RowsParams P
     for (int i = 0; i < kMaxPairs; ++i)
 #pragma unroll
       for (int e = 0; e < 4; ++e) wacc[m][i][0][e] = wacc[m][i][1][e] = 0.f;
+  auto put = [&](float* at, float x0, float x1) {
+    if (P.add) {
+      const float2 v = *reinterpret_cast<const float2*>(P.add + (at - P.dX));
+      x0 += v.x;
+      x1 += v.y;
+    }
+    *reinterpret_cast<float2*>(at) = make_float2(x0, x1);
+  };
   int b = 0;
   while (walk.in(job)) {
     const RowTile nxt = walk.valid(walk.step(job));
@@ -289,8 +299,9 @@ __global__ void __launch_bounds__(kRThreads) rows_grad_kernel(const RowsParams P
             if (p < D16) {
 #pragma unroll
               for (int nt = 0; nt < 2; ++nt) {
-                if (m0 + g < rows) *reinterpret_cast<float2*>(out + p * 16 + nt * 8) = make_float2(acc[i][nt][0], acc[i][nt][1]);
-                if (m0 + g + 8 < rows) *reinterpret_cast<float2*>(out + 8 * d + p * 16 + nt * 8) = make_float2(acc[i][nt][2], acc[i][nt][3]);
+                const int at = p * 16 + nt * 8;
+                if (m0 + g < rows) put(out + at, acc[i][nt][0], acc[i][nt][1]);
+                if (m0 + g + 8 < rows) put(out + 8 * d + at, acc[i][nt][2], acc[i][nt][3]);
               }
             }
           }
@@ -347,6 +358,19 @@ __global__ void __launch_bounds__(kRThreads) rows_grad_kernel(const RowsParams P
         }
       }
     }
+}
+
+// hi + lo = scale * src, 4 values per thread and step
+__global__ void __launch_bounds__(256) split_rows_kernel(const float4* src, uint2* hi, uint2* lo, size_t n4, float scale) {
+  chain_wait();
+  chain_release();
+  for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < n4; i += (size_t)gridDim.x * 256) {
+    float4 v = src[i];
+    v.x *= scale; v.y *= scale; v.z *= scale; v.w *= scale;
+    const uint32_t a = pack2(v.x, v.y), b = pack2(v.z, v.w);
+    hi[i] = make_uint2(a, b);
+    lo[i] = make_uint2(pack2(v.x - bf16_lo(a), v.y - bf16_hi(a)), pack2(v.z - bf16_lo(b), v.w - bf16_hi(b)));
+  }
 }
 
 size_t project_smem(int d, int n) { return (size_t)d * (2 * n + 16) + 2 * kRT * (2 * (size_t)d + 16) + (size_t)kRT * (2 * n + 16); }
@@ -421,6 +445,21 @@ int rows_gradients(const Plan& p, const void* items, const int32_t* lengths, con
   P.groups = p.U; P.rows_per_group = p.L; P.tiles_per_group = (p.L + kRT - 1) / kRT; P.na = p.dqk; P.nb = p.d;
   P.X = (const bf16*)items; P.Wa = (const bf16*)Wk; P.Wb = (const bf16*)Wv; P.lengths = lengths; P.cand_offsets = cand_offsets;
   P.N = p.N; P.Ahi = dK_hi; P.Alo = dK_lo; P.Bhi = dV_hi; P.Blo = dV_lo; P.dX = d_items; P.dWa = dWk; P.dWb = dWv;
+  LASER_ROWS_DISPATCH(launch_grad)
+}
+
+int rows_gradients_cands(const Plan& p, const void* cands, const void* Wq, const float* dQf, __nv_bfloat16* hi, __nv_bfloat16* lo,
+                         const float* dT0, float* d_cands, float* dWq, cudaStream_t st) {
+  {
+    const size_t n4 = (size_t)p.N * p.dqk / 4;
+    LaunchScope ls("bwd_split_rows", st);
+    LASER_CUDA_OK(launch_chained(split_rows_kernel, dim3((unsigned)std::min<size_t>((n4 + 255) / 256, 4 * device_sms())), dim3(256), 0,
+                                 st, (const float4*)dQf, (uint2*)hi, (uint2*)lo, n4, p.inv_gamma));
+  }
+  RowsParams P = {};
+  P.groups = 1; P.rows_per_group = p.N; P.tiles_per_group = (p.N + kRT - 1) / kRT; P.na = p.dqk;
+  P.X = (const bf16*)cands; P.Wa = P.Wb = (const bf16*)Wq; P.N = p.N; P.Ahi = P.Bhi = hi; P.Alo = P.Blo = lo;
+  P.add = dT0; P.dX = d_cands; P.dWa = P.dWb = dWq;
   LASER_ROWS_DISPATCH(launch_grad)
 }
 
