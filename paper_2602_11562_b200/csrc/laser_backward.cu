@@ -2,12 +2,14 @@
 // weight matrix.  The paper trains the model (section "Experimental Settings") without printing backward formulas; what
 // is computed here is the chain rule through Eq. 7 (layers last to first) and then through Eq. 10-12 and Eq. 8-9.
 //
-// Inputs are read in their dtype, everything else is fp32.  Two versions: FP32 ALUs throughout (either dtype), and, for
-// bf16 batches, the batched matrix products on the tensor cores with TF32 operands (gemm_tf32_kernel) plus the gate
-// contractions, the recomputed H' and the GSTA attention with bf16 operands (laser_backward_mma.cu).  The forward intermediates are recomputed and kept (projections, H', and per GSTA layer
-// the running target, Q, the key-folded query Qt_h = W_k[:, h] Q_h / tau, the attention weights and the weighted sums
-// m_h = sum_j a_j s_j), all dense steps are batched matrix products over the N candidates (or the U L item rows), and
-// three kernels do what is not a matrix product:
+// Inputs are read in their dtype, everything else is fp32.  Four routes (backward_t):
+//   FP32 ALUs           every fp32 batch, bf16 on request: laser_backward_simt.cu and sta_bwd_kernel below
+//   one candidate       bf16, at most one per user: laser_backward_stream.cu, the attention in laser_backward_gsta.cu
+//   candidate lists     bf16, 8 or more per user: laser_backward_rows.cu, _mma.cu, _gsta.cu
+//   everything else     bf16 of other widths or counts, or no layer: the batched TF32 products and the attention kernels below
+// On the last one the forward intermediates are recomputed and kept (projections, H', and per GSTA layer the running target, Q,
+// the key-folded query Qt_h = W_k[:, h] Q_h / tau, the attention weights and the weighted sums m_h = sum_j a_j s_j), all dense
+// steps are batched matrix products over the N candidates (or the U L item rows), and three kernels do what is not a product:
 //   gsta_attn_fwd   per candidate: e_{j,h} = s_j . Qt_h, a = softmax_j, m_h = sum_j a_{j,h} s_j
 //   gsta_attn_bwd   per candidate: da_j = s_j . dm_h, de = a (da - sum a da), dQt_h = sum_j de_j s_j,
 //                   ds_j += de_j Qt_h + a_j dm_h
