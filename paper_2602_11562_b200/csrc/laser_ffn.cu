@@ -258,13 +258,26 @@ __global__ void __launch_bounds__(kFfnThreads, 1) ffn_tc_kernel(FfnParams P) {
   };
 
   if (warp == 18 && P.zero_empty) {
-    // Rows of H' of empty segments, candidates dealt over the blocks: this kernel is bound by its MMAs, so the stores ride
-    // along (64 x 256 candidates, 39 of 100 segments empty, d = 128: 25 us of a call as a kernel of its own).
-    for (int u = 0; u < P.U; ++u) {
-      const RowUser s = row_user(P, u);
-      const int n = (P.Lp - s.nseg) * (d >> 3);
-      for (int c = (bidx + G - s.c0 % G) % G; c < s.nc && n > 0; c += G) {
-        uint4* out = reinterpret_cast<uint4*>(P.H + ((size_t)(s.c0 + c) * P.Lp + s.nseg) * d);
+    // Rows of H' of empty segments: this kernel is bound by its MMAs, so the stores ride along.  Candidates are dealt over the
+    // blocks one by one (users differ in their empty segments); 32 of a block's are looked up at a time, one per lane, so that
+    // the walk costs a search of log2(U) steps per 32 candidates whatever the number of users (a walk over the users: 1168 us at
+    // 4000 of them with two candidates each, 23 so).  As a kernel of its own the zeros take 31 us of 572 at 64 x 256 candidates,
+    // 39 of 100 segments empty, d = 128; here the call takes 561.
+    for (unsigned base = bidx; base < (unsigned)P.N; base += 32u * G) {
+      const unsigned mine = base + (unsigned)lane * G;
+      int first = P.Lp;                                  // its first empty segment
+      if (mine < (unsigned)P.N) {
+        int lo = 0, hi = P.U - 1;                        // largest u with cand_offsets[u] <= mine
+        while (lo < hi) {
+          const int mid = (lo + hi + 1) >> 1;
+          if (P.cand_offsets[mid] <= (int)mine) lo = mid; else hi = mid - 1;
+        }
+        const RowUser s = row_user(P, lo);
+        if ((int)mine >= s.c0 && (int)mine < s.c0 + s.nc) first = s.nseg;
+      }
+      for (int k = 0; k < 32 && base + (unsigned)k * G < (unsigned)P.N; ++k) {
+        const int seg = __shfl_sync(0xffffffffu, first, k), n = (P.Lp - seg) * (d >> 3);
+        uint4* out = reinterpret_cast<uint4*>(P.H + ((size_t)(base + (unsigned)k * G) * P.Lp + seg) * d);
         for (int i = lane; i < n; i += 32) out[i] = make_uint4(0, 0, 0, 0);
       }
     }
