@@ -1197,7 +1197,7 @@ int backward_stream_all(const Plan& p, const T* items, const int32_t* lengths, c
   bf16 *Hhi = reinterpret_cast<bf16*>(s.Hp), *Hlo = Hhi + (size_t)N * p.Lp * d;
   BWD_OK(backward_stream_forward(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, nullptr, Hhi, Hlo, ws, stream_scratch, st));
   const GstaPlanes G = train_planes(p, s);
-  BWD_OK(gsta_train(p, 2, Hhi, Hlo, lengths, cand_offsets, cands, Wg, dz, G, s.dHp, train_scratch, st));
+  BWD_OK(gsta_train(p, 2, Hhi, Hlo, lengths, cand_offsets, cands, Wg, dz, G, s.dHp, nullptr, train_scratch, st));
   const float* p_sums = nullptr;
   BWD_OK(backward_stream(p, items, lengths, cand_offsets, Wv, s.dHp, d_items, dWv, &p_sums, ws, stream_scratch, st));
 #undef BWD_OK
@@ -1221,9 +1221,10 @@ int backward_stream_all(const Plan& p, const T* items, const int32_t* lengths, c
 }
 
 // Candidate lists, bf16, M > 0: gates, stacked attention and every product over the item rows on the MMAs.
-bool backward_lists_supported(const Plan& p) {
-  return sta_bwd_mma_supported(p) && sta_fwd_mma_supported(p) && gsta_train_supported(p, 1) && rows_mma_supported(p);
+bool lists_attention_supported(const Plan& p) {
+  return sta_bwd_mma_supported(p) && sta_fwd_mma_supported(p) && gsta_train_supported(p, 1) && 2 * p.M * p.H <= 64;
 }
+bool backward_lists_supported(const Plan& p) { return lists_attention_supported(p) && rows_mma_supported(p); }
 int backward_lists(const Plan& p, const bf16* items, const int32_t* lengths, const bf16* cands, const int32_t* cand_offsets,
                    const bf16* Wq, const bf16* Wk, const bf16* Wv, const bf16* Wg, const float* dz, float* d_items,
                    float* d_cands, float* dWq, float* dWk, float* dWv, float* dWg, char* ws, cudaStream_t st) {
@@ -1243,7 +1244,7 @@ int backward_lists(const Plan& p, const bf16* items, const int32_t* lengths, con
   BWD_OK(rows_project_cands(p, cands, Wq, 0.5f * p.inv_gamma, Qb, st));
   BWD_OK(rows_project_items(p, items, lengths, cand_offsets, Wk, Wv, Kb, Vb, st));
   BWD_OK(sta_fwd_mma(p, lengths, cand_offsets, nullptr, true, mma_scratch, st));
-  BWD_OK(gsta_train(p, 1, Hb, nullptr, lengths, cand_offsets, cands, Wg, dz, G, dSb, train_scratch, st));
+  BWD_OK(gsta_train(p, 1, Hb, nullptr, lengths, cand_offsets, cands, Wg, dz, G, nullptr, dSb, train_scratch, st));
   BWD_OK(gsta_weight_sums(p, G, dWg, st));
   BWD_OK(sta_bwd_mma_split(p, lengths, cand_offsets, s.dQf, dKh, dKl, dVh, dVl, mma_scratch, st));
   BWD_OK(rows_gradients(p, items, lengths, cand_offsets, Wk, Wv, dKh, dKl, dVh, dVl, d_items, dWk, dWv, st));
@@ -1285,8 +1286,8 @@ int backward_t(const Plan& p, const T* items, const int32_t* lengths, const T* c
   // ---- forward, kept in fp32: projections and H' (the FP32-ALU forward kernels), then the GSTA layers
   char* mma_scratch = ws + p.total + s.total;
   const bool mma = tensor && sta_bwd_mma_supported(p);     // (users with very few candidates keep the FP32 gate kernels)
-  const bool stream = tensor && backward_stream_supported(p);   // one candidate per user: no keys or values of the items
-  const bool train = mma && sta_fwd_mma_supported(p) && gsta_train_supported(p, 1);   // the stacked attention as well
+  const bool stream = tensor && backward_stream_supported(p);   // one candidate per user and no layer: no keys or values of the items
+  const bool train = mma && lists_attention_supported(p);   // the stacked attention as well
   char* train_scratch = mma_scratch + sta_bwd_mma_scratch_bytes(p);
   if (stream) {
     BWD_OK(gemm<T, T>(gx, N, dqk, d, cands, d, false, Wq, dqk, false, Qf, dqk, p.inv_gamma, false, false));
@@ -1327,7 +1328,7 @@ int backward_t(const Plan& p, const T* items, const int32_t* lengths, const T* c
     sta_mma_segment_arrays(p, mma_scratch, &Hb, &dSb);
     const GstaPlanes G = train_planes(p, s);
     dT0 = G.dT0;
-    BWD_OK(gsta_train(p, 1, Hb, nullptr, lengths, cand_offsets, cands, Wg, dz, G, dSb, train_scratch, st));
+    BWD_OK(gsta_train(p, 1, Hb, nullptr, lengths, cand_offsets, cands, Wg, dz, G, nullptr, dSb, train_scratch, st));
     BWD_OK(gsta_weight_sums(p, G, dWg, st));
   } else {
     {

@@ -26,13 +26,15 @@ struct GstaPlanes {
   float* dT0;
 };
 
-// Tensor cores (laser_backward_gsta.cu), bf16 inputs: np = 1: segment vectors S0 in bf16, dS [N, Lp, d] leaves as bf16;
-// np = 2: segment vectors S0 + S1 (bf16 high and low parts of fp32 values), dS leaves as fp32.  Rows of empty segments are
-// neither read nor written.  gsta_weight_sums adds the layers' weight gradients from what gsta_train left in G.
+// Tensor cores (laser_backward_gsta.cu), bf16 inputs: np = 1: segment vectors S0 in bf16; np = 2: segment vectors S0 + S1 (bf16
+// high and low parts of fp32 values).  dS [N, Lp, d] leaves as fp32 in dS32 (np = 2) or rounded to bf16 in dS16, whichever is not
+// null.  Rows of empty segments are neither read nor written.  gsta_weight_sums adds the layers' weight gradients from what
+// gsta_train left in G.
 bool gsta_train_supported(const Plan& p, int np);
 size_t gsta_train_scratch_bytes(const Plan& p, int np);
 int gsta_train(const Plan& p, int np, const void* S0, const void* S1, const int32_t* lengths, const int32_t* cand_offsets,
-               const void* cands, const void* Wg, const float* dz, const GstaPlanes& G, void* dS, char* scratch, cudaStream_t st);
+               const void* cands, const void* Wg, const float* dz, const GstaPlanes& G, float* dS32, __nv_bfloat16* dS16, char* scratch,
+               cudaStream_t st);
 int gsta_weight_sums(const Plan& p, const GstaPlanes& G, float* dWg, cudaStream_t st);
 
 // Products over the item rows on the tensor cores (laser_backward_rows.cu), users' valid rows only, bf16 inputs: K and V (or

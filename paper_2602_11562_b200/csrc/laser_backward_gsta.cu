@@ -32,7 +32,7 @@ constexpr int kTW = 8, kTThreads = kTW * 32;      // warps per block: one or two
 constexpr int kTRows = 16;                        // candidates per tile = rows of the dense MMAs; segments per chunk
 
 struct TrainParams {
-  int N, U, L, S, Lp, H, M, cpb, slots, nb;       // slots = 2 M H; nb staging buffers per warp
+  int N, U, L, S, Lp, H, M, cpb, slots, nb, kb;   // slots = 2 M H; nb staging buffers per warp, kb of them hold slot rows
   float inv_tau;
   const bf16 *S0, *S1;                            // [N, Lp, d] segment vectors: high (or only) and low parts
   const bf16* cands;
@@ -44,8 +44,8 @@ struct TrainParams {
   bf16 *rows0, *rows1;                            // [N, slots, d] qt and dm per slot (high, low)
   float* ad32;                                    // [N, Lp, slots] de and a per slot (NP = 2)
   bf16* ad16;                                     // the same as the bf16 operand it becomes (NP = 1)
-  bf16* dS16;                                     // [N, Lp, d] out (NP = 1)
-  float* dS32;                                    // [N, Lp, d] out (NP = 2)
+  bf16* dS16;                                     // [N, Lp, d] out, rounded to bf16, or
+  float* dS32;                                    // [N, Lp, d] out, fp32 (NP = 2, dS16 null)
 };
 
 // Weight images in MMA fragment order (see laser_gsta_img.cuh), each matrix as stored (B[k][n] = W[k][n]) and transposed.
@@ -604,91 +604,115 @@ __global__ void __launch_bounds__(kTThreads, 2) gsta_train_kernel(const __grid_c
   }
 
   // =============================================================================================== dH'
-  // rows = segments, k = slots: A from the de / a array, B = the candidate's slot rows (staged once: slots <= 64)
+  // rows = segments, k = slots: A from the de / a array, B = the candidate's slot rows, staged once if all of them fit the
+  // buffers and otherwise kb steps of 16 at a time for every 16 segments (any number of layers and heads, with the sums
+  // of all features in registers).  One candidate per user, d = 128, 8 heads: 256 users of 1000 items in 100 segments, 2 layers,
+  // 369 us a call (616 with the attention on the FP32 ALUs); 2048 users of 500 items 872 (1172).
   const int KS = (P.slots + 15) >> 4;
-  const bool staged = P.nb > KS;                                     // 16 staging rows are left beside the slot rows
+  const bool resident = P.kb >= KS, out16 = NP == 1 || P.dS16 != nullptr;
+  const bool staged = out16 && (!resident || P.nb > KS);             // 16 rows of a buffer are free for the result
+  uint8_t* result = resident ? mine + 16 * KS * NP * RS : mine;
   const int mi = lane >> 3, lr = lane & 7;
   const uint32_t s_trans = ((mi & 1) * 8 + lr) * RS + (mi >> 1) * 16;
+  const uint32_t s_plane = P.kb * 16 * RS;
+  auto stage_slots = [&](int cand, int k0) {                         // steps k0 .. k0 + kb - 1, planes of 16 kb rows
+    const int n = 16 * min(P.kb, KS - k0) * 2 * D16;
+#pragma unroll
+    for (int pl = 0; pl < NP; ++pl) {
+      const bf16* src = (pl ? P.rows1 : P.rows0) + ((size_t)cand * P.slots + k0 * 16) * d;
+      for (int i = lane; i < n; i += 32) {
+        const int r = i / (2 * D16), q = i % (2 * D16);
+        const bool ok = k0 * 16 + r < P.slots;
+        cp16(mine_a + pl * s_plane + r * RS + q * 16, ok ? (const void*)(src + r * d + q * 8) : (const void*)P.S0, ok ? 16u : 0u);
+      }
+    }
+    cp_commit();
+    cp_wait<0>();
+    __syncwarp();
+  };
 #pragma unroll 1
   for (int sl = 0; sl < n_slots; ++sl) {
     const int c = warp + kTW * sl, cand = c_base + c, nv = nv_s[c];
     if (cand >= c_end) continue;
     __syncwarp();
-    for (int i = lane; i < 16 * KS * 2 * D16 * NP; i += 32) {        // planes of 16 KS rows
-      const int pl = i / (16 * KS * 2 * D16), r = (i - pl * (16 * KS * 2 * D16)) / (2 * D16), q = i % (2 * D16);
-      const bf16* src = (pl ? P.rows1 : P.rows0) + ((size_t)cand * P.slots + r) * d + q * 8;
-      cp16(mine_a + (pl * 16 * KS + r) * RS + q * 16, r < P.slots ? (const void*)src : (const void*)P.S0, r < P.slots ? 16u : 0u);
-    }
-    cp_commit();
-    cp_wait<0>();
-    __syncwarp();
+    if (resident && nv > 0) stage_slots(cand, 0);
     for (int j0 = 0; j0 < nv; j0 += kTRows) {
-      uint32_t ah[4][4], al[4][4];
+      float x[D16][2][4];
 #pragma unroll
-      for (int ks = 0; ks < 4; ++ks) {
-        if (ks >= KS) break;
+      for (int jp = 0; jp < D16; ++jp)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) x[jp][0][e] = x[jp][1][e] = 0.f;
+#pragma unroll 1
+      for (int ks = 0; ks < KS; ++ks) {
+        uint32_t ah[4], al[4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
           const int j = j0 + g + (e & 1) * 8, s = ks * 16 + 2 * t + (e >> 1) * 8;
           const bool in = j < nv && s < P.slots;
           const size_t at = ((size_t)cand * Lp + j) * P.slots + s;
           if constexpr (NP == 1) {
-            ah[ks][e] = in ? *reinterpret_cast<const uint32_t*>(P.ad16 + at) : 0u;
+            ah[e] = in ? *reinterpret_cast<const uint32_t*>(P.ad16 + at) : 0u;
           } else {
             const float2 v = in ? *reinterpret_cast<const float2*>(P.ad32 + at) : make_float2(0.f, 0.f);
-            split2(v.x, v.y, ah[ks][e], al[ks][e]);
+            split2(v.x, v.y, ah[e], al[e]);
           }
         }
-      }
+        const int k = ks % P.kb;
+        if (!resident && k == 0) {
+          __syncwarp();                                              // every lane is done with the rows before
+          stage_slots(cand, ks);
+        }
+        const uint32_t row = mine_a + k * 16 * RS + s_trans;
 #pragma unroll
-      for (int jp = 0; jp < D16; ++jp) {
-        float c0[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-        for (int ks = 0; ks < 4; ++ks) {
-          if (ks >= KS) break;
+        for (int jp = 0; jp < D16; ++jp) {
           uint32_t b[4];
-          ldsm_x4_t(b, mine_a + ks * 16 * RS + s_trans + jp * 32);
-          mma16816(c0, ah[ks][0], ah[ks][1], ah[ks][2], ah[ks][3], b[0], b[1]);
-          mma16816(c1, ah[ks][0], ah[ks][1], ah[ks][2], ah[ks][3], b[2], b[3]);
+          ldsm_x4_t(b, row + jp * 32);
+          mma16816(x[jp][0], ah[0], ah[1], ah[2], ah[3], b[0], b[1]);
+          mma16816(x[jp][1], ah[0], ah[1], ah[2], ah[3], b[2], b[3]);
           if constexpr (NP == 2) {
-            mma16816(c0, al[ks][0], al[ks][1], al[ks][2], al[ks][3], b[0], b[1]);
-            mma16816(c1, al[ks][0], al[ks][1], al[ks][2], al[ks][3], b[2], b[3]);
-            ldsm_x4_t(b, mine_a + (16 * KS + ks * 16) * RS + s_trans + jp * 32);
-            mma16816(c0, ah[ks][0], ah[ks][1], ah[ks][2], ah[ks][3], b[0], b[1]);
-            mma16816(c1, ah[ks][0], ah[ks][1], ah[ks][2], ah[ks][3], b[2], b[3]);
-          }
-        }
-        if (NP == 1 && staged) {                                     // through shared memory: whole rows leave in 16-byte pieces
-          uint8_t* o = mine + 16 * KS * RS + g * RS + jp * 32 + 4 * t;
-          *reinterpret_cast<uint32_t*>(o) = pack2(c0[0], c0[1]);
-          *reinterpret_cast<uint32_t*>(o + 16) = pack2(c1[0], c1[1]);
-          *reinterpret_cast<uint32_t*>(o + 8 * RS) = pack2(c0[2], c0[3]);
-          *reinterpret_cast<uint32_t*>(o + 8 * RS + 16) = pack2(c1[2], c1[3]);
-          continue;
-        }
-#pragma unroll
-        for (int hf = 0; hf < 2; ++hf) {
-          const int j = j0 + g + hf * 8;
-          if (j >= nv) continue;
-          const size_t at = ((size_t)cand * Lp + j) * d + jp * 16 + 2 * t;
-          if constexpr (NP == 1) {
-            *reinterpret_cast<uint32_t*>(P.dS16 + at) = pack2(c0[2 * hf], c0[2 * hf + 1]);
-            *reinterpret_cast<uint32_t*>(P.dS16 + at + 8) = pack2(c1[2 * hf], c1[2 * hf + 1]);
-          } else {
-            *reinterpret_cast<float2*>(P.dS32 + at) = make_float2(c0[2 * hf], c0[2 * hf + 1]);
-            *reinterpret_cast<float2*>(P.dS32 + at + 8) = make_float2(c1[2 * hf], c1[2 * hf + 1]);
+            mma16816(x[jp][0], al[0], al[1], al[2], al[3], b[0], b[1]);
+            mma16816(x[jp][1], al[0], al[1], al[2], al[3], b[2], b[3]);
+            ldsm_x4_t(b, row + s_plane + jp * 32);
+            mma16816(x[jp][0], ah[0], ah[1], ah[2], ah[3], b[0], b[1]);
+            mma16816(x[jp][1], ah[0], ah[1], ah[2], ah[3], b[2], b[3]);
           }
         }
       }
-      if (NP == 1 && staged) {
+      if (staged) {                                                  // through shared memory: whole rows leave in 16-byte pieces
+        if (!resident) __syncwarp();
+#pragma unroll
+        for (int jp = 0; jp < D16; ++jp) {
+          uint8_t* o = result + g * RS + jp * 32 + 4 * t;
+          *reinterpret_cast<uint32_t*>(o) = pack2(x[jp][0][0], x[jp][0][1]);
+          *reinterpret_cast<uint32_t*>(o + 16) = pack2(x[jp][1][0], x[jp][1][1]);
+          *reinterpret_cast<uint32_t*>(o + 8 * RS) = pack2(x[jp][0][2], x[jp][0][3]);
+          *reinterpret_cast<uint32_t*>(o + 8 * RS + 16) = pack2(x[jp][1][2], x[jp][1][3]);
+        }
         __syncwarp();
         bf16* out = P.dS16 + ((size_t)cand * Lp + j0) * d;
 #pragma unroll
         for (int i = 0; i < D16; ++i) {
           const int piece = i * 32 + lane, r = piece / (2 * D16), q = piece - r * (2 * D16);
-          if (j0 + r < nv) *reinterpret_cast<uint4*>(out + r * d + q * 8) = ld16(mine + (16 * KS + r) * RS + q * 16);
+          if (j0 + r < nv) *reinterpret_cast<uint4*>(out + r * d + q * 8) = ld16(result + r * RS + q * 16);
         }
         __syncwarp();
+        continue;
+      }
+#pragma unroll
+      for (int hf = 0; hf < 2; ++hf) {
+        const int j = j0 + g + hf * 8;
+        if (j >= nv) continue;
+#pragma unroll
+        for (int jp = 0; jp < D16; ++jp) {
+          const size_t at = ((size_t)cand * Lp + j) * d + jp * 16 + 2 * t;
+          if (out16) {
+            *reinterpret_cast<uint32_t*>(P.dS16 + at) = pack2(x[jp][0][2 * hf], x[jp][0][2 * hf + 1]);
+            *reinterpret_cast<uint32_t*>(P.dS16 + at + 8) = pack2(x[jp][1][2 * hf], x[jp][1][2 * hf + 1]);
+          } else {
+            *reinterpret_cast<float2*>(P.dS32 + at) = make_float2(x[jp][0][2 * hf], x[jp][0][2 * hf + 1]);
+            *reinterpret_cast<float2*>(P.dS32 + at + 8) = make_float2(x[jp][1][2 * hf], x[jp][1][2 * hf + 1]);
+          }
+        }
       }
     }
   }
@@ -831,9 +855,6 @@ TrainScratch carve_train(const Plan& p, int np, char* base) {
   return s;
 }
 
-int train_slot_steps(const Plan& p) { return (2 * p.M * p.H + 15) / 16; }
-int train_buffers(const Plan& p, int np) { return std::max(np == 1 ? 2 : 1, train_slot_steps(p)); }
-
 template <int D16, int NP>
 int launch_train(TrainParams P, const Plan& p, const TrainScratch& s, const void* Wg, const int32_t* lengths,
                  const int32_t* cand_offsets, cudaStream_t st) {
@@ -885,17 +906,32 @@ int launch_sums(const Plan& p, const GstaPlanes& G, float* dWg, cudaStream_t st)
   return LASER_OK;
 }
 
-size_t train_smem(const Plan& p, int np) {
+int train_slot_steps(const Plan& p) { return (2 * p.M * p.H + 15) / 16; }
+
+size_t train_smem(const Plan& p, int np, int nb) {
   const size_t RS = 2 * p.d + 16;
   return 2 * (size_t)kTRows * RS + 2 * np * (size_t)kTRows * (p.H * RS + (p.H % 2 ? 0 : 16)) + RS + kTRows * sizeof(int) + 48 +
-         (size_t)kTW * train_buffers(p, np) * kTRows * RS * np;
+         (size_t)kTW * nb * kTRows * RS * np;
+}
+
+constexpr size_t kTrainSmemMax = 226 * 1024, kSmemPerSm = 228 * 1024, kSmemPerBlock = 1024;    // (the last: reserved by the system)
+int train_blocks_per_sm(const Plan& p, int np, int nb) { return (int)std::min<size_t>(2, kSmemPerSm / (train_smem(p, np, nb) + kSmemPerBlock)); }
+
+// Staging buffers of a warp: two (the next 16 segments arrive while these are worked on), one where the second would cost a
+// block per SM or does not fit, and as many as the slot rows need where that costs nothing.
+int train_buffers(const Plan& p, int np) {
+  auto free_of_charge = [&](int nb, int base) {
+    return train_smem(p, np, nb) <= kTrainSmemMax && train_blocks_per_sm(p, np, nb) == train_blocks_per_sm(p, np, base);
+  };
+  const int base = np == 1 || free_of_charge(2, 1) ? 2 : 1, all = train_slot_steps(p);
+  return all > base && free_of_charge(all, base) ? all : base;
 }
 
 }  // namespace
 
 bool gsta_train_supported(const Plan& p, int np) {
   return p.dtype == LASER_BF16 && p.M > 0 && p.d % 16 == 0 && p.d >= 16 && p.d <= 128 && p.H <= 8 && p.dvh % 16 == 0 &&
-         train_slot_steps(p) <= 4 && train_smem(p, np) <= 226 * 1024;
+         train_smem(p, np, np == 1 ? 2 : 1) <= kTrainSmemMax;
 }
 size_t gsta_train_scratch_bytes(const Plan& p, int np) { return gsta_train_supported(p, np) ? carve_train(p, np, nullptr).total : 0; }
 
@@ -913,14 +949,16 @@ size_t gsta_train_scratch_bytes(const Plan& p, int np) { return gsta_train_suppo
   }
 
 int gsta_train(const Plan& p, int np, const void* S0, const void* S1, const int32_t* lengths, const int32_t* cand_offsets,
-               const void* cands, const void* Wg, const float* dz, const GstaPlanes& G, void* dS, char* scratch, cudaStream_t st) {
+               const void* cands, const void* Wg, const float* dz, const GstaPlanes& G, float* dS32, __nv_bfloat16* dS16, char* scratch,
+               cudaStream_t st) {
   const TrainScratch s = carve_train(p, np, scratch);
   TrainParams P = {};
   P.N = p.N; P.U = p.U; P.L = p.L; P.S = p.S; P.Lp = p.Lp; P.H = p.H; P.M = p.M; P.slots = 2 * p.M * p.H; P.nb = train_buffers(p, np);
+  P.kb = std::min(P.nb, train_slot_steps(p));
   P.inv_tau = p.inv_tau;
   P.S0 = (const bf16*)S0; P.S1 = (const bf16*)S1; P.cands = (const bf16*)cands; P.dz = dz;
   P.img = s.img; P.nseg = s.nseg; P.G = G; P.stat = s.stat; P.rows0 = s.rows0; P.rows1 = s.rows1; P.ad16 = s.ad16; P.ad32 = s.ad32;
-  P.dS16 = (bf16*)dS; P.dS32 = (float*)dS;
+  P.dS16 = dS16; P.dS32 = dS32;
 #define LASER_TRAIN_CALL(D) (np == 1 ? launch_train<D, 1>(P, p, s, Wg, lengths, cand_offsets, st) : launch_train<D, 2>(P, p, s, Wg, lengths, cand_offsets, st))
   LASER_TRAIN_DISPATCH(LASER_TRAIN_CALL)
 #undef LASER_TRAIN_CALL

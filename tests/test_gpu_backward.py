@@ -28,7 +28,7 @@ CASES = [
 ]
 
 
-def _check(case_kw, seed, path, bar, want_kernel=None):
+def _check(case_kw, seed, path, bar, want_kernel=None, want_kernels=()):
     kw = dict(case_kw)
     std = kw.pop("emb_std", "one" if kw["d"] <= 32 else "inv_sqrt_d")
     w = make_custom(seed=seed, emb_std=std, **kw)
@@ -48,6 +48,7 @@ def _check(case_kw, seed, path, bar, want_kernel=None):
     assert P.laser_check_status(ws) == 0
     if want_kernel is not None:
         assert ("bwd_sta_mma" in names) == want_kernel, names
+    assert set(want_kernels) <= set(names), names
     worst = {}
     for k, r in ref.items():
         g = got[k].cpu().numpy().astype(np.float64)
@@ -175,15 +176,18 @@ STREAM_CASES = [
     dict(U=3, C=1, L=1100, d=128, H=8, S=17, M=1, dtype="bf16", lengths=[1100, 1099, 16]),
     dict(U=2, C=1, L=400, d=96, H=3, S=10, M=2, dtype="bf16", lengths=[400, 211]),
     dict(U=640, C=1, L=40, d=64, H=2, S=10, M=2, dtype="bf16"),
-    dict(U=7, C=1, L=330, d=128, H=8, S=10, M=3, dtype="bf16"),                              # 48 slots, three staging buffers
+    dict(U=7, C=1, L=330, d=128, H=8, S=10, M=3, dtype="bf16"),                              # 48 slots in steps of 16 through one staging buffer
     dict(U=3000, C=1, L=24, d=32, H=1, S=8, M=1, dtype="bf16"),                              # 16 candidates per attention block
     dict(U=2100, C=1, L=36, d=32, H=2, S=2, M=1, dtype="bf16"),                              # two row tiles, no table of users
+    dict(U=9, C=1, L=300, d=128, H=8, S=20, M=2, dtype="bf16", lengths=[300, 299, 161, 160, 1, 0, 33, 300, 20]),   # 32 slots, one buffer
+    dict(U=6, C=1, L=200, d=96, H=6, S=10, M=3, dtype="bf16"),                               # 36 slots, the last step partly filled
+    dict(U=5, C=1, L=90, d=64, H=4, S=10, M=7, dtype="bf16"),                                # seven layers
 ]
 
 
 @pytest.mark.parametrize("case", range(len(STREAM_CASES)))
 def test_backward_one_candidate_matches_oracle(case):
-    worst = _check(STREAM_CASES[case], 1300 + case, P.PATH_AUTO, 2e-3, want_kernel=False)
+    worst = _check(STREAM_CASES[case], 1300 + case, P.PATH_AUTO, 2e-3, want_kernel=False, want_kernels=("bs_fwd", "gsta_train", "bs_bwd"))
     print("backward, one candidate per user, worst error / largest entry:", {k: f"{v:.2e}" for k, v in worst.items()})
 
 
