@@ -1220,20 +1220,37 @@ int backward_stream_all(const Plan& p, const T* items, const int32_t* lengths, c
   return gsta_weight_sums(p, G, dWg, st);
 }
 
-// Candidate lists, bf16, M > 0: gates, stacked attention and every product over the item rows on the MMAs.
-bool lists_attention_supported(const Plan& p) {
-  return sta_bwd_mma_supported(p) && sta_fwd_mma_supported(p) && gsta_train_supported(p, 1) && 2 * p.M * p.H <= 64;
+// bf16 parts of a segment vector in the stacked attention of candidate lists (0: not on the MMAs).  One part: H', the key-folded
+// queries and the attention's weights are rounded to bf16, which the widths of 32, 64 and 128 with at most 128 segments and 64
+// (layer, head) slots take.  Two parts: the attention is as good as in fp32.  8 users x 64 candidates, d = 96, 3 heads, 3 layers,
+// 2-norm errors of d_items | dW_q with one part 3.4e-3 | 2.2e-3, with two 2.4e-3 | 1.4e-3, on the FP32 ALUs 2.4e-3 | 1.4e-3 (what
+// is left is the bf16 of the gates); 64 users x 256 candidates, 2048 items, d = 96, 3 heads: the call 539 against 627 us.
+int lists_parts(const Plan& p) {
+  const int np = (p.d == 32 || p.d == 64 || p.d == 128) && p.Lp <= 128 && 2 * p.M * p.H <= 64 ? 1 : 2;
+  return sta_bwd_mma_supported(p) && sta_fwd_mma_supported(p) && gsta_train_supported(p, np) ? np : 0;
 }
-bool backward_lists_supported(const Plan& p) { return lists_attention_supported(p) && rows_mma_supported(p); }
+// The recomputed H' and its stacked attention, forward and backward, on that many parts: leaves the bf16 dH' for the gate kernel
+// and adds the layers' weight gradients.
+int lists_attention(const Plan& p, int np, const BwdScratch& s, const int32_t* lengths, const int32_t* cand_offsets, const bf16* cands,
+                    const bf16* Wg, const float* dz, const GstaPlanes& G, float* dWg, char* mma_scratch, char* train_scratch,
+                    cudaStream_t st) {
+  bf16 *Hb = reinterpret_cast<bf16*>(s.Hp), *Hl = np == 2 ? Hb + (size_t)p.N * p.Lp * p.d : nullptr;
+  int rc = sta_fwd_mma(p, lengths, cand_offsets, nullptr, Hb, Hl, mma_scratch, st);
+  if (rc == LASER_OK)
+    rc = gsta_train(p, np, Hb, Hl, lengths, cand_offsets, cands, Wg, dz, G, nullptr, sta_mma_segment_gradients(p, mma_scratch), train_scratch, st);
+  return rc == LASER_OK ? gsta_weight_sums(p, G, dWg, st) : rc;
+}
+
+// Candidate lists, bf16, M > 0: gates, stacked attention and every product over the item rows on the MMAs.
+bool backward_lists_supported(const Plan& p) { return lists_parts(p) > 0 && rows_mma_supported(p); }
 int backward_lists(const Plan& p, const bf16* items, const int32_t* lengths, const bf16* cands, const int32_t* cand_offsets,
                    const bf16* Wq, const bf16* Wk, const bf16* Wv, const bf16* Wg, const float* dz, float* d_items,
                    float* d_cands, float* dWq, float* dWk, float* dWv, float* dWg, char* ws, cudaStream_t st) {
   const size_t N = p.N, d = p.d, M = p.M, dqk = p.dqk, UL = (size_t)p.U * p.L;
   const BwdScratch s = carve_scratch(p, ws + p.total);
   char *mma_scratch = ws + p.total + s.total, *train_scratch = mma_scratch + sta_bwd_mma_scratch_bytes(p);
-  bf16 *Qb, *Kb, *Vb, *Hb, *dSb;
+  bf16 *Qb, *Kb, *Vb;
   sta_mma_operand_arrays(p, mma_scratch, &Qb, &Kb, &Vb);
-  sta_mma_segment_arrays(p, mma_scratch, &Hb, &dSb);
   bf16 *dKh = reinterpret_cast<bf16*>(s.dK), *dKl = dKh + UL * dqk, *dVh = reinterpret_cast<bf16*>(s.dV), *dVl = dVh + UL * d;
   const GstaPlanes G = train_planes(p, s);
   int rc;
@@ -1243,9 +1260,7 @@ int backward_lists(const Plan& p, const bf16* items, const int32_t* lengths, con
   BWD_OK(zero_arrays(Z, st));
   BWD_OK(rows_project_cands(p, cands, Wq, 0.5f * p.inv_gamma, Qb, st));
   BWD_OK(rows_project_items(p, items, lengths, cand_offsets, Wk, Wv, Kb, Vb, st));
-  BWD_OK(sta_fwd_mma(p, lengths, cand_offsets, nullptr, true, mma_scratch, st));
-  BWD_OK(gsta_train(p, 1, Hb, nullptr, lengths, cand_offsets, cands, Wg, dz, G, nullptr, dSb, train_scratch, st));
-  BWD_OK(gsta_weight_sums(p, G, dWg, st));
+  BWD_OK(lists_attention(p, lists_parts(p), s, lengths, cand_offsets, cands, Wg, dz, G, dWg, mma_scratch, train_scratch, st));
   BWD_OK(sta_bwd_mma_split(p, lengths, cand_offsets, s.dQf, dKh, dKl, dVh, dVl, mma_scratch, st));
   BWD_OK(rows_gradients(p, items, lengths, cand_offsets, Wk, Wv, dKh, dKl, dVh, dVl, d_items, dWk, dWv, st));
   // (Qt and dM are not used on this route; each holds N rows of H d floats, and d_qk <= 2 H d)
@@ -1287,7 +1302,7 @@ int backward_t(const Plan& p, const T* items, const int32_t* lengths, const T* c
   char* mma_scratch = ws + p.total + s.total;
   const bool mma = tensor && sta_bwd_mma_supported(p);     // (users with very few candidates keep the FP32 gate kernels)
   const bool stream = tensor && backward_stream_supported(p);   // one candidate per user and no layer: no keys or values of the items
-  const bool train = mma && lists_attention_supported(p);   // the stacked attention as well
+  const int parts = tensor ? lists_parts(p) : 0;           // the stacked attention on the MMAs as well
   char* train_scratch = mma_scratch + sta_bwd_mma_scratch_bytes(p);
   if (stream) {
     BWD_OK(gemm<T, T>(gx, N, dqk, d, cands, d, false, Wq, dqk, false, Qf, dqk, p.inv_gamma, false, false));
@@ -1312,7 +1327,8 @@ int backward_t(const Plan& p, const T* items, const int32_t* lengths, const T* c
       BWD_OK(gemm<T, T>(gx, (int)UL, d, d, items, d, false, Wv, d, false, Vf, d, 1.f, false, false));
     }
     if (mma) BWD_OK(sta_mma_operands(p, Qf, kv_ready ? nullptr : Kf, kv_ready ? nullptr : Vf, mma_scratch, st));
-    if (mma && sta_fwd_mma_supported(p)) BWD_OK(sta_fwd_mma(p, lengths, cand_offsets, train ? nullptr : s.Hp, train, mma_scratch, st));
+    if (parts) {                                             // (with the attention, below)
+    } else if (mma && sta_fwd_mma_supported(p)) BWD_OK(sta_fwd_mma(p, lengths, cand_offsets, s.Hp, nullptr, nullptr, mma_scratch, st));
     else if (p.dqh == 16 && (dvh == 16 || dvh == 32 || dvh == 64) && p.H <= 32) BWD_OK(simt_attend_f32(p, lengths, cand_offsets, s.Hp, ws, st));
     else BWD_OK(simt_sta_f32(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, s.Hp, ws, st));
   } else if (p.dqh == 16 && (dvh == 16 || dvh == 32 || dvh == 64) && p.H <= 32) {
@@ -1323,14 +1339,16 @@ int backward_t(const Plan& p, const T* items, const int32_t* lengths, const T* c
   }
   const size_t Nd = (size_t)N * d, NHd = Nd * H;
   float* dT0 = s.dT;
-  if (train) {
-    bf16 *Hb, *dSb;
-    sta_mma_segment_arrays(p, mma_scratch, &Hb, &dSb);
-    const GstaPlanes G = train_planes(p, s);
-    dT0 = G.dT0;
-    BWD_OK(gsta_train(p, 1, Hb, nullptr, lengths, cand_offsets, cands, Wg, dz, G, nullptr, dSb, train_scratch, st));
-    BWD_OK(gsta_weight_sums(p, G, dWg, st));
-  } else {
+  bool attended = false;
+  if constexpr (sizeof(T) == 2) {
+    if (parts) {
+      const GstaPlanes G = train_planes(p, s);
+      dT0 = G.dT0;
+      BWD_OK(lists_attention(p, parts, s, lengths, cand_offsets, cands, Wg, dz, G, dWg, mma_scratch, train_scratch, st));
+      attended = true;
+    }
+  }
+  if (!attended) {
     {
       LaunchScope ls("bwd_to_f32", st);
       to_f32_kernel<T><<<296, 256, 0, st>>>(cands, s.T, Nd);
@@ -1406,7 +1424,7 @@ int backward_t(const Plan& p, const T* items, const int32_t* lengths, const T* c
   }
   if (stream) {
   } else if (mma) {
-    BWD_OK(sta_bwd_mma(p, train ? nullptr : s.dHp, lengths, cand_offsets, s.dQf, s.dK, s.dV, mma_scratch, st));
+    BWD_OK(sta_bwd_mma(p, attended ? nullptr : s.dHp, lengths, cand_offsets, s.dQf, s.dK, s.dV, mma_scratch, st));
   } else {
     BWD_OK(launch_sta_bwd(p, Qf, Kf, Vf, s.dHp, lengths, cand_offsets, s.dQf, s.dK, s.dV, st));
   }
@@ -1430,7 +1448,7 @@ int backward_t(const Plan& p, const T* items, const int32_t* lengths, const T* c
 
 size_t backward_scratch_bytes(const Plan& p) {
   return carve_scratch(p, nullptr).total + sta_bwd_mma_scratch_bytes(p) + backward_stream_scratch_bytes(p) +
-         std::max(gsta_train_scratch_bytes(p, 1), gsta_train_scratch_bytes(p, 2));
+         (backward_stream_supported(p) ? gsta_train_scratch_bytes(p, 2) : lists_parts(p) ? gsta_train_scratch_bytes(p, lists_parts(p)) : 0);
 }
 
 bool backward_tensor_supported(const Plan& p) { return p.dtype == LASER_BF16; }

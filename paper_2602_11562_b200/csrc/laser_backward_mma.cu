@@ -297,7 +297,7 @@ struct FwdMmaParams {
   const bf16 *Qb, *Kb, *Vb;
   const int32_t *lengths, *cand_offsets;
   float* Hp;                                     // fp32 H' (null: not wanted)
-  bf16* Hb;                                      // bf16 H' for the attention kernels below (null: not wanted)
+  bf16 *Hb, *Hl;                                 // H' rounded to bf16, and what the rounding left (null: not wanted)
   int L, d, dqk, H, S, Lp, N, rows;              // rows = staged rows per block (min(S, L) rounded up to 16)
 };
 
@@ -386,20 +386,26 @@ __global__ void __launch_bounds__(kBwdWarps * 32) sta_fwd_mma_kernel(const FwdMm
         if (r0 < C) *reinterpret_cast<float2*>(P.Hp + at + (size_t)r0 * row + c) = make_float2(acc[j][0], acc[j][1]);
         if (r1 < C) *reinterpret_cast<float2*>(P.Hp + at + (size_t)r1 * row + c) = make_float2(acc[j][2], acc[j][3]);
       }
-      if (P.Hb) {                                                  // through shared memory: 16-byte pieces of a candidate's row
-        unsigned char* o = smem + P.rows * (KS + VS) + warp * 16 * VS + g * VS + c * 2;
-        *reinterpret_cast<uint32_t*>(o) = pack2(acc[j][0], acc[j][1]);
-        *reinterpret_cast<uint32_t*>(o + 8 * VS) = pack2(acc[j][2], acc[j][3]);
-      }
     }
-    if (P.Hb) {
+    for (bf16* out = P.Hb; out; out = out == P.Hb ? P.Hl : nullptr) {   // through shared memory: 16-byte pieces of a candidate's row
+      unsigned char* tile = smem + P.rows * (KS + VS) + warp * 16 * VS;
+#pragma unroll
+      for (int j = 0; j < 2 * DV16; ++j)
+#pragma unroll
+        for (int hf = 0; hf < 2; ++hf) {
+          float &x = acc[j][2 * hf], &y = acc[j][2 * hf + 1];
+          const uint32_t v = pack2(x, y);
+          *reinterpret_cast<uint32_t*>(tile + (g + 8 * hf) * VS + (j * 8 + 2 * t) * 2) = v;
+          x -= bf16_lo(v);
+          y -= bf16_hi(v);
+        }
       __syncwarp();
 #pragma unroll
       for (int i = 0; i < DV16; ++i) {
         const int piece = i * 32 + lane, r = piece / (2 * DV16), q = piece - r * (2 * DV16);
         if (c0 + r < C)
-          *reinterpret_cast<uint4*>(P.Hb + at + (size_t)(c0 + r) * row + q * 8) =
-              *reinterpret_cast<const uint4*>(smem + P.rows * (KS + VS) + warp * 16 * VS + r * VS + q * 16);
+          *reinterpret_cast<uint4*>(out + at + (size_t)(c0 + r) * row + q * 8) =
+              *reinterpret_cast<const uint4*>(tile + r * VS + q * 16);
       }
       __syncwarp();
     }
@@ -453,7 +459,7 @@ int cast(const float* src, bf16* dst, size_t n, float scale, cudaStream_t st) {
 }
 
 struct MmaScratch {
-  bf16 *Qb, *Kb, *Vb, *dSb, *Hb;
+  bf16 *Qb, *Kb, *Vb, *dSb;
   size_t total;
 };
 MmaScratch carve_mma(const Plan& p, char* base) {
@@ -469,7 +475,6 @@ MmaScratch carve_mma(const Plan& p, char* base) {
   s.Kb = take(UL * p.dqk);
   s.Vb = take(UL * p.d);
   s.dSb = take((size_t)p.N * p.Lp * p.d);
-  s.Hb = take((size_t)p.N * p.Lp * p.d);
   s.total = off;
   return s;
 }
@@ -505,14 +510,10 @@ bool sta_fwd_mma_supported(const Plan& p) {
   return sta_bwd_mma_supported(p) && fwd_smem(p) <= kFwdSmemMax && (long long)p.Lp * p.H <= 0x7fffffffLL;
 }
 
-void sta_mma_segment_arrays(const Plan& p, char* scratch, __nv_bfloat16** Hb, __nv_bfloat16** dSb) {
-  const MmaScratch s = carve_mma(p, scratch);
-  *Hb = s.Hb;
-  *dSb = s.dSb;
-}
+__nv_bfloat16* sta_mma_segment_gradients(const Plan& p, char* scratch) { return carve_mma(p, scratch).dSb; }
 
-int sta_fwd_mma(const Plan& p, const int32_t* lengths, const int32_t* cand_offsets, float* Hp, bool bf16_copy, char* scratch,
-                cudaStream_t st) {
+int sta_fwd_mma(const Plan& p, const int32_t* lengths, const int32_t* cand_offsets, float* Hp, __nv_bfloat16* Hb, __nv_bfloat16* Hl,
+                char* scratch, cudaStream_t st) {
   MmaShape sh;
   if (!mma_shape(p, &sh) || !sta_fwd_mma_supported(p)) return LASER_ERR_UNSUPPORTED;
   const MmaScratch s = carve_mma(p, scratch);
@@ -520,7 +521,8 @@ int sta_fwd_mma(const Plan& p, const int32_t* lengths, const int32_t* cand_offse
   P.Qb = s.Qb; P.Kb = s.Kb; P.Vb = s.Vb;
   P.lengths = lengths; P.cand_offsets = cand_offsets;
   P.Hp = Hp;
-  P.Hb = bf16_copy ? s.Hb : nullptr;
+  P.Hb = Hb;
+  P.Hl = Hl;
   P.L = p.L; P.d = p.d; P.dqk = p.dqk; P.H = p.H; P.S = p.S; P.Lp = p.Lp; P.N = p.N;
   P.rows = (std::min(p.S, p.L) + 15) / 16 * 16;
   const size_t smem = fwd_smem(p);

@@ -92,7 +92,7 @@ int backward(const Plan& p, const void* items, const int32_t* lengths, const voi
              float* d_cands, float* dWq, float* dWk, float* dWv, float* dWg, char* ws, cudaStream_t st, bool tensor);
 // Tensor-core kernels of the backward pass (laser_backward_mma.cu), all on bf16 copies kept in `scratch`
 // (sta_bwd_mma_scratch_bytes): sta_mma_operands makes the copies of Qf (Q / gamma), Kf and Vf; sta_fwd_mma recomputes H'
-// in fp32 from them (rows of empty segments are left as they are); sta_bwd_mma copies dHp (null: the bf16 copy is there
+// from them (rows of empty segments are left as they are); sta_bwd_mma copies dHp (null: the bf16 copy is there
 // already), writes the dK / dV rows of valid items (the rest must hold zeros) and adds to dQf.
 bool sta_bwd_mma_supported(const Plan& p);
 bool sta_fwd_mma_supported(const Plan& p);
@@ -101,10 +101,11 @@ int sta_mma_operands(const Plan& p, const float* Qf, const float* Kf, const floa
 // The bf16 Q / (2 gamma) [N, d_qk], K [U L, d_qk] and V [U L, d] arrays inside `scratch`, for a producer that writes them directly (it then passes
 // Kf = Vf = null to sta_mma_operands).
 void sta_mma_operand_arrays(const Plan& p, char* scratch, __nv_bfloat16** Qb, __nv_bfloat16** Kb, __nv_bfloat16** Vb);
-// The bf16 H' that sta_fwd_mma leaves (bf16_copy) and the bf16 dH' that sta_bwd_mma reads, [N, L', d] each.
-void sta_mma_segment_arrays(const Plan& p, char* scratch, __nv_bfloat16** Hb, __nv_bfloat16** dSb);
-int sta_fwd_mma(const Plan& p, const int32_t* lengths, const int32_t* cand_offsets, float* Hp, bool bf16_copy, char* scratch,
-                cudaStream_t st);
+// The bf16 dH' that sta_bwd_mma reads, [N, L', d].
+__nv_bfloat16* sta_mma_segment_gradients(const Plan& p, char* scratch);
+// H' as fp32 (Hp), or rounded to bf16 (Hb) and, with Hl, what the rounding left (null: not wanted).
+int sta_fwd_mma(const Plan& p, const int32_t* lengths, const int32_t* cand_offsets, float* Hp, __nv_bfloat16* Hb, __nv_bfloat16* Hl,
+                char* scratch, cudaStream_t st);
 int sta_bwd_mma(const Plan& p, const float* dHp, const int32_t* lengths, const int32_t* cand_offsets, float* dQf,
                 float* dK, float* dV, char* scratch, cudaStream_t st);
 // The same with dK and dV as bf16 high and low parts.

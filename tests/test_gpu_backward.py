@@ -204,3 +204,38 @@ def test_backward_users_without_a_candidate():
     for k, r in ref.items():
         assert np.max(np.abs(got[k].cpu().numpy() - r)) <= 2e-3 * np.max(np.abs(r)), k
     assert not got["d_items"][1].any() and not got["d_items"][4].any()
+
+
+# Candidate lists whose attention works on bf16 pairs: widths other than 32, 64 and 128, more than 128 segments, more than 64 slots.
+# (lists of 8 and more candidates; d_qk of 192 takes the products of the general route)
+PAIR_CASES = [
+    dict(U=2, C=21, L=170, d=96, H=6, S=10, M=3, dtype="bf16", lengths=[170, 161]),           # 36 slots
+    dict(U=3, C=17, L=330, d=48, H=3, S=2, M=2, dtype="bf16", lengths=[330, 31, 0]),          # 165 segments
+    dict(U=2, C=300, L=260, d=64, H=2, S=2, M=1, dtype="bf16", lengths=[260, 3]),             # 130 segments, 16 candidates per block
+    dict(U=2, C=9, L=64, d=128, H=8, S=16, M=5, dtype="bf16", lengths=[64, 40]),              # 80 slots, one staging buffer
+    dict(U=2, C=12, L=50, d=32, H=2, S=10, M=17, dtype="bf16", lengths=[50, 21], emb_std="inv_sqrt_d"),   # 68 slots: 17 layers
+    dict(U=2, C=10, L=90, d=96, H=6, S=9, M=1, dtype="bf16", lengths=[90, 90], d_qh=32),
+    dict(U=1, C=40, L=120, d=112, H=7, S=40, M=2, dtype="bf16", lengths=[115]),
+    dict(U=1, C=33, L=64, d=16, H=1, S=16, M=2, dtype="bf16", lengths=[64], emb_std="inv_sqrt_d"),
+]
+
+
+@pytest.mark.parametrize("case", range(len(PAIR_CASES)))
+def test_backward_lists_on_pairs_match_oracle(case):
+    _check(PAIR_CASES[case], 1500 + case, P.PATH_AUTO, TENSOR_BAR, want_kernel=True, want_kernels=("bwd_sta_fwd_mma", "gsta_train"))
+
+
+def test_backward_lists_on_pairs_keep_fp32_attention():
+    """dWq of long users: the bf16 roundings of K and of the gates' gradients differ from item to item and average out over the
+    items, those of the stacked attention (H', query, weights, de) are common to the items of a segment and do not.  2-norm error
+    with pairs 7e-4 .. 9e-4 (as with the FP32 attention kernels), with bf16 operands 1.9e-3; the bar lies between."""
+    w = make_custom(U=3, C=96, L=4000, d=96, H=6, S=100, M=1, dtype="bf16", seed=1550, lengths=[4000, 3150, 2222])
+    s = w.spec
+    dz = np.random.default_rng(1551).standard_normal((w.N, s.d)).astype(np.float32)
+    ref = backward_oracle.backward(w.items, w.lengths, w.cands, w.cand_offsets, w.Wq, w.Wk, w.Wv, w.Wg, s.S, s.H,
+                                   dz.astype(np.float64), w.gamma, w.tau)["dWq"]
+    b = P.DeviceBatch.from_workload(w)
+    got = P.laser_backward(b.cfg, *b.args(), b.Wg, torch.from_numpy(dz).cuda())["dWq"].cpu().numpy()
+    err = float(np.linalg.norm(got - ref) / np.linalg.norm(ref))
+    print(f"dWq, 2-norm error {err:.2e}")
+    assert err <= 1.3e-3
