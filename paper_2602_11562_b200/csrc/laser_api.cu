@@ -1,4 +1,5 @@
 // extern "C" entry points: argument validation, path selection, workspace carve-up, dispatch.
+#include <cuda.h>
 #include <math.h>
 #include <string.h>
 
@@ -47,7 +48,20 @@ int device_sms() {
   return n;
 }
 
-// One slot per (kernel, device), open addressing (a full table only costs a repeated driver call).  The attribute is raised
+unsigned current_context() {
+  using GetId = CUresult (*)(CUcontext, unsigned long long*);
+  static const GetId get_id = []() -> GetId {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    const bool ok = cudaGetDriverEntryPoint("cuCtxGetId", &f, cudaEnableDefault, &q) == cudaSuccess && q == cudaDriverEntryPointSuccess;
+    return ok ? reinterpret_cast<GetId>(f) : nullptr;
+  }();
+  unsigned long long id = 0;
+  return get_id && get_id(nullptr, &id) == CUDA_SUCCESS && id < (1ull << 16) ? (unsigned)id : 0u;
+}
+
+// One slot per (kernel, context), open addressing (a full table only costs a repeated driver call).  By context, not by device:
+// a second context on the device, or the one after a reset, starts with the kernel's default.  The attribute is raised
 // under a lock and never lowered, so that threads with launches of different sizes do not undo each other's.
 cudaError_t allow_smem_ptr(const void* kernel, int bytes) {
   struct Slot {
@@ -56,12 +70,10 @@ cudaError_t allow_smem_ptr(const void* kernel, int bytes) {
   };
   constexpr unsigned kSlots = 1024;
   static Slot slots[kSlots];
-  int dev = 0;
-  const cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  const uintptr_t key = reinterpret_cast<uintptr_t>(kernel) ^ ((uintptr_t)dev << 56);
+  const unsigned ctx = current_context();
+  const uintptr_t key = reinterpret_cast<uintptr_t>(kernel) ^ ((uintptr_t)ctx << 48);      // (host pointers have 48 bits)
   Slot* mine = nullptr;
-  for (unsigned i = 0; i < 16 && !mine; ++i) {
+  for (unsigned i = 0; i < 16 && !mine && ctx; ++i) {
     Slot& s = slots[((key >> 4) * 0x9E3779B97F4A7C15ull >> 32) + i & (kSlots - 1)];
     uintptr_t empty = 0;
     if (s.key.load(std::memory_order_acquire) == key || s.key.compare_exchange_strong(empty, key) || empty == key) mine = &s;

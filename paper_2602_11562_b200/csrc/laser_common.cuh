@@ -213,7 +213,9 @@ inline cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 bloc
 
 // SM count of the current device, asked of the driver once per device.
 int device_sms();
-// Lets `kernel` use `bytes` of dynamic shared memory on the current device.  The attribute is set on the first call with
+// A number that no other context of this process has or had (0: none is current, or it has no such number: nothing to cache by).
+unsigned current_context();
+// Lets `kernel` use `bytes` of dynamic shared memory in the current context.  The attribute is set on the first call with
 // a larger size only: the driver call would otherwise be a good part of what a small call costs on the host.
 cudaError_t allow_smem_ptr(const void* kernel, int bytes);
 template <typename... KArgs>
