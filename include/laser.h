@@ -253,9 +253,9 @@ LASER_API int laser_backward(const laser_config* cfg, const void* items, const i
  *   - cfg->path is ignored; items .. Hprime are as for laser_sta_forward.
  *   - status_out: optional DEVICE int32; if non-NULL the device-side status word of this call (LASER_OK or
  *     LASER_ERR_BAD_INPUT) is copied to it on the stream after the kernels.
- *   - The first call on each device looks up the array's device address (with that device current); make
+ *   - The first call in each context looks up the array's device address (with that context current); make
  *     that first call outside any stream capture.
- *   - All calls on a device share the one array, which keeps the previous call's contents (only the status
+ *   - All calls in a context share the one array, which keeps the previous call's contents (only the status
  *     word is cleared per call): two calls that overlap on the GPU (different streams or threads) race.
  *     Serialise them on one stream or with events. */
 #define LASER_STATIC_SCRATCH_BYTES (8u << 20)

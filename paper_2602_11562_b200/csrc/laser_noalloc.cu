@@ -15,26 +15,31 @@ namespace laser {
 namespace {
 
 constexpr size_t kStaticScratchBytes = LASER_STATIC_SCRATCH_BYTES;
-constexpr int kMaxDevices = 64;
+constexpr unsigned kMaxContexts = 64;
 
 // The scratch itself.  In host code this name is only a host-side stand-in for the symbol, NOT a device
 // address: host code must go through cudaGetSymbolAddress (below) and hand the result to the kernels.
 static __device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBytes];
 
 std::mutex g_mu;
-char* g_scratch_ptr[kMaxDevices];   // device address of g_static_scratch on each device, once resolved
+struct { unsigned ctx; char* ptr; } g_scratch[kMaxContexts];   // device address of g_static_scratch by context, once resolved
+unsigned g_next;                                               // entry that is overwritten next
 
-// Resolves, once per device and with that device current, where g_static_scratch lives on the current device.
-int static_scratch_for_current_device(char** out) {
-  int dev = -1;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return LASER_ERR_CUDA;
+// Where g_static_scratch lives in the current context.  (Every context has its own copy: one that came after a reset, or beside
+// another on the same device, must not be given the address that the library had in the other.)
+int static_scratch_for_current_context(char** out) {
+  const unsigned ctx = current_context();
   std::lock_guard<std::mutex> lock(g_mu);
-  if (!g_scratch_ptr[dev]) {
-    void* ptr = nullptr;
-    if (cudaGetSymbolAddress(&ptr, g_static_scratch) != cudaSuccess || !ptr) return LASER_ERR_CUDA;
-    g_scratch_ptr[dev] = static_cast<char*>(ptr);
-  }
-  *out = g_scratch_ptr[dev];
+  for (const auto& e : g_scratch)
+    if (ctx && e.ctx == ctx) {
+      *out = e.ptr;
+      return LASER_OK;
+    }
+  void* ptr = nullptr;
+  if (cudaGetSymbolAddress(&ptr, g_static_scratch) != cudaSuccess || !ptr) return LASER_ERR_CUDA;
+  *out = static_cast<char*>(ptr);
+  const unsigned now = current_context();                      // (the first call of a thread may have made one current)
+  if (now) g_scratch[g_next++ % kMaxContexts] = {now, *out};
   return LASER_OK;
 }
 
@@ -70,7 +75,7 @@ extern "C" int laser_sta_forward_static(const laser_config* cfg, const void* ite
       if (!q || (reinterpret_cast<uintptr_t>(q) & 15u)) return LASER_ERR_INVALID_ARG;
   }
   char* scratch = nullptr;
-  if ((rc = static_scratch_for_current_device(&scratch)) != LASER_OK) return rc;
+  if ((rc = static_scratch_for_current_context(&scratch)) != LASER_OK) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   // The array keeps whatever the previous call left in it.  Only the status word must start at zero (the first
   // kernel clears it): Q, K and V are fully rewritten for every row that is read afterwards.

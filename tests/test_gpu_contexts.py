@@ -79,7 +79,7 @@ print("contexts ok")
 """
 
 
-@pytest.mark.parametrize("mode", ["f32", "bf16"])
+@pytest.mark.parametrize("mode", ["f32", "bf16", "static"])
 def test_calls_in_several_contexts_agree(mode, repo_root):
     env = dict(os.environ, PYTHONPATH=repo_root)
     r = subprocess.run([sys.executable, "-c", CHILD, mode], cwd=repo_root, env=env, capture_output=True, text=True, timeout=300)
