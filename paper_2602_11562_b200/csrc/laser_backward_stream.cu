@@ -204,17 +204,16 @@ __global__ void __launch_bounds__(kBThreads) bs_fwd_kernel(BsParams P) {
 //
 // A job is (16-segment tile, user, head), tiles slowest and users in the launch order (longest first): the tiles that exist
 // are the first ones of each tile index, so the warps' shares are equal to within a job.  Candidate and segment count of a
-// user come from a table that the block fills once: looked up per job they were two dependent round trips to memory in front
-// of the rows' own.
-constexpr int kBsTable = 2048;
+// user are two dependent round trips to memory in front of the rows' own, unless the block fills a table of them first
+// (tabled; see launch_rows).
 
 // (NPC: the most column pairs a head has; KA: k-tiles requested together.  Half a matrix of columns at most leaves the
 // registers for all of a row tile's k-tiles: r -> s 68 -> 58 us, with the high and low products interleaved.)
 template <int D16, int NPC, int KA, bool to_y>
-__global__ void __launch_bounds__(256, 2) bs_rows_kernel(BsParams P) {
+__global__ void __launch_bounds__(256, 2) bs_rows_kernel(BsParams P, int tabled) {
   constexpr int d = 16 * D16, WS = 2 * d + 16;
   extern __shared__ __align__(128) uint8_t smem[];
-  __shared__ int2 table[kBsTable];                          // (candidate, segments) by launch position
+  int2* table = reinterpret_cast<int2*>(smem + d * WS);     // (candidate, segments) by launch position
   chain_wait();
   chain_release();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3, H = P.H, dvh = d / H;
@@ -228,7 +227,6 @@ __global__ void __launch_bounds__(256, 2) bs_rows_kernel(BsParams P) {
     const int cand = one_candidate(P, P.order ? min(max(P.order[pos], 0), P.U - 1) : pos, &len);
     return make_int2(cand, cand >= 0 ? (len + P.S - 1) / P.S : 0);
   };
-  const bool tabled = P.U <= kBsTable;
   if (tabled)
     for (int i = tid; i < P.U; i += 256) table[i] = look_up(i);
   cp_wait<0>();
@@ -669,11 +667,19 @@ BsParams bs_params(const Plan& p, const BsScratch& s, const void* items, const i
 
 template <int D16, int NPC, int KA, bool to_y>
 int launch_rows(const Plan& p, const BsParams& P, cudaStream_t st) {
-  const size_t smem = (size_t)p.d * (2 * p.d + 16);
-  const long long jobs = (long long)p.U * ((p.Lp + 15) / 16) * p.H;
+  // A table of the users costs a block U look-ups and saves it one per job, of which it has U tiles H / (2 SMs): whatever the
+  // number of users, it pays where a user has many jobs.  Both launches together, without | with it, us: 2 jobs per user (9000
+  // users, d = 64) 50 | 87, 8 (4096 users) 72 | 77, 14 (2048 users, d = 128) 117 | 116, 16 (2048 users, d = 64) 70 | 68, 24 (4096
+  // users, d = 128) 254 | 226, 28 (1024 users) 95 | 87, 32 (2048 users) 166 | 142.
+  constexpr size_t kHalfSm = (228 / 2 - 1) * 1024;          // (two blocks per SM beside each other)
+  const int tiles = (p.Lp + 15) / 16;
+  const size_t w_bytes = (size_t)p.d * (2 * p.d + 16), table = (size_t)p.U * sizeof(int2);
+  const bool tabled = tiles * p.H > 16 && w_bytes + table <= kHalfSm;
+  const size_t smem = w_bytes + (tabled ? table : 0);
+  const long long jobs = (long long)p.U * tiles * p.H;
   auto kernel = bs_rows_kernel<D16, NPC, KA, to_y>;
   LASER_CUDA_OK(allow_smem(kernel, smem));
-  LASER_CUDA_OK(launch_chained(kernel, dim3((unsigned)std::min<long long>((jobs + 7) / 8, 2 * device_sms())), dim3(256), smem, st, P));
+  LASER_CUDA_OK(launch_chained(kernel, dim3((unsigned)std::min<long long>((jobs + 7) / 8, 2 * device_sms())), dim3(256), smem, st, P, tabled ? 1 : 0));
   return LASER_OK;
 }
 

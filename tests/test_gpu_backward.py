@@ -178,10 +178,11 @@ STREAM_CASES = [
     dict(U=640, C=1, L=40, d=64, H=2, S=10, M=2, dtype="bf16"),
     dict(U=7, C=1, L=330, d=128, H=8, S=10, M=3, dtype="bf16"),                              # 48 slots in steps of 16 through one staging buffer
     dict(U=3000, C=1, L=24, d=32, H=1, S=8, M=1, dtype="bf16"),                              # 16 candidates per attention block
-    dict(U=2100, C=1, L=36, d=32, H=2, S=2, M=1, dtype="bf16"),                              # two row tiles, no table of users
+    dict(U=2100, C=1, L=36, d=32, H=2, S=2, M=1, dtype="bf16"),                              # two row tiles, users looked up per job
     dict(U=9, C=1, L=300, d=128, H=8, S=20, M=2, dtype="bf16", lengths=[300, 299, 161, 160, 1, 0, 33, 300, 20]),   # 32 slots, one buffer
     dict(U=6, C=1, L=200, d=96, H=6, S=10, M=3, dtype="bf16"),                               # 36 slots, the last step partly filled
     dict(U=5, C=1, L=90, d=64, H=4, S=10, M=7, dtype="bf16"),                                # seven layers
+    dict(U=2600, C=1, L=68, d=64, H=4, S=1, M=1, dtype="bf16"),                              # a table of more users than threads and blocks: 20 jobs each
 ]
 
 
