@@ -356,19 +356,23 @@ __global__ void __launch_bounds__(kMaxThreads) sta_regs_kernel(const float* __re
 
 template <typename TO, int DVH>
 int launch_sta_regs(const Plan& p, const int32_t* lengths, const int32_t* cand_offsets, TO* Hp, char* ws, cudaStream_t st) {
-  // up to four warps per (tile, head), each with at least four items of a chunk
-  const int per_chunk = p.S < kStaItems ? p.S : kStaItems;
+  // Up to four warps per (tile, head), each with at least four items of a chunk, while there are few of them: with 8 warps per SM and
+  // more two, with 32 one.  One | two | four, us: 5 users x 61 candidates (640 warps) 21 | 17 | 15; 20 x 60, segments of 60 (1120) 29
+  // | 23 | 25; 32 x 3, d = 128 (2560) 18 | 15 | 22; 4 x 300 (2720) 23 | 21 | 25; 40 x 60 (5120) 31 | 33 | 39; 256 x 6, segments of
+  // 20 (25600) 60 | 76 | 150.
+  const int per_chunk = p.S < kStaItems ? p.S : kStaItems, ctiles = (p.maxC + kStaCands - 1) / kStaCands;
+  const long long warps = (long long)p.Lp * ctiles * p.U * p.H, sms = device_sms();
+  const int most = warps > 32 * sms ? 1 : warps > 8 * sms ? 2 : 4;
   int parts = 1;
-  while (parts < 4 && 2 * parts * p.H <= 16 && per_chunk / (2 * parts) >= 4) parts *= 2;
+  while (parts < most && 2 * parts * p.H <= 16 && per_chunk / (2 * parts) >= 4) parts *= 2;
   const size_t smem = ((size_t)kStaItems * (p.dqk + p.d) + (size_t)(parts - 1) * p.H * DVH * 33) * sizeof(float);
   if (smem > 200 * 1024) return LASER_ERR_UNSUPPORTED;
   auto kernel = p.H <= 16 ? sta_regs_kernel<TO, DVH, 512> : sta_regs_kernel<TO, DVH, 1024>;
   LASER_CUDA_OK(allow_smem(kernel, smem));
   LaunchScope ls("sta_simt", st);
-  LASER_CUDA_OK(launch_chained(kernel, dim3(p.Lp, (p.maxC + kStaCands - 1) / kStaCands, p.U),
-                               dim3(32 * p.H * parts), smem, st, (const float*)(ws + p.off_q), (const float*)(ws + p.off_k),
-                               (const float*)(ws + p.off_v), (const int*)lengths, (const int*)cand_offsets, Hp, p.L, p.d,
-                               p.dqk, p.H, p.S, p.Lp, p.N, parts, (const int*)p.item_offsets,
+  LASER_CUDA_OK(launch_chained(kernel, dim3(p.Lp, ctiles, p.U), dim3(32 * p.H * parts), smem, st,
+                               (const float*)(ws + p.off_q), (const float*)(ws + p.off_k), (const float*)(ws + p.off_v),
+                               (const int*)lengths, (const int*)cand_offsets, Hp, p.L, p.d, p.dqk, p.H, p.S, p.Lp, p.N, parts, (const int*)p.item_offsets,
                                reinterpret_cast<int*>(ws + p.off_status)));
   return LASER_OK;
 }

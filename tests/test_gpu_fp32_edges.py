@@ -17,6 +17,8 @@ CASES = [
     dict(U=3, C=400, L=64, d=32, H=2, S=16, M=2),                    # enough candidates for four per block, a partial block
     dict(U=1, C=3, L=1680, d=64, H=2, S=2, M=1),                     # segment vectors that fit only without row padding
     dict(U=1, C=5, L=40, d=256, H=4, S=20, M=1, d_qh=16),            # as many columns as threads
+    dict(U=300, C=3, L=40, d=64, H=4, S=20, M=1),                    # two item parts: 2400 warps without
+    dict(U=700, C=2, L=40, d=64, H=4, S=20, M=1),                    # one: 5600 warps
 ]
 
 
