@@ -1034,9 +1034,12 @@ int launch_sta_bwd(const Plan& p, const float* Qf, const float* Kf, const float*
   const int cps = (min(p.S, L) + kChunk - 1) / kChunk;
   const int dqh = dqk / H;
   const int variant = (dqh == 16 && dvh == 32) ? 2 : (dqh == 16 && dvh == 16) ? 1 : 0;   // register-resident head slices
-  // up to four warps per (32 items, head): small batches run about one block per SM and are bound by a warp's serial walk
+  // Up to four warps per (32 items, head): small batches run about one block per SM and are bound by a warp's serial walk (6 users
+  // x 45 candidates: 48, 29, 23 us with one, two, four).  Where two already fill the SMs' warps, four only add their sums (40 users x
+  // 40 candidates: 74, 72, 89), and two want at least eight candidates each (20: 50, 43, 56; but 5: 35, 50; 7: 136, 183).
+  const bool crowded = 2ll * Lp * cps * U * H > 16ll * device_sms();
   int parts = 1;
-  while (variant && parts < 4 && 2 * parts * H <= 16 && p.maxC >= 4 * parts) parts *= 2;
+  while (variant && parts < (crowded ? 2 : 4) && 2 * parts * H <= 16 && p.maxC >= (crowded ? 16 : 4) * parts) parts *= 2;
   auto smem_of = [&](int step) {
     return ((parts > 1 ? (size_t)H * (dqh + dvh) * 33 : 0) + (variant ? (size_t)kChunk * (dqk + 1) : 2 * (size_t)kChunk * (dqk + 1 + d + 1)) +
             (size_t)step * (dqk + d + H * 33)) * sizeof(float);

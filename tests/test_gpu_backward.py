@@ -25,6 +25,8 @@ CASES = [
     dict(U=3, C=399, L=48, d=32, H=2, S=16, M=2, dtype="f32", lengths=[48, 17, 33]),       # four candidates per attention block, a partial one
     dict(U=1, C=6, L=30, d=64, H=4, S=7, M=7, dtype="f32", lengths=[30]),                  # more products than one launch takes
     dict(U=2, C=3, L=33, d=256, H=4, S=16, M=1, dtype="f32", lengths=[33, 32], d_qh=16),   # as many columns as threads
+    dict(U=150, C=17, L=128, d=32, H=2, S=32, M=1, dtype="f32"),                           # many gate blocks: two warps share their items
+    dict(U=150, C=5, L=128, d=64, H=2, S=32, M=1, dtype="bf16"),                           # and with few candidates one
 ]
 
 
@@ -151,6 +153,12 @@ def test_backward_of_users_with_few_candidates_keeps_the_fp32_gate_kernels():
     # one candidate per user (the one-candidate serving shape): the matrix products still run on the tensor cores
     kw = dict(U=40, C=1, L=128, d=64, H=2, S=32, M=1, dtype="bf16", lengths=[128] * 20 + [77] * 19 + [0])
     _check(kw, 1300, P.PATH_AUTO, TENSOR_BAR, want_kernel=False)
+
+
+def test_backward_of_few_candidates_in_many_blocks():
+    # bf16, 2 .. 7 candidates per user: FP32 gates, one warp per (32 items, head); FP32 sums of two item parts (1600 warps) and of one
+    for U in (100, 400):
+        _check(dict(U=U, C=3, L=64, d=64, H=4, S=16, M=1, dtype="bf16"), 1330 + U, P.PATH_AUTO, 2e-3, want_kernel=False, want_kernels=("bwd_sta", "sta_simt"))
 
 
 def test_backward_tensor_path_on_request_only_where_it_exists():
