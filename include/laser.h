@@ -217,13 +217,16 @@ LASER_API int laser_sta_softmax_forward(const laser_config* cfg, const void* ite
  *   LASER_PATH_SIMT                 FP32 ALUs throughout, either dtype: every gradient within 1e-4 of its largest entry.
  *   LASER_PATH_AUTO / _STREAM       fp32 batches as above.  bf16 batches on the tensor cores, fp32 accumulation throughout.
  *                                   Candidate lists (max_cands_per_user >= 8, d_qk / H in {16, 32}, d / H in {16, 32, 64}): the
- *                                   contractions through the gates, the recomputed H' and the attention itself with bf16
- *                                   operands, as the forward's tensor-core path rounds them, the dense products with 16-bit
- *                                   (bf16 pairs) or TF32 operands: every gradient within 2e-2 of its largest entry while the
- *                                   attention logits stay within a few nats (at tens of nats the bf16 rounding of a segment
- *                                   vector alone moves a softmax weight by several per cent: ask for the FP32 ALUs).  One
- *                                   candidate per user: 16-bit or TF32 operands everywhere (2e-3).  Fewer than 8 candidates, or
- *                                   other widths: FP32 gates and attention, TF32 products.
+ *                                   contractions through the gates and the recomputed H' with bf16 operands, as the forward's
+ *                                   tensor-core path rounds them, the dense products with 16-bit (bf16 pairs) or TF32 operands:
+ *                                   every gradient within 2e-2 of its largest entry.  The stacked attention runs on the tensor
+ *                                   cores for d <= 128 and H <= 8, any number of layers and segments: with bf16 operands for d =
+ *                                   32, 64 or 128, at most 128 segments and 2 M H <= 64, while the logits stay within a few nats (at
+ *                                   tens of nats the bf16 rounding of a segment vector alone moves a softmax weight by several per
+ *                                   cent: ask for the FP32 ALUs), and with 16-bit operands for all others; beyond d = 128 or H = 8
+ *                                   on the FP32 ALUs.  One candidate per user (d_qk / H and d / H multiples of 16, d <= 128, H <= 8):
+ *                                   16-bit or TF32 operands everywhere (2e-3).  Fewer than 8 candidates, or other widths: FP32
+ *                                   gates and attention, TF32 products.
  *   LASER_PATH_TENSOR               as LASER_PATH_AUTO for bf16 batches; LASER_ERR_UNSUPPORTED for fp32 batches.
  *   dz          [N, d] fp32            IN
  *   d_items     [U, L, d] fp32         OUT (rows of padding are zero)

@@ -149,10 +149,9 @@ def test_backward_full_size_configs_sampled_users(name, users):
         assert not got["d_items"][u, int(w.lengths[u]):].any()
 
 
-def test_backward_of_users_with_few_candidates_keeps_the_fp32_gate_kernels():
-    # one candidate per user (the one-candidate serving shape): the matrix products still run on the tensor cores
+def test_backward_of_one_candidate_per_user_takes_the_streaming_kernels():
     kw = dict(U=40, C=1, L=128, d=64, H=2, S=32, M=1, dtype="bf16", lengths=[128] * 20 + [77] * 19 + [0])
-    _check(kw, 1300, P.PATH_AUTO, TENSOR_BAR, want_kernel=False)
+    _check(kw, 1300, P.PATH_AUTO, TENSOR_BAR, want_kernel=False, want_kernels=("bs_fwd", "gsta_train", "bs_bwd", "bs_wv"))
 
 
 def test_backward_of_few_candidates_in_many_blocks():
