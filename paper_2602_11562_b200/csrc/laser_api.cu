@@ -64,6 +64,7 @@ unsigned current_context() {
 // a second context on the device, or the one after a reset, starts with the kernel's default.  The attribute is raised
 // under a lock and never lowered, so that threads with launches of different sizes do not undo each other's.
 cudaError_t allow_smem_ptr(const void* kernel, int bytes) {
+  if (bytes <= 40 * 1024) return cudaSuccess;      // (any kernel may use 48 KB, its static share included, unasked)
   struct Slot {
     std::atomic<uintptr_t> key;
     std::atomic<int> bytes;
@@ -199,10 +200,11 @@ static int run_sta(const Plan& p, const void* items, const int32_t* lengths, con
 }
 
 static int run_gsta(const Plan& p, const void* Hp, const int32_t* lengths, const int32_t* cand_offsets,
-                    const void* cands, const void* Wg, void* z, char* ws, cudaStream_t st, bool images_ready) {
+                    const void* cands, const void* Wg, void* z, char* ws, cudaStream_t st, bool images_ready,
+                    bool follows_call) {
   switch (p.path) {
-    case LASER_PATH_SIMT: return simt_gsta(p, Hp, lengths, cand_offsets, cands, Wg, z, ws, st);
-    case LASER_PATH_TENSOR: return tensor_gsta(p, Hp, lengths, cand_offsets, cands, Wg, z, ws, st, images_ready);
+    case LASER_PATH_SIMT: return simt_gsta(p, Hp, lengths, cand_offsets, cands, Wg, z, ws, st, follows_call);
+    case LASER_PATH_TENSOR: return tensor_gsta(p, Hp, lengths, cand_offsets, cands, Wg, z, ws, st, images_ready, follows_call);
     case LASER_PATH_STREAM: return gsta_mma(p, Hp, lengths, cand_offsets, cands, Wg, z, ws, st, images_ready);
     default: return LASER_ERR_UNSUPPORTED;
   }
@@ -216,7 +218,7 @@ static int forward_impl(const Plan& p, const void* items, const int32_t* lengths
   const bool side_images = p.M > 0 && p.path != LASER_PATH_SIMT && gsta_mma_supported(p);
   const int rc = run_sta(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, Hp, ws, st, side_images ? Wg : nullptr);
   if (rc != LASER_OK) return rc;
-  return run_gsta(p, Hp, lengths, cand_offsets, cands, Wg, z, ws, st, side_images);
+  return run_gsta(p, Hp, lengths, cand_offsets, cands, Wg, z, ws, st, side_images, true);
 }
 
 }  // namespace laser
@@ -262,7 +264,7 @@ int laser_gsta_forward(const laser_config* cfg, const void* Hprime, const int32_
   char* ws = static_cast<char*>(workspace);
   if ((rc = clear_status(p, ws, st)) != LASER_OK) return rc;
   if (p.N == 0) return LASER_OK;
-  return run_gsta(p, Hprime, lengths, cand_offsets, cands, Wgsta, z, ws, st, false);
+  return run_gsta(p, Hprime, lengths, cand_offsets, cands, Wgsta, z, ws, st, false, false);
 }
 
 int laser_forward(const laser_config* cfg, const void* items, const int32_t* lengths, const void* cands,
@@ -458,7 +460,7 @@ int laser_forward_ffn(const laser_config* cfg, const void* items, const int32_t*
   if (rc != LASER_OK) return rc;
   rc = ffn_forward(p, ffn, Hp, lengths, cand_offsets, ws, ws + p.total, st);
   if (rc != LASER_OK) return rc;
-  return run_gsta(p, Hp, lengths, cand_offsets, cands, Wgsta, z, ws, st, side_images);
+  return run_gsta(p, Hp, lengths, cand_offsets, cands, Wgsta, z, ws, st, side_images, true);
 }
 
 namespace {

@@ -71,11 +71,17 @@ int simt_sta_softmax(const Plan& p, const void* items, const int32_t* lengths, c
                      const int32_t* cand_offsets, const void* Wq, const void* Wk, const void* Wv, void* Hprime, char* ws,
                      cudaStream_t st);
 int simt_gsta(const Plan& p, const void* Hprime, const int32_t* lengths, const int32_t* cand_offsets, const void* cands,
-              const void* Wg, void* z, char* ws, cudaStream_t st);
+              const void* Wg, void* z, char* ws, cudaStream_t st, bool follows_call);
+// The same for the widths in use (laser_simt_gsta.cu); LASER_ERR_UNSUPPORTED for all other shapes.
+int gsta_f32(const Plan& p, const void* Hprime, const int32_t* lengths, const int32_t* cand_offsets, const void* cands,
+             const void* Wg, void* z, char* ws, cudaStream_t st, bool follows_call);
 // Eq. 8-9 on the FP32 ALUs (fp32 Q / gamma, K, V at off_q, off_k, off_v), and the segment sums alone, from fp32 Q / gamma, K, V at off_q, off_k, off_v (16-wide query heads, 16-, 32- or 64-wide value
 // heads; else LASER_ERR_UNSUPPORTED).
 int simt_project(const Plan& p, const void* items, const int32_t* lengths, const void* cands, const void* Wq,
                  const void* Wk, const void* Wv, char* ws, cudaStream_t st);
+// The same with larger tiles, for batches of many rows (laser_simt_proj.cu); LASER_ERR_UNSUPPORTED for widths it does not take.
+int simt_project_tiles(const Plan& p, const void* items, const int32_t* lengths, const void* cands, const void* Wq, const void* Wk,
+                       const void* Wv, char* ws, cudaStream_t st);
 int simt_attend_f32(const Plan& p, const int32_t* lengths, const int32_t* cand_offsets, float* Hprime32, char* ws,
                     cudaStream_t st);
 // STA on the FP32 ALUs with an fp32 H' whatever the I/O dtype; leaves fp32 Q / gamma, K, V at off_q, off_k, off_v.
@@ -123,7 +129,7 @@ int tensor_sta(const Plan& p, const void* items, const int32_t* lengths, const v
 // Launches the bounded-wait self-test block (laser_tensor.cu); the status word is the first word of ws.
 int tensor_wait_selftest(char* ws, int poll_limit, cudaStream_t st);
 int tensor_gsta(const Plan& p, const void* Hprime, const int32_t* lengths, const int32_t* cand_offsets,
-                const void* cands, const void* Wg, void* z, char* ws, cudaStream_t st, bool images_ready);
+                const void* cands, const void* Wg, void* z, char* ws, cudaStream_t st, bool images_ready, bool follows_call);
 
 // Fused warp-MMA GSTA kernel for bf16 (laser_gsta.cu); needs gsta_mma_image_bytes(p) of scratch at off_gimg.
 bool gsta_mma_supported(const Plan& p);

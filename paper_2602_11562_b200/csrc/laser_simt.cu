@@ -14,12 +14,11 @@ constexpr int kStaThreads = 128;
 constexpr int kStaMaxJ = 64;      // columns per thread = d/4 <= 64  (d <= 256)
 constexpr int kGstaThreads = 256;
 
-// Eq. 4 / Eq. 8-9 in one launch: Q = t W_q / gamma for the candidates (the first q_tiles blocks of grid.x), K = H W_k and
-// V = H W_v for every user's valid items (padded [U, L, .] outputs).  A block owns 32 rows x 32 columns, a thread eight rows
-// of one column: the weights come straight from L2, a warp reading one 128-byte row piece per step, sixteen steps in flight;
-// the rows sit in shared memory and are read as 128-bit broadcasts.  Small batches are latency-bound, and the column
-// tiles spread them over more SMs than blocks that own all columns did (one user of 256 items, d = 32: two launches of
-// 4.5 us each before, one of 3 us now).  Block 0 clears the status word for the kernels behind this one.
+// Eq. 4 / Eq. 8-9 in one launch, for widths that the tiled kernels (laser_simt_proj.cu) do not take: Q = t W_q / gamma for the
+// candidates (the first q_tiles blocks of grid.x), K = H W_k and V = H W_v for every user's valid items (padded [U, L, .]
+// outputs).  A block owns 32 rows x 32 columns, a thread eight rows of one column: the weights come straight from L2, a warp
+// reading one 128-byte row piece per step, sixteen steps in flight; the rows sit in shared memory and are read as 128-bit
+// broadcasts.  Block 0 clears the status word for the kernels behind this one.
 struct ProjParams {
   const void *items, *cands, *Wq, *Wk, *Wv;
   float *Q, *K, *V;
@@ -377,14 +376,15 @@ int launch_sta_regs(const Plan& p, const int32_t* lengths, const int32_t* cand_o
   return LASER_OK;
 }
 
-// One block per CB candidates.  Eq. 7 in the reassociated form (exact in real arithmetic):
+// One block per CB candidates, for widths that gsta_f32_kernel (laser_simt_gsta.cu) does not take.  Eq. 7 in the reassociated form
+// (exact in real arithmetic):
 //   q = t W_q;  qt_h = W_k[:, head h] q_h  (so that (s_j W_k)_h . q_h = s_j . qt_h);  e_{j,h} = s_j . qt_h / tau;
 //   a = softmax_j(e);  m_h = sum_j a_{j,h} s_j;  o[head h] = m_h W_v[:, head h];  t += o.
 // Small batches are bound by the latency of these phases, so each of them spreads its outputs AND its sums over all 256
 // threads: the two d x d products split the contraction index into `parts` partial sums, a score belongs to four lanes,
 // each with a quarter of the features (segment vectors sit in rows padded by four words, so the eight rows a warp reads at a
 // time do not share banks).  With more candidates than two blocks per SM, a block takes CB of them and reads every weight
-// once for all (two layers, d = 64, four heads, 16 segments, 140 candidates: 68 -> 14 us).
+// once for all.
 template <typename T, int CB>
 __global__ void __launch_bounds__(kGstaThreads)
 gsta_simt_kernel(const T* __restrict__ Hp, const int* __restrict__ lengths, const int* __restrict__ cand_offsets,
@@ -549,6 +549,8 @@ template <typename T>
 int simt_project_t(const Plan& p, const T* items, const int32_t* lengths, const T* cands, const T* Wq, const T* Wk,
                    const T* Wv, char* ws, cudaStream_t st) {
   if (p.N == 0 || p.U == 0) return LASER_OK;
+  const int rc = simt_project_tiles(p, items, lengths, cands, Wq, Wk, Wv, ws, st);
+  if (rc != LASER_ERR_UNSUPPORTED) return rc;
   ProjParams P;
   P.items = items; P.cands = cands; P.Wq = Wq; P.Wk = Wk; P.Wv = Wv;
   P.Q = reinterpret_cast<float*>(ws + p.off_q);
@@ -699,7 +701,9 @@ int simt_sta_softmax(const Plan& p, const void* items, const int32_t* lengths, c
 }
 
 int simt_gsta(const Plan& p, const void* Hprime, const int32_t* lengths, const int32_t* cand_offsets, const void* cands,
-              const void* Wg, void* z, char* ws, cudaStream_t st) {
+              const void* Wg, void* z, char* ws, cudaStream_t st, bool follows_call) {
+  const int rc = gsta_f32(p, Hprime, lengths, cand_offsets, cands, Wg, z, ws, st, follows_call);
+  if (rc != LASER_ERR_UNSUPPORTED) return rc;
   if (p.dtype == LASER_F32)
     return simt_gsta_t<float>(p, (const float*)Hprime, lengths, cand_offsets, (const float*)cands, (const float*)Wg,
                               (float*)z, ws, st);

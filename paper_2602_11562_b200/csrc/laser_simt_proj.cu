@@ -1,0 +1,211 @@
+// Eq. 4 / Eq. 8-9 for batches of many rows on the fp32 path: Q = t W_q / gamma of the candidates, K = H W_k and V = H W_v of every
+// user's valid items, all fp32.  A block owns 64 rows x 64 columns with all of the contraction in shared memory (one barrier);
+// the first q_tiles blocks of grid.x take the candidates, block 0 clears the status word for the kernels behind this one.  Widths
+// that are no multiples of 4 (fp32) or 16 (bf16) keep proj_simt_kernel (laser_simt.cu), whose 32 x 32 tiles read each weight from L2
+// per 8 multiply-adds.  us of the two (CUDA events, about 6 too long; 40 users of up to 2700 items, 62 % valid): d = 64 fp32 101 -> 40,
+// d = 128 with 128 query columns 341 -> 125 (half of the FP32 rate); 5 users of up to 777, d = 64: 13 -> 10; 2 users of up to 4000,
+// d = d_qk = 128, bf16 42 -> 11.
+//
+//   proj_tile_f32_kernel  fp32 inputs: a thread has 8 x 4 outputs (its rows lie 8 apart, so that the two rows that a warp reads at
+//                         a time start in different banks), 12 shared-memory reads of 16 bytes per 128 multiply-adds.
+//   proj_tile_mma_kernel  bf16 inputs: warp-level MMAs.  Products of bf16 values are exact in fp32 and the sums are fp32, so Q, K
+//                         and V are those of the FP32 ALUs up to the order of the sums.  Bound by the fp32 stores.
+#include "laser_common.cuh"
+#include "laser_mma.cuh"
+
+namespace laser {
+namespace {
+
+using bf16 = __nv_bfloat16;
+using namespace mma;
+
+constexpr int kRows = 64, kCols = 64, kThreads = 128;
+
+struct TileParams {
+  const void *items, *cands, *Wq, *Wk, *Wv;
+  float *Q, *K, *V;
+  const int *lengths, *row_off;          // row_off: packed item layout (null: padded)
+  int* status;
+  int U, L, N, d, dqk, q_tiles, tiles_per_user;
+  float inv_gamma;
+};
+
+struct Tile {
+  int rows, n_cols;                      // rows == 0: nothing to do
+  size_t in_row, out_row;
+  bool is_q;
+};
+__device__ __forceinline__ Tile find_tile(const TileParams& P) {
+  Tile t;
+  t.is_q = (int)blockIdx.x < P.q_tiles;
+  t.n_cols = t.is_q ? P.dqk : P.dqk + P.d;
+  if (t.is_q) {
+    const int r0 = blockIdx.x * kRows;
+    t.rows = min(kRows, P.N - r0);
+    t.in_row = t.out_row = r0;
+  } else {
+    const int x = blockIdx.x - P.q_tiles, u = x / P.tiles_per_user, r0 = (x - u * P.tiles_per_user) * kRows;
+    int len = P.lengths[u];              // (invalid lengths and row offsets are reported by the STA kernel)
+    if (len < 0 || len > P.L) len = 0;
+    if (P.row_off && len > 0 && (P.row_off[u] < 0 || P.row_off[u] > P.row_off[P.U] - len)) len = 0;
+    t.rows = max(0, min(kRows, len - r0));
+    t.in_row = (P.row_off ? (size_t)P.row_off[u] : (size_t)u * P.L) + r0;
+    t.out_row = (size_t)u * P.L + r0;
+  }
+  if ((int)blockIdx.y * kCols >= t.n_cols) t.rows = 0;
+  return t;
+}
+// Column col of [W_q], or of [W_k | W_v]: its place in its matrix, and in that matrix's output
+template <typename T>
+__device__ __forceinline__ const T* weights_at(const TileParams& P, bool is_q, int col, int* ld) {
+  const bool first = col < P.dqk;
+  *ld = first ? P.dqk : P.d;
+  return static_cast<const T*>(is_q ? P.Wq : first ? P.Wk : P.Wv) + (first ? col : col - P.dqk);
+}
+__device__ __forceinline__ float* output_at(const TileParams& P, const Tile& t, int col, int* ld) {
+  const bool first = col < P.dqk;
+  *ld = first ? P.dqk : P.d;
+  return (t.is_q ? P.Q : first ? P.K : P.V) + t.out_row * *ld + (first ? col : col - P.dqk);
+}
+
+__global__ void __launch_bounds__(kThreads) proj_tile_f32_kernel(TileParams P) {      // d and d_qk multiples of 4
+  extern __shared__ __align__(16) float xs[];   // [64][d + 4] rows, then [d][64] weights
+  chain_wait();
+  chain_release();
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) set_status(P.status, 0);
+  const Tile tile = find_tile(P);
+  if (tile.rows == 0) return;
+  const int d = P.d, xp = d + 4, d4 = d >> 2, tid = threadIdx.x, tx = tid & 15, ty = tid >> 4, col = blockIdx.y * kCols + tx * 4;
+  float* ws = xs + kRows * xp;
+  const float* X = static_cast<const float*>(tile.is_q ? P.cands : P.items) + tile.in_row * d;
+  for (int i = tid; i < kRows * d4; i += kThreads) {
+    const int r = i / d4, c = i - r * d4;
+    cp16(smem_addr(xs + r * xp + c * 4), r < tile.rows ? X + (size_t)i * 4 : X, r < tile.rows ? 16u : 0u);
+  }
+  {
+    int ldw;
+    const bool in = col < tile.n_cols;
+    const float* W = weights_at<float>(P, tile.is_q, in ? col : 0, &ldw);
+    for (int k = ty; k < d; k += kThreads / 16) cp16(smem_addr(ws + k * kCols + tx * 4), W + (size_t)k * ldw, in ? 16u : 0u);
+  }
+  cp_commit();
+  cp_wait<0>();
+  __syncthreads();
+  float acc[8][4];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.f;
+  const float *xr = xs + ty * xp, *wr = ws + tx * 4;
+#pragma unroll 2
+  for (int k = 0; k < d; k += 4) {
+    float4 w[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) w[e] = *reinterpret_cast<const float4*>(wr + (k + e) * kCols);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const float4 x = *reinterpret_cast<const float4*>(xr + i * 8 * xp + k);
+      const float xv[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        acc[i][0] = fmaf(xv[e], w[e].x, acc[i][0]);
+        acc[i][1] = fmaf(xv[e], w[e].y, acc[i][1]);
+        acc[i][2] = fmaf(xv[e], w[e].z, acc[i][2]);
+        acc[i][3] = fmaf(xv[e], w[e].w, acc[i][3]);
+      }
+    }
+  }
+  if (col >= tile.n_cols) return;
+  int ldy;
+  float* Y = output_at(P, tile, col, &ldy);
+  const float scale = tile.is_q ? P.inv_gamma : 1.f;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int r = ty + 8 * i;
+    if (r < tile.rows)
+      *reinterpret_cast<float4*>(Y + (size_t)r * ldy) = make_float4(acc[i][0] * scale, acc[i][1] * scale, acc[i][2] * scale, acc[i][3] * scale);
+  }
+}
+
+__global__ void __launch_bounds__(kThreads) proj_tile_mma_kernel(TileParams P) {      // d a multiple of 16, d_qk of 8
+  extern __shared__ __align__(128) uint8_t xb[];  // [64][2 d + 16] bytes, then [d][144]
+  constexpr int WS = kCols * 2 + 16;
+  chain_wait();
+  chain_release();
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) set_status(P.status, 0);
+  const Tile tile = find_tile(P);
+  if (tile.rows == 0) return;
+  const int d = P.d, XS = 2 * d + 16, d8 = d >> 3, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, col0 = blockIdx.y * kCols;
+  const uint32_t xa = smem_addr(xb), wa = xa + kRows * XS;
+  const bf16* X = static_cast<const bf16*>(tile.is_q ? P.cands : P.items) + tile.in_row * d;
+  for (int i = tid; i < kRows * d8; i += kThreads) {
+    const int r = i / d8, c = i - r * d8;
+    cp16(xa + r * XS + c * 16, r < tile.rows ? X + (size_t)i * 8 : X, r < tile.rows ? 16u : 0u);
+  }
+  {
+    int ldw;
+    const int c8 = tid & 7, col = col0 + c8 * 8;
+    const bool in = col < tile.n_cols;
+    const bf16* W = weights_at<bf16>(P, tile.is_q, in ? col : 0, &ldw);
+    for (int k = tid >> 3; k < d; k += kThreads / 8) cp16(wa + k * WS + c8 * 16, W + (size_t)k * ldw, in ? 16u : 0u);
+  }
+  cp_commit();
+  cp_wait<0>();
+  __syncthreads();
+  float acc[8][4];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.f;
+  const uint32_t a_at = xa + ((lane & 7) + ((lane >> 3) & 1) * 8 + warp * 16) * XS + (lane >> 4) * 16;
+  const uint32_t b_at = wa + ((lane & 7) + ((lane >> 3) & 1) * 8) * WS + (lane >> 4) * 16;
+  for (int kt = 0; kt < d >> 4; ++kt) {
+    uint32_t a[4];
+    ldsm_x4(a, a_at + kt * 32);
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+      uint32_t w[4];
+      ldsm_x4_t(w, b_at + kt * 16 * WS + p * 32);
+      mma16816(acc[2 * p], a[0], a[1], a[2], a[3], w[0], w[1]);
+      mma16816(acc[2 * p + 1], a[0], a[1], a[2], a[3], w[2], w[3]);
+    }
+  }
+  const float scale = tile.is_q ? P.inv_gamma : 1.f;
+  const int g = lane >> 2, t = lane & 3, r0 = warp * 16 + g;
+#pragma unroll
+  for (int p = 0; p < 8; ++p) {
+    const int col = col0 + p * 8;
+    if (col >= tile.n_cols) break;
+    int ldy;
+    float* Y = output_at(P, tile, col, &ldy) + 2 * t;
+    if (r0 < tile.rows) *reinterpret_cast<float2*>(Y + (size_t)r0 * ldy) = make_float2(acc[p][0] * scale, acc[p][1] * scale);
+    if (r0 + 8 < tile.rows) *reinterpret_cast<float2*>(Y + (size_t)(r0 + 8) * ldy) = make_float2(acc[p][2] * scale, acc[p][3] * scale);
+  }
+}
+
+}  // namespace
+
+int simt_project_tiles(const Plan& p, const void* items, const int32_t* lengths, const void* cands, const void* Wq, const void* Wk,
+                       const void* Wv, char* ws, cudaStream_t st) {
+  const bool f32 = p.dtype == LASER_F32;
+  if (f32 ? p.d % 4 || p.dqk % 4 : p.d % 16 || p.dqk % 8) return LASER_ERR_UNSUPPORTED;
+  const size_t smem = f32 ? ((size_t)kRows * (p.d + 4) + (size_t)p.d * kCols) * sizeof(float)
+                          : (size_t)kRows * (2 * p.d + 16) + (size_t)p.d * (kCols * 2 + 16);
+  if (smem > 200 * 1024) return LASER_ERR_UNSUPPORTED;
+  TileParams P;
+  P.items = items; P.cands = cands; P.Wq = Wq; P.Wk = Wk; P.Wv = Wv;
+  P.Q = reinterpret_cast<float*>(ws + p.off_q);
+  P.K = reinterpret_cast<float*>(ws + p.off_k);
+  P.V = reinterpret_cast<float*>(ws + p.off_v);
+  P.lengths = lengths; P.row_off = p.item_offsets;
+  P.status = reinterpret_cast<int*>(ws + p.off_status);
+  P.U = p.U; P.L = p.L; P.N = p.N; P.d = p.d; P.dqk = p.dqk; P.inv_gamma = p.inv_gamma;
+  P.q_tiles = (p.N + kRows - 1) / kRows;
+  P.tiles_per_user = (p.L + kRows - 1) / kRows;
+  const long long tiles = P.q_tiles + (long long)p.U * P.tiles_per_user;
+  const int col_tiles = (p.dqk + p.d + kCols - 1) / kCols;
+  if (tiles > 0x7fffffffLL || col_tiles > 65535) return LASER_ERR_UNSUPPORTED;
+  auto kernel = f32 ? proj_tile_f32_kernel : proj_tile_mma_kernel;
+  LASER_CUDA_OK(allow_smem(kernel, smem));
+  LaunchScope ls("proj_tile", st);
+  LASER_CUDA_OK(launch_chained(kernel, dim3((unsigned)tiles, col_tiles), dim3(kThreads), smem, st, P));
+  return LASER_OK;
+}
+
+}  // namespace laser

@@ -1250,9 +1250,9 @@ int tensor_wait_selftest(char* ws, int poll_limit, cudaStream_t st) {
 }
 
 int tensor_gsta(const Plan& p, const void* Hprime, const int32_t* lengths, const int32_t* cand_offsets,
-                const void* cands, const void* Wg, void* z, char* ws, cudaStream_t st, bool images_ready) {
+                const void* cands, const void* Wg, void* z, char* ws, cudaStream_t st, bool images_ready, bool follows_call) {
   if (gsta_mma_supported(p)) return gsta_mma(p, Hprime, lengths, cand_offsets, cands, Wg, z, ws, st, images_ready);
-  return simt_gsta(p, Hprime, lengths, cand_offsets, cands, Wg, z, ws, st);
+  return simt_gsta(p, Hprime, lengths, cand_offsets, cands, Wg, z, ws, st, follows_call);
 }
 
 }  // namespace laser

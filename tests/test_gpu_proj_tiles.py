@@ -1,0 +1,45 @@
+"""The tiled projections of the fp32 path at the edges of their tiles (64 rows, 64 columns), fp32 and bf16 inputs, padded and packed
+items: through H' against the float64 oracle."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2602_11562_b200 as P
+from oracle import laser_oracle
+from workloads import make_custom
+
+pytestmark = pytest.mark.gpu
+
+CASES = [
+    dict(U=1, C=1, L=1, d=16, H=1, S=1, d_qh=16, lengths=[1]),
+    dict(U=3, C=64, L=64, d=64, H=4, S=16, d_qh=16),                              # whole tiles
+    dict(U=3, C=65, L=129, d=96, H=6, S=40, d_qh=16, lengths=[129, 0, 64]),       # one row past a tile, an empty user
+    dict(U=2, C=5, L=63, d=128, H=8, S=21, d_qh=16, lengths=[63, 1]),
+    dict(U=2, C=9, L=70, d=48, H=2, S=10, d_qh=8),                                # columns 0 .. 15 keys, then values
+    dict(U=2, C=9, L=70, d=20, H=2, S=10, d_qh=10),                               # fp32 only: multiples of 4
+]
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("case", range(len(CASES)))
+def test_projection_tiles(case, dtype):
+    w = make_custom(seed=2300 + case, dtype=dtype, M=1, emb_std="inv_sqrt_d", **CASES[case])
+    s = w.spec
+    b = P.DeviceBatch.from_workload(w, path=P.PATH_SIMT)
+    ws = torch.empty(P.laser_workspace_bytes(b.cfg), dtype=torch.uint8, device="cuda")
+    ws.fill_(0xFF)
+    Hp = P.laser_forward(b.cfg, *b.args(), b.Wg, workspace=ws, want_hprime=True)[0]
+    assert P.laser_check_status(ws) == 0
+    ref = laser_oracle.sta_forward(w.items, w.lengths, w.cands, w.cand_offsets, w.Wq, w.Wk, w.Wv, s.S, s.H, w.gamma)
+    got = Hp.float().cpu().numpy().astype(np.float64)
+    # fp32: at most 128-term sums of O(1) products, twice; bf16: the result alone is rounded (2^-9 of it)
+    tol = 2e-5 if dtype == "f32" else 2.0 ** -8
+    assert np.isfinite(got).all() and np.max(np.abs(got - ref) / np.maximum(1.0, np.abs(ref))) <= tol
+    valid = torch.arange(s.L, device="cuda")[None, :] < b.lengths[:, None]
+    starts = torch.cat([torch.zeros(1, dtype=torch.int32, device="cuda"), b.lengths.cumsum(0).int()])
+    packed = P.laser_forward_packed(b.cfg, b.items[valid].contiguous(), starts, b.lengths, b.cands, b.cand_offsets, b.Wq, b.Wk,
+                                    b.Wv, b.Wg, workspace=ws)
+    padded = P.laser_forward(b.cfg, *b.args(), b.Wg, workspace=ws)
+    assert P.laser_check_status(ws) == 0
+    z0, z1 = (x[0] if isinstance(x, tuple) else x for x in (padded, packed))
+    assert torch.equal(z0, z1)
