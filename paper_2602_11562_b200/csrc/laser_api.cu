@@ -398,7 +398,6 @@ int laser_backward(const laser_config* cfg, const void* items, const int32_t* le
   if (p.M > 0 && (rc = check_ptrs({Wgsta, dWgsta})) != LASER_OK) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   char* ws = static_cast<char*>(workspace);
-  if ((rc = clear_status(p, ws, st)) != LASER_OK) return rc;
   return backward(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, Wgsta, dz, d_items, d_cands, dWq, dWk, dWv, dWgsta,
                   ws, st, tensor);
 }

@@ -26,6 +26,22 @@
 
 namespace laser {
 namespace {
+__global__ void __launch_bounds__(256) zero_kernel(const __grid_constant__ ZeroList Z) {
+  zero_share(Z, (unsigned long long)blockIdx.x * 256 + threadIdx.x, (unsigned long long)gridDim.x * 256);
+}
+}  // namespace
+
+int zero_arrays(const ZeroList& Z, cudaStream_t st) {
+  unsigned long long total = 0;
+  for (int i = 0; i < Z.count; ++i) total += Z.n[i];
+  if (total == 0) return LASER_OK;
+  LaunchScope ls("bwd_zero", st);
+  zero_kernel<<<(int)std::min<unsigned long long>((total / 4 + 255) / 256 + 1, 8ull * device_sms()), 256, 0, st>>>(Z);
+  LASER_CUDA_OK(cudaGetLastError());
+  return LASER_OK;
+}
+
+namespace {
 
 using bf16 = __nv_bfloat16;
 
@@ -822,25 +838,19 @@ gsta_attn_bwd_kernel(const float* __restrict__ Hp, const float* __restrict__ Qt,
   }
 }
 
-// One block per (user, 32 consecutive items of one segment), thread (item n, head h); the block walks the user's
-// candidates, `step` at a time between two block-wide barriers.  Qf holds q / gamma, so the score is Qf_h . k_n
-// and dQf is the gradient with respect to q / gamma.  dK, dV rows of this chunk are written once (no other block touches
-// them); dQf is summed over the chunks atomically: the per-item terms de_n of a step go through shared memory and thread
-// (candidate, head, component) adds up its 32 items while the next step's rows are loaded.
+// One block per (user, 32 consecutive items of one segment), thread (item n, head h), for head widths that sta_bwd_f32
+// (laser_backward_f32.cu) does not take: any widths, everything in shared memory.  The block walks the user's candidates, `step` at
+// a time between two block-wide barriers.  Qf holds q / gamma, so the score is Qf_h . k_n and dQf is the gradient with respect to
+// q / gamma.  dK, dV rows of this chunk are written once (no other block touches them); dQf is summed over the chunks
+// atomically: the per-item terms de_n of a step go through shared memory and thread (candidate, head, component) adds up its 32
+// items while the next step's rows are loaded.
 constexpr int kChunk = 32;
 constexpr int kCandsPerStep = 16, kCandsPerStepMin = 4;      // the smaller one where shared memory is short
-// `parts` warps share a (32 items, head): part k takes candidates k, k + parts, ... of a step (register variant only).
-// DQH, DVH > 0: the head widths are compile-time constants and thread (item, head) keeps its key / value slices and
-// their gradient accumulators in registers (shared memory then holds only the keys for the query-side sums and the
-// step's candidate rows); 0, 0: any widths, everything in shared memory.
-template <int DQH, int DVH>
 __global__ void sta_bwd_kernel(const float* __restrict__ Qf, const float* __restrict__ Kf, const float* __restrict__ Vf,
                                const float* __restrict__ dHp, const int* __restrict__ lengths,
                                const int* __restrict__ cand_offsets, float* __restrict__ dQf, float* __restrict__ dKf,
                                float* __restrict__ dVf, int L, int d, int dqk, int H, int S, int Lp, int N,
-                               int chunks_per_seg, int step, int parts) {
-  constexpr bool kRegs = DQH > 0;
-  constexpr int kR = kRegs ? DQH : 1, kV = kRegs ? DVH : 1;
+                               int chunks_per_seg, int step) {
   extern __shared__ __align__(16) float sm[];
   const int u = blockIdx.y, seg = blockIdx.x / chunks_per_seg, ck = blockIdx.x - seg * chunks_per_seg;
   const int len = lengths[u], off0 = cand_offsets[u], off1 = cand_offsets[u + 1];
@@ -848,47 +858,24 @@ __global__ void sta_bwd_kernel(const float* __restrict__ Qf, const float* __rest
   const int n0 = seg * S + ck * kChunk, n_end = min(min((seg + 1) * S, L), len);
   if (n0 >= n_end) return;
   const int cnt = min(kChunk, n_end - n0);
-  const int dqh = kRegs ? DQH : dqk / H, dvh = kRegs ? DVH : d / H, kld = dqk + 1, vld = d + 1;
+  const int dqh = dqk / H, dvh = d / H, kld = dqk + 1, vld = d + 1;
   float* Ks = sm;                                                  // [32][dqk + 1]
-  float* Vs = Ks + kChunk * kld;                                   // [32][d + 1]      (shared-memory variant only)
-  float* dKs = Vs + (kRegs ? 0 : kChunk * vld);                    // [32][dqk + 1]    (shared-memory variant only)
-  float* dVs = dKs + (kRegs ? 0 : kChunk * kld);                   // [32][d + 1]      (shared-memory variant only)
-  float* qs = dVs + (kRegs ? 0 : kChunk * vld);                    // [step][dqk]
-  float* ds = qs + step * dqk;                            // [step][d]
-  float* des = ds + step * d;                             // [step][H][33]: de of (candidate, head, item)
-  const int tid = threadIdx.x, nt = blockDim.x, n = tid & 31, h = (tid >> 5) % H, part = (tid >> 5) / H;
-  float* red = des + step * H * 33;                                // [H][DQH + DVH][33]: one part's sums (parts > 1)
+  float* Vs = Ks + kChunk * kld;                                   // [32][d + 1]
+  float* dKs = Vs + kChunk * vld;                                  // [32][dqk + 1]
+  float* dVs = dKs + kChunk * kld;                                 // [32][d + 1]
+  float* qs = dVs + kChunk * vld;                                  // [step][dqk]
+  float* ds = qs + step * dqk;                                     // [step][d]
+  float* des = ds + step * d;                                      // [step][H][33]: de of (candidate, head, item)
+  const int tid = threadIdx.x, nt = blockDim.x, n = tid & 31, h = tid >> 5;
   for (int i = tid; i < kChunk * dqk; i += nt) {
     const int r = i / dqk, a = i - r * dqk;
     Ks[r * kld + a] = r < cnt ? Kf[((size_t)u * L + n0 + r) * dqk + a] : 0.f;
-    if (!kRegs) dKs[r * kld + a] = 0.f;
+    dKs[r * kld + a] = 0.f;
   }
-  if (!kRegs) {
-    for (int i = tid; i < kChunk * d; i += nt) {
-      const int r = i / d, a = i - r * d;
-      Vs[r * vld + a] = r < cnt ? Vf[((size_t)u * L + n0 + r) * d + a] : 0.f;
-      dVs[r * vld + a] = 0.f;
-    }
-  }
-  float kreg[kR], vreg[kV], dk[kR], dv[kV];
-  if (kRegs) {
-    const bool live = n < cnt;
-    const float4* kp = reinterpret_cast<const float4*>(Kf + ((size_t)u * L + n0 + n) * dqk + h * dqh);
-    const float4* vp = reinterpret_cast<const float4*>(Vf + ((size_t)u * L + n0 + n) * d + h * dvh);
-#pragma unroll
-    for (int a = 0; a < kR / 4; ++a) {
-      const float4 x = live ? kp[a] : make_float4(0.f, 0.f, 0.f, 0.f);
-      kreg[4 * a] = x.x; kreg[4 * a + 1] = x.y; kreg[4 * a + 2] = x.z; kreg[4 * a + 3] = x.w;
-    }
-#pragma unroll
-    for (int v = 0; v < kV / 4; ++v) {
-      const float4 x = live ? vp[v] : make_float4(0.f, 0.f, 0.f, 0.f);
-      vreg[4 * v] = x.x; vreg[4 * v + 1] = x.y; vreg[4 * v + 2] = x.z; vreg[4 * v + 3] = x.w;
-    }
-#pragma unroll
-    for (int a = 0; a < kR; ++a) dk[a] = 0.f;
-#pragma unroll
-    for (int v = 0; v < kV; ++v) dv[v] = 0.f;
+  for (int i = tid; i < kChunk * d; i += nt) {
+    const int r = i / d, a = i - r * d;
+    Vs[r * vld + a] = r < cnt ? Vf[((size_t)u * L + n0 + r) * d + a] : 0.f;
+    dVs[r * vld + a] = 0.f;
   }
   // the query-side sums of the step whose de terms sit in `des`: candidates c_lo .. c_lo + n_c - 1
   auto reduce_dq = [&](int c_lo, int n_c) {
@@ -912,85 +899,30 @@ __global__ void sta_bwd_kernel(const float* __restrict__ Qf, const float* __rest
       ds[i] = dHp[((size_t)(c + cc) * Lp + seg) * d + x];
     }
     __syncthreads();                       // (also: the previous step's sums have been read out of `des`)
-    {
-      for (int cc = part; cc < n_c; cc += parts) {
-        const float* q = qs + cc * dqk + h * dqh;
-        const float* g_out = ds + cc * d + h * dvh;
-        float e = 0.f, dg = 0.f;
-        if (kRegs) {
-          float qv[kR], gv[kV];
-#pragma unroll
-          for (int a = 0; a < kR / 4; ++a) {
-            const float4 x = reinterpret_cast<const float4*>(q)[a];
-            qv[4 * a] = x.x; qv[4 * a + 1] = x.y; qv[4 * a + 2] = x.z; qv[4 * a + 3] = x.w;
-          }
-#pragma unroll
-          for (int v = 0; v < kV / 4; ++v) {
-            const float4 x = reinterpret_cast<const float4*>(g_out)[v];
-            gv[4 * v] = x.x; gv[4 * v + 1] = x.y; gv[4 * v + 2] = x.z; gv[4 * v + 3] = x.w;
-          }
-#pragma unroll
-          for (int a = 0; a < kR; ++a) e = fmaf(qv[a], kreg[a], e);
-#pragma unroll
-          for (int v = 0; v < kV; ++v) dg = fmaf(gv[v], vreg[v], dg);
-          const float g = n < cnt ? 1.f / (1.f + expf(-e)) : 0.f;
-          const float de = dg * g * (1.f - g);
-#pragma unroll
-          for (int v = 0; v < kV; ++v) dv[v] = fmaf(g, gv[v], dv[v]);
-#pragma unroll
-          for (int a = 0; a < kR; ++a) dk[a] = fmaf(de, qv[a], dk[a]);
-          des[(cc * H + h) * 33 + n] = de;
-        } else {
-          for (int a = 0; a < dqh; ++a) e = fmaf(q[a], Ks[n * kld + h * dqh + a], e);
-          for (int v = 0; v < dvh; ++v) dg = fmaf(g_out[v], Vs[n * vld + h * dvh + v], dg);
-          const float g = n < cnt ? 1.f / (1.f + expf(-e)) : 0.f;
-          const float de = dg * g * (1.f - g);
-          for (int v = 0; v < dvh; ++v) dVs[n * vld + h * dvh + v] = fmaf(g, g_out[v], dVs[n * vld + h * dvh + v]);
-          for (int a = 0; a < dqh; ++a) dKs[n * kld + h * dqh + a] = fmaf(de, q[a], dKs[n * kld + h * dqh + a]);
-          des[(cc * H + h) * 33 + n] = de;
-        }
-      }
+    for (int cc = 0; cc < n_c; ++cc) {
+      const float* q = qs + cc * dqk + h * dqh;
+      const float* g_out = ds + cc * d + h * dvh;
+      float e = 0.f, dg = 0.f;
+      for (int a = 0; a < dqh; ++a) e = fmaf(q[a], Ks[n * kld + h * dqh + a], e);
+      for (int v = 0; v < dvh; ++v) dg = fmaf(g_out[v], Vs[n * vld + h * dvh + v], dg);
+      const float g = n < cnt ? 1.f / (1.f + expf(-e)) : 0.f;
+      const float de = dg * g * (1.f - g);
+      for (int v = 0; v < dvh; ++v) dVs[n * vld + h * dvh + v] = fmaf(g, g_out[v], dVs[n * vld + h * dvh + v]);
+      for (int a = 0; a < dqh; ++a) dKs[n * kld + h * dqh + a] = fmaf(de, q[a], dKs[n * kld + h * dqh + a]);
+      des[(cc * H + h) * 33 + n] = de;
     }
     prev_lo = c;
     prev_n = n_c;
   }
   __syncthreads();
   if (prev_n > 0) reduce_dq(prev_lo, prev_n);
-  if (kRegs) {
-    for (int k = 1; k < parts; ++k) {      // part 0 collects the other parts' sums, one after the other
-      float* mine = red + (size_t)h * (kR + kV) * 33 + n;
-      __syncthreads();
-      if (part == k) {
-#pragma unroll
-        for (int a = 0; a < kR; ++a) mine[a * 33] = dk[a];
-#pragma unroll
-        for (int v = 0; v < kV; ++v) mine[(kR + v) * 33] = dv[v];
-      }
-      __syncthreads();
-      if (part == 0) {
-#pragma unroll
-        for (int a = 0; a < kR; ++a) dk[a] += mine[a * 33];
-#pragma unroll
-        for (int v = 0; v < kV; ++v) dv[v] += mine[(kR + v) * 33];
-      }
-    }
-    if (part == 0 && n < cnt) {
-      float4* kp = reinterpret_cast<float4*>(dKf + ((size_t)u * L + n0 + n) * dqk + h * dqh);
-      float4* vp = reinterpret_cast<float4*>(dVf + ((size_t)u * L + n0 + n) * d + h * dvh);
-#pragma unroll
-      for (int a = 0; a < kR / 4; ++a) kp[a] = make_float4(dk[4 * a], dk[4 * a + 1], dk[4 * a + 2], dk[4 * a + 3]);
-#pragma unroll
-      for (int v = 0; v < kV / 4; ++v) vp[v] = make_float4(dv[4 * v], dv[4 * v + 1], dv[4 * v + 2], dv[4 * v + 3]);
-    }
-  } else {
-    for (int i = tid; i < cnt * dqk; i += nt) {
-      const int r = i / dqk, a = i - r * dqk;
-      dKf[((size_t)u * L + n0 + r) * dqk + a] = dKs[r * kld + a];
-    }
-    for (int i = tid; i < cnt * d; i += nt) {
-      const int r = i / d, a = i - r * d;
-      dVf[((size_t)u * L + n0 + r) * d + a] = dVs[r * vld + a];
-    }
+  for (int i = tid; i < cnt * dqk; i += nt) {
+    const int r = i / dqk, a = i - r * dqk;
+    dKf[((size_t)u * L + n0 + r) * dqk + a] = dKs[r * kld + a];
+  }
+  for (int i = tid; i < cnt * d; i += nt) {
+    const int r = i / d, a = i - r * d;
+    dVf[((size_t)u * L + n0 + r) * d + a] = dVs[r * vld + a];
   }
 }
 
@@ -1030,29 +962,21 @@ BwdScratch carve_scratch(const Plan& p, char* base) {
 // The gate kernel of the FP32 ALUs: dK, dV rows of valid items, adds to dQf (all of them zeroed before).
 int launch_sta_bwd(const Plan& p, const float* Qf, const float* Kf, const float* Vf, const float* dHp, const int32_t* lengths,
                    const int32_t* cand_offsets, float* dQf, float* dK, float* dV, cudaStream_t st) {
-  const int L = p.L, d = p.d, H = p.H, dqk = p.dqk, dvh = p.dvh, Lp = p.Lp, N = p.N, U = p.U;
+  const int rc = sta_bwd_f32(p, Qf, Kf, Vf, dHp, lengths, cand_offsets, dQf, dK, dV, st);
+  if (rc != LASER_ERR_UNSUPPORTED) return rc;
+  const int L = p.L, d = p.d, H = p.H, dqk = p.dqk, Lp = p.Lp, N = p.N, U = p.U;
   const int cps = (min(p.S, L) + kChunk - 1) / kChunk;
-  const int dqh = dqk / H;
-  const int variant = (dqh == 16 && dvh == 32) ? 2 : (dqh == 16 && dvh == 16) ? 1 : 0;   // register-resident head slices
-  // Up to four warps per (32 items, head): small batches run about one block per SM and are bound by a warp's serial walk (6 users
-  // x 45 candidates: 48, 29, 23 us with one, two, four).  Where two already fill the SMs' warps, four only add their sums (40 users x
-  // 40 candidates: 74, 72, 89), and two want at least eight candidates each (20: 50, 43, 56; but 5: 35, 50; 7: 136, 183).
-  const bool crowded = 2ll * Lp * cps * U * H > 16ll * device_sms();
-  int parts = 1;
-  while (variant && parts < (crowded ? 2 : 4) && 2 * parts * H <= 16 && p.maxC >= (crowded ? 16 : 4) * parts) parts *= 2;
   auto smem_of = [&](int step) {
-    return ((parts > 1 ? (size_t)H * (dqh + dvh) * 33 : 0) + (variant ? (size_t)kChunk * (dqk + 1) : 2 * (size_t)kChunk * (dqk + 1 + d + 1)) +
-            (size_t)step * (dqk + d + H * 33)) * sizeof(float);
+    return (2 * (size_t)kChunk * (dqk + 1 + d + 1) + (size_t)step * (dqk + d + H * 33)) * sizeof(float);
   };
-  // (a step costs two barriers and a round trip to L2 whatever it holds: 6 users x 23 candidates 40 -> 22 us with 16)
+  // (a step costs two barriers and a round trip to L2 whatever it holds)
   const int step = smem_of(kCandsPerStep) <= 72 * 1024 ? kCandsPerStep : kCandsPerStepMin;
   const size_t smem = smem_of(step);
   if (smem > 200 * 1024 || (long long)Lp * cps > 0x7fffffffLL || U > 65535 || H > 32) return LASER_ERR_UNSUPPORTED;
-  auto kernel = variant == 2 ? sta_bwd_kernel<16, 32> : variant == 1 ? sta_bwd_kernel<16, 16> : sta_bwd_kernel<0, 0>;
-  LASER_CUDA_OK(allow_smem(kernel, smem));
+  LASER_CUDA_OK(allow_smem(sta_bwd_kernel, smem));
   LaunchScope ls("bwd_sta", st);
-  kernel<<<dim3(Lp * cps, U), 32 * H * parts, smem, st>>>(Qf, Kf, Vf, dHp, lengths, cand_offsets, dQf, dK, dV, L, d, dqk,
-                                                  H, p.S, Lp, N, cps, step, parts);
+  sta_bwd_kernel<<<dim3(Lp * cps, U), 32 * H, smem, st>>>(Qf, Kf, Vf, dHp, lengths, cand_offsets, dQf, dK, dV, L, d, dqk, H, p.S, Lp,
+                                                          N, cps, step);
   LASER_CUDA_OK(cudaGetLastError());
   return LASER_OK;
 }
@@ -1061,33 +985,6 @@ int launch_sta_bwd(const Plan& p, const float* Qf, const float* Kf, const float*
 GstaPlanes train_planes(const Plan& p, const BwdScratch& s) {
   auto h = [](float* q) { return reinterpret_cast<bf16*>(q); };
   return {h(s.T), h(s.Q), h(s.dT), h(s.dQ), h(s.Mh), h(s.dQt), s.dT + p.M * (size_t)p.N * p.d};
-}
-
-// Several arrays set to zero by one launch.
-struct ZeroList {
-  float* p[8];
-  unsigned long long n[8];
-  int count;
-  void add(float* q, size_t len) {
-    if (len) { p[count] = q; n[count++] = len; }
-  }
-};
-__global__ void __launch_bounds__(256) zero_kernel(const __grid_constant__ ZeroList Z) {
-  for (int a = 0; a < Z.count; ++a) {
-    float4* q = reinterpret_cast<float4*>(Z.p[a]);           // (16-byte aligned arrays)
-    const unsigned long long n4 = Z.n[a] / 4, i0 = (unsigned long long)blockIdx.x * 256 + threadIdx.x;
-    for (unsigned long long i = i0; i < n4; i += (unsigned long long)gridDim.x * 256) q[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (i0 < (Z.n[a] & 3)) Z.p[a][n4 * 4 + i0] = 0.f;
-  }
-}
-int zero_arrays(const ZeroList& Z, cudaStream_t st) {
-  unsigned long long total = 0;
-  for (int i = 0; i < Z.count; ++i) total += Z.n[i];
-  if (total == 0) return LASER_OK;
-  LaunchScope ls("bwd_zero", st);
-  zero_kernel<<<(int)std::min<unsigned long long>((total / 4 + 255) / 256 + 1, 8ull * device_sms()), 256, 0, st>>>(Z);
-  LASER_CUDA_OK(cudaGetLastError());
-  return LASER_OK;
 }
 
 // Products collected for as few launches as possible.
@@ -1164,12 +1061,14 @@ int backward_simt(const Plan& p, const T* items, const int32_t* lengths, const T
 #define BWD_OK(...) do { rc = (__VA_ARGS__); if (rc != LASER_OK) return rc; } while (0)
   ZeroList Z = {};
   Z.add(dWq, (size_t)d * dqk); Z.add(dWk, (size_t)d * dqk); Z.add(dWv, (size_t)d * d); Z.add(dWg, (size_t)M * 3 * d * d);
-  Z.add(s.dQf, (size_t)N * dqk); Z.add(s.dK, (size_t)UL * dqk); Z.add(s.dV, (size_t)UL * d);
-  BWD_OK(zero_arrays(Z, st));
+  Z.add(s.dQf, (size_t)N * dqk);
+  Z.add(ws + p.off_status, kStatusWords);
+  if (!sta_bwd_f32_supported(p)) { Z.add(s.dK, (size_t)UL * dqk); Z.add(s.dV, (size_t)UL * d); }     // (it writes every row)
   if (p.dqh == 16 && (dvh == 16 || dvh == 32 || dvh == 64) && H <= 32) {
-    BWD_OK(simt_project(p, items, lengths, cands, Wq, Wk, Wv, ws, st));
+    BWD_OK(simt_project(p, items, lengths, cands, Wq, Wk, Wv, ws, st, &Z));
     BWD_OK(simt_attend_f32(p, lengths, cand_offsets, s.Hp, ws, st));
   } else {
+    BWD_OK(zero_arrays(Z, st));
     BWD_OK(simt_sta_f32(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, s.Hp, ws, st));
   }
   const GstaTrain G = {s.T, s.Q, s.dT, s.dQ, s.Mh, s.dQt, s.dT + M * (size_t)N * d};
@@ -1196,6 +1095,7 @@ int backward_stream_all(const Plan& p, const T* items, const int32_t* lengths, c
   ZeroList Z = {};
   Z.add(dWq, (size_t)d * dqk); Z.add(dWk, (size_t)d * dqk); Z.add(dWv, (size_t)d * d); Z.add(dWg, (size_t)M * 3 * d * d);
   Z.add(backward_stream_sums(p, stream_scratch), (size_t)N * H * d);
+  Z.add(ws + p.off_status, kStatusWords);
   BWD_OK(zero_arrays(Z, st));
   bf16 *Hhi = reinterpret_cast<bf16*>(s.Hp), *Hlo = Hhi + (size_t)N * p.Lp * d;
   BWD_OK(backward_stream_forward(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, nullptr, Hhi, Hlo, ws, stream_scratch, st));
@@ -1260,6 +1160,7 @@ int backward_lists(const Plan& p, const bf16* items, const int32_t* lengths, con
 #define BWD_OK(...) do { rc = (__VA_ARGS__); if (rc != LASER_OK) return rc; } while (0)
   ZeroList Z = {};
   Z.add(dWq, d * dqk); Z.add(dWk, d * dqk); Z.add(dWv, d * d); Z.add(dWg, M * 3 * d * d); Z.add(s.dQf, N * dqk);
+  Z.add(ws + p.off_status, kStatusWords);
   BWD_OK(zero_arrays(Z, st));
   BWD_OK(rows_project_cands(p, cands, Wq, 0.5f * p.inv_gamma, Qb, st));
   BWD_OK(rows_project_items(p, items, lengths, cand_offsets, Wk, Wv, Kb, Vb, st));
@@ -1287,6 +1188,7 @@ int backward_t(const Plan& p, const T* items, const int32_t* lengths, const T* c
       return backward_lists(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, Wg, dz, d_items, d_cands, dWq, dWk, dWv, dWg, ws, st);
   }
   // (d_items: with candidates present its first matrix product writes every row, padding included)
+  LASER_CUDA_OK(cudaMemsetAsync(ws + p.off_status, 0, kStatusWords * sizeof(int), st));      // (the other routes' first launch does)
   if (N == 0 || U == 0) LASER_CUDA_OK(cudaMemsetAsync(d_items, 0, UL * d * sizeof(float), st));
   LASER_CUDA_OK(cudaMemsetAsync(dWq, 0, (size_t)d * dqk * sizeof(float), st));
   LASER_CUDA_OK(cudaMemsetAsync(dWk, 0, (size_t)d * dqk * sizeof(float), st));

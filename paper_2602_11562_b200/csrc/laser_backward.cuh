@@ -20,6 +20,14 @@ bool gsta_train_simt_supported(const Plan& p);
 int gsta_train_simt(const Plan& p, const float* Hp, const int32_t* lengths, const int32_t* cand_offsets, const void* cands,
                     const void* Wg, const float* dz, const GstaTrain& G, float* dHp, cudaStream_t st);
 
+// The same for the widths in use (laser_backward_f32.cu), and the gates: every row of dK and dV, adds to dQf (zeroed before).
+// LASER_ERR_UNSUPPORTED for all other shapes.
+int gsta_train_f32(const Plan& p, const float* Hp, const int32_t* lengths, const int32_t* cand_offsets, const void* cands,
+                   const void* Wg, const float* dz, const GstaTrain& G, float* dHp, cudaStream_t st);
+bool sta_bwd_f32_supported(const Plan& p);
+int sta_bwd_f32(const Plan& p, const float* Qf, const float* Kf, const float* Vf, const float* dHp, const int32_t* lengths,
+                const int32_t* cand_offsets, float* dQf, float* dK, float* dV, cudaStream_t st);
+
 // The same for the tensor-core kernel, as bf16 high and low parts: arrays of [2][M, N, d] and [2][M, N, H, d].
 struct GstaPlanes {
   __nv_bfloat16 *T, *Q, *dT, *dQ, *Mh, *dQt;

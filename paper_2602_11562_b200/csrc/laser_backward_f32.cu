@@ -1,0 +1,547 @@
+// FP32-ALU kernels of the backward pass for the widths in use: the stacked attention of a candidate forward and backward in one
+// kernel (d = 32, 64, 96, 128), and the gates (16-wide query heads, 16-, 32- or 64-wide value heads).  Other shapes take the
+// general kernels (laser_backward_simt.cu, laser_backward.cu).
+#include <cooperative_groups.h>
+
+#include <algorithm>
+#include <type_traits>
+
+#include "laser_backward.cuh"
+#include "laser_common.cuh"
+#include "laser_mma.cuh"
+#include "laser_simt_dense.cuh"
+
+namespace laser {
+namespace {
+
+using bf16 = __nv_bfloat16;
+using namespace dense;
+
+// ------------------------------------------------------------------------------------------------ stacked attention
+// Formulas as at gsta_train_simt_kernel (laser_backward_simt.cu).  Everything of CB candidates stays in shared memory: segment
+// vectors, and per layer t, q, qt, m, dm, the attention weights a and their gradients de.  The gradient of the segment vectors,
+//   ds_j = sum over layers and heads of de_{j,h} qt_h + a_{j,h} dm_h,
+// is formed once at the end, eight segments of four features per thread, instead of a read-modify-write of global memory per layer.
+struct TrainParams {
+  const float* Hp;
+  const void *cands, *Wg;
+  const float* dz;
+  const int *lengths, *cand_offsets;
+  GstaTrain G;
+  float* dHp;
+  int U, L, S, Lp, LpP, M, N;            // LpP: L' rounded up to a multiple of 4
+  float inv_tau;
+};
+
+template <int D, int H, int CB>
+__host__ __device__ constexpr int train_red_floats() {
+  return Weighted<D, H, CB>::kFloats > 8 * CB * D ? Weighted<D, H, CB>::kFloats : 8 * CB * D;
+}
+template <int D, int H, int CB>
+__host__ __device__ constexpr size_t train_floats(int Lp, int LpP, int M) {
+  return (size_t)CB * ((size_t)(M + 1) * D + (size_t)M * D + 3 * (size_t)M * H * (D + 4) + (size_t)H * (D + 4) + 2 * D +
+                       2 * (size_t)M * H * LpP + H + (size_t)Lp * (D + 4)) + train_red_floats<D, H, CB>() + 4;
+}
+
+template <typename T, int D, int H, int CB>
+__global__ void __launch_bounds__(kThreads, 2) gsta_train_f32_kernel(const TrainParams P) {
+  constexpr int DS = D + 4, kCols = D / 4, HF = D == 96 ? 3 : 1;        // HF: slices of a row in products with W^T
+  extern __shared__ __align__(16) float sm[];
+  __shared__ int s_nv[CB];
+  const int Lp = P.Lp, LpP = P.LpP, M = P.M, c_base = blockIdx.x * CB, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  float* t = sm;                                 // [M + 1][CB][D]
+  float* q = t + (M + 1) * CB * D;               // [M][CB][D]
+  float* qt = q + M * CB * D;                    // [M][CB][H][DS]
+  float* m = qt + M * CB * H * DS;               // [M][CB][H][DS]
+  float* dm = m + M * CB * H * DS;               // [M][CB][H][DS]
+  float* dqt = dm + M * CB * H * DS;             // [CB][H][DS]
+  float* dt = dqt + CB * H * DS;                 // [CB][D]
+  float* dq = dt + CB * D;                       // [CB][D]
+  float* a = dq + CB * D;                        // [M][CB][H][LpP]
+  float* de = a + M * CB * H * LpP;              // [M][CB][H][LpP]
+  float* red = de + M * CB * H * LpP;
+  float* Hs = red + train_red_floats<D, H, CB>();       // [CB][Lp][DS]
+  float* mdm = Hs + (size_t)CB * Lp * DS;        // [CB][H]
+  const T* Wg = static_cast<const T*>(P.Wg);
+  ProductNN<T, D, CB> nn;
+  ProductNT<T, D, H, CB> nt;
+  ProductNT<T, D, HF, CB> ntf;
+  nn.load(Wg, tid);
+  if (tid < CB) {
+    const int cand = c_base + tid;
+    int nv = 0;
+    if (cand < P.N) {
+      int lo = 0, hi = P.U - 1;                  // the last user whose first candidate is <= cand
+      while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (P.cand_offsets[mid] <= cand) lo = mid; else hi = mid - 1;
+      }
+      const int len = P.lengths[lo];
+      nv = len <= 0 || len > P.L ? 0 : min((len + P.S - 1) / P.S, Lp);
+    }
+    s_nv[tid] = nv;
+  }
+  const int live = min(CB, P.N - c_base) * D;    // elements of the candidates' rows
+  for (int i = tid; i < CB * D; i += kThreads) {
+    t[i] = i < live ? to_f32<T>(static_cast<const T*>(P.cands)[(size_t)c_base * D + i]) : 0.f;
+    dt[i] = i < live ? P.dz[(size_t)c_base * D + i] : 0.f;
+  }
+  __syncthreads();
+  stage_segments<float, D, CB, DS>(Hs, P.Hp, s_nv, c_base, Lp, tid);
+
+  auto keep = [&](float* dst, const float* src) {          // [CB][D] to the candidates' rows
+    for (int i = tid * 4; i < live; i += kThreads * 4)
+      *reinterpret_cast<float4*>(dst + (size_t)c_base * D + i) = *reinterpret_cast<const float4*>(src + i);
+  };
+  auto keep_heads = [&](float* dst, const float* src) {    // [CB][H][DS] to [N, H, D]
+    for (int i = tid; i < live * H / 4; i += kThreads)
+      *reinterpret_cast<float4*>(dst + (size_t)c_base * H * D + i * 4) =
+          *reinterpret_cast<const float4*>(src + i / kCols * DS + i % kCols * 4);
+  };
+  auto put4 = [&](float* y) {
+    return [=](int i, const float (&s)[4]) { *reinterpret_cast<float4*>(y + i) = make_float4(s[0], s[1], s[2], s[3]); };
+  };
+  const size_t Nd = (size_t)P.N * D;
+
+  for (int l = 0; l < M; ++l) {
+    const T *Wk = Wg + (size_t)(l * 3 + 1) * D * D, *Wv = Wk + D * D;
+    float *tl = t + l * CB * D, *ql = q + l * CB * D, *qtl = qt + l * CB * H * DS, *ml = m + l * CB * H * DS, *al = a + l * CB * H * LpP;
+    nn.run([&](int c, int) { return (const float*)(tl + c * D); }, red, tid);
+    nt.load(Wk, tid);
+    __syncthreads();
+    nn.finish(red, tid, put4(ql));
+    __syncthreads();
+    nt.run(ql, tid, [&](int c, int h, int i, float v) { qtl[(c * H + h) * DS + i] = v * P.inv_tau; });
+    keep(P.G.T + l * Nd, tl);
+    keep(P.G.Q + l * Nd, ql);
+    __syncthreads();
+    scores<D, H, CB, DS>(Hs, qtl, s_nv, Lp, LpP, 1.f, al, tid);
+    __syncthreads();
+    softmax<H, CB>(al, s_nv, LpP, tid);
+    __syncthreads();
+    Weighted<D, H, CB>::template run<DS>(Hs, al, s_nv, Lp, LpP, red, tid);
+    nn.load(Wv, tid);
+    __syncthreads();
+    Weighted<D, H, CB>::template finish<DS>(red, ml, tid);
+    __syncthreads();
+    nn.run([&](int c, int j) { return (const float*)(ml + (c * H + j / (D / H)) * DS); }, red, tid);
+    if (l + 1 < M) nn.load(Wv + D * D, tid);
+    keep_heads(P.G.Mh + l * Nd * H, ml);
+    __syncthreads();
+    nn.finish(red, tid, [&](int i, const float (&s)[4]) {
+      const float4 v = *reinterpret_cast<const float4*>(tl + i);
+      *reinterpret_cast<float4*>(tl + CB * D + i) = make_float4(v.x + s[0], v.y + s[1], v.z + s[2], v.w + s[3]);
+    });
+    __syncthreads();
+  }
+  nt.load(Wg + (size_t)((M - 1) * 3 + 2) * D * D, tid);
+  for (int l = M - 1; l >= 0; --l) {
+    const T *Wq = Wg + (size_t)(l * 3) * D * D, *Wk = Wq + D * D;
+    float *ml = m + l * CB * H * DS, *dml = dm + l * CB * H * DS, *al = a + l * CB * H * LpP, *del = de + l * CB * H * LpP;
+    keep(P.G.dT + l * Nd, dt);
+    nt.run(dt, tid, [&](int c, int h, int i, float v) { dml[(c * H + h) * DS + i] = v; });
+    __syncthreads();
+    scores<D, H, CB, DS>(Hs, dml, s_nv, Lp, LpP, 1.f, del, tid);
+    for (int ch = warp; ch < CB * H; ch += kWarps) {       // sum_j a_j (s_j . dm) = m . dm
+      float v = 0.f;
+#pragma unroll
+      for (int i = 0; i < D; i += 32) v = fmaf(ml[ch * DS + i + lane], dml[ch * DS + i + lane], v);
+      v = warp_sum(v);
+      if (lane == 0) mdm[ch] = v;
+    }
+    __syncthreads();
+    for (int ch = warp; ch < CB * H; ch += kWarps) {
+      const int n = s_nv[ch / H];
+      const float x = mdm[ch];
+      for (int j = lane; j < n; j += 32) del[ch * LpP + j] = al[ch * LpP + j] * (del[ch * LpP + j] - x);
+    }
+    __syncthreads();
+    Weighted<D, H, CB>::template run<DS>(Hs, del, s_nv, Lp, LpP, red, tid);
+    nn.load(Wk, tid);
+    __syncthreads();
+    Weighted<D, H, CB>::template finish<DS>(red, dqt, tid);
+    __syncthreads();
+    nn.run([&](int c, int j) { return (const float*)(dqt + (c * H + j / (D / H)) * DS); }, red, tid);
+    ntf.load(Wq, tid);
+    keep_heads(P.G.dQt + l * Nd * H, dqt);
+    __syncthreads();
+    nn.finish(red, tid, [&](int i, const float (&s)[4]) {
+      *reinterpret_cast<float4*>(dq + i) = make_float4(s[0] * P.inv_tau, s[1] * P.inv_tau, s[2] * P.inv_tau, s[3] * P.inv_tau);
+    });
+    __syncthreads();
+    ntf.run(dq, tid, [&](int c, int h, int i, float v) { red[(h * CB + c) * D + i] = v; });
+    if (l > 0) nt.load(Wq - D * D, tid);                   // W_v of the layer before
+    keep(P.G.dQ + l * Nd, dq);
+    __syncthreads();
+    for (int i = tid; i < CB * D; i += kThreads) {
+      float v = dt[i];
+#pragma unroll
+      for (int h = 0; h < HF; ++h) v += red[h * CB * D + i];
+      dt[i] = v;
+    }
+    __syncthreads();
+  }
+  keep(P.G.dT0, dt);
+  // gradient of the segment vectors: thread = (eight segments, four features)
+  constexpr int kJ = 8;
+  for (int c = 0; c < CB && c_base + c < P.N; ++c) {
+    const int nv = s_nv[c], groups = (Lp + kJ - 1) / kJ;
+    float* out = P.dHp + (size_t)(c_base + c) * Lp * D;
+    for (int o = tid; o < groups * kCols; o += kThreads) {
+      const int j0 = o / kCols * kJ, i = o % kCols * 4;
+      float acc[kJ][4];
+#pragma unroll
+      for (int j = 0; j < kJ; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
+      if (j0 < nv) {
+        for (int lh = 0; lh < M * H; ++lh) {
+          const int r = lh / H * CB * H + c * H + lh % H;
+          float qv[4], mv[4];
+          lds4(qv, qt + r * DS + i);
+          lds4(mv, dm + r * DS + i);
+#pragma unroll
+          for (int k = 0; k < kJ; k += 4) {
+            float ev[4], av[4];
+            if (j0 + k < LpP) {
+              lds4(ev, de + r * LpP + j0 + k);
+              lds4(av, a + r * LpP + j0 + k);
+#pragma unroll
+              for (int e = 0; e < 4; ++e)
+#pragma unroll
+                for (int x = 0; x < 4; ++x) acc[k + e][x] = fmaf(ev[e], qv[x], fmaf(av[e], mv[x], acc[k + e][x]));
+            }
+          }
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < kJ; ++j)
+        if (j0 + j < Lp) {
+          const bool in = j0 + j < nv;                     // (rows of empty segments receive no gradient)
+          *reinterpret_cast<float4*>(out + (size_t)(j0 + j) * D + i) =
+              in ? make_float4(acc[j][0], acc[j][1], acc[j][2], acc[j][3]) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    }
+  }
+}
+
+constexpr size_t kMost = 226 * 1024;
+
+template <typename T, int D, int H, int CB>
+int launch_train_cb(const Plan& p, const TrainParams& P, cudaStream_t st) {
+  const size_t smem = train_floats<D, H, CB>(P.Lp, P.LpP, P.M) * sizeof(float);
+  LASER_CUDA_OK(allow_smem(gsta_train_f32_kernel<T, D, H, CB>, smem));
+  LaunchScope ls("gsta_train_simt", st);
+  gsta_train_f32_kernel<T, D, H, CB><<<(p.N + CB - 1) / CB, kThreads, smem, st>>>(P);
+  LASER_CUDA_OK(cudaGetLastError());
+  return LASER_OK;
+}
+
+template <typename T, int D, int H>
+int launch_train(const Plan& p, const TrainParams& P, cudaStream_t st) {
+  const int sms = device_sms();
+  // Candidates per block as in the forward kernel (launch, laser_simt_gsta.cu).  us (CUDA events, about 6 too long; one | two | four):
+  // 270 candidates, d = 64, two heads 17 | 19 | 25; 400, four heads 31 | 23 | 29; 992, d = 32 41 | 27 | 19; 1400, d = 64, four heads 64 | 48 |
+  // 48; 4590, d = 64, one head, three layers 220 | 142 | 101.
+  if (p.N > 6 * sms && train_floats<D, H, 4>(P.Lp, P.LpP, P.M) * 4 <= kMost / 2) return launch_train_cb<T, D, H, 4>(p, P, st);
+  if (p.N > 2 * sms && train_floats<D, H, 2>(P.Lp, P.LpP, P.M) * 4 <= kMost) return launch_train_cb<T, D, H, 2>(p, P, st);
+  if (train_floats<D, H, 1>(P.Lp, P.LpP, P.M) * 4 > kMost) return LASER_ERR_UNSUPPORTED;
+  return launch_train_cb<T, D, H, 1>(p, P, st);
+}
+
+template <typename T>
+int dispatch_train(const Plan& p, const TrainParams& P, cudaStream_t st) {
+  switch (p.d * 16 + p.H) {
+    case 32 * 16 + 1: return launch_train<T, 32, 1>(p, P, st);
+    case 32 * 16 + 2: return launch_train<T, 32, 2>(p, P, st);
+    case 64 * 16 + 1: return launch_train<T, 64, 1>(p, P, st);
+    case 64 * 16 + 2: return launch_train<T, 64, 2>(p, P, st);
+    case 64 * 16 + 4: return launch_train<T, 64, 4>(p, P, st);
+    case 96 * 16 + 3: return launch_train<T, 96, 3>(p, P, st);
+    case 96 * 16 + 6: return launch_train<T, 96, 6>(p, P, st);
+    case 128 * 16 + 1: return launch_train<T, 128, 1>(p, P, st);
+    case 128 * 16 + 2: return launch_train<T, 128, 2>(p, P, st);
+    case 128 * 16 + 4: return launch_train<T, 128, 4>(p, P, st);
+    case 128 * 16 + 8: return launch_train<T, 128, 8>(p, P, st);
+    default: return LASER_ERR_UNSUPPORTED;
+  }
+}
+
+// ------------------------------------------------------------------------------------------------ gates
+// dK, dV and dQf from dH' (formulas as at sta_bwd_kernel, laser_backward.cu).  One block = 32 consecutive items of a user, whatever
+// segments they belong to (a lane reads its own segment's rows of dH'; blocks of one segment each leave 20 of 32 lanes idle
+// when segments have 12 items); warp = (head, part), thread = item with its key and value slices and their gradients in
+// registers.  The candidates pass 16 (or 8, 4) at a time; the next ones' rows are on their way (cp.async) while a step is computed.  The `parts`
+// warps of a head share a step's candidates.  The query side, dQ_h = de K_h, is a 16 x 16 x 32 product per step and head: a warp's
+// thread owns a 4 x 4 tile of it over a slice of the items and reads 16 bytes per shared-memory access (before, one value of it:
+// two reads per multiply-add, most of the kernel).
+// Few blocks (small batches): a cluster of `csplit` blocks shares the candidates, and their dK and dV meet through distributed
+// shared memory in a fixed order, so that d_items does not depend on the order of anything.
+struct GateParams {
+  const float *Qf, *Kf, *Vf, *dHp;
+  const int *lengths, *cand_offsets;
+  float *dQf, *dKf, *dVf;
+  int L, d, dqk, H, S, Lp, N, step, parts, span;           // span: segments that 32 consecutive items can touch
+};
+constexpr int kItems = 32, kStepMax = 16, kDeP = 36;       // kDeP: pitch of a candidate's 32 de values
+
+template <int DVH, int kMaxThreads>
+__global__ void __launch_bounds__(kMaxThreads) sta_bwd_f32_kernel(const GateParams P) {
+  constexpr int DQ = 16;
+  namespace cg = cooperative_groups;
+  extern __shared__ __align__(16) float sm[];
+  const int u = blockIdx.y, n0 = blockIdx.x * kItems, rank = blockIdx.z, ranks = gridDim.z;
+  const int L = P.L, d = P.d, dqk = P.dqk, H = P.H, S = P.S, step = P.step, parts = P.parts;
+  const int len = P.lengths[u], off0 = P.cand_offsets[u], off1 = P.cand_offsets[u + 1];
+  const int tid = threadIdx.x, nt = blockDim.x, n = tid & 31, warp = tid >> 5, h = warp % H, part = warp / H;
+  const bool usable = len > 0 && len <= L && off0 >= 0 && off1 > off0 && off1 <= P.N;
+  const int cnt = usable ? min(kItems, len - n0) : 0, rows_here = min(kItems, L - n0);
+  if (cnt < rows_here) {                                    // rows of items that receive no gradient
+    const int first = max(cnt, 0);
+    float *k0 = P.dKf + ((size_t)u * L + n0 + first) * dqk, *v0 = P.dVf + ((size_t)u * L + n0 + first) * d;
+    if (rank == 0) {
+      for (int i = tid; i < (rows_here - first) * dqk; i += nt) k0[i] = 0.f;
+      for (int i = tid; i < (rows_here - first) * d; i += nt) v0[i] = 0.f;
+    }
+    if (cnt <= 0) return;                                   // (all blocks of the cluster alike)
+  }
+  const int seg0 = n0 / S, nsp = (n0 + cnt - 1) / S - seg0 + 1;        // segments of the valid items
+  const int gp = d + 4, kld = dqk + 4;
+  const int grows = P.span;
+  float* Ks = sm;                                           // [32][kld]
+  float* qs = Ks + kItems * kld;                            // [2][step][dqk]
+  float* ds = qs + 2 * step * dqk;                          // [2][step][span][gp]
+  float* des = ds + (size_t)2 * step * grows * gp;          // [H][16][kDeP]
+  // this block's candidates
+  const int per = (off1 - off0 + ranks - 1) / ranks, c_lo = off0 + rank * per, c_hi = min(off1, c_lo + per);
+  auto fetch = [&](int c, int b) {
+    const int n_c = min(step, c_hi - c);
+    for (int i = tid; i < n_c * dqk / 4; i += nt) mma::cp16(mma::smem_addr(qs + b * step * dqk + i * 4), P.Qf + (size_t)c * dqk + i * 4, 16u);
+    const int d4 = d >> 2, row4 = nsp * d4;
+    for (int i = tid; i < n_c * row4; i += nt) {
+      const int cc = i / row4, r = i - cc * row4, sg = r / d4, x = r - sg * d4;
+      mma::cp16(mma::smem_addr(ds + ((size_t)(b * step + cc) * grows + sg) * gp + x * 4),
+                P.dHp + ((size_t)(c + cc) * P.Lp + seg0) * d + r * 4, 16u);
+    }
+  };
+  if (c_lo < c_hi) fetch(c_lo, 0);
+  mma::cp_commit();
+  for (int i = tid; i < kItems * dqk / 4; i += nt) {
+    const int r = i / (dqk / 4), x = i - r * (dqk / 4);
+    *reinterpret_cast<float4*>(Ks + r * kld + x * 4) =
+        r < cnt ? *reinterpret_cast<const float4*>(P.Kf + ((size_t)u * L + n0 + r) * dqk + x * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  for (int i = tid; i < H * kStepMax * kDeP; i += nt) des[i] = 0.f;
+  float kreg[DQ], vreg[DVH], dk[DQ], dv[DVH];
+  const bool live = n < cnt;
+#pragma unroll
+  for (int a = 0; a < DQ; a += 4) {
+    float x[4] = {0.f, 0.f, 0.f, 0.f};
+    if (live) unpack4(x, *reinterpret_cast<const float4*>(P.Kf + ((size_t)u * L + n0 + n) * dqk + h * DQ + a));
+#pragma unroll
+    for (int e = 0; e < 4; ++e) { kreg[a + e] = x[e]; dk[a + e] = 0.f; }
+  }
+#pragma unroll
+  for (int v = 0; v < DVH; v += 4) {
+    float x[4] = {0.f, 0.f, 0.f, 0.f};
+    if (live) unpack4(x, *reinterpret_cast<const float4*>(P.Vf + ((size_t)u * L + n0 + n) * d + h * DVH + v));
+#pragma unroll
+    for (int e = 0; e < 4; ++e) { vreg[v + e] = x[e]; dv[v + e] = 0.f; }
+  }
+  const int sl = live ? (n0 + n) / S - seg0 : 0;
+  int b = 0;
+  for (int c = c_lo; c < c_hi; c += step, b ^= 1) {
+    const int n_c = min(step, c_hi - c);
+    mma::cp_wait<0>();
+    __syncthreads();                       // this step's rows are there; the previous step's de terms have been read
+    if (c + step < c_hi) fetch(c + step, b ^ 1);
+    mma::cp_commit();
+    // K candidates cc, cc + parts, ... at once: their chains of dependent operations run side by side
+    auto gates = [&](int cc, auto count) {
+      constexpr int K = decltype(count)::value;
+      float qv[K][DQ], gv[K][DVH], g[K], de[K];
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        const float* qp = qs + (b * step + cc + k * parts) * dqk + h * DQ;
+        const float* op = ds + ((size_t)(b * step + cc + k * parts) * grows + sl) * gp + h * DVH;
+#pragma unroll
+        for (int a = 0; a < DQ; a += 4) unpack4(*reinterpret_cast<float(*)[4]>(qv[k] + a), *reinterpret_cast<const float4*>(qp + a));
+#pragma unroll
+        for (int v = 0; v < DVH; v += 4) unpack4(*reinterpret_cast<float(*)[4]>(gv[k] + v), *reinterpret_cast<const float4*>(op + v));
+      }
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        float e0 = 0.f, e1 = 0.f, g0 = 0.f, g1 = 0.f;
+#pragma unroll
+        for (int a = 0; a < DQ; a += 2) { e0 = fmaf(qv[k][a], kreg[a], e0); e1 = fmaf(qv[k][a + 1], kreg[a + 1], e1); }
+#pragma unroll
+        for (int v = 0; v < DVH; v += 2) { g0 = fmaf(gv[k][v], vreg[v], g0); g1 = fmaf(gv[k][v + 1], vreg[v + 1], g1); }
+        g[k] = live ? 1.f / (1.f + expf(-(e0 + e1))) : 0.f;
+        de[k] = (g0 + g1) * g[k] * (1.f - g[k]);
+        des[(h * kStepMax + cc + k * parts) * kDeP + n] = de[k];
+      }
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+#pragma unroll
+        for (int v = 0; v < DVH; ++v) dv[v] = fmaf(g[k], gv[k][v], dv[v]);
+#pragma unroll
+        for (int a = 0; a < DQ; ++a) dk[a] = fmaf(de[k], qv[k][a], dk[a]);
+      }
+    };
+    int cc = part;
+    if constexpr (DVH < 64)
+      for (; cc + parts < n_c; cc += 2 * parts) gates(cc, std::integral_constant<int, 2>());
+    for (; cc < n_c; cc += parts) gates(cc, std::integral_constant<int, 1>());
+    for (; cc < step; cc += parts) des[(h * kStepMax + cc) * kDeP + n] = 0.f;
+    __syncthreads();
+    {
+      // dQ_h of the step: thread = (items slice, candidates cg + 4 i, components 4 ag ..); the two halves of a warp and the parts of a
+      // head take different items
+      const int ag = n & 3, cgp = n >> 2 & 3, slice = part * 2 + (n >> 4), per_slice = kItems / (2 * parts);
+      float acc[4][4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.f;
+      const float* ep = des + (h * kStepMax + cgp) * kDeP;
+      const float* kp = Ks + h * DQ + ag * 4;
+      for (int r = slice * per_slice; r < (slice + 1) * per_slice; r += 4) {
+        float kv[4][4];
+#pragma unroll
+        for (int x = 0; x < 4; ++x) lds4(kv[x], kp + (r + x) * kld);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          float ev[4];
+          lds4(ev, ep + i * 4 * kDeP + r);
+#pragma unroll
+          for (int x = 0; x < 4; ++x)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) acc[i][e] = fmaf(ev[x], kv[x][e], acc[i][e]);
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[i][e] += __shfl_xor_sync(0xffffffffu, acc[i][e], 16);
+        const int cc = cgp + 4 * i;
+        if (n < 16 && cc < n_c) mma::red_add4(P.dQf + (size_t)(c + cc) * dqk + h * DQ + ag * 4, acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+      }
+    }
+  }
+  mma::cp_wait<0>();
+  // sums of the parts and of the cluster's blocks, in a fixed order, through [parts][32 items][H (16 + DVH) + 1]
+  if (parts > 1 || ranks > 1) {
+    const int width = H * (DQ + DVH), pitch = width + 1, warps = nt >> 5;
+    const cg::cluster_group cluster = cg::this_cluster();
+    __syncthreads();                       // (everything else in shared memory has been read)
+    float* mine = sm + (size_t)(part * kItems + n) * pitch + h * (DQ + DVH);
+#pragma unroll
+    for (int a = 0; a < DQ; ++a) mine[a] = dk[a];
+#pragma unroll
+    for (int v = 0; v < DVH; ++v) mine[DQ + v] = dv[v];
+    if (ranks > 1 && parts > 1) {          // the parts first: the other blocks read one sum
+      __syncthreads();
+      for (int r = warp; r < cnt; r += warps)
+        for (int x = n; x < width; x += 32) {
+          float v = sm[(size_t)r * pitch + x];
+          for (int k = 1; k < parts; ++k) v += sm[(size_t)(k * kItems + r) * pitch + x];
+          sm[(size_t)r * pitch + x] = v;
+        }
+    }
+    if (ranks > 1) cluster.sync(); else __syncthreads();
+    // this block's share of the items, a warp per item
+    const int lo = cnt * rank / ranks, hi = cnt * (rank + 1) / ranks;
+    for (int r = lo + warp; r < hi; r += warps)
+      for (int x = n; x < width; x += 32) {
+        float v = 0.f;
+        if (ranks > 1) {
+          for (int k = 0; k < ranks; ++k) v += cluster.map_shared_rank(sm, k)[(size_t)r * pitch + x];
+        } else {
+          for (int k = 0; k < parts; ++k) v += sm[(size_t)(k * kItems + r) * pitch + x];
+        }
+        const int hh = x / (DQ + DVH), comp = x - hh * (DQ + DVH);
+        if (comp < DQ) P.dKf[((size_t)u * L + n0 + r) * dqk + hh * DQ + comp] = v;
+        else P.dVf[((size_t)u * L + n0 + r) * d + hh * DVH + comp - DQ] = v;
+      }
+    if (ranks > 1) cluster.sync();         // (no block leaves while others read its sums)
+  } else if (live) {
+    float* kp = P.dKf + ((size_t)u * L + n0 + n) * dqk + h * DQ;
+    float* vp = P.dVf + ((size_t)u * L + n0 + n) * d + h * DVH;
+#pragma unroll
+    for (int a = 0; a < DQ; a += 4) *reinterpret_cast<float4*>(kp + a) = make_float4(dk[a], dk[a + 1], dk[a + 2], dk[a + 3]);
+#pragma unroll
+    for (int v = 0; v < DVH; v += 4) *reinterpret_cast<float4*>(vp + v) = make_float4(dv[v], dv[v + 1], dv[v + 2], dv[v + 3]);
+  }
+}
+
+bool gate_plan(const Plan& p, GateParams* params, int* split, size_t* smem) {
+  GateParams& P = *params;
+  if (p.dqh != 16 || (p.dvh != 16 && p.dvh != 32 && p.dvh != 64) || p.U > 65535) return false;
+  if (p.H > (p.dvh == 16 ? 16 : 8)) return false;
+  P.L = p.L; P.d = p.d; P.dqk = p.dqk; P.H = p.H; P.S = p.S; P.Lp = p.Lp; P.N = p.N;
+  P.span = std::min((kItems - 2 + p.S) / p.S + 1, p.Lp);
+  // Too few blocks for four warps per SM: clusters of blocks share a user's candidates, at least eight each, in fours or eights (in
+  // twos they gain nothing); then warps of a block do, with at least sixteen each.  us (CUDA events, about 6 too long), `parts` /
+  // `csplit`: 6 users x 45 candidates, two heads, 114 blocks 25 (1/1), 25 (1/2), 19 (1/4), 19 (4/1); 30 x 153, one head, 120 blocks
+  // 105 (1/1), 29 (1/8), 35 (4/2); 1 x 1000, 2 blocks 476 (1/1), 68 (1/8), 31 (4/8); 20 x 20, four heads, 640 blocks 21 (1/1), 37
+  // (1/2), 39 (2/1).
+  const long long warps = (long long)((p.L + kItems - 1) / kItems) * p.U * p.H, want = 4ll * device_sms();
+  int csplit = 1;
+  while (csplit < 8 && warps * csplit < want && p.maxC >= 16 * csplit) csplit *= 2;
+  if (csplit == 2) csplit = 1;
+  P.parts = 1;
+  while (2 * P.parts * p.H <= 8 && warps * csplit * P.parts < want && p.maxC / csplit >= 32 * P.parts) P.parts *= 2;
+  auto smem_of = [&](int step) {
+    const size_t loop = (size_t)kItems * (p.dqk + 4) + 2 * (size_t)step * (p.dqk + (size_t)P.span * (p.d + 4)) + (size_t)p.H * kStepMax * kDeP;
+    const size_t sums = P.parts > 1 || csplit > 1 ? (size_t)P.parts * kItems * (p.H * (16 + p.dvh) + 1) : 0;
+    return std::max(loop, sums) * sizeof(float);
+  };
+  P.step = kStepMax;
+  while (P.step > 4 && smem_of(P.step) > 100 * 1024) P.step /= 2;
+  *smem = smem_of(P.step);
+  *split = csplit;
+  return *smem <= 200 * 1024;
+}
+
+}  // namespace
+
+int gsta_train_f32(const Plan& p, const float* Hp, const int32_t* lengths, const int32_t* cand_offsets, const void* cands,
+                   const void* Wg, const float* dz, const GstaTrain& G, float* dHp, cudaStream_t st) {
+  TrainParams P;
+  P.Hp = Hp; P.cands = cands; P.Wg = Wg; P.dz = dz; P.lengths = lengths; P.cand_offsets = cand_offsets; P.G = G; P.dHp = dHp;
+  P.U = p.U; P.L = p.L; P.S = p.S; P.Lp = p.Lp; P.LpP = (p.Lp + 3) & ~3; P.M = p.M; P.N = p.N; P.inv_tau = p.inv_tau;
+  return p.dtype == LASER_F32 ? dispatch_train<float>(p, P, st) : dispatch_train<bf16>(p, P, st);
+}
+
+bool sta_bwd_f32_supported(const Plan& p) {
+  GateParams P;
+  int csplit;
+  size_t smem;
+  return gate_plan(p, &P, &csplit, &smem);
+}
+
+int sta_bwd_f32(const Plan& p, const float* Qf, const float* Kf, const float* Vf, const float* dHp, const int32_t* lengths,
+                const int32_t* cand_offsets, float* dQf, float* dK, float* dV, cudaStream_t st) {
+  GateParams P;
+  int csplit;
+  size_t smem;
+  if (!gate_plan(p, &P, &csplit, &smem)) return LASER_ERR_UNSUPPORTED;
+  P.Qf = Qf; P.Kf = Kf; P.Vf = Vf; P.dHp = dHp; P.lengths = lengths; P.cand_offsets = cand_offsets; P.dQf = dQf; P.dKf = dK; P.dVf = dV;
+  auto kernel = p.dvh == 64   ? sta_bwd_f32_kernel<64, 256>
+                : p.dvh == 32 ? sta_bwd_f32_kernel<32, 256>
+                : p.H <= 8    ? sta_bwd_f32_kernel<16, 256>
+                              : sta_bwd_f32_kernel<16, 512>;
+  LASER_CUDA_OK(allow_smem(kernel, smem));
+  LaunchScope ls("bwd_sta", st);
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = attr.val.clusterDim.y = 1;
+  attr.val.clusterDim.z = csplit;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((p.L + kItems - 1) / kItems, p.U, csplit);
+  cfg.blockDim = dim3(32 * p.H * P.parts);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  LASER_CUDA_OK(cudaLaunchKernelEx(&cfg, kernel, P));
+  return LASER_OK;
+}
+
+}  // namespace laser

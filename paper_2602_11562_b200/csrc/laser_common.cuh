@@ -63,6 +63,26 @@ class LaunchScope {
   int slot_;
 };
 
+// Several arrays to be set to zero (16-byte aligned), and one worker's share of that.
+struct ZeroList {
+  float* p[8];
+  unsigned long long n[8];
+  int count;
+  void add(void* q, size_t len) {
+    if (len) { p[count] = static_cast<float*>(q); n[count++] = len; }
+  }
+};
+__device__ __forceinline__ void zero_share(const ZeroList& Z, unsigned long long worker, unsigned long long workers) {
+  for (int a = 0; a < Z.count; ++a) {
+    float4* q = reinterpret_cast<float4*>(Z.p[a]);
+    const unsigned long long n4 = Z.n[a] / 4;
+    for (unsigned long long i = worker; i < n4; i += workers) q[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (worker < (Z.n[a] & 3)) Z.p[a][n4 * 4 + worker] = 0.f;
+  }
+}
+
+int zero_arrays(const ZeroList& Z, cudaStream_t st);      // as a launch of its own (laser_backward.cu)
+
 // --- per-path launchers (each returns LASER_OK / LASER_ERR_*) -------------------------------------------------------
 int simt_sta(const Plan& p, const void* items, const int32_t* lengths, const void* cands, const int32_t* cand_offsets,
              const void* Wq, const void* Wk, const void* Wv, void* Hprime, char* ws, cudaStream_t st);
@@ -75,13 +95,14 @@ int simt_gsta(const Plan& p, const void* Hprime, const int32_t* lengths, const i
 // The same for the widths in use (laser_simt_gsta.cu); LASER_ERR_UNSUPPORTED for all other shapes.
 int gsta_f32(const Plan& p, const void* Hprime, const int32_t* lengths, const int32_t* cand_offsets, const void* cands,
              const void* Wg, void* z, char* ws, cudaStream_t st, bool follows_call);
-// Eq. 8-9 on the FP32 ALUs (fp32 Q / gamma, K, V at off_q, off_k, off_v), and the segment sums alone, from fp32 Q / gamma, K, V at off_q, off_k, off_v (16-wide query heads, 16-, 32- or 64-wide value
-// heads; else LASER_ERR_UNSUPPORTED).
+// Eq. 8-9 on the FP32 ALUs (fp32 Q / gamma, K, V at off_q, off_k, off_v), and the segment sums alone, from fp32 Q / gamma, K, V at off_q,
+// off_k, off_v (16-wide query heads, 16-, 32- or 64-wide value heads; else LASER_ERR_UNSUPPORTED).
+// zero: arrays that the same launch sets to zero (null: none).
 int simt_project(const Plan& p, const void* items, const int32_t* lengths, const void* cands, const void* Wq,
-                 const void* Wk, const void* Wv, char* ws, cudaStream_t st);
+                 const void* Wk, const void* Wv, char* ws, cudaStream_t st, const ZeroList* zero = nullptr);
 // The same with larger tiles, for batches of many rows (laser_simt_proj.cu); LASER_ERR_UNSUPPORTED for widths it does not take.
 int simt_project_tiles(const Plan& p, const void* items, const int32_t* lengths, const void* cands, const void* Wq, const void* Wk,
-                       const void* Wv, char* ws, cudaStream_t st);
+                       const void* Wv, char* ws, cudaStream_t st, const ZeroList* zero);
 int simt_attend_f32(const Plan& p, const int32_t* lengths, const int32_t* cand_offsets, float* Hprime32, char* ws,
                     cudaStream_t st);
 // STA on the FP32 ALUs with an fp32 H' whatever the I/O dtype; leaves fp32 Q / gamma, K, V at off_q, off_k, off_v.

@@ -547,10 +547,11 @@ gsta_simt_kernel(const T* __restrict__ Hp, const int* __restrict__ lengths, cons
 // Eq. 8-9 in fp32: Q / gamma, K, V into the workspace (off_q, off_k, off_v).
 template <typename T>
 int simt_project_t(const Plan& p, const T* items, const int32_t* lengths, const T* cands, const T* Wq, const T* Wk,
-                   const T* Wv, char* ws, cudaStream_t st) {
+                   const T* Wv, char* ws, cudaStream_t st, const ZeroList* zero = nullptr) {
   if (p.N == 0 || p.U == 0) return LASER_OK;
-  const int rc = simt_project_tiles(p, items, lengths, cands, Wq, Wk, Wv, ws, st);
+  int rc = simt_project_tiles(p, items, lengths, cands, Wq, Wk, Wv, ws, st, zero);
   if (rc != LASER_ERR_UNSUPPORTED) return rc;
+  if (zero && (rc = zero_arrays(*zero, st)) != LASER_OK) return rc;
   ProjParams P;
   P.items = items; P.cands = cands; P.Wq = Wq; P.Wk = Wk; P.Wv = Wv;
   P.Q = reinterpret_cast<float*>(ws + p.off_q);
@@ -672,12 +673,12 @@ int simt_sta_f32(const Plan& p, const void* items, const int32_t* lengths, const
 }
 
 int simt_project(const Plan& p, const void* items, const int32_t* lengths, const void* cands, const void* Wq,
-                 const void* Wk, const void* Wv, char* ws, cudaStream_t st) {
+                 const void* Wk, const void* Wv, char* ws, cudaStream_t st, const ZeroList* zero) {
   if (p.dtype == LASER_F32)
     return simt_project_t<float>(p, (const float*)items, lengths, (const float*)cands, (const float*)Wq, (const float*)Wk,
-                                 (const float*)Wv, ws, st);
+                                 (const float*)Wv, ws, st, zero);
   using B = __nv_bfloat16;
-  return simt_project_t<B>(p, (const B*)items, lengths, (const B*)cands, (const B*)Wq, (const B*)Wk, (const B*)Wv, ws, st);
+  return simt_project_t<B>(p, (const B*)items, lengths, (const B*)cands, (const B*)Wq, (const B*)Wk, (const B*)Wv, ws, st, zero);
 }
 
 int simt_attend_f32(const Plan& p, const int32_t* lengths, const int32_t* cand_offsets, float* Hprime32, char* ws,

@@ -168,10 +168,10 @@ struct ProductNT {
 
 // The warps of a block are dealt to its candidates: kWarps / CB each.
 
-// y[c][h][j] = scale s_j . x[c][h] for the nv[c] segment vectors of candidate c (Hs: rows of pitch ds, Lp rows per candidate),
-// four lanes per segment, all heads at once.
+// y[c][h][j] = scale s_j . x[c][h] for the nv[c] segment vectors of candidate c (Hs: Lp rows of pitch DS per candidate; y: rows of
+// pitch yp), four lanes per segment, all heads at once.
 template <int D, int H, int CB, int DS>
-__device__ __forceinline__ void scores(const float* Hs, const float* x, const int* nv, int Lp, float scale, float* y, int tid) {
+__device__ __forceinline__ void scores(const float* Hs, const float* x, const int* nv, int Lp, int yp, float scale, float* y, int tid) {
   constexpr int kPer = kWarps / CB;
   const int warp = tid >> 5, lane = tid & 31, c = warp / kPer, p = lane & 3, n = nv[c];
   const float* xc = x + (size_t)c * H * DS + p * 4;
@@ -201,18 +201,18 @@ __device__ __forceinline__ void scores(const float* Hs, const float* x, const in
     if (j < n) {
 #pragma unroll
       for (int h = 0; h < H; ++h)
-        if ((h & 3) == p) y[((size_t)c * H + h) * Lp + j] = acc[h] * scale;
+        if ((h & 3) == p) y[((size_t)c * H + h) * yp + j] = acc[h] * scale;
     }
   }
 }
 
-// softmax over a candidate's segments, one warp per (candidate, head); a candidate without segments has no weights
+// softmax over a candidate's segments (rows of pitch ep), one warp per (candidate, head); a candidate without segments has no weights
 template <int H, int CB>
-__device__ __forceinline__ void softmax(float* e, const int* nv, int Lp, int tid) {
+__device__ __forceinline__ void softmax(float* e, const int* nv, int ep, int tid) {
   const int warp = tid >> 5, lane = tid & 31;
   for (int ch = warp; ch < CB * H; ch += kWarps) {
     const int n = nv[ch / H];
-    float* ec = e + (size_t)ch * Lp;
+    float* ec = e + (size_t)ch * ep;
     float mx = -INFINITY, s = 0.f;
     for (int j = lane; j < n; j += 32) mx = fmaxf(mx, ec[j]);
     mx = warp_max(mx);
@@ -226,14 +226,14 @@ __device__ __forceinline__ void softmax(float* e, const int* nv, int Lp, int tid
   }
 }
 
-// y[c][h] = sum_j w[c][h][j] s_j: a group of D / 4 lanes (four features each) takes every kGroups-th segment of its
-// candidate, all heads at once; the groups' sums meet in `red` (weighted_floats).
+// y[c][h] = sum_j w[c][h][j] s_j (w: rows of pitch wp): a group of D / 4 lanes (four features each) takes every kGroups-th segment of its
+// candidate, all heads at once; the groups' sums meet in `red` (kFloats).
 template <int D, int H, int CB>
 struct Weighted {
   static constexpr int kPer = kWarps / CB, kCols = D / 4, kInWarp = 32 / kCols, kGroups = kPer * kInWarp;
   static constexpr int kFloats = CB * kGroups * H * D;                 // of `red`
   template <int DS>
-  __device__ __forceinline__ static void run(const float* Hs, const float* w, const int* nv, int Lp, float* red, int tid) {
+  __device__ __forceinline__ static void run(const float* Hs, const float* w, const int* nv, int Lp, int wp, float* red, int tid) {
     const int warp = tid >> 5, lane = tid & 31, c = warp / kPer, sub = lane / kCols, n = nv[c];
     if (kInWarp * kCols < 32 && sub >= kInWarp) return;
     const int grp = warp % kPer * kInWarp + sub, i = lane % kCols * 4;
@@ -241,14 +241,14 @@ struct Weighted {
 #pragma unroll
     for (int h = 0; h < H; ++h) acc[h][0] = acc[h][1] = acc[h][2] = acc[h][3] = 0.f;
     const float* s = Hs + (size_t)c * Lp * DS + i;
-    const float* wc = w + (size_t)c * H * Lp;
+    const float* wc = w + (size_t)c * H * wp;
 #pragma unroll 4
     for (int j = grp; j < n; j += kGroups) {
       float sv[4];
       lds4(sv, s + (size_t)j * DS);
 #pragma unroll
       for (int h = 0; h < H; ++h) {
-        const float a = wc[h * Lp + j];
+        const float a = wc[h * wp + j];
 #pragma unroll
         for (int e = 0; e < 4; ++e) acc[h][e] = fmaf(a, sv[e], acc[h][e]);
       }
@@ -289,13 +289,6 @@ __device__ __forceinline__ void stage_segments(float* Hs, const T* Hp, const int
     unpack4(v, *reinterpret_cast<const typename Raw4<T>::type*>(src + 4 * i));
     *reinterpret_cast<float4*>(dst + i / kCols * DS + i % kCols * 4) = make_float4(v[0], v[1], v[2], v[3]);
   }
-}
-
-// Shapes with a compile-time kernel: f.template operator()<D, H>() for (d, heads), false for the others.
-inline bool supported(int d, int H) {
-  if (H < 1 || d % 32 || d > 128 || d % H) return false;
-  const int dh = d / H;
-  return dh == 16 || dh == 32 || (dh == 64 && d != 96) || (dh == 128);
 }
 
 }  // namespace dense

@@ -98,11 +98,11 @@ __global__ void __launch_bounds__(kThreads, 2) gsta_f32_kernel(const GstaF32Para
     __syncthreads();
     nt.run(q, tid, [&](int c, int h, int i, float v) { qt[(c * H + h) * DS + i] = v; });
     __syncthreads();
-    scores<D, H, CB, DS>(Hs, qt, s_nv, Lp, P.inv_tau, e, tid);
+    scores<D, H, CB, DS>(Hs, qt, s_nv, Lp, Lp, P.inv_tau, e, tid);
     __syncthreads();
     softmax<H, CB>(e, s_nv, Lp, tid);
     __syncthreads();
-    Weighted<D, H, CB>::template run<DS>(Hs, e, s_nv, Lp, red, tid);
+    Weighted<D, H, CB>::template run<DS>(Hs, e, s_nv, Lp, Lp, red, tid);
     nn.load(Wv, tid);
     __syncthreads();
     Weighted<D, H, CB>::template finish<DS>(red, qt, tid);
@@ -131,7 +131,7 @@ template <typename T, int D, int H, int CB>
 int launch_cb(const Plan& p, const GstaF32Params& P, cudaStream_t st) {
   const size_t smem = smem_bytes<D, H, CB>(p.Lp);
   LASER_CUDA_OK(allow_smem(gsta_f32_kernel<T, D, H, CB>, smem));
-  LaunchScope ls("gsta_f32", st);
+  LaunchScope ls("gsta_simt", st);
   LASER_CUDA_OK(launch_chained(gsta_f32_kernel<T, D, H, CB>, dim3((p.N + CB - 1) / CB), dim3(kThreads), smem, st, P));
   return LASER_OK;
 }

@@ -28,7 +28,15 @@ struct TileParams {
   int* status;
   int U, L, N, d, dqk, q_tiles, tiles_per_user;
   float inv_gamma;
+  ZeroList zero;                         // arrays that this launch also sets to zero
 };
+__device__ __forceinline__ void housekeeping(const TileParams& P) {
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) set_status(P.status, 0);
+  if (P.zero.count > 0) {
+    const unsigned long long block = (unsigned long long)blockIdx.y * gridDim.x + blockIdx.x;
+    zero_share(P.zero, block * kThreads + threadIdx.x, (unsigned long long)gridDim.x * gridDim.y * kThreads);
+  }
+}
 
 struct Tile {
   int rows, n_cols;                      // rows == 0: nothing to do
@@ -68,11 +76,11 @@ __device__ __forceinline__ float* output_at(const TileParams& P, const Tile& t, 
   return (t.is_q ? P.Q : first ? P.K : P.V) + t.out_row * *ld + (first ? col : col - P.dqk);
 }
 
-__global__ void __launch_bounds__(kThreads) proj_tile_f32_kernel(TileParams P) {      // d and d_qk multiples of 4
+__global__ void __launch_bounds__(kThreads) proj_tile_f32_kernel(const __grid_constant__ TileParams P) {      // d and d_qk multiples of 4
   extern __shared__ __align__(16) float xs[];   // [64][d + 4] rows, then [d][64] weights
   chain_wait();
   chain_release();
-  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) set_status(P.status, 0);
+  housekeeping(P);
   const Tile tile = find_tile(P);
   if (tile.rows == 0) return;
   const int d = P.d, xp = d + 4, d4 = d >> 2, tid = threadIdx.x, tx = tid & 15, ty = tid >> 4, col = blockIdx.y * kCols + tx * 4;
@@ -125,12 +133,12 @@ __global__ void __launch_bounds__(kThreads) proj_tile_f32_kernel(TileParams P) {
   }
 }
 
-__global__ void __launch_bounds__(kThreads) proj_tile_mma_kernel(TileParams P) {      // d a multiple of 16, d_qk of 8
+__global__ void __launch_bounds__(kThreads) proj_tile_mma_kernel(const __grid_constant__ TileParams P) {      // d a multiple of 16, d_qk of 8
   extern __shared__ __align__(128) uint8_t xb[];  // [64][2 d + 16] bytes, then [d][144]
   constexpr int WS = kCols * 2 + 16;
   chain_wait();
   chain_release();
-  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) set_status(P.status, 0);
+  housekeeping(P);
   const Tile tile = find_tile(P);
   if (tile.rows == 0) return;
   const int d = P.d, XS = 2 * d + 16, d8 = d >> 3, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, col0 = blockIdx.y * kCols;
@@ -182,13 +190,14 @@ __global__ void __launch_bounds__(kThreads) proj_tile_mma_kernel(TileParams P) {
 }  // namespace
 
 int simt_project_tiles(const Plan& p, const void* items, const int32_t* lengths, const void* cands, const void* Wq, const void* Wk,
-                       const void* Wv, char* ws, cudaStream_t st) {
+                       const void* Wv, char* ws, cudaStream_t st, const ZeroList* zero) {
   const bool f32 = p.dtype == LASER_F32;
   if (f32 ? p.d % 4 || p.dqk % 4 : p.d % 16 || p.dqk % 8) return LASER_ERR_UNSUPPORTED;
   const size_t smem = f32 ? ((size_t)kRows * (p.d + 4) + (size_t)p.d * kCols) * sizeof(float)
                           : (size_t)kRows * (2 * p.d + 16) + (size_t)p.d * (kCols * 2 + 16);
   if (smem > 200 * 1024) return LASER_ERR_UNSUPPORTED;
-  TileParams P;
+  TileParams P = {};
+  if (zero) P.zero = *zero;
   P.items = items; P.cands = cands; P.Wq = Wq; P.Wk = Wk; P.Wv = Wv;
   P.Q = reinterpret_cast<float*>(ws + p.off_q);
   P.K = reinterpret_cast<float*>(ws + p.off_k);
@@ -203,7 +212,7 @@ int simt_project_tiles(const Plan& p, const void* items, const int32_t* lengths,
   if (tiles > 0x7fffffffLL || col_tiles > 65535) return LASER_ERR_UNSUPPORTED;
   auto kernel = f32 ? proj_tile_f32_kernel : proj_tile_mma_kernel;
   LASER_CUDA_OK(allow_smem(kernel, smem));
-  LaunchScope ls("proj_tile", st);
+  LaunchScope ls("proj_simt", st);
   LASER_CUDA_OK(launch_chained(kernel, dim3((unsigned)tiles, col_tiles), dim3(kThreads), smem, st, P));
   return LASER_OK;
 }

@@ -1,0 +1,48 @@
+"""The fp32 backward kernels at the sizes where their work is split differently: gates whose 32 items cross segments, candidates shared by
+a cluster of blocks or by the warps of a head, one to four candidates per block in the stacked attention, every width."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2602_11562_b200 as P
+from oracle import backward_oracle
+from workloads import make_custom
+
+pytestmark = pytest.mark.gpu
+
+CASES = [
+    dict(U=2, C=9, L=70, d=32, H=1, S=1, M=1),                        # every item its own segment
+    dict(U=2, C=17, L=65, d=32, H=2, S=7, M=2, lengths=[65, 33]),     # 32 items touch five or six segments; one item past a block
+    dict(U=3, C=5, L=96, d=64, H=1, S=31, M=2, lengths=[96, 0, 1]),   # 64-wide value heads, users without or with one item
+    dict(U=1, C=70, L=64, d=128, H=2, S=64, M=1),                     # a cluster of eight, 64-wide heads, an uneven last share
+    dict(U=1, C=300, L=33, d=64, H=2, S=16, M=1),                     # a cluster of eight and two warps per head
+    dict(U=2, C=33, L=40, d=128, H=4, S=20, M=2),                     # a cluster of four, 32-wide heads
+    dict(U=1, C=40, L=40, d=96, H=6, S=13, M=3),                      # products with transposed 96-wide matrices
+    dict(U=1, C=20, L=50, d=128, H=8, S=9, M=1),
+    dict(U=1, C=12, L=30, d=128, H=1, S=9, M=1),                      # 128-wide head: general gates, new stacked attention
+    dict(U=4, C=100, L=20, d=32, H=1, S=5, M=1),                      # two candidates per block
+    dict(U=9, C=100, L=20, d=64, H=4, S=5, M=2),                      # four, a partial block
+    dict(U=1, C=4, L=40, d=96, H=2, S=9, M=1),                        # 48-wide heads: general kernels throughout
+]
+
+
+@pytest.mark.parametrize("case", range(len(CASES)))
+def test_fp32_backward_edges(case):
+    w = make_custom(seed=2500 + case, dtype="f32", d_qh=16, emb_std="inv_sqrt_d", **CASES[case])
+    s = w.spec
+    dz = np.random.default_rng(case).standard_normal((w.N, s.d)).astype(np.float32)
+    ref = backward_oracle.backward(w.items, w.lengths, w.cands, w.cand_offsets, w.Wq, w.Wk, w.Wv, w.Wg, s.S, s.H,
+                                   dz.astype(np.float64), w.gamma, w.tau)
+    b = P.DeviceBatch.from_workload(w)
+    ws = torch.empty(P.laser_backward_workspace_bytes(b.cfg), dtype=torch.uint8, device="cuda")
+    runs = []
+    for fill in (0xFF, 0x7F):                                          # nothing left in the workspace may matter
+        ws.fill_(fill)
+        got = P.laser_backward(b.cfg, *b.args(), b.Wg, torch.from_numpy(dz).cuda(), workspace=ws)
+        assert P.laser_check_status(ws) == 0
+        runs.append(got)
+    for k, r in ref.items():
+        g = runs[0][k].cpu().numpy().astype(np.float64)
+        # fp32 sums of a few hundred products through three or four steps: 1e-4 of the largest entry, as for the other shapes
+        assert np.isfinite(g).all() and np.max(np.abs(g - r)) <= 1e-4 * max(float(np.max(np.abs(r))), 1e-30), k
+    assert torch.equal(runs[0]["d_items"], runs[1]["d_items"])         # (sums with atomics go into the other gradients only)
