@@ -1,6 +1,8 @@
 // Interfaces between the source files of the backward pass.  The kernels of the two tensor-core routes are chained (the next
-// one's blocks are placed while the last blocks of this one run: 1.2 % of a call of 0.75-0.85 ms).  Those of the FP32 route are
-// not: their grids are smaller than the GPU, and blocks placed early crowd the SMs that happen to be idle (83 -> 88 us).
+// one's blocks are placed while the last blocks of this one run: 1.2 % of a call of 0.75-0.85 ms).  Those of the FP32 route and of the
+// FP32 forward are chained too, but (the segment sums apart) they let their successor start only as they end: their grids are
+// smaller than the GPU, and blocks placed early crowd the SMs that happen to be idle.  6 users x 45 candidates, backward: early
+// release everywhere 60.8 us, no chaining 55.3, this 49.4; 2 x 63 of 2507 items, forward: 38.1 and 34.7.
 #pragma once
 
 #include "laser_common.cuh"

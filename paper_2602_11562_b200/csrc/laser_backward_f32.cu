@@ -66,7 +66,7 @@ __global__ void __launch_bounds__(kThreads, 2) gsta_train_f32_kernel(const Train
   ProductNN<T, D, CB> nn;
   ProductNT<T, D, H, CB> nt;
   ProductNT<T, D, HF, CB> ntf;
-  nn.load(Wg, tid);
+  nn.load(Wg, tid);                              // (inputs: complete before the first kernel of the call has started)
   if (tid < CB) {
     const int cand = c_base + tid;
     int nv = 0;
@@ -86,6 +86,7 @@ __global__ void __launch_bounds__(kThreads, 2) gsta_train_f32_kernel(const Train
     t[i] = i < live ? to_f32<T>(static_cast<const T*>(P.cands)[(size_t)c_base * D + i]) : 0.f;
     dt[i] = i < live ? P.dz[(size_t)c_base * D + i] : 0.f;
   }
+  chain_wait();                                  // (no early release of the next kernel: laser_backward.cuh)
   __syncthreads();
   stage_segments<float, D, CB, DS>(Hs, P.Hp, s_nv, c_base, Lp, tid);
 
@@ -230,8 +231,7 @@ int launch_train_cb(const Plan& p, const TrainParams& P, cudaStream_t st) {
   const size_t smem = train_floats<D, H, CB>(P.Lp, P.LpP, P.M) * sizeof(float);
   LASER_CUDA_OK(allow_smem(gsta_train_f32_kernel<T, D, H, CB>, smem));
   LaunchScope ls("gsta_train_simt", st);
-  gsta_train_f32_kernel<T, D, H, CB><<<(p.N + CB - 1) / CB, kThreads, smem, st>>>(P);
-  LASER_CUDA_OK(cudaGetLastError());
+  LASER_CUDA_OK(launch_chained(gsta_train_f32_kernel<T, D, H, CB>, dim3((p.N + CB - 1) / CB), dim3(kThreads), smem, st, P));
   return LASER_OK;
 }
 
@@ -290,6 +290,7 @@ __global__ void __launch_bounds__(kMaxThreads) sta_bwd_f32_kernel(const GatePara
   extern __shared__ __align__(16) float sm[];
   const int u = blockIdx.y, n0 = blockIdx.x * kItems, rank = blockIdx.z, ranks = gridDim.z;
   const int L = P.L, d = P.d, dqk = P.dqk, H = P.H, S = P.S, step = P.step, parts = P.parts;
+  chain_wait();
   const int len = P.lengths[u], off0 = P.cand_offsets[u], off1 = P.cand_offsets[u + 1];
   const int tid = threadIdx.x, nt = blockDim.x, n = tid & 31, warp = tid >> 5, h = warp % H, part = warp / H;
   const bool usable = len > 0 && len <= L && off0 >= 0 && off1 > off0 && off1 <= P.N;
@@ -529,17 +530,19 @@ int sta_bwd_f32(const Plan& p, const float* Qf, const float* Kf, const float* Vf
                               : sta_bwd_f32_kernel<16, 512>;
   LASER_CUDA_OK(allow_smem(kernel, smem));
   LaunchScope ls("bwd_sta", st);
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = attr.val.clusterDim.y = 1;
-  attr.val.clusterDim.z = csplit;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = csplit;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((p.L + kItems - 1) / kItems, p.U, csplit);
   cfg.blockDim = dim3(32 * p.H * P.parts);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
   LASER_CUDA_OK(cudaLaunchKernelEx(&cfg, kernel, P));
   return LASER_OK;
 }

@@ -369,6 +369,7 @@ __device__ __forceinline__ void put4(float* sm, const float (&v)[4], bool k_majo
 
 __global__ void __launch_bounds__(256) products_kernel(const __grid_constant__ ProductList L) {
   __shared__ __align__(16) float As[2][kStep * (kTile + 4)], Bs[2][kStep * (kTile + 4)];
+  chain_wait();
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   int which = 0;
   while (which + 1 < L.n && (int)blockIdx.x >= L.first[which + 1]) ++which;
@@ -462,8 +463,7 @@ int run_products(Product* list, int n, cudaStream_t st) {
     L.first[L.n] = (int)blocks;
     if (blocks == 0) continue;
     LaunchScope ls("bwd_products", st);
-    products_kernel<<<(unsigned)blocks, 256, 0, st>>>(L);
-    LASER_CUDA_OK(cudaGetLastError());
+    LASER_CUDA_OK(launch_chained(products_kernel, dim3((unsigned)blocks), dim3(256), 0, st, L));
   }
   return LASER_OK;
 }

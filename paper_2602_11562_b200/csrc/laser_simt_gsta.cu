@@ -43,10 +43,7 @@ __global__ void __launch_bounds__(kThreads, 2) gsta_f32_kernel(const GstaF32Para
   float* Hs = red + red_floats<D, H, CB>();  // [CB][Lp][DS]
   float* e = Hs + (size_t)CB * Lp * DS;      // [CB][H][Lp]
   const T* Wg = static_cast<const T*>(P.Wg);
-  if (!P.early) {
-    chain_wait();
-    chain_release();
-  }
+  if (!P.early) chain_wait();
   ProductNN<T, D, CB> nn;
   ProductNT<T, D, H, CB> nt;
   if (P.M > 0) nn.load(Wg, tid);
@@ -74,10 +71,7 @@ __global__ void __launch_bounds__(kThreads, 2) gsta_f32_kernel(const GstaF32Para
   }
   for (int i = tid; i < CB * D; i += kThreads)
     t[i] = c_base + i / D < P.N ? to_f32<T>(static_cast<const T*>(P.cands)[(size_t)c_base * D + i]) : 0.f;
-  if (P.early) {
-    chain_wait();
-    chain_release();
-  }
+  if (P.early) chain_wait();
   __syncthreads();
   if (tid < CB && s_nv[tid] == -2) {
     report_status(P.status, LASER_ERR_BAD_INPUT);

@@ -78,8 +78,7 @@ __device__ __forceinline__ float* output_at(const TileParams& P, const Tile& t, 
 
 __global__ void __launch_bounds__(kThreads) proj_tile_f32_kernel(const __grid_constant__ TileParams P) {      // d and d_qk multiples of 4
   extern __shared__ __align__(16) float xs[];   // [64][d + 4] rows, then [d][64] weights
-  chain_wait();
-  chain_release();
+  chain_wait();                          // (no early release of the next kernel: laser_backward.cuh)
   housekeeping(P);
   const Tile tile = find_tile(P);
   if (tile.rows == 0) return;
@@ -136,8 +135,7 @@ __global__ void __launch_bounds__(kThreads) proj_tile_f32_kernel(const __grid_co
 __global__ void __launch_bounds__(kThreads) proj_tile_mma_kernel(const __grid_constant__ TileParams P) {      // d a multiple of 16, d_qk of 8
   extern __shared__ __align__(128) uint8_t xb[];  // [64][2 d + 16] bytes, then [d][144]
   constexpr int WS = kCols * 2 + 16;
-  chain_wait();
-  chain_release();
+  chain_wait();                          // (no early release of the next kernel: laser_backward.cuh)
   housekeeping(P);
   const Tile tile = find_tile(P);
   if (tile.rows == 0) return;
