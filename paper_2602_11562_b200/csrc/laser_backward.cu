@@ -1100,7 +1100,7 @@ int backward_stream_all(const Plan& p, const T* items, const int32_t* lengths, c
   bf16 *Hhi = reinterpret_cast<bf16*>(s.Hp), *Hlo = Hhi + (size_t)N * p.Lp * d;
   BWD_OK(backward_stream_forward(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, nullptr, Hhi, Hlo, ws, stream_scratch, st));
   const GstaPlanes G = train_planes(p, s);
-  BWD_OK(gsta_train(p, 2, Hhi, Hlo, lengths, cand_offsets, cands, Wg, dz, G, s.dHp, nullptr, train_scratch, st));
+  BWD_OK(gsta_train(p, 2, Hhi, Hlo, lengths, cand_offsets, cands, Wg, dz, G, s.dHp, nullptr, train_scratch, st, false));
   const float* p_sums = nullptr;
   BWD_OK(backward_stream(p, items, lengths, cand_offsets, Wv, s.dHp, d_items, dWv, &p_sums, ws, stream_scratch, st));
 #undef BWD_OK
@@ -1132,16 +1132,17 @@ int lists_parts(const Plan& p) {
   const int np = (p.d == 32 || p.d == 64 || p.d == 128) && p.Lp <= 128 && 2 * p.M * p.H <= 64 ? 1 : 2;
   return sta_bwd_mma_supported(p) && sta_fwd_mma_supported(p) && gsta_train_supported(p, np) ? np : 0;
 }
-// The recomputed H' and its stacked attention, forward and backward, on that many parts: leaves the bf16 dH' for the gate kernel
-// and adds the layers' weight gradients.
+// The recomputed H' and its stacked attention, forward and backward, on that many parts: leaves the bf16 dH' for the gate kernel and,
+// in G, what gsta_weight_sums adds up.
 int lists_attention(const Plan& p, int np, const BwdScratch& s, const int32_t* lengths, const int32_t* cand_offsets, const bf16* cands,
-                    const bf16* Wg, const float* dz, const GstaPlanes& G, float* dWg, char* mma_scratch, char* train_scratch,
-                    cudaStream_t st) {
+                    const bf16* Wg, const float* dz, const GstaPlanes& G, char* mma_scratch, char* train_scratch, cudaStream_t st,
+                    bool prepared) {
   bf16 *Hb = reinterpret_cast<bf16*>(s.Hp), *Hl = np == 2 ? Hb + (size_t)p.N * p.Lp * p.d : nullptr;
   int rc = sta_fwd_mma(p, lengths, cand_offsets, nullptr, Hb, Hl, mma_scratch, st);
   if (rc == LASER_OK)
-    rc = gsta_train(p, np, Hb, Hl, lengths, cand_offsets, cands, Wg, dz, G, nullptr, sta_mma_segment_gradients(p, mma_scratch), train_scratch, st);
-  return rc == LASER_OK ? gsta_weight_sums(p, G, dWg, st) : rc;
+    rc = gsta_train(p, np, Hb, Hl, lengths, cand_offsets, cands, Wg, dz, G, nullptr, sta_mma_segment_gradients(p, mma_scratch), train_scratch, st,
+                    prepared);
+  return rc;
 }
 
 // Candidate lists, bf16, M > 0: gates, stacked attention and every product over the item rows on the MMAs.
@@ -1161,14 +1162,14 @@ int backward_lists(const Plan& p, const bf16* items, const int32_t* lengths, con
   ZeroList Z = {};
   Z.add(dWq, d * dqk); Z.add(dWk, d * dqk); Z.add(dWv, d * d); Z.add(dWg, M * 3 * d * d); Z.add(s.dQf, N * dqk);
   Z.add(ws + p.off_status, kStatusWords);
-  BWD_OK(zero_arrays(Z, st));
-  BWD_OK(rows_project_cands(p, cands, Wq, 0.5f * p.inv_gamma, Qb, st));
-  BWD_OK(rows_project_items(p, items, lengths, cand_offsets, Wk, Wv, Kb, Vb, st));
-  BWD_OK(lists_attention(p, lists_parts(p), s, lengths, cand_offsets, cands, Wg, dz, G, dWg, mma_scratch, train_scratch, st));
+  const int np = lists_parts(p);
+  BWD_OK(rows_project(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, 0.5f * p.inv_gamma, Qb, Kb, Vb, Z,
+                      gsta_train_prep(p, np, Wg, lengths, cand_offsets, train_scratch), st));
+  BWD_OK(lists_attention(p, np, s, lengths, cand_offsets, cands, Wg, dz, G, mma_scratch, train_scratch, st, true));
   BWD_OK(sta_bwd_mma_split(p, lengths, cand_offsets, s.dQf, dKh, dKl, dVh, dVl, mma_scratch, st));
-  BWD_OK(rows_gradients(p, items, lengths, cand_offsets, Wk, Wv, dKh, dKl, dVh, dVl, d_items, dWk, dWv, st));
-  // (Qt and dM are not used on this route; each holds N rows of H d floats, and d_qk <= 2 H d)
-  BWD_OK(rows_gradients_cands(p, cands, Wq, s.dQf, reinterpret_cast<bf16*>(s.Qt), reinterpret_cast<bf16*>(s.dM), G.dT0, d_cands, dWq, st));
+  BWD_OK(rows_gradients(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, s.dQf, dKh, dKl, dVh, dVl, G.dT0, d_items, d_cands, dWq, dWk,
+                        dWv, st));
+  BWD_OK(gsta_weight_sums(p, G, dWg, st));
 #undef BWD_OK
   return LASER_OK;
 }
@@ -1249,7 +1250,8 @@ int backward_t(const Plan& p, const T* items, const int32_t* lengths, const T* c
     if (parts) {
       const GstaPlanes G = train_planes(p, s);
       dT0 = G.dT0;
-      BWD_OK(lists_attention(p, parts, s, lengths, cand_offsets, cands, Wg, dz, G, dWg, mma_scratch, train_scratch, st));
+      BWD_OK(lists_attention(p, parts, s, lengths, cand_offsets, cands, Wg, dz, G, mma_scratch, train_scratch, st, false));
+      BWD_OK(gsta_weight_sums(p, G, dWg, st));
       attended = true;
     }
   }

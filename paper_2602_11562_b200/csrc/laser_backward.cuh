@@ -6,6 +6,7 @@
 #pragma once
 
 #include "laser_common.cuh"
+#include "laser_gsta_img.cuh"
 
 namespace laser {
 
@@ -40,26 +41,28 @@ struct GstaPlanes {
 // high and low parts of fp32 values).  dS [N, Lp, d] leaves as fp32 in dS32 (np = 2) or rounded to bf16 in dS16, whichever is not
 // null.  Rows of empty segments are neither read nor written.  gsta_weight_sums adds the layers' weight gradients from what
 // gsta_train left in G.
+// prepared: an earlier launch of the call did the work of gsta_train_prep(..) (train_prep_share, and gsta_build_order where it asks
+// for an order).
 bool gsta_train_supported(const Plan& p, int np);
 size_t gsta_train_scratch_bytes(const Plan& p, int np);
+TrainPrep gsta_train_prep(const Plan& p, int np, const void* Wg, const int32_t* lengths, const int32_t* cand_offsets, char* scratch);
 int gsta_train(const Plan& p, int np, const void* S0, const void* S1, const int32_t* lengths, const int32_t* cand_offsets,
                const void* cands, const void* Wg, const float* dz, const GstaPlanes& G, float* dS32, __nv_bfloat16* dS16, char* scratch,
-               cudaStream_t st);
+               cudaStream_t st, bool prepared);
 int gsta_weight_sums(const Plan& p, const GstaPlanes& G, float* dWg, cudaStream_t st);
 
-// Products over the item rows on the tensor cores (laser_backward_rows.cu), users' valid rows only, bf16 inputs: K and V (or
-// scale Q of the candidates) as bf16; every row of d_items (zeros for padding) and the sums into dWk, dWv from dK and dV
-// given as bf16 high and low parts.
+// Products over the item rows on the tensor cores (laser_backward_rows.cu), users' valid rows only, bf16 inputs.  rows_project: K, V
+// and q_scale Q as bf16; the same launch sets arrays to zero and runs gsta_train's preparation.  rows_gradients: every row of d_items
+// (zeros for padding) and the sums into dWk, dWv from dK and dV as bf16 high and low parts; d_cands = dT0 + dQf W_q^T / gamma and
+// dWq += T^T dQf / gamma.
 bool rows_mma_supported(const Plan& p);
-int rows_project_items(const Plan& p, const void* items, const int32_t* lengths, const int32_t* cand_offsets, const void* Wk,
-                       const void* Wv, __nv_bfloat16* Kb, __nv_bfloat16* Vb, cudaStream_t st);
-int rows_project_cands(const Plan& p, const void* cands, const void* Wq, float scale, __nv_bfloat16* Qb, cudaStream_t st);
-int rows_gradients(const Plan& p, const void* items, const int32_t* lengths, const int32_t* cand_offsets, const void* Wk,
-                   const void* Wv, const __nv_bfloat16* dK_hi, const __nv_bfloat16* dK_lo, const __nv_bfloat16* dV_hi,
-                   const __nv_bfloat16* dV_lo, float* d_items, float* dWk, float* dWv, cudaStream_t st);
-// d_cands = dT0 + dQf W_q^T / gamma and dWq += T^T dQf / gamma; hi, lo: room for N rows of d_qk bf16 each.
-int rows_gradients_cands(const Plan& p, const void* cands, const void* Wq, const float* dQf, __nv_bfloat16* hi, __nv_bfloat16* lo,
-                         const float* dT0, float* d_cands, float* dWq, cudaStream_t st);
+int rows_project(const Plan& p, const void* items, const int32_t* lengths, const void* cands, const int32_t* cand_offsets, const void* Wq,
+                 const void* Wk, const void* Wv, float q_scale, __nv_bfloat16* Qb, __nv_bfloat16* Kb, __nv_bfloat16* Vb,
+                 const ZeroList& zero, const TrainPrep& prep, cudaStream_t st);
+int rows_gradients(const Plan& p, const void* items, const int32_t* lengths, const void* cands, const int32_t* cand_offsets, const void* Wq,
+                   const void* Wk, const void* Wv, const float* dQf, const __nv_bfloat16* dK_hi, const __nv_bfloat16* dK_lo,
+                   const __nv_bfloat16* dV_hi, const __nv_bfloat16* dV_lo, const float* dT0, float* d_items, float* d_cands, float* dWq,
+                   float* dWk, float* dWv, cudaStream_t st);
 
 // A dense product on the FP32 ALUs: C[m][n] = D[m][n] + alpha (sum_k A(m, k) B(k, n) + sum_k A2(m, k) B2(k, n)), or, with
 // atomic, C += alpha A B in slices of the contraction.  A(m, k) = ta ? A[k lda + m] : A[m lda + k], B(k, n) = tb ?

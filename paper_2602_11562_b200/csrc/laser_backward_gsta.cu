@@ -48,38 +48,13 @@ struct TrainParams {
   float* dS32;                                    // [N, Lp, d] out, fp32 (NP = 2, dS16 null)
 };
 
-// Weight images in MMA fragment order (see laser_gsta_img.cuh), each matrix as stored (B[k][n] = W[k][n]) and transposed.
-__global__ void __launch_bounds__(256) train_prep_kernel(const bf16* Wg, uint4* img, int d, int M, const int* lengths,
-                                                         const int* cand_offsets, int U, int N, int L, int S, int Lp, int cpb,
-                                                         int* nseg, int* order, int* keys) {
+__global__ void __launch_bounds__(256) train_prep_kernel(const __grid_constant__ TrainPrep P) {
+  __shared__ int bins[kGstaSortWords];
   chain_wait();
   chain_release();
-  const int n_blocks = gridDim.x - (order ? 1 : 0);
-  if ((int)blockIdx.x == n_blocks) {
-    gsta_build_order(lengths, cand_offsets, U, N, L, S, Lp, cpb, order, keys);
-    return;
-  }
-  const int D16 = d >> 4, total = M * 6 * D16 * D16 * 32, workers = n_blocks * 256;
-  const int worker = blockIdx.x * 256 + threadIdx.x;
-  for (int i = worker; i < total; i += workers) {
-    const int lane = i & 31;
-    int r = i >> 5;
-    const int p = r % D16; r /= D16;
-    const int kt = r % D16; r /= D16;
-    const bool trans = r & 1;
-    const uint16_t* W = reinterpret_cast<const uint16_t*>(Wg) + (size_t)(r >> 1) * d * d;
-    const int g = lane >> 2, t = lane & 3;
-    uint32_t v[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int n = (2 * p + (q >> 1)) * 8 + g, k = kt * 16 + 2 * t + (q & 1) * 8;
-      const uint32_t lo = trans ? W[(size_t)n * d + k] : W[(size_t)k * d + n];
-      const uint32_t hi = trans ? W[(size_t)n * d + k + 1] : W[(size_t)(k + 1) * d + n];
-      v[q] = lo | (hi << 16);
-    }
-    img[i] = make_uint4(v[0], v[1], v[2], v[3]);
-  }
-  gsta_build_nseg(lengths, cand_offsets, U, N, L, S, Lp, nullptr, nseg, worker >> 5, workers >> 5, threadIdx.x & 31);
+  const int n_blocks = gridDim.x - (P.order ? 1 : 0);
+  if ((int)blockIdx.x == n_blocks) gsta_build_order(P.lengths, P.cand_offsets, P.U, P.N, P.L, P.S, P.Lp, P.cpb, P.order, P.keys, bins);
+  else train_prep_share(P, blockIdx.x * 256 + threadIdx.x, n_blocks * 256);
 }
 
 // x -> (high, low) bf16 pairs of two floats
@@ -855,20 +830,19 @@ TrainScratch carve_train(const Plan& p, int np, char* base) {
   return s;
 }
 
+// 8 candidates per block (one per warp) while all blocks still run at once, two per SM
+int train_cpb(const Plan& p) { return (p.N + 7) / 8 <= 2 * device_sms() ? 8 : kTRows; }
+
 template <int D16, int NP>
-int launch_train(TrainParams P, const Plan& p, const TrainScratch& s, const void* Wg, const int32_t* lengths,
-                 const int32_t* cand_offsets, cudaStream_t st) {
-  const int sms = device_sms();
-  // 8 candidates per block (one per warp) while all blocks still run at once, two per SM
-  P.cpb = (p.N + 7) / 8 <= 2 * sms ? 8 : kTRows;
+int launch_train(TrainParams P, const TrainPrep& prep, const Plan& p, bool prepared, cudaStream_t st) {
+  P.cpb = prep.cpb;
+  P.order = prep.order;
   const int blocks = (p.N + P.cpb - 1) / P.cpb;
-  P.order = blocks > 2 * sms ? s.order : nullptr;
-  {
+  if (!prepared) {
     const int total = p.M * 6 * D16 * D16 * 32;
     LaunchScope ls("gsta_train_prep", st);
-    LASER_CUDA_OK(launch_chained(train_prep_kernel, dim3(std::min((total + 255) / 256, 4 * sms) + (P.order ? 1 : 0)), dim3(256), 0,
-                                 st, (const bf16*)Wg, s.img, p.d, p.M, lengths, cand_offsets, p.U, p.N, p.L, p.S, p.Lp, P.cpb,
-                                 s.nseg, P.order ? s.order : nullptr, s.keys));
+    LASER_CUDA_OK(launch_chained(train_prep_kernel, dim3(std::min((total + 255) / 256, 4 * device_sms()) + (prep.order ? 1 : 0)), dim3(256),
+                                 0, st, prep));
   }
   const size_t smem = TrainSmem<D16, NP>::bytes(p.H, P.nb);
   LASER_CUDA_OK(allow_smem(gsta_train_kernel<D16, NP>, smem));
@@ -946,10 +920,22 @@ size_t gsta_train_scratch_bytes(const Plan& p, int np) { return gsta_train_suppo
     default: return LASER_ERR_UNSUPPORTED; \
   }
 
+TrainPrep gsta_train_prep(const Plan& p, int np, const void* Wg, const int32_t* lengths, const int32_t* cand_offsets, char* scratch) {
+  const TrainScratch s = carve_train(p, np, scratch);
+  TrainPrep P;
+  P.Wg = (const bf16*)Wg; P.img = s.img; P.lengths = lengths; P.cand_offsets = cand_offsets;
+  P.d = p.d; P.M = p.M; P.U = p.U; P.N = p.N; P.L = p.L; P.S = p.S; P.Lp = p.Lp; P.cpb = train_cpb(p);
+  P.nseg = s.nseg;
+  P.order = (p.N + P.cpb - 1) / P.cpb > 2 * device_sms() ? s.order : nullptr;
+  P.keys = s.keys;
+  return P;
+}
+
 int gsta_train(const Plan& p, int np, const void* S0, const void* S1, const int32_t* lengths, const int32_t* cand_offsets,
                const void* cands, const void* Wg, const float* dz, const GstaPlanes& G, float* dS32, __nv_bfloat16* dS16, char* scratch,
-               cudaStream_t st) {
+               cudaStream_t st, bool prepared) {
   const TrainScratch s = carve_train(p, np, scratch);
+  const TrainPrep prep = gsta_train_prep(p, np, Wg, lengths, cand_offsets, scratch);
   TrainParams P = {};
   P.N = p.N; P.U = p.U; P.L = p.L; P.S = p.S; P.Lp = p.Lp; P.H = p.H; P.M = p.M; P.slots = 2 * p.M * p.H; P.nb = train_buffers(p, np);
   P.kb = std::min(P.nb, train_slot_steps(p));
@@ -957,7 +943,7 @@ int gsta_train(const Plan& p, int np, const void* S0, const void* S1, const int3
   P.S0 = (const bf16*)S0; P.S1 = (const bf16*)S1; P.cands = (const bf16*)cands; P.dz = dz;
   P.img = s.img; P.nseg = s.nseg; P.G = G; P.stat = s.stat; P.rows0 = s.rows0; P.rows1 = s.rows1; P.ad16 = s.ad16; P.ad32 = s.ad32;
   P.dS16 = dS16; P.dS32 = dS32;
-#define LASER_TRAIN_CALL(D) (np == 1 ? launch_train<D, 1>(P, p, s, Wg, lengths, cand_offsets, st) : launch_train<D, 2>(P, p, s, Wg, lengths, cand_offsets, st))
+#define LASER_TRAIN_CALL(D) (np == 1 ? launch_train<D, 1>(P, prep, p, prepared, st) : launch_train<D, 2>(P, prep, p, prepared, st))
   LASER_TRAIN_DISPATCH(LASER_TRAIN_CALL)
 #undef LASER_TRAIN_CALL
 }

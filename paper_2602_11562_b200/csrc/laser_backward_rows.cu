@@ -1,13 +1,13 @@
 // The dense products of the backward pass over the item rows (bf16 inputs, warp-level MMAs), in two kernels that touch only
 // the users' valid rows:
 //
-//   rows_project_kernel   Y = scale X [W_a | W_b] as bf16: K and V of the recomputed forward (X read once for both), or Q
+//   rows_project_kernel   Y = scale X [W_a | W_b] as bf16: K and V of the recomputed forward (X read once for both), and Q
 //   rows_grad_kernel      d_items = dK W_k^T + dV W_v^T (zero rows for padding), dW_k += X^T dK, dW_v += X^T dV, all from one
-//                         read of X, dK and dV; or d_cands = dt_0 + dQ W_q^T, dW_q += T^T dQ (16384 candidates: 37 us as two
+//                         read of X, dK and dV; and d_cands = dt_0 + dQ W_q^T, dW_q += T^T dQ (16384 candidates: 37 us as two
 //                         products on the FP32 ALUs)
 //
 // dK and dV arrive as bf16 high and low parts (16 bits; TF32 operands, 11 bits, before), so every operand tile is copied to
-// shared memory as it is and read with ldmatrix; the weights stay in shared memory for the block's lifetime, the weight
+// shared memory as it is and read with ldmatrix; dQ, summed in fp32, is split on its way into shared memory; the weights stay in shared memory for the block's lifetime, the weight
 // gradients in its registers until one atomic add per element at the end.
 // Bound by HBM: 0.64 and 1.5 KB per valid row at d = 128, d_qk = 64.  Six kernels over all rows, padding included, and two
 // memsets before: 470 us at 64 users of 512 .. 4096 of 4096 rows.
@@ -15,6 +15,7 @@
 
 #include "laser_backward.cuh"
 #include "laser_common.cuh"
+#include "laser_gsta_img.cuh"
 #include "laser_mma.cuh"
 
 namespace laser {
@@ -37,9 +38,31 @@ struct RowsParams {
   float scale;
   // gradients
   const bf16 *Ahi, *Alo, *Bhi, *Blo;                 // dK [.., na], dV [.., nb]: high and low parts
+  const float* A32;                                  // not null: the gradient [.., na] in fp32 instead, times scale (nb = 0)
   const float* add;                                  // not null: dX = add + the products
   float *dX, *dWa, *dWb;
 };
+
+// The items and the candidates in one launch: blocks first[r] .. first[r] + blocks[r] - 1 work on r.  A grid that fills the GPU takes
+// one after the other (both ranges are all blocks); where each has few tiles they run beside one another.
+struct RowsPair {
+  RowsParams r[2];
+  int first[2], blocks[2];
+};
+RowsPair pair_up(const RowsParams& items, const RowsParams& cands, long long most, unsigned* grid) {
+  RowsPair P;
+  P.r[0] = items;
+  P.r[1] = cands;
+  long long jobs[2];
+  for (int r = 0; r < 2; ++r) jobs[r] = (long long)P.r[r].groups * P.r[r].tiles_per_group;
+  const bool apart = jobs[0] + jobs[1] <= most;
+  for (int r = 0; r < 2; ++r) {
+    P.blocks[r] = (int)std::min(jobs[r], most);
+    P.first[r] = apart && r == 1 ? P.blocks[0] : 0;
+  }
+  *grid = apart ? P.blocks[0] + P.blocks[1] : std::max(P.blocks[0], P.blocks[1]);
+  return P;
+}
 
 // Rows of a group that take part (a user without candidates, or with invalid inputs, has none).
 __device__ __forceinline__ int valid_rows(const RowsParams& P, int u) {
@@ -56,20 +79,20 @@ __device__ __forceinline__ void fill_table(const RowsParams& P, int* table, int 
   __syncthreads();
 }
 
-// Tile `tile` of group `u`.  A block takes every gridDim.x-th one, groups fastest: the tiles that only long users have come
+// Tile `tile` of group `u`.  Block `block` of `blocks` takes every blocks-th one, groups fastest: the tiles that only long users have come
 // last, spread over the blocks.  (A cursor instead of a tile number: divisions were a third of the gradient kernel's instructions.)
 struct RowTile { int tile, u; };
 struct RowWalk {
   const RowsParams& P;
   const int* table;
-  int dt, du;
-  __device__ __forceinline__ RowWalk(const RowsParams& params, const int* t) : P(params), table(t) {
-    dt = gridDim.x / P.groups;
-    du = gridDim.x - dt * P.groups;
+  int dt, du, block;
+  __device__ __forceinline__ RowWalk(const RowsParams& params, const int* t, int b, int blocks) : P(params), table(t), block(b) {
+    dt = blocks / P.groups;
+    du = blocks - dt * P.groups;
   }
   __device__ __forceinline__ RowTile first() const {
-    const int tile = blockIdx.x / P.groups;
-    return {tile, (int)blockIdx.x - tile * P.groups};
+    const int tile = block / P.groups;
+    return {tile, block - tile * P.groups};
   }
   __device__ __forceinline__ bool in(RowTile c) const { return c.tile < P.tiles_per_group; }
   __device__ __forceinline__ RowTile step(RowTile c) const {
@@ -91,12 +114,8 @@ struct RowWalk {
 };
 
 template <int D16>
-__global__ void __launch_bounds__(kRThreads, 2) rows_project_kernel(const RowsParams P) {
+__device__ __forceinline__ void project_rows(const RowsParams& P, int block, int blocks, uint8_t* smem, int* table) {
   constexpr int d = 16 * D16, XS = 2 * d + 16;
-  extern __shared__ __align__(128) uint8_t smem[];
-  __shared__ int table[kTableGroups];
-  chain_wait();
-  chain_release();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
   const int n = P.na + P.nb, WS = 2 * n + 16;                        // bytes per row of [W_a | W_b] and of the output tile
   uint8_t* Ws = smem;                                                // [d][WS]
@@ -107,7 +126,7 @@ __global__ void __launch_bounds__(kRThreads, 2) rows_project_kernel(const RowsPa
     cp16(smem_addr(Ws) + k * WS + c * 2, c < P.na ? P.Wa + (size_t)k * P.na + c : P.Wb + (size_t)k * P.nb + c - P.na, 16u);
   }
   fill_table(P, table, tid);
-  const RowWalk walk(P, table);
+  const RowWalk walk(P, table, block, blocks);
   auto stage = [&](RowTile j, int b) {
     const int rows = walk.rows(j);
     const bf16* src = P.X + walk.row0(j) * d;
@@ -178,15 +197,44 @@ __global__ void __launch_bounds__(kRThreads, 2) rows_project_kernel(const RowsPa
   cp_wait<0>();
 }
 
+// The set-up of the backward pass of candidate lists in one launch: both projections, the arrays that are summed into set to zero
+// (the status word among them), and in `prep_blocks` blocks of their own what the stacked attention wants (one more sorts its blocks).
+// Four launches and a memset before: the small batches are bound by their number.
+struct ProjectParams {
+  RowsPair rows;
+  ZeroList zero;
+  TrainPrep prep;
+  int row_blocks, prep_blocks;
+};
 template <int D16>
-__global__ void __launch_bounds__(kRThreads) rows_grad_kernel(const RowsParams P, int nbuf) {
-  constexpr int d = 16 * D16, XS = 2 * d + 16;
-  // a warp's share of the weight gradients: kM tiles of 16 features, column pairs wpart, wpart + kParts, ...
-  constexpr int kM = D16 % 2 == 0 ? 2 : 1, kParts = 16 * kM / D16, kMaxPairs = (16 + kParts - 1) / kParts;
+__global__ void __launch_bounds__(kRThreads, 2) rows_project_kernel(const __grid_constant__ ProjectParams P) {
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ int table[kTableGroups];
   chain_wait();
   chain_release();
+  const int block = blockIdx.x, tid = threadIdx.x;
+  zero_share(P.zero, (unsigned long long)block * kRThreads + tid, (unsigned long long)gridDim.x * kRThreads);
+  if (block >= P.row_blocks) {
+    const int b = block - P.row_blocks;
+    if (b < P.prep_blocks) train_prep_share(P.prep, b * kRThreads + tid, P.prep_blocks * kRThreads);
+    else gsta_build_order(P.prep.lengths, P.prep.cand_offsets, P.prep.U, P.prep.N, P.prep.L, P.prep.S, P.prep.Lp, P.prep.cpb,
+                          P.prep.order, P.prep.keys, reinterpret_cast<int*>(smem));
+    return;
+  }
+#pragma unroll 1
+  for (int r = 0; r < 2; ++r) {
+    const int b = block - P.rows.first[r];
+    if (b < 0 || b >= P.rows.blocks[r]) continue;
+    project_rows<D16>(P.rows.r[r], b, P.rows.blocks[r], smem, table);
+    __syncthreads();                       // (the next rows' weights and tiles replace these)
+  }
+}
+
+template <int D16>
+__device__ __forceinline__ void row_gradients(const RowsParams& P, int block, int blocks, int nbuf, uint8_t* smem, int* table) {
+  constexpr int d = 16 * D16, XS = 2 * d + 16;
+  // a warp's share of the weight gradients: kM tiles of 16 features, column pairs wpart, wpart + kParts, ...
+  constexpr int kM = D16 % 2 == 0 ? 2 : 1, kParts = 16 * kM / D16, kMaxPairs = (16 + kParts - 1) / kParts;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
   const int n = P.na + P.nb, WS = 2 * n + 16, pairs = n >> 4;
   uint8_t* Ws = smem;                                                // [d][WS]  [W_k | W_v]
@@ -197,7 +245,7 @@ __global__ void __launch_bounds__(kRThreads) rows_grad_kernel(const RowsParams P
     cp16(smem_addr(Ws) + k * WS + c * 2, c < P.na ? P.Wa + (size_t)k * P.na + c : P.Wb + (size_t)k * P.nb + c - P.na, 16u);
   }
   fill_table(P, table, tid);
-  const RowWalk walk(P, table);
+  const RowWalk walk(P, table, block, blocks);
   const int g_c = lane * 8, g_ld = g_c < P.na ? P.na : P.nb;                 // this lane's 8 columns of [dK | dV]
   const bf16 *g_hi = g_c < P.na ? P.Ahi + g_c : P.Bhi + g_c - P.na, *g_lo = g_c < P.na ? P.Alo + g_c : P.Blo + g_c - P.na;
   auto stage = [&](RowTile j, int b) {
@@ -208,7 +256,19 @@ __global__ void __launch_bounds__(kRThreads) rows_grad_kernel(const RowsParams P
       const int r = i / (2 * D16), q = i - r * (2 * D16);
       cp16(smem_addr(Xs) + b * kRT * XS + r * XS + q * 16, r < rows ? x + r * d + q * 8 : P.X, r < rows ? 16u : 0u);
     }
-    if (g_c < n) {                                                   // a warp per row, 8 columns per lane
+    if (P.A32) {                                                     // fp32: split into its parts on the way
+      for (int i = tid; i < kRT * (n / 4); i += kRThreads) {
+        const int r = i / (n / 4), q = i - r * (n / 4);
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (r < rows) v = *reinterpret_cast<const float4*>(P.A32 + (row0 + r) * n + q * 4);
+        v.x *= P.scale; v.y *= P.scale; v.z *= P.scale; v.w *= P.scale;
+        const uint32_t h0 = pack2(v.x, v.y), h1 = pack2(v.z, v.w);
+        uint8_t* at = Gs + (size_t)b * 2 * kRT * WS + r * WS + q * 8;
+        *reinterpret_cast<uint2*>(at) = make_uint2(h0, h1);
+        *reinterpret_cast<uint2*>(at + kRT * WS) =
+            make_uint2(pack2(v.x - bf16_lo(h0), v.y - bf16_hi(h0)), pack2(v.z - bf16_lo(h1), v.w - bf16_hi(h1)));
+      }
+    } else if (g_c < n) {                                            // a warp per row, 8 columns per lane
       const bf16 *hi = g_hi + row0 * g_ld, *lo = g_lo + row0 * g_ld;
       uint32_t dst = smem_addr(Gs) + b * 2 * kRT * WS + warp * WS + g_c * 2;
 #pragma unroll
@@ -360,16 +420,18 @@ __global__ void __launch_bounds__(kRThreads) rows_grad_kernel(const RowsParams P
     }
 }
 
-// hi + lo = scale * src, 4 values per thread and step
-__global__ void __launch_bounds__(256) split_rows_kernel(const float4* src, uint2* hi, uint2* lo, size_t n4, float scale) {
+template <int D16>
+__global__ void __launch_bounds__(kRThreads) rows_grad_kernel(const __grid_constant__ RowsPair P, int nbuf0, int nbuf1) {
+  extern __shared__ __align__(128) uint8_t smem[];
+  __shared__ int table[kTableGroups];
   chain_wait();
   chain_release();
-  for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < n4; i += (size_t)gridDim.x * 256) {
-    float4 v = src[i];
-    v.x *= scale; v.y *= scale; v.z *= scale; v.w *= scale;
-    const uint32_t a = pack2(v.x, v.y), b = pack2(v.z, v.w);
-    hi[i] = make_uint2(a, b);
-    lo[i] = make_uint2(pack2(v.x - bf16_lo(a), v.y - bf16_hi(a)), pack2(v.z - bf16_lo(b), v.w - bf16_hi(b)));
+#pragma unroll 1
+  for (int r = 0; r < 2; ++r) {
+    const int b = (int)blockIdx.x - P.first[r];
+    if (b < 0 || b >= P.blocks[r]) continue;
+    row_gradients<D16>(P.r[r], b, P.blocks[r], r ? nbuf1 : nbuf0, smem, table);
+    __syncthreads();                       // (the next rows' weights and tiles replace these)
   }
 }
 
@@ -379,39 +441,53 @@ size_t grad_smem(int d, int n, int nbuf) {
 }
 constexpr size_t kRowsSmemMax = 226 * 1024;
 
+struct ProjectJob {
+  RowsParams items, cands;
+  ZeroList zero;
+  TrainPrep prep;
+};
 template <int D16>
-int launch_project(const RowsParams& P, cudaStream_t st) {
-  const size_t smem = project_smem(16 * D16, P.na + P.nb);
+int launch_project(const ProjectJob& J, cudaStream_t st) {
+  const size_t smem = project_smem(16 * D16, std::max(J.items.na + J.items.nb, J.cands.na));
   LASER_CUDA_OK(allow_smem(rows_project_kernel<D16>, smem));
-  const long long jobs = (long long)P.groups * P.tiles_per_group;
-  const int per_sm = smem <= 112 * 1024 ? 2 : 1;
+  const int per_sm = smem <= 112 * 1024 ? 2 : 1, sms = device_sms();
+  ProjectParams P;
+  unsigned grid;
+  P.rows = pair_up(J.items, J.cands, (long long)per_sm * sms, &grid);
+  P.zero = J.zero;
+  P.prep = J.prep;
+  P.row_blocks = (int)grid;
+  P.prep_blocks = std::min((J.prep.M * 6 * D16 * D16 * 32 + kRThreads - 1) / kRThreads, sms);
   LaunchScope ls("bwd_rows_project", st);
-  LASER_CUDA_OK(launch_chained(rows_project_kernel<D16>, dim3((unsigned)std::min<long long>(jobs, (long long)per_sm * device_sms())),
-                               dim3(kRThreads), smem, st, P));
+  LASER_CUDA_OK(launch_chained(rows_project_kernel<D16>, dim3(grid + P.prep_blocks + (J.prep.order ? 1 : 0)), dim3(kRThreads), smem, st, P));
   return LASER_OK;
 }
+struct GradJob {
+  RowsParams items, cands;
+};
 template <int D16>
-int launch_grad(const RowsParams& P, cudaStream_t st) {
-  const int n = P.na + P.nb, nbuf = grad_smem(16 * D16, n, 2) <= kRowsSmemMax ? 2 : 1;
-  const size_t smem = grad_smem(16 * D16, n, nbuf);
+int launch_grad(const GradJob& J, cudaStream_t st) {
+  const int n0 = J.items.na + J.items.nb, n1 = J.cands.na;
+  auto buffers = [](int n) { return grad_smem(16 * D16, n, 2) <= kRowsSmemMax ? 2 : 1; };
+  const size_t smem = std::max(grad_smem(16 * D16, n0, buffers(n0)), grad_smem(16 * D16, n1, buffers(n1)));
   LASER_CUDA_OK(allow_smem(rows_grad_kernel<D16>, smem));
-  const long long jobs = (long long)P.groups * P.tiles_per_group;
+  unsigned grid;
+  const RowsPair P = pair_up(J.items, J.cands, device_sms(), &grid);
   LaunchScope ls("bwd_rows_grad", st);
-  LASER_CUDA_OK(launch_chained(rows_grad_kernel<D16>, dim3((unsigned)std::min<long long>(jobs, device_sms())), dim3(kRThreads), smem, st,
-                               P, nbuf));
+  LASER_CUDA_OK(launch_chained(rows_grad_kernel<D16>, dim3(grid), dim3(kRThreads), smem, st, P, buffers(n0), buffers(n1)));
   return LASER_OK;
 }
 
 #define LASER_ROWS_DISPATCH(fn)               \
   switch (p.d / 16) {                         \
-    case 1: return fn<1>(P, st);              \
-    case 2: return fn<2>(P, st);              \
-    case 3: return fn<3>(P, st);              \
-    case 4: return fn<4>(P, st);              \
-    case 5: return fn<5>(P, st);              \
-    case 6: return fn<6>(P, st);              \
-    case 7: return fn<7>(P, st);              \
-    case 8: return fn<8>(P, st);              \
+    case 1: return fn<1>(J, st);              \
+    case 2: return fn<2>(J, st);              \
+    case 3: return fn<3>(J, st);              \
+    case 4: return fn<4>(J, st);              \
+    case 5: return fn<5>(J, st);              \
+    case 6: return fn<6>(J, st);              \
+    case 7: return fn<7>(J, st);              \
+    case 8: return fn<8>(J, st);              \
     default: return LASER_ERR_UNSUPPORTED;    \
   }
 
@@ -422,44 +498,44 @@ bool rows_mma_supported(const Plan& p) {
          grad_smem(p.d, p.dqk + p.d, 1) <= kRowsSmemMax && (long long)p.U * ((p.L + kRT - 1) / kRT) < (1ll << 30);
 }
 
-int rows_project_items(const Plan& p, const void* items, const int32_t* lengths, const int32_t* cand_offsets, const void* Wk,
-                       const void* Wv, __nv_bfloat16* Kb, __nv_bfloat16* Vb, cudaStream_t st) {
+static RowsParams item_rows(const Plan& p, const void* items, const int32_t* lengths, const int32_t* cand_offsets, const void* Wk,
+                            const void* Wv) {
   RowsParams P = {};
   P.groups = p.U; P.rows_per_group = p.L; P.tiles_per_group = (p.L + kRT - 1) / kRT; P.na = p.dqk; P.nb = p.d;
   P.X = (const bf16*)items; P.Wa = (const bf16*)Wk; P.Wb = (const bf16*)Wv; P.lengths = lengths; P.cand_offsets = cand_offsets;
-  P.N = p.N; P.Ya = Kb; P.Yb = Vb; P.scale = 1.f;
+  P.N = p.N; P.scale = 1.f;
+  return P;
+}
+static RowsParams cand_rows(const Plan& p, const void* cands, const void* Wq, float scale) {
+  RowsParams P = {};
+  P.groups = 1; P.rows_per_group = p.N; P.tiles_per_group = (p.N + kRT - 1) / kRT; P.na = p.dqk;
+  P.X = (const bf16*)cands; P.Wa = P.Wb = (const bf16*)Wq; P.N = p.N; P.scale = scale;
+  return P;
+}
+
+int rows_project(const Plan& p, const void* items, const int32_t* lengths, const void* cands, const int32_t* cand_offsets, const void* Wq,
+                 const void* Wk, const void* Wv, float q_scale, __nv_bfloat16* Qb, __nv_bfloat16* Kb, __nv_bfloat16* Vb,
+                 const ZeroList& zero, const TrainPrep& prep, cudaStream_t st) {
+  ProjectJob J;
+  J.items = item_rows(p, items, lengths, cand_offsets, Wk, Wv);
+  J.items.Ya = Kb; J.items.Yb = Vb;
+  J.cands = cand_rows(p, cands, Wq, q_scale);
+  J.cands.Ya = Qb;
+  J.zero = zero;
+  J.prep = prep;
   LASER_ROWS_DISPATCH(launch_project)
 }
 
-int rows_project_cands(const Plan& p, const void* cands, const void* Wq, float scale, __nv_bfloat16* Qb, cudaStream_t st) {
-  RowsParams P = {};
-  P.groups = 1; P.rows_per_group = p.N; P.tiles_per_group = (p.N + kRT - 1) / kRT; P.na = p.dqk;
-  P.X = (const bf16*)cands; P.Wa = P.Wb = (const bf16*)Wq; P.N = p.N; P.Ya = Qb; P.scale = scale;
-  LASER_ROWS_DISPATCH(launch_project)
-}
-
-int rows_gradients(const Plan& p, const void* items, const int32_t* lengths, const int32_t* cand_offsets, const void* Wk,
-                   const void* Wv, const __nv_bfloat16* dK_hi, const __nv_bfloat16* dK_lo, const __nv_bfloat16* dV_hi,
-                   const __nv_bfloat16* dV_lo, float* d_items, float* dWk, float* dWv, cudaStream_t st) {
-  RowsParams P = {};
-  P.groups = p.U; P.rows_per_group = p.L; P.tiles_per_group = (p.L + kRT - 1) / kRT; P.na = p.dqk; P.nb = p.d;
-  P.X = (const bf16*)items; P.Wa = (const bf16*)Wk; P.Wb = (const bf16*)Wv; P.lengths = lengths; P.cand_offsets = cand_offsets;
-  P.N = p.N; P.Ahi = dK_hi; P.Alo = dK_lo; P.Bhi = dV_hi; P.Blo = dV_lo; P.dX = d_items; P.dWa = dWk; P.dWb = dWv;
-  LASER_ROWS_DISPATCH(launch_grad)
-}
-
-int rows_gradients_cands(const Plan& p, const void* cands, const void* Wq, const float* dQf, __nv_bfloat16* hi, __nv_bfloat16* lo,
-                         const float* dT0, float* d_cands, float* dWq, cudaStream_t st) {
-  {
-    const size_t n4 = (size_t)p.N * p.dqk / 4;
-    LaunchScope ls("bwd_split_rows", st);
-    LASER_CUDA_OK(launch_chained(split_rows_kernel, dim3((unsigned)std::min<size_t>((n4 + 255) / 256, 4 * device_sms())), dim3(256), 0,
-                                 st, (const float4*)dQf, (uint2*)hi, (uint2*)lo, n4, p.inv_gamma));
-  }
-  RowsParams P = {};
-  P.groups = 1; P.rows_per_group = p.N; P.tiles_per_group = (p.N + kRT - 1) / kRT; P.na = p.dqk;
-  P.X = (const bf16*)cands; P.Wa = P.Wb = (const bf16*)Wq; P.N = p.N; P.Ahi = P.Bhi = hi; P.Alo = P.Blo = lo;
-  P.add = dT0; P.dX = d_cands; P.dWa = P.dWb = dWq;
+int rows_gradients(const Plan& p, const void* items, const int32_t* lengths, const void* cands, const int32_t* cand_offsets, const void* Wq,
+                   const void* Wk, const void* Wv, const float* dQf, const __nv_bfloat16* dK_hi, const __nv_bfloat16* dK_lo,
+                   const __nv_bfloat16* dV_hi, const __nv_bfloat16* dV_lo, const float* dT0, float* d_items, float* d_cands, float* dWq,
+                   float* dWk, float* dWv, cudaStream_t st) {
+  GradJob J;
+  J.items = item_rows(p, items, lengths, cand_offsets, Wk, Wv);
+  J.items.Ahi = dK_hi; J.items.Alo = dK_lo; J.items.Bhi = dV_hi; J.items.Blo = dV_lo;
+  J.items.dX = d_items; J.items.dWa = dWk; J.items.dWb = dWv;
+  J.cands = cand_rows(p, cands, Wq, p.inv_gamma);
+  J.cands.A32 = dQf; J.cands.add = dT0; J.cands.dX = d_cands; J.cands.dWa = J.cands.dWb = dWq;
   LASER_ROWS_DISPATCH(launch_grad)
 }
 

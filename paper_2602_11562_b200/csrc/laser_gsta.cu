@@ -52,7 +52,8 @@ __global__ void __launch_bounds__(256) gsta_prep_kernel(GstaParams P) {
   chain_release();
   const int n_blocks = gridDim.x - (P.build_order ? 1 : 0);          // blocks that build images and segment counts
   if ((int)blockIdx.x == n_blocks) {
-    gsta_build_order(P.lengths, P.cand_offsets, P.U, P.N, P.L, P.S, P.Lp, P.cpb, P.order, P.order_keys);
+    __shared__ int bins[kGstaSortWords];
+    gsta_build_order(P.lengths, P.cand_offsets, P.U, P.N, P.L, P.S, P.Lp, P.cpb, P.order, P.order_keys, bins);
     return;
   }
   gsta_build_images(P.Wg, P.img, P.d, P.M, blockIdx.x * blockDim.x + threadIdx.x, n_blocks * blockDim.x);

@@ -63,13 +63,13 @@ __device__ __forceinline__ void gsta_build_nseg(const int* lengths, const int* c
 
 // Counting sort, largest key first: order[0 .. n - 1] = the indices 0 .. n - 1 by descending key(i) (keys in
 // 0 .. kGstaOrderBins - 1; equal keys land in arbitrary order).  Run by ONE thread block (all of its threads call this, at
-// least one warp); keys: n ints of scratch.
+// least one warp); keys: n ints of scratch; bins: kGstaSortWords words of shared memory.
 constexpr int kGstaOrderBins = 1024;
+constexpr int kGstaSortWords = kGstaOrderBins + kGstaOrderBins / 32;      // bin k at k + k / 32: lane-strided walks stay conflict-free
 template <class KeyFn>
-__device__ __forceinline__ void sort_desc_by_key(int n, KeyFn key_of, int* order, int* keys) {
-  __shared__ int bins[kGstaOrderBins + kGstaOrderBins / 32];      // bin k at k + k / 32: lane-strided walks stay conflict-free
+__device__ __forceinline__ void sort_desc_by_key(int n, KeyFn key_of, int* order, int* keys, int* bins) {
   const int tid = threadIdx.x, nt = blockDim.x;
-  for (int i = tid; i < kGstaOrderBins + kGstaOrderBins / 32; i += nt) bins[i] = 0;
+  for (int i = tid; i < kGstaSortWords; i += nt) bins[i] = 0;
   __syncthreads();
   constexpr int kBatch = 8;                      // independent loads first, then the atomics: the passes are latency-bound
   for (int b0 = tid; b0 < n; b0 += kBatch * nt) {
@@ -122,7 +122,7 @@ __device__ __forceinline__ void sort_desc_by_key(int n, KeyFn key_of, int* order
 // or offsets are reported elsewhere; here they are clamped, so `order` is a permutation of 0 .. n_blocks - 1 whatever
 // the inputs hold.
 __device__ __forceinline__ void gsta_build_order(const int* lengths, const int* cand_offsets, int U, int N, int L, int S,
-                                                 int Lp, int cpb, int* order, int* keys) {
+                                                 int Lp, int cpb, int* order, int* keys, int* bins) {
   const int n_blocks = (N + cpb - 1) / cpb;
   sort_desc_by_key(n_blocks, [&](int b) {
     const int c = b * cpb;
@@ -133,7 +133,40 @@ __device__ __forceinline__ void gsta_build_order(const int* lengths, const int* 
     }
     const int len = min(max(lengths[lo], 0), L);
     return min((len + S - 1) / S, Lp);
-  }, order, keys);
+  }, order, keys, bins);
+}
+
+// What the backward pass's stacked attention wants before it starts: every matrix in fragment order as stored (B[k][n] = W[k][n]) and
+// transposed, the segment counts, and (order not null) the launch order of its blocks.
+struct TrainPrep {
+  const __nv_bfloat16* Wg;
+  uint4* img;                                     // [M][3][2][d/16][d/16][32]
+  const int *lengths, *cand_offsets;
+  int d, M, U, N, L, S, Lp, cpb;
+  int *nseg, *order, *keys;
+};
+// Called by whole warps with ranks worker = 0 .. workers - 1; the order is built by a block of its own (gsta_build_order).
+__device__ __forceinline__ void train_prep_share(const TrainPrep& P, int worker, int workers) {
+  const int D16 = P.d >> 4, total = P.M * 6 * D16 * D16 * 32, d = P.d;
+  for (int i = worker; i < total; i += workers) {
+    const int lane = i & 31;
+    int r = i >> 5;
+    const int p = r % D16; r /= D16;
+    const int kt = r % D16; r /= D16;
+    const bool trans = r & 1;
+    const uint16_t* W = reinterpret_cast<const uint16_t*>(P.Wg) + (size_t)(r >> 1) * d * d;
+    const int g = lane >> 2, t = lane & 3;
+    uint32_t v[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int n = (2 * p + (q >> 1)) * 8 + g, k = kt * 16 + 2 * t + (q & 1) * 8;
+      const uint32_t lo = trans ? W[(size_t)n * d + k] : W[(size_t)k * d + n];
+      const uint32_t hi = trans ? W[(size_t)n * d + k + 1] : W[(size_t)(k + 1) * d + n];
+      v[q] = lo | (hi << 16);
+    }
+    P.img[i] = make_uint4(v[0], v[1], v[2], v[3]);
+  }
+  gsta_build_nseg(P.lengths, P.cand_offsets, P.U, P.N, P.L, P.S, P.Lp, nullptr, P.nseg, worker >> 5, workers >> 5, threadIdx.x & 31);
 }
 
 }  // namespace laser

@@ -81,8 +81,9 @@ __global__ void __launch_bounds__(kPreWarps * 32) stream_pre_kernel(StreamParams
     // the last block sorts the users by length, longest first: the attention kernel's grid runs in several waves of
     // blocks whose time is proportional to the user's length, and its last wave should be made of the shortest
     const float per_row = (float)(kGstaOrderBins - 1) / (float)P.L;
+    __shared__ int bins[kGstaSortWords];
     sort_desc_by_key(P.U, [&](int u) { return (int)((float)min(max(P.lengths[u], 0), P.L) * per_row); }, P.order,
-                     P.order_keys);
+                     P.order_keys, bins);
     return;
   }
   if (wg >= user_warps) {

@@ -188,7 +188,8 @@ __global__ void __launch_bounds__(1024) tc_prep_kernel(TcParams P) {
     return;
   }
   if (P.gorder && blockIdx.x == gridDim.x - 1) {   // one extra block when the GSTA kernel wants its blocks sorted
-    gsta_build_order(P.lengths, P.cand_offsets, P.U, P.N, P.L, P.S, P.Lp, P.gcpb, P.gorder, P.gorder_keys);
+    __shared__ int bins[kGstaSortWords];
+    gsta_build_order(P.lengths, P.cand_offsets, P.U, P.N, P.L, P.S, P.Lp, P.gcpb, P.gorder, P.gorder_keys, bins);
     return;
   }
   // remaining blocks: weight images, grid-stride
