@@ -97,7 +97,7 @@ static int resolve_path(const Plan& p, int requested) {
   }
   if (requested == LASER_PATH_SIMT) return LASER_PATH_SIMT;
   if (requested == LASER_PATH_TENSOR) return tensor_supported(p) ? (int)LASER_PATH_TENSOR : (int)LASER_ERR_UNSUPPORTED;
-  if (requested == LASER_PATH_STREAM) return (p.maxC <= 1 && stream_supported(p)) ? (int)LASER_PATH_STREAM : (int)LASER_ERR_UNSUPPORTED;
+  if (requested == LASER_PATH_STREAM) return (p.maxC <= 1 && stream_supported(p) && stream_in_one_pass(p)) ? (int)LASER_PATH_STREAM : (int)LASER_ERR_UNSUPPORTED;
   return LASER_ERR_INVALID_ARG;
 }
 

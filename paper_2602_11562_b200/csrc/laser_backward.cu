@@ -1096,11 +1096,12 @@ int backward_stream_all(const Plan& p, const T* items, const int32_t* lengths, c
   Z.add(dWq, (size_t)d * dqk); Z.add(dWk, (size_t)d * dqk); Z.add(dWv, (size_t)d * d); Z.add(dWg, (size_t)M * 3 * d * d);
   Z.add(backward_stream_sums(p, stream_scratch), (size_t)N * H * d);
   Z.add(ws + p.off_status, kStatusWords);
-  BWD_OK(zero_arrays(Z, st));
+  const TrainPrep prep = gsta_train_prep(p, 2, Wg, lengths, cand_offsets, train_scratch);
   bf16 *Hhi = reinterpret_cast<bf16*>(s.Hp), *Hlo = Hhi + (size_t)N * p.Lp * d;
-  BWD_OK(backward_stream_forward(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, nullptr, Hhi, Hlo, ws, stream_scratch, st));
+  BWD_OK(backward_stream_forward(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, nullptr, Hhi, Hlo, ws, stream_scratch, st, &Z,
+                                 &prep));
   const GstaPlanes G = train_planes(p, s);
-  BWD_OK(gsta_train(p, 2, Hhi, Hlo, lengths, cand_offsets, cands, Wg, dz, G, s.dHp, nullptr, train_scratch, st, false));
+  BWD_OK(gsta_train(p, 2, Hhi, Hlo, lengths, cand_offsets, cands, Wg, dz, G, s.dHp, nullptr, train_scratch, st, true));
   const float* p_sums = nullptr;
   BWD_OK(backward_stream(p, items, lengths, cand_offsets, Wv, s.dHp, d_items, dWv, &p_sums, ws, stream_scratch, st));
 #undef BWD_OK
@@ -1212,7 +1213,8 @@ int backward_t(const Plan& p, const T* items, const int32_t* lengths, const T* c
   char* train_scratch = mma_scratch + sta_bwd_mma_scratch_bytes(p);
   if (stream) {
     BWD_OK(gemm<T, T>(gx, N, dqk, d, cands, d, false, Wq, dqk, false, Qf, dqk, p.inv_gamma, false, false));
-    BWD_OK(backward_stream_forward(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, s.Hp, nullptr, nullptr, ws, mma_scratch, st));
+    BWD_OK(backward_stream_forward(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, s.Hp, nullptr, nullptr, ws, mma_scratch, st,
+                                   nullptr, nullptr));
   } else if (tensor) {
     // (sta_fwd_mma writes every row of H' that is read later: all candidates of every non-empty segment)
     if (!(mma && sta_fwd_mma_supported(p))) LASER_CUDA_OK(cudaMemsetAsync(s.Hp, 0, (size_t)N * Lp * d * sizeof(float), st));

@@ -745,9 +745,11 @@ size_t backward_stream_scratch_bytes(const Plan& p) { return backward_stream_sup
 
 int backward_stream_forward(const Plan& p, const void* items, const int32_t* lengths, const void* cands,
                             const int32_t* cand_offsets, const void* Wq, const void* Wk, const void* Wv, float* Hp,
-                            __nv_bfloat16* Hp_hi, __nv_bfloat16* Hp_lo, char* ws, char* scratch, cudaStream_t st) {
+                            __nv_bfloat16* Hp_hi, __nv_bfloat16* Hp_lo, char* ws, char* scratch, cudaStream_t st,
+                            const ZeroList* zero, const TrainPrep* prep) {
   const BsScratch s = carve_bs(p, scratch);
-  const int rc = stream_fold(p, lengths, cands, cand_offsets, Wq, Wk, Wv, s.u, s.fold, reinterpret_cast<int*>(ws + p.off_status), st);
+  const int rc = stream_fold(p, lengths, cands, cand_offsets, Wq, Wk, Wv, s.u, s.fold, reinterpret_cast<int*>(ws + p.off_status), st,
+                             zero, prep);
   if (rc != LASER_OK) return rc;
   BsParams P = bs_params(p, s, items, lengths, cand_offsets, Wv, ws);
   P.s = Hp; P.s_hi = Hp_hi; P.s_lo = Hp_lo;

@@ -165,17 +165,21 @@ int gsta_mma(const Plan& p, const void* Hprime, const int32_t* lengths, const in
 
 // One-candidate-per-user STA (laser_stream.cu); needs stream_scratch_bytes(p) of scratch at off_su.  Its GSTA is gsta_mma.
 bool stream_supported(const Plan& p);
+bool stream_in_one_pass(const Plan& p);
 size_t stream_scratch_bytes(const Plan& p);
 int stream_sta(const Plan& p, const void* items, const int32_t* lengths, const void* cands, const int32_t* cand_offsets,
                const void* Wq, const void* Wk, const void* Wv, void* Hprime, char* ws, cudaStream_t st,
                const void* Wg_images);
 
 // u [U, H, d] (fp32) = W_k[:, h] (t W_q)_h / gamma for the candidate of every user (zero rows without one), and the users'
-// launch order, longest first; scratch: stream_fold_bytes(p).
+// launch order, longest first; scratch: stream_fold_bytes(p).  The same launch sets arrays to zero and runs gsta_train's
+// preparation (null: neither).
+struct TrainPrep;
 size_t stream_fold_bytes(const Plan& p);
 const int* stream_fold_order(const Plan& p, const char* scratch);   // null: index order
 int stream_fold(const Plan& p, const int32_t* lengths, const void* cands, const int32_t* cand_offsets, const void* Wq,
-                const void* Wk, const void* Wv, float* u, char* scratch, int* status, cudaStream_t st);
+                const void* Wk, const void* Wv, float* u, char* scratch, int* status, cudaStream_t st, const ZeroList* zero,
+                const TrainPrep* prep);
 
 // Backward pass of batches with at most one candidate per user (laser_backward_stream.cu).  _forward recomputes H' (fp32, or,
 // with Hp null, its bf16 high and low parts; rows of non-empty segments only); the other writes every row of d_items, adds to dWv and leaves
@@ -185,7 +189,8 @@ size_t backward_stream_scratch_bytes(const Plan& p);
 float* backward_stream_sums(const Plan& p, char* scratch);      // p of backward_stream, [N, H, d]: zeroed by the caller
 int backward_stream_forward(const Plan& p, const void* items, const int32_t* lengths, const void* cands,
                             const int32_t* cand_offsets, const void* Wq, const void* Wk, const void* Wv, float* Hp,
-                            __nv_bfloat16* Hp_hi, __nv_bfloat16* Hp_lo, char* ws, char* scratch, cudaStream_t st);
+                            __nv_bfloat16* Hp_hi, __nv_bfloat16* Hp_lo, char* ws, char* scratch, cudaStream_t st,
+                            const ZeroList* zero, const TrainPrep* prep);
 int backward_stream(const Plan& p, const void* items, const int32_t* lengths, const int32_t* cand_offsets, const void* Wv,
                     const float* dHp, float* d_items, float* dWv, const float** p_sums, char* ws, char* scratch,
                     cudaStream_t st);

@@ -20,6 +20,8 @@
 //                        survive the bf16 operands to about 16 bits.  After the item loop the block multiplies all
 //                        its segment sums by W_v (MMA, rows = segments) and writes H'.
 //   GSTA                 the shared fused GSTA kernel (laser_gsta.cu) on that H'.
+#include <algorithm>
+
 #include "laser_common.cuh"
 #include "laser_gsta_img.cuh"
 #include "laser_mma.cuh"
@@ -53,6 +55,9 @@ struct StreamParams {
   int* order;                     // [U] users by descending length (null: blocks take the users in index order)
   int* order_keys;                // [U] scratch of the sort
   int* status;
+  int chunk;                      // segments whose sums the attention kernel holds at a time
+  ZeroList zero;                  // backward pass: arrays that the pre kernel sets to zero, and what the stacked attention wants
+  TrainPrep prep;                 // (img null: not wanted)
 };
 
 // Candidate of user u, or -1 when it has none (or its offsets / length are invalid).
@@ -69,28 +74,35 @@ __device__ __forceinline__ int user_candidate(const StreamParams& P, int u, int*
 }
 
 template <int D16>
-__global__ void __launch_bounds__(kPreWarps * 32) stream_pre_kernel(StreamParams P, int user_warps) {
+__global__ void __launch_bounds__(kPreWarps * 32) stream_pre_kernel(const __grid_constant__ StreamParams P, int user_warps) {
   constexpr int d = D16 * 16;
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  const int wg = blockIdx.x * kPreWarps + (threadIdx.x >> 5);
   const int dqk = P.dqk, H = P.H, dqh = dqk / H;
   chain_wait();
   chain_release();
   if (blockIdx.x == 0 && threadIdx.x == 0) set_status(P.status, 0);   // (the attention kernel checks every user and reports)
-  if (P.order && blockIdx.x == gridDim.x - 1) {
-    // the last block sorts the users by length, longest first: the attention kernel's grid runs in several waves of
+  zero_share(P.zero, (unsigned long long)blockIdx.x * (kPreWarps * 32) + threadIdx.x, (unsigned long long)gridDim.x * (kPreWarps * 32));
+  const int sorts = (P.order ? 1 : 0) + (P.prep.order ? 1 : 0), plain = gridDim.x - sorts;
+  if ((int)blockIdx.x < sorts) {                 // (first: they take longest)
+    __shared__ int bins[kGstaSortWords];
+    if (!P.order || blockIdx.x == 1) {
+      gsta_build_order(P.prep.lengths, P.prep.cand_offsets, P.prep.U, P.prep.N, P.prep.L, P.prep.S, P.prep.Lp, P.prep.cpb, P.prep.order,
+                       P.prep.keys, bins);
+      return;
+    }
+    // one block sorts the users by length, longest first: the attention kernel's grid runs in several waves of
     // blocks whose time is proportional to the user's length, and its last wave should be made of the shortest
     const float per_row = (float)(kGstaOrderBins - 1) / (float)P.L;
-    __shared__ int bins[kGstaSortWords];
     sort_desc_by_key(P.U, [&](int u) { return (int)((float)min(max(P.lengths[u], 0), P.L) * per_row); }, P.order,
                      P.order_keys, bins);
     return;
   }
+  const int wg = ((int)blockIdx.x - sorts) * kPreWarps + (threadIdx.x >> 5);
   if (wg >= user_warps) {
     // spare warps: W_v image, entry (kt, p, lane) = {b0, b1 of column tile 2p, b0, b1 of column tile 2p+1},
     // B[k][n] = W_v[k][n]; and the GSTA weight images when GSTA follows
     const int worker = (wg - user_warps) * 32 + lane;
-    const int n_workers = (((int)gridDim.x - (P.order ? 1 : 0)) * kPreWarps - user_warps) * 32;
+    const int n_workers = (plain * kPreWarps - user_warps) * 32;
     const int total = D16 * D16 * 32;
     const uint16_t* W = reinterpret_cast<const uint16_t*>(P.Wv);
     for (int i = worker; i < total; i += n_workers) {
@@ -105,14 +117,16 @@ __global__ void __launch_bounds__(kPreWarps * 32) stream_pre_kernel(StreamParams
       P.imgv[i] = make_uint4(v[0], v[1], v[2], v[3]);
     }
     if (P.Wg) gsta_build_images(P.Wg, P.gimg, d, P.M, worker, n_workers);
+    if (P.prep.img) train_prep_share(P.prep, worker, n_workers);
     return;
   }
-  // users 16 wg + g (MMA rows g) and 16 wg + g + 8 (rows g + 8); a user without a candidate is a zero row
-  const int uA = wg * 16 + g, uB = uA + 8;
+  // warp = (16 users, head): users 16 ug + g (MMA rows g) and 16 ug + g + 8 (rows g + 8); a user without a candidate is a zero row
+  const int ug = wg / H, h = wg - ug * H;
+  const int uA = ug * 16 + g, uB = uA + 8;
   int lenA = 0, lenB = 0;
   const int cA = uA < P.U ? user_candidate(P, uA, &lenA, false) : -1;
   const int cB = uB < P.U ? user_candidate(P, uB, &lenB, false) : -1;
-  if (P.Wg && t == 0) {                                  // segment counts of these users' candidates for the GSTA kernel
+  if (P.Wg && t == 0 && h == 0) {                                  // segment counts of these users' candidates for the GSTA kernel
     if (cA >= 0) P.gnseg[cA] = min((lenA + P.S - 1) / P.S, P.Lp);
     if (cB >= 0) P.gnseg[cB] = min((lenB + P.S - 1) / P.S, P.Lp);
   }
@@ -126,45 +140,43 @@ __global__ void __launch_bounds__(kPreWarps * 32) stream_pre_kernel(StreamParams
     ta[kt][3] = cB >= 0 ? *reinterpret_cast<const uint32_t*>(P.cands + (size_t)cB * d + k + 8) : 0u;
   }
   const uint16_t* Wq = reinterpret_cast<const uint16_t*>(P.Wq);
-  for (int h = 0; h < H; ++h) {
-    float uacc[2 * D16][4];                              // u_h of the 16 users: (user g | g + 8, features 8 nt + 2t..)
+  float uacc[2 * D16][4];                              // u_h of the 16 users: (user g | g + 8, features 8 nt + 2t..)
 #pragma unroll
-    for (int nt = 0; nt < 2 * D16; ++nt) uacc[nt][0] = uacc[nt][1] = uacc[nt][2] = uacc[nt][3] = 0.f;
-    for (int a0 = h * dqh; a0 < (h + 1) * dqh; a0 += 16) {
-      // 16 columns of q = t W_q / gamma   (Eq. 4 / Eq. 8)
-      float qc[2][4] = {};
+  for (int nt = 0; nt < 2 * D16; ++nt) uacc[nt][0] = uacc[nt][1] = uacc[nt][2] = uacc[nt][3] = 0.f;
+  for (int a0 = h * dqh; a0 < (h + 1) * dqh; a0 += 16) {
+    // 16 columns of q = t W_q / gamma   (Eq. 4 / Eq. 8)
+    float qc[2][4] = {};
 #pragma unroll
-      for (int kt = 0; kt < D16; ++kt) {
+    for (int kt = 0; kt < D16; ++kt) {
 #pragma unroll
-        for (int nt = 0; nt < 2; ++nt) {
-          const uint16_t* w = Wq + (size_t)(kt * 16 + 2 * t) * dqk + a0 + nt * 8 + g;
-          const uint32_t b0 = (uint32_t)w[0] | ((uint32_t)w[dqk] << 16);
-          const uint32_t b1 = (uint32_t)w[8 * dqk] | ((uint32_t)w[9 * dqk] << 16);
-          mma16816(qc[nt], ta[kt][0], ta[kt][1], ta[kt][2], ta[kt][3], b0, b1);
-        }
-      }
-      // the accumulator layout of two 8-column tiles is the A layout of one 16-wide k-tile; high and low bf16 parts
-      uint32_t qh[4], ql[4];
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const float x0 = qc[r >> 1][(r & 1) * 2] * P.inv_gamma, x1 = qc[r >> 1][(r & 1) * 2 + 1] * P.inv_gamma;
-        qh[r] = pack2(x0, x1);
-        ql[r] = pack2(x0 - bf16_lo(qh[r]), x1 - bf16_hi(qh[r]));
-      }
-      // u_h[i] += sum_{a in this chunk} W_k[i][a] q[a]: B[k = a][n = i] = W_k[i][a0 + k]
-#pragma unroll
-      for (int nt = 0; nt < 2 * D16; ++nt) {
-        const bf16* w = P.Wk + (size_t)(nt * 8 + g) * dqk + a0 + 2 * t;
-        const uint32_t b0 = *reinterpret_cast<const uint32_t*>(w), b1 = *reinterpret_cast<const uint32_t*>(w + 8);
-        mma16816(uacc[nt], qh[0], qh[1], qh[2], qh[3], b0, b1);
-        mma16816(uacc[nt], ql[0], ql[1], ql[2], ql[3], b0, b1);
+      for (int nt = 0; nt < 2; ++nt) {
+        const uint16_t* w = Wq + (size_t)(kt * 16 + 2 * t) * dqk + a0 + nt * 8 + g;
+        const uint32_t b0 = (uint32_t)w[0] | ((uint32_t)w[dqk] << 16);
+        const uint32_t b1 = (uint32_t)w[8 * dqk] | ((uint32_t)w[9 * dqk] << 16);
+        mma16816(qc[nt], ta[kt][0], ta[kt][1], ta[kt][2], ta[kt][3], b0, b1);
       }
     }
+    // the accumulator layout of two 8-column tiles is the A layout of one 16-wide k-tile; high and low bf16 parts
+    uint32_t qh[4], ql[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const float x0 = qc[r >> 1][(r & 1) * 2] * P.inv_gamma, x1 = qc[r >> 1][(r & 1) * 2 + 1] * P.inv_gamma;
+      qh[r] = pack2(x0, x1);
+      ql[r] = pack2(x0 - bf16_lo(qh[r]), x1 - bf16_hi(qh[r]));
+    }
+    // u_h[i] += sum_{a in this chunk} W_k[i][a] q[a]: B[k = a][n = i] = W_k[i][a0 + k]
 #pragma unroll
     for (int nt = 0; nt < 2 * D16; ++nt) {
-      if (uA < P.U) *reinterpret_cast<float2*>(P.u + ((size_t)uA * H + h) * d + nt * 8 + 2 * t) = make_float2(uacc[nt][0], uacc[nt][1]);
-      if (uB < P.U) *reinterpret_cast<float2*>(P.u + ((size_t)uB * H + h) * d + nt * 8 + 2 * t) = make_float2(uacc[nt][2], uacc[nt][3]);
+      const bf16* w = P.Wk + (size_t)(nt * 8 + g) * dqk + a0 + 2 * t;
+      const uint32_t b0 = *reinterpret_cast<const uint32_t*>(w), b1 = *reinterpret_cast<const uint32_t*>(w + 8);
+      mma16816(uacc[nt], qh[0], qh[1], qh[2], qh[3], b0, b1);
+      mma16816(uacc[nt], ql[0], ql[1], ql[2], ql[3], b0, b1);
     }
+  }
+#pragma unroll
+  for (int nt = 0; nt < 2 * D16; ++nt) {
+    if (uA < P.U) *reinterpret_cast<float2*>(P.u + ((size_t)uA * H + h) * d + nt * 8 + 2 * t) = make_float2(uacc[nt][0], uacc[nt][1]);
+    if (uB < P.U) *reinterpret_cast<float2*>(P.u + ((size_t)uB * H + h) * d + nt * 8 + 2 * t) = make_float2(uacc[nt][2], uacc[nt][3]);
   }
 }
 
@@ -177,8 +189,9 @@ __device__ __forceinline__ float sigmoid_fast(float x) {
   return r;
 }
 
-template <int D16>
-__global__ void __launch_bounds__(kSThreads) stream_sta_kernel(StreamParams P) {
+// kChunks: more segments than fit in shared memory at a time.
+template <int D16, bool kChunks>
+__global__ void __launch_bounds__(kSThreads) stream_sta_kernel(const __grid_constant__ StreamParams P) {
   constexpr int d = D16 * 16;
   constexpr int RS = 2 * d + 16;                 // bytes per staged row (the padding keeps ldmatrix conflict-free)
   extern __shared__ __align__(128) uint8_t smem[];
@@ -191,10 +204,50 @@ __global__ void __launch_bounds__(kSThreads) stream_sta_kernel(StreamParams P) {
   const int cand = user_candidate(P, u, &len);
   if (cand < 0) return;
   const int nv = (len + P.S - 1) / P.S;          // non-empty segments
-  const int Lp16 = (P.Lp + 15) & ~15;
-  uint8_t* Rhi = smem;                           // [Lp16][H] rows: bf16 high part of r_{i,h}
-  uint8_t* Rlo = Rhi + (size_t)Lp16 * H * RS;    // same shape: bf16 low part
-  uint8_t* ring = Rlo + (size_t)Lp16 * H * RS + (size_t)warp * kSStages * kSRows * RS;
+  const int chunk = P.chunk;                     // segments whose sums are held at a time: all L', or a multiple of 16
+  uint8_t* Rhi = smem;                           // [chunk][H] rows: bf16 high part of r_{i,h}
+  uint8_t* Rlo = Rhi + (size_t)chunk * H * RS;   // same shape: bf16 low part
+  uint8_t* ring = Rlo + (size_t)chunk * H * RS + (size_t)warp * kSStages * kSRows * RS;
+  // (the product with W_v reads segments in sixteens: where all L' are held, up to 15 H <= 120 rows past the end of Rlo lie in the
+  // ring's 256, which nothing writes by then, and what it makes of them is not stored)
+  static_assert(kSW * kSStages * kSRows >= 15 * 8, "rows past the last segment stay inside the block's shared memory");
+
+  // s_i[head h] = r_{i,h} W_v[:, head h] for the segments s0 .. s1 - 1 in shared memory: a warp takes 16 columns (of one head) at a
+  // time, with all of their weights in flight at once, for all segments (a read per k-step and head, each waited for, was most of a
+  // short user's time: 3119 users of 180 items, d = 128, eight heads, segments of nine, 439 -> 220 us)
+  auto product = [&](int s0, int s1) {
+    const uint32_t arow = (lane & 7) + ((lane >> 3) & 1) * 8, akc = lane >> 4;
+    constexpr int kShare = D16 < kSW ? kSW / D16 : 1;      // narrow widths: warps that share 16 columns take every kShare-th sixteen
+    const int mine = D16 < kSW ? warp / D16 : 0;
+    if (mine >= kShare) return;
+    for (int p = D16 < kSW ? warp % D16 : warp; p < D16; p += kSW) {
+      uint4 b[D16];
+#pragma unroll
+      for (int kt = 0; kt < D16; ++kt) b[kt] = __ldg(P.imgv + (kt * D16 + p) * 32 + lane);
+      const int h = p * 16 / dvh;
+      for (int m0 = s0 + 16 * mine; m0 < s1; m0 += 16 * kShare) {
+        float acc[2][4] = {};
+        const size_t o = (size_t)((m0 - s0 + arow) * H + h) * RS + akc * 16;
+#pragma unroll
+        for (int kt = 0; kt < D16; ++kt) {
+          uint32_t ah[4], al[4];
+          ldsm_x4(ah, smem_addr(Rhi + o) + kt * 32);
+          ldsm_x4(al, smem_addr(Rlo + o) + kt * 32);
+          mma16816(acc[0], ah[0], ah[1], ah[2], ah[3], b[kt].x, b[kt].y);
+          mma16816(acc[0], al[0], al[1], al[2], al[3], b[kt].x, b[kt].y);
+          mma16816(acc[1], ah[0], ah[1], ah[2], ah[3], b[kt].z, b[kt].w);
+          mma16816(acc[1], al[0], al[1], al[2], al[3], b[kt].z, b[kt].w);
+        }
+        const int i0 = m0 + g, i1 = i0 + 8;
+        bf16* out = P.Hp + ((size_t)cand * P.Lp + i0) * d + p * 16 + 2 * t;
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt) {
+          if (i0 < s1) *reinterpret_cast<uint32_t*>(out + nt * 8) = pack2(acc[nt][0], acc[nt][1]);
+          if (i1 < s1) *reinterpret_cast<uint32_t*>(out + 8 * d + nt * 8) = pack2(acc[nt][2], acc[nt][3]);
+        }
+      }
+    }
+  };
 
   if (nv > 0) {
     // A fragments of U: row h = high part of u_h, row h + 8 = low part
@@ -257,99 +310,72 @@ __global__ void __launch_bounds__(kSThreads) stream_sta_kernel(StreamParams P) {
     int stage = 0;
     const uint32_t off1 = ((lane & 7) + ((lane >> 4) & 1) * 8) * RS + ((lane >> 3) & 1) * 16;   // [item][k] operand
     const uint32_t off2 = ((lane & 7) + ((lane >> 3) & 1) * 8) * RS + (lane >> 4) * 16;         // [item][col], transposed
-    for (int seg = warp; seg < nv; seg += kSW) {
-      float racc[2 * D16][4];
+    // (a chunk of several is a multiple of the warps: a warp's segments, and the copies it has in flight, simply go on)
+    for (int s0 = 0; s0 < nv; s0 += chunk) {
+      const int s1 = kChunks ? min(nv, s0 + chunk) : nv;
+      if (kChunks && s0 > 0) __syncthreads();    // the previous chunk's sums have been read
+      for (int seg = s0 + warp; seg < s1; seg += kSW) {
+        float racc[2 * D16][4];
 #pragma unroll
-      for (int j = 0; j < 2 * D16; ++j) racc[j][0] = racc[j][1] = racc[j][2] = racc[j][3] = 0.f;
-      const int ngrp = groups_of(seg);
-      for (int grp = 0; grp < ngrp; ++grp) {
-        cp_wait<kSStages - 2>();
-        __syncwarp();
-        if (f_valid) issue((stage + kSStages - 1) % kSStages);
-        cp_commit();
-        const uint32_t sb = ring_addr + stage * (kSRows * RS);
-        // scores (Eq. 10 before the sigmoid): rows = heads (high / low parts), columns = the 16 items
-        float sc[2][4] = {};
+        for (int j = 0; j < 2 * D16; ++j) racc[j][0] = racc[j][1] = racc[j][2] = racc[j][3] = 0.f;
+        const int ngrp = groups_of(seg);
+        for (int grp = 0; grp < ngrp; ++grp) {
+          cp_wait<kSStages - 2>();
+          __syncwarp();
+          if (f_valid) issue((stage + kSStages - 1) % kSStages);
+          cp_commit();
+          const uint32_t sb = ring_addr + stage * (kSRows * RS);
+          // scores (Eq. 10 before the sigmoid): rows = heads (high / low parts), columns = the 16 items
+          float sc[2][4] = {};
 #pragma unroll
-        for (int kt = 0; kt < D16; ++kt) {
-          uint32_t b[4];
-          ldsm_x4(b, sb + off1 + kt * 32);
-          mma16816(sc[0], ua[kt][0], ua[kt][1], ua[kt][2], ua[kt][3], b[0], b[1]);
-          mma16816(sc[1], ua[kt][0], ua[kt][1], ua[kt][2], ua[kt][3], b[2], b[3]);
+          for (int kt = 0; kt < D16; ++kt) {
+            uint32_t b[4];
+            ldsm_x4(b, sb + off1 + kt * 32);
+            mma16816(sc[0], ua[kt][0], ua[kt][1], ua[kt][2], ua[kt][3], b[0], b[1]);
+            mma16816(sc[1], ua[kt][0], ua[kt][1], ua[kt][2], ua[kt][3], b[2], b[3]);
+          }
+          // gates; a zero row has score 0, gate 1/2 and contributes 1/2 * 0 = 0, so no mask is needed here
+          uint32_t ga[4] = {0u, 0u, 0u, 0u};
+          if (g < H) {
+#pragma unroll
+            for (int nt = 0; nt < 2; ++nt) {
+              const float g0 = sigmoid_fast(sc[nt][0] + sc[nt][2]), g1 = sigmoid_fast(sc[nt][1] + sc[nt][3]);
+              ga[2 * nt] = pack2(g0, g1);
+              ga[2 * nt + 1] = pack2(g0 - bf16_lo(ga[2 * nt]), g1 - bf16_hi(ga[2 * nt]));
+            }
+          }
+          // r += G X  (Eq. 11-12 with the value projection postponed): rows = heads, k = items, columns = d
+#pragma unroll
+          for (int jp = 0; jp < D16; ++jp) {
+            uint32_t b[4];
+            ldsm_x4_t(b, sb + off2 + jp * 32);
+            mma16816(racc[2 * jp], ga[0], ga[1], ga[2], ga[3], b[0], b[1]);
+            mma16816(racc[2 * jp + 1], ga[0], ga[1], ga[2], ga[3], b[2], b[3]);
+          }
+          stage = (stage + 1) % kSStages;
         }
-        // gates; a zero row has score 0, gate 1/2 and contributes 1/2 * 0 = 0, so no mask is needed here
-        uint32_t ga[4] = {0u, 0u, 0u, 0u};
         if (g < H) {
 #pragma unroll
-          for (int nt = 0; nt < 2; ++nt) {
-            const float g0 = sigmoid_fast(sc[nt][0] + sc[nt][2]), g1 = sigmoid_fast(sc[nt][1] + sc[nt][3]);
-            ga[2 * nt] = pack2(g0, g1);
-            ga[2 * nt + 1] = pack2(g0 - bf16_lo(ga[2 * nt]), g1 - bf16_hi(ga[2 * nt]));
+          for (int j = 0; j < 2 * D16; ++j) {
+            const float r0 = racc[j][0] + racc[j][2], r1 = racc[j][1] + racc[j][3];
+            const uint32_t hi = pack2(r0, r1);
+            const uint32_t lo = pack2(r0 - bf16_lo(hi), r1 - bf16_hi(hi));
+            const size_t o = (size_t)((seg - s0) * H + g) * RS + (j * 8 + 2 * t) * 2;
+            *reinterpret_cast<uint32_t*>(Rhi + o) = hi;
+            *reinterpret_cast<uint32_t*>(Rlo + o) = lo;
           }
         }
-        // r += G X  (Eq. 11-12 with the value projection postponed): rows = heads, k = items, columns = d
-#pragma unroll
-        for (int jp = 0; jp < D16; ++jp) {
-          uint32_t b[4];
-          ldsm_x4_t(b, sb + off2 + jp * 32);
-          mma16816(racc[2 * jp], ga[0], ga[1], ga[2], ga[3], b[0], b[1]);
-          mma16816(racc[2 * jp + 1], ga[0], ga[1], ga[2], ga[3], b[2], b[3]);
-        }
-        stage = (stage + 1) % kSStages;
       }
-      if (g < H) {
-#pragma unroll
-        for (int j = 0; j < 2 * D16; ++j) {
-          const float r0 = racc[j][0] + racc[j][2], r1 = racc[j][1] + racc[j][3];
-          const uint32_t hi = pack2(r0, r1);
-          const uint32_t lo = pack2(r0 - bf16_lo(hi), r1 - bf16_hi(hi));
-          const size_t o = (size_t)(seg * H + g) * RS + (j * 8 + 2 * t) * 2;
-          *reinterpret_cast<uint32_t*>(Rhi + o) = hi;
-          *reinterpret_cast<uint32_t*>(Rlo + o) = lo;
-        }
+      if (s1 == nv) cp_wait<0>();
+      if constexpr (kChunks) {
+        __syncthreads();
+        product(s0, s1);
       }
     }
-    cp_wait<0>();
   }
-  __syncthreads();
-
-  // s_i[head h] = r_{i,h} W_v[:, head h]: one unit = (16 segments, head)
-  {
-    const int NP = dvh >> 4;                      // 16-column pairs per head
-    const int units = ((nv + 15) >> 4) * H;
-    const uint32_t arow = (lane & 7) + ((lane >> 3) & 1) * 8, akc = lane >> 4;
-    for (int unit = warp; unit < units; unit += kSW) {
-      const int mt = unit / H, h = unit - mt * H;
-      float acc[2 * D16][4];
-#pragma unroll
-      for (int j = 0; j < 2 * D16; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
-#pragma unroll
-      for (int kt = 0; kt < D16; ++kt) {
-        uint32_t ah[4], al[4];
-        const size_t o = (size_t)((mt * 16 + arow) * H + h) * RS + (kt * 2 + akc) * 16;
-        ldsm_x4(ah, smem_addr(Rhi + o));
-        ldsm_x4(al, smem_addr(Rlo + o));
-#pragma unroll
-        for (int p = 0; p < D16; ++p) {
-          if (p < NP) {
-            const uint4 b = __ldg(P.imgv + (kt * D16 + h * NP + p) * 32 + lane);
-            mma16816(acc[2 * p], ah[0], ah[1], ah[2], ah[3], b.x, b.y);
-            mma16816(acc[2 * p], al[0], al[1], al[2], al[3], b.x, b.y);
-            mma16816(acc[2 * p + 1], ah[0], ah[1], ah[2], ah[3], b.z, b.w);
-            mma16816(acc[2 * p + 1], al[0], al[1], al[2], al[3], b.z, b.w);
-          }
-        }
-      }
-      const int s0 = mt * 16 + g, s1 = s0 + 8;
-#pragma unroll
-      for (int j = 0; j < 2 * D16; ++j) {
-        if (j < 2 * NP) {
-          const int col = h * dvh + j * 8 + 2 * t;
-          if (s0 < nv) *reinterpret_cast<uint32_t*>(P.Hp + ((size_t)cand * P.Lp + s0) * d + col) = pack2(acc[j][0], acc[j][1]);
-          if (s1 < nv) *reinterpret_cast<uint32_t*>(P.Hp + ((size_t)cand * P.Lp + s1) * d + col) = pack2(acc[j][2], acc[j][3]);
-        }
-      }
-    }
+  if constexpr (!kChunks) {
+    __syncthreads();
+    product(0, nv);
   }
   if (P.zero_empty) {
     const int vec = d / 8;
@@ -360,24 +386,41 @@ __global__ void __launch_bounds__(kSThreads) stream_sta_kernel(StreamParams P) {
   }
 }
 
-size_t stream_smem_bytes(int d, int H, int Lp) {
+// (rows for L' segments, not for a multiple of 16: one segment and eight heads take 74 KB, three blocks per SM, instead of 139; with
+// the product's weights in flight at once 3349 users of 28 items, d = 128 240 -> 88 us)
+size_t stream_smem_bytes(int d, int H, int segs) {
   const size_t RS = 2 * (size_t)d + 16;
-  const size_t Lp16 = ((size_t)Lp + 15) & ~(size_t)15;
-  return 2 * Lp16 * H * RS + (size_t)kSW * kSStages * kSRows * RS;
+  return 2 * (size_t)segs * H * RS + (size_t)kSW * kSStages * kSRows * RS;
+}
+
+// Segments held at a time: all, or as many sixteens as leave room for two blocks per SM (at least one).  (Where all of them at once
+// did not fit 200 KB the general kernels projected every item: 1090 users of 1480 items, d = 96, six heads, 114 segments, the call
+// 1553 -> 102 us.)
+int stream_chunk(int d, int H, int Lp) {
+  const size_t two = 112 * 1024;
+  if (stream_smem_bytes(d, H, Lp) <= two) return Lp;
+  int c = 16;
+  while (c + 16 < Lp && stream_smem_bytes(d, H, c + 16) <= two) c += 16;
+  return c;
 }
 
 template <int D16>
 int launch_stream(const StreamParams& P, cudaStream_t st) {
-  const size_t smem = stream_smem_bytes(P.d, P.H, P.Lp);
-  LASER_CUDA_OK(allow_smem(stream_sta_kernel<D16>, smem));
+  const size_t smem = stream_smem_bytes(P.d, P.H, P.chunk);
+  auto kernel = P.chunk < P.Lp ? stream_sta_kernel<D16, true> : stream_sta_kernel<D16, false>;
+  LASER_CUDA_OK(allow_smem(kernel, smem));
   LaunchScope ls("stream_sta", st);
-  LASER_CUDA_OK(launch_chained(stream_sta_kernel<D16>, dim3(P.U), dim3(kSThreads), smem, st, P));
+  LASER_CUDA_OK(launch_chained(kernel, dim3(P.U), dim3(kSThreads), smem, st, P));
   return LASER_OK;
 }
 
 int launch_pre(const StreamParams& P, cudaStream_t st) {
-  const int user_warps = (P.U + 15) / 16;
-  const dim3 grid((user_warps + kPreWarps - 1) / kPreWarps + 2 + (P.order ? 1 : 0)), block(kPreWarps * 32);
+  const int user_warps = (P.U + 15) / 16 * P.H;
+  // spare blocks for the weight images, an entry or two per thread (two blocks for all of them took 26 us at d = 128, three layers)
+  const int D16 = P.d / 16, entries = (1 + (P.Wg ? 3 * P.M : 0) + (P.prep.img ? 6 * P.M : 0)) * D16 * D16 * 32;
+  const int spare = std::max(2, std::min((entries + kPreWarps * 64 - 1) / (kPreWarps * 64), 2 * device_sms()));
+  const int sorts = (P.order ? 1 : 0) + (P.prep.order ? 1 : 0);
+  const dim3 grid((user_warps + kPreWarps - 1) / kPreWarps + spare + sorts), block(kPreWarps * 32);
   LaunchScope ls("stream_pre", st);
   cudaError_t e;
   switch (P.d / 16) {
@@ -402,9 +445,10 @@ bool stream_supported(const Plan& p) {
   if (p.d % 16 || p.d < 16 || p.d > 128) return false;
   if (p.H > 8 || p.dvh % 16) return false;
   if (p.dqh % 16) return false;                    // the query fold works on 16-column chunks of a head
-  if (!gsta_mma_supported(p)) return false;
-  return stream_smem_bytes(p.d, p.H, p.Lp) <= 200 * 1024;
+  return gsta_mma_supported(p);
 }
+// Every segment's sums in shared memory at once: the shapes for which LASER_PATH_STREAM may be asked for.
+bool stream_in_one_pass(const Plan& p) { return stream_smem_bytes(p.d, p.H, (p.Lp + 15) & ~15) <= 200 * 1024; }
 
 size_t stream_scratch_bytes(const Plan& p) {   // u, the W_v image, the launch order of the users and its sort keys
   return align_up((size_t)p.U * p.H * p.d * sizeof(float)) + align_up((size_t)p.d * p.d * 2) +
@@ -424,8 +468,11 @@ const int* stream_fold_order(const Plan& p, const char* scratch) {
   return stream_wants_order(p) ? reinterpret_cast<const int*>(scratch + align_up((size_t)p.d * p.d * 2)) : nullptr;
 }
 int stream_fold(const Plan& p, const int32_t* lengths, const void* cands, const int32_t* cand_offsets, const void* Wq,
-                const void* Wk, const void* Wv, float* u, char* scratch, int* status, cudaStream_t st) {
+                const void* Wk, const void* Wv, float* u, char* scratch, int* status, cudaStream_t st, const ZeroList* zero,
+                const TrainPrep* prep) {
   StreamParams P = {};
+  if (zero) P.zero = *zero;
+  if (prep) P.prep = *prep;
   P.U = p.U; P.L = p.L; P.d = p.d; P.dqk = p.dqk; P.H = p.H; P.S = p.S; P.Lp = p.Lp; P.N = p.N; P.M = p.M;
   P.inv_gamma = p.inv_gamma;
   P.cands = (const bf16*)cands; P.Wq = (const bf16*)Wq; P.Wk = (const bf16*)Wk; P.Wv = (const bf16*)Wv;
@@ -442,7 +489,7 @@ int stream_sta(const Plan& p, const void* items, const int32_t* lengths, const v
                const void* Wq, const void* Wk, const void* Wv, void* Hprime, char* ws, cudaStream_t st,
                const void* Wg_images) {
   if (p.N == 0 || p.U == 0) return LASER_OK;
-  StreamParams P;
+  StreamParams P = {};
   P.Wg = (const bf16*)Wg_images;
   P.gimg = reinterpret_cast<uint4*>(ws + p.off_gimg);
   P.gnseg = reinterpret_cast<int*>(ws + p.off_gimg + gsta_nseg_offset(p));
@@ -465,6 +512,7 @@ int stream_sta(const Plan& p, const void* items, const int32_t* lengths, const v
                                      align_up((size_t)p.d * p.d * 2));
     P.order_keys = P.order + p.U;
   }
+  P.chunk = stream_chunk(p.d, p.H, p.Lp);
   int rc = launch_pre(P, st);
   if (rc != LASER_OK) return rc;
   switch (p.d / 16) {

@@ -1,0 +1,51 @@
+"""One candidate per user: more segments than the attention kernel holds at a time (several chunks of them, a short last one), fewer than a
+sixteen, users without items; against the float64 oracle, with and without H' asked for, padded and packed."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2602_11562_b200 as P
+from workloads import make_custom
+
+from _util import err_metric, oracle_forward, to_np
+
+pytestmark = pytest.mark.gpu
+
+CASES = [
+    dict(U=3, C=1, L=500, d=128, H=8, S=9, M=2, lengths=[500, 0, 145]),       # 56 segments, sixteen at a time
+    dict(U=4, C=1, L=330, d=96, H=6, S=5, M=1, lengths=[330, 80, 81, 1]),     # 66 segments; whole chunks, and one segment more
+    dict(U=2, C=1, L=600, d=128, H=2, S=5, M=1),                              # 120 segments
+    dict(U=5, C=1, L=40, d=128, H=8, S=40, M=1),                              # one segment: rows past it are not the block's
+    dict(U=2, C=1, L=27, d=64, H=4, S=1, M=2),                                # 27 segments of one item, all at once
+]
+
+
+@pytest.mark.parametrize("case", range(len(CASES)))
+def test_segments_in_chunks(case):
+    w = make_custom(seed=2700 + case, dtype="bf16", d_qh=16, emb_std="inv_sqrt_d", **CASES[case])
+    Hr, zr = oracle_forward(w)
+    b = P.DeviceBatch.from_workload(w)
+    ws = torch.empty(P.laser_workspace_bytes(b.cfg), dtype=torch.uint8, device="cuda")
+    ws.fill_(0xFF)
+    P.laser_profile_enable(True)
+    try:
+        Hp, z = P.laser_forward(b.cfg, *b.args(), b.Wg, workspace=ws, want_hprime=True)
+        assert P.laser_check_status(ws) == 0
+        assert "stream_sta" in [n for n, _ in P.laser_profile_read()]
+    finally:
+        P.laser_profile_enable(False)
+    # fp32 sums of bf16 pairs, rounded once: half a unit in the last place of bf16 (2^-9) and a little
+    assert err_metric(to_np(Hp), Hr) <= 2.0 ** -8 and err_metric(to_np(z), zr) <= 2e-2
+    z2 = P.laser_forward(b.cfg, *b.args(), b.Wg, workspace=ws)
+    valid = torch.arange(w.spec.L, device="cuda")[None, :] < b.lengths[:, None]
+    starts = torch.cat([torch.zeros(1, dtype=torch.int32, device="cuda"), b.lengths.cumsum(0).int()])
+    z3 = P.laser_forward_packed(b.cfg, b.items[valid].contiguous(), starts, b.lengths, b.cands, b.cand_offsets, b.Wq, b.Wk, b.Wv, b.Wg,
+                                workspace=ws)
+    assert P.laser_check_status(ws) == 0
+    for other in (z2, z3):
+        assert torch.equal(z, other[0] if isinstance(other, tuple) else other)
+
+
+def test_asking_for_the_path_is_refused_as_before():
+    w = make_custom(seed=1, dtype="bf16", d_qh=16, **dict(CASES[0], U=1, lengths=[500]))
+    assert P.laser_workspace_bytes(P.DeviceBatch.from_workload(w, path=P.PATH_STREAM).cfg) == 0
