@@ -433,7 +433,7 @@ int laser_ffn_forward(const laser_config* cfg, const laser_ffn_params* ffn, void
   char* ws = static_cast<char*>(workspace);
   if ((rc = clear_status(p, ws, st)) != LASER_OK) return rc;
   if (p.N == 0) return LASER_OK;
-  return ffn_forward(p, ffn, Hprime, lengths, cand_offsets, ws, ws + p.total, st);
+  return ffn_forward(p, ffn, Hprime, lengths, cand_offsets, ws, ws + p.total, st, false);
 }
 
 int laser_forward_ffn(const laser_config* cfg, const void* items, const int32_t* lengths, const void* cands,
@@ -455,9 +455,21 @@ int laser_forward_ffn(const laser_config* cfg, const void* items, const int32_t*
   void* Hp = Hprime ? Hprime : (void*)(ws + p.off_hp);
   const bool side_images = p.M > 0 && p.path != LASER_PATH_SIMT && gsta_mma_supported(p);
   p.zero_in_ffn = Hprime && p.path == LASER_PATH_TENSOR && ffn_on_tensor_cores(p, ffn->d_hidden);
+  // the set-up of the feed-forward step beside STA's own kernels
+  struct FfnSetup : SideLaunches {
+    const Plan* p;
+    const laser_ffn_params* ffn;
+    const int32_t *lengths, *cand_offsets;
+    char* ws;
+    cudaStream_t st;
+    int launch(int which) override { return ffn_side_launch(*p, ffn, lengths, cand_offsets, ws, ws + p->total, st, which); }
+  } setup;
+  setup.p = &p; setup.ffn = ffn; setup.lengths = lengths; setup.cand_offsets = cand_offsets; setup.ws = ws; setup.st = st;
+  const bool beside = p.path != LASER_PATH_SIMT && p.U > 0 && ffn_on_tensor_cores(p, ffn->d_hidden);
+  if (beside) p.side = &setup;
   rc = run_sta(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, Hp, ws, st, side_images ? Wgsta : nullptr);
   if (rc != LASER_OK) return rc;
-  rc = ffn_forward(p, ffn, Hp, lengths, cand_offsets, ws, ws + p.total, st);
+  rc = ffn_forward(p, ffn, Hp, lengths, cand_offsets, ws, ws + p.total, st, beside);
   if (rc != LASER_OK) return rc;
   return run_gsta(p, Hp, lengths, cand_offsets, cands, Wgsta, z, ws, st, side_images, true);
 }

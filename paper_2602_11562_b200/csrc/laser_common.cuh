@@ -29,6 +29,7 @@ struct Plan {
   float inv_gamma, inv_tau;
   size_t esize;
   bool zero_in_ffn;                // the FFN kernel writes the zero rows of empty segments, STA's extra kernel does not
+  struct SideLaunches* side;       // launches that the STA path makes room for between its own (null: none)
   const int32_t* item_offsets;     // packed item layout: first row of every user ([U + 1]); null = padded [U, L, d]
   // workspace byte offsets
   size_t off_status;
@@ -44,6 +45,13 @@ struct Plan {
   // every region of the carve-up (byte offset, bytes in use), in order: what a call may write inside the workspace
   int n_regions;
   size_t reg_off[kMaxRegions], reg_size[kMaxRegions];
+};
+
+// Launches of a later part of the call that depend on its inputs only, or on one another.  The STA path makes launch(0) right after its
+// first kernel and launch(1) after its second.  Such a kernel does its work before it waits for the kernel in front of it, beside
+// which it therefore runs, and waits for it before it ends, so that what follows may rely on both.
+struct SideLaunches {
+  virtual int launch(int which) = 0;
 };
 
 inline size_t align_up(size_t x, size_t a = kAlign) { return (x + a - 1) / a * a; }
@@ -204,7 +212,10 @@ bool ffn_supported(const Plan& p, int hid);
 bool ffn_on_tensor_cores(const Plan& p, int hid);
 size_t ffn_scratch_bytes(const Plan& p, int hid);
 int ffn_forward(const Plan& p, const laser_ffn_params* f, void* H, const int32_t* lengths, const int32_t* cand_offsets,
-                char* ws, char* scratch, cudaStream_t st);
+                char* ws, char* scratch, cudaStream_t st, bool prepared);
+// The set-up kernels of the tensor-core version as side launches of the STA path (which = 0, 1); ffn_forward is then told so.
+int ffn_side_launch(const Plan& p, const laser_ffn_params* f, const int32_t* lengths, const int32_t* cand_offsets, char* ws, char* scratch,
+                    cudaStream_t st, int which);
 
 // --- device helpers ---------------------------------------------------------------------------------------------------
 template <typename T> __device__ __forceinline__ float to_f32(T v);

@@ -50,6 +50,7 @@ struct FfnParams {
   int* rowmap;                                // [N * Lp] compact row -> row of H' (first counters[0] entries valid)
   int* status;
   int zero_empty;                             // also write the zero rows of empty segments
+  int beside;                                 // the set-up kernels run beside kernels of the STA path (SideLaunches)
 };
 
 struct RowUser {
@@ -103,7 +104,7 @@ __device__ void scan_rows(const PT& P, int* status) {
     const RowUser s = row_user(P, u);
     a += s.nc * s.nseg;
   }
-  if (bad) report_status(status, LASER_ERR_BAD_INPUT);
+  if (bad && status) report_status(status, LASER_ERR_BAD_INPUT);
   sa[tid] = a;
   __syncthreads();
   for (int off = 1; off < n_act; off <<= 1) {
@@ -124,14 +125,11 @@ __device__ void scan_rows(const PT& P, int* status) {
   }
 }
 
-__global__ void __launch_bounds__(1024) ffn_prep_kernel(FfnParams P, int build_images) {
-  chain_wait();
-  chain_release();
+__device__ __forceinline__ void ffn_prep(const FfnParams& P) {
   if (blockIdx.x == 0) {
-    scan_rows(P, P.status);
+    scan_rows(P, P.beside ? nullptr : P.status);     // (STA's kernels make the same checks, and one of them is clearing the word now)
     return;
   }
-  if (!build_images) return;
   const int nthreads = (gridDim.x - 1) * blockDim.x;
   const int g = (blockIdx.x - 1) * blockDim.x + threadIdx.x;
   for (int i = g; i < P.d; i += nthreads) {
@@ -150,14 +148,25 @@ __global__ void __launch_bounds__(1024) ffn_prep_kernel(FfnParams P, int build_i
     P.img2[(h / kChunk) * chunk_elems + canon_off(e, h % kChunk, kChunk)] = P.W2[i];
   }
 }
+// Beside the STA path's first kernel (production shape: ffn_prep and ffn_map took 15 of 590 us behind one another and behind STA's
+// kernels; a batch of 390 candidates, d = 32: 8 of 48): what it reads are inputs, what it writes the call before has done with,
+// since no block of it starts before every block of that kernel has seen the call before complete.
+__global__ void __launch_bounds__(1024) ffn_prep_kernel(const __grid_constant__ FfnParams P) {
+  if (!P.beside) chain_wait();
+  chain_release();
+  ffn_prep(P);
+  if (P.beside) chain_wait();
+}
 
 // Compact row -> row of H', for every valid row (the main kernel reads it with coalesced loads).
-__global__ void __launch_bounds__(256) ffn_map_kernel(FfnParams P) {
-  chain_wait();
+// Beside the STA path's second kernel, whose blocks have all seen ffn_prep_kernel complete when this one's start.
+__global__ void __launch_bounds__(256) ffn_map_kernel(const __grid_constant__ FfnParams P) {
+  if (!P.beside) chain_wait();
   chain_release();
   const int total = P.counters[0];
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x)
     P.rowmap[i] = global_row(P, i, total);
+  if (P.beside) chain_wait();
 }
 
 // ------------------------------------------------------------------------------------------------------- tensor kernel
@@ -722,16 +731,11 @@ bool ffn_supported(const Plan& p, int hid) {
   return ((size_t)2 * kSimtRows * p.d + (size_t)kSimtRows * hid) * sizeof(float) <= 200 * 1024;
 }
 
-int ffn_forward(const Plan& p, const laser_ffn_params* f, void* H, const int32_t* lengths, const int32_t* cand_offsets,
-                char* ws, char* scratch, cudaStream_t st) {
-  if (p.N == 0 || p.U == 0) return LASER_OK;
+namespace {
+FfnParams ffn_params(const Plan& p, const laser_ffn_params* f, void* H, const int32_t* lengths, const int32_t* cand_offsets, char* ws,
+                     char* scratch) {
   const int hid = f->d_hidden;
-  if (!ffn_supported(p, hid)) return LASER_ERR_UNSUPPORTED;
-  if (!ffn_on_tensor_cores(p, hid)) {
-    if (p.dtype == LASER_F32) return ffn_simt<float>(p, f, H, lengths, cand_offsets, ws, scratch, st);
-    return ffn_simt<bf16>(p, f, H, lengths, cand_offsets, ws, scratch, st);
-  }
-  FfnParams P;
+  FfnParams P = {};
   P.U = p.U; P.N = p.N; P.L = p.L; P.Lp = p.Lp; P.S = p.S; P.d = p.d; P.hid = hid; P.NJ = hid / kChunk; P.maxC = p.maxC;
   P.eps = f->ln_eps > 0.f ? f->ln_eps : 1e-5f;
   P.H = (bf16*)H;
@@ -746,15 +750,43 @@ int ffn_forward(const Plan& p, const laser_ffn_params* f, void* H, const int32_t
   P.rowmap = (int*)((char*)P.lnv + align_up((size_t)3 * p.d * sizeof(float)));
   P.status = (int*)(ws + p.off_status);
   P.zero_empty = p.zero_in_ffn ? 1 : 0;
-  {
+  return P;
+}
+
+int ffn_setup_launch(const Plan& p, const FfnParams& P, int which, cudaStream_t st) {
+  if (which == 0) {
     LaunchScope ls("ffn_prep", st);
-    LASER_CUDA_OK(launch_chained(ffn_prep_kernel, dim3(1 + 16), dim3(1024), 0, st, P, 1));
-  }
-  {
+    LASER_CUDA_OK(launch_chained(ffn_prep_kernel, dim3(1 + 16), dim3(1024), 0, st, P));
+  } else {
     const long long rows_max = (long long)p.N * p.Lp;
     const int grid = (int)(rows_max < 256LL * 4 * device_sms() ? (rows_max + 255) / 256 : 4 * device_sms());
     LaunchScope ls("ffn_map", st);
     LASER_CUDA_OK(launch_chained(ffn_map_kernel, dim3(grid > 0 ? grid : 1), dim3(256), 0, st, P));
+  }
+  return LASER_OK;
+}
+}  // namespace
+
+int ffn_side_launch(const Plan& p, const laser_ffn_params* f, const int32_t* lengths, const int32_t* cand_offsets, char* ws, char* scratch,
+                    cudaStream_t st, int which) {
+  FfnParams P = ffn_params(p, f, nullptr, lengths, cand_offsets, ws, scratch);
+  P.beside = 1;
+  return ffn_setup_launch(p, P, which, st);
+}
+
+int ffn_forward(const Plan& p, const laser_ffn_params* f, void* H, const int32_t* lengths, const int32_t* cand_offsets,
+                char* ws, char* scratch, cudaStream_t st, bool prepared) {
+  if (p.N == 0 || p.U == 0) return LASER_OK;
+  const int hid = f->d_hidden;
+  if (!ffn_supported(p, hid)) return LASER_ERR_UNSUPPORTED;
+  if (!ffn_on_tensor_cores(p, hid)) {
+    if (p.dtype == LASER_F32) return ffn_simt<float>(p, f, H, lengths, cand_offsets, ws, scratch, st);
+    return ffn_simt<bf16>(p, f, H, lengths, cand_offsets, ws, scratch, st);
+  }
+  const FfnParams P = ffn_params(p, f, H, lengths, cand_offsets, ws, scratch);
+  for (int which = 0; which < 2 && !prepared; ++which) {
+    const int rc = ffn_setup_launch(p, P, which, st);
+    if (rc != LASER_OK) return rc;
   }
   {
     const size_t smem = ffn_tc_smem(p.d, hid);

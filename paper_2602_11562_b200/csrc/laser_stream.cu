@@ -514,6 +514,7 @@ int stream_sta(const Plan& p, const void* items, const int32_t* lengths, const v
   }
   P.chunk = stream_chunk(p.d, p.H, p.Lp);
   int rc = launch_pre(P, st);
+  if (rc == LASER_OK && p.side) rc = p.side->launch(0);
   if (rc != LASER_OK) return rc;
   switch (p.d / 16) {
     case 1: rc = launch_stream<1>(P, st); break;
@@ -526,6 +527,7 @@ int stream_sta(const Plan& p, const void* items, const int32_t* lengths, const v
     case 8: rc = launch_stream<8>(P, st); break;
     default: return LASER_ERR_UNSUPPORTED;
   }
+  if (rc == LASER_OK && p.side) rc = p.side->launch(1);
   if (rc != LASER_OK) return rc;
   LASER_CUDA_OK(cudaGetLastError());
   return LASER_OK;

@@ -1217,6 +1217,8 @@ int tensor_sta(const Plan& p, const void* items, const int32_t* lengths, const v
     LaunchScope ls("tc_prep", st);
     LASER_CUDA_OK(launch_chained(tc_prep_kernel, dim3(1 + 32 + (P.gorder ? 1 : 0)), dim3(1024), 0, st, P));
   }
+  int rc = p.side ? p.side->launch(0) : LASER_OK;
+  if (rc != LASER_OK) return rc;
   {
     const size_t smem = ((size_t)p.dqk * p.d + 3 * (size_t)kCandTile * p.d) * 2;   // W_k^T | W_q^T, W_v^T, two staging buffers
     LASER_CUDA_OK(allow_smem(tc_proj_kernel, smem));
@@ -1227,6 +1229,7 @@ int tensor_sta(const Plan& p, const void* items, const int32_t* lengths, const v
     const int use_tma = !P.item_off && P.IT >= 32 && encode_item_map(p, P.IT, items, &item_map) ? 1 : 0;
     LASER_CUDA_OK(launch_chained(tc_proj_kernel, dim3(P.proj_grid), dim3(kProjThreads), smem, st, P, item_map, use_tma));
   }
+  if (p.side && (rc = p.side->launch(1)) != LASER_OK) return rc;
   if (user_wants_hp && !p.zero_in_ffn) {
     LaunchScope ls("tc_zero_empty", st);
     LASER_CUDA_OK(launch_chained(tc_zero_empty_kernel, dim3(p.Lp, p.U), dim3(256), 0, st, P));
