@@ -520,7 +520,20 @@ struct HostItemRoute {
   const void* alias;                     // kGather: device alias of items_h
 };
 constexpr size_t kCopyWorth = 384 * 1024, kGatherWorth = 256 * 1024;
+constexpr size_t kShortItems = 2 * 1024 * 1024;      // padded items that travel with the small arrays (a kernel reads at 50 GB/s, a copy at 55)
 constexpr int kGatherThreads = 256;
+
+// Where the device reads or writes pinned (or registered) host memory in place; null for any other memory, and where 16-byte accesses
+// would not be aligned.
+void* device_alias(const void* h) {
+  if (reinterpret_cast<uintptr_t>(h) & 15) return nullptr;
+  cudaPointerAttributes attr;
+  if (cudaPointerGetAttributes(&attr, h) != cudaSuccess) {
+    cudaGetLastError();                  // (no device, or a runtime that rejects pageable pointers: not an error here)
+    return nullptr;
+  }
+  return attr.type == cudaMemoryTypeHost && (reinterpret_cast<uintptr_t>(attr.devicePointer) & 15) == 0 ? attr.devicePointer : nullptr;
+}
 
 HostItemRoute host_item_route(const Plan& p, const void* items_h, const int32_t* lengths_h) {
   HostItemRoute r;
@@ -540,20 +553,60 @@ HostItemRoute host_item_route(const Plan& p, const void* items_h, const int32_t*
   }
   if (rows > 0x7fffffffLL) return r;
   const size_t need = (size_t)rows * row;
-  if (items_h && row % 16 == 0 && (reinterpret_cast<uintptr_t>(items_h) & 15) == 0 && need + kGatherWorth < padded) {
-    cudaPointerAttributes attr;
-    if (cudaPointerGetAttributes(&attr, items_h) == cudaSuccess) {
-      if (attr.type == cudaMemoryTypeHost && attr.devicePointer) {
-        r.kind = kGather;
-        r.alias = attr.devicePointer;
-      }
-    } else {
-      cudaGetLastError();                // (no device, or a runtime that rejects pageable pointers: not an error here)
-    }
-  }
+  if (items_h && row % 16 == 0 && need + kGatherWorth < padded && (r.alias = device_alias(items_h)) != nullptr) r.kind = kGather;
   if (r.kind == kPadded && need + copies * kCopyWorth < padded) r.kind = kRuns;
   if (r.kind != kPadded) r.bytes = need;
   return r;
+}
+
+// The small arrays of a call (lengths, offsets, candidates, weights, short item arrays) from pinned host memory in one launch:
+// a copy each cost 4-5 us of the stream, one after the other.  A block copies 16 KB of one array; the last block of the grid also
+// makes the row offsets (null: not wanted), from the lengths as they lie on the host.
+struct HostSegs {
+  const void* src[8];
+  void* dst[8];
+  unsigned long long bytes[8];
+  unsigned first[9];                     // first block of each array
+  int count;
+};
+constexpr unsigned kSegBytes = 16 * 1024;
+__global__ void __launch_bounds__(kGatherThreads) host_fetch_kernel(const __grid_constant__ HostSegs G, const int32_t* lengths, int U, int L,
+                                                                    int32_t* row_off) {
+  chain_wait();
+  const int tid = threadIdx.x;
+  if (blockIdx.x < G.first[G.count]) {
+    int a = 0;
+    while (blockIdx.x >= G.first[a + 1]) ++a;
+    const unsigned long long lo = (unsigned long long)(blockIdx.x - G.first[a]) * kSegBytes, n = min((unsigned long long)kSegBytes, G.bytes[a] - lo);
+    const char* src = static_cast<const char*>(G.src[a]) + lo;
+    char* dst = static_cast<char*>(G.dst[a]) + lo;
+    const unsigned n16 = (unsigned)(n / 16);
+#pragma unroll 4
+    for (unsigned i = tid; i < n16; i += kGatherThreads) reinterpret_cast<uint4*>(dst)[i] = reinterpret_cast<const uint4*>(src)[i];
+    for (unsigned i = n16 * 16 + tid; i < n; i += kGatherThreads) dst[i] = src[i];
+    return;
+  }
+  __shared__ int part[kGatherThreads / 32];
+  int run = 0;                           // rows before this round's users
+  for (int u0 = 0; u0 < U; u0 += kGatherThreads) {
+    const int u = u0 + tid, len = u < U ? min(max(lengths[u], 0), L) : 0;
+    int incl = len;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, incl, o);
+      if ((tid & 31) >= o) incl += v;
+    }
+    if ((tid & 31) == 31) part[tid >> 5] = incl;
+    __syncthreads();
+    int before = run, total = 0;
+    for (int w = 0; w < kGatherThreads / 32; ++w) {
+      if (w < tid >> 5) before += part[w];
+      total += part[w];
+    }
+    if (u < U) row_off[u] = before + incl - len;
+    run += total;
+    __syncthreads();
+  }
+  if (tid == 0) row_off[U] = run;
 }
 
 // First row of every user in the gap-free array: exclusive prefix sums of the lengths, clamped to [0, L] as the host
@@ -644,13 +697,44 @@ int laser_forward_host(const laser_config* cfg, const void* items_h, const int32
     if (!bytes) return cudaSuccess;
     return cudaMemcpyAsync(ws + off, src, bytes, cudaMemcpyHostToDevice, st);
   };
-  LASER_CUDA_OK(h2d(s.lengths, lengths_h, s.b_lengths));
-  LASER_CUDA_OK(h2d(s.offs, cand_offsets_h, s.b_offs));
+  const HostItemRoute route = host_item_route(p, items_h, lengths_h);
+  // everything but long item arrays by one kernel where all of it is pinned, else by a copy each
+  HostSegs G = {};
+  bool fetched = p.N > 0 && p.U > 0;
+  auto seg = [&](size_t off, const void* src, size_t bytes) {
+    if (!fetched || bytes == 0) return;
+    const void* alias = device_alias(src);
+    if (!alias) { fetched = false; return; }
+    G.src[G.count] = alias;
+    G.dst[G.count] = ws + off;
+    G.bytes[G.count] = bytes;
+    G.first[G.count + 1] = G.first[G.count] + (unsigned)((bytes + kSegBytes - 1) / kSegBytes);
+    ++G.count;
+  };
+  const bool short_items = route.kind == kPadded && s.b_items <= kShortItems;
+  seg(s.lengths, lengths_h, s.b_lengths);
+  seg(s.offs, cand_offsets_h, s.b_offs);
+  if (fetched) {
+    seg(s.cands, cands_h, s.b_cands);
+    seg(s.wq, Wq_h, s.b_wq);
+    seg(s.wk, Wk_h, s.b_wk);
+    seg(s.wv, Wv_h, s.b_wv);
+    if (p.M > 0) seg(s.wg, Wgsta_h, s.b_wg);
+    if (short_items) seg(s.items, items_h, s.b_items);
+  }
+  if (fetched) {
+    LaunchScope ls("host_fetch", st);
+    LASER_CUDA_OK(launch_chained(host_fetch_kernel, dim3(G.first[G.count] + (route.kind == kPadded ? 0 : 1)), dim3(kGatherThreads), 0, st, G,
+                                 static_cast<const int32_t*>(G.src[0]), p.U, p.L, reinterpret_cast<int32_t*>(ws + s.item_offs)));
+  } else {
+    LASER_CUDA_OK(h2d(s.lengths, lengths_h, s.b_lengths));
+    LASER_CUDA_OK(h2d(s.offs, cand_offsets_h, s.b_offs));
+  }
   if (p.N > 0) {
-    const HostItemRoute route = host_item_route(p, items_h, lengths_h);
-    if (route.kind == kPadded) LASER_CUDA_OK(h2d(s.items, items_h, s.b_items));
-    else {
-      {
+    if (route.kind == kPadded) {
+      if (!fetched || !short_items) LASER_CUDA_OK(h2d(s.items, items_h, s.b_items));
+    } else {
+      if (!fetched) {
         LaunchScope ls("host_row_offsets", st);
         LASER_CUDA_OK(launch_chained(host_row_offsets_kernel, dim3(1), dim3(1024), 0, st,
                                      reinterpret_cast<const int32_t*>(ws + s.lengths), p.U, p.L,
@@ -682,17 +766,22 @@ int laser_forward_host(const laser_config* cfg, const void* items_h, const int32
       }
       p.item_offsets = reinterpret_cast<const int32_t*>(ws + s.item_offs);
     }
-    LASER_CUDA_OK(h2d(s.cands, cands_h, s.b_cands));
-    LASER_CUDA_OK(h2d(s.wq, Wq_h, s.b_wq));
-    LASER_CUDA_OK(h2d(s.wk, Wk_h, s.b_wk));
-    LASER_CUDA_OK(h2d(s.wv, Wv_h, s.b_wv));
-    LASER_CUDA_OK(h2d(s.wg, Wgsta_h, s.b_wg));
+    if (!fetched) {
+      LASER_CUDA_OK(h2d(s.cands, cands_h, s.b_cands));
+      LASER_CUDA_OK(h2d(s.wq, Wq_h, s.b_wq));
+      LASER_CUDA_OK(h2d(s.wk, Wk_h, s.b_wk));
+      LASER_CUDA_OK(h2d(s.wv, Wv_h, s.b_wv));
+      LASER_CUDA_OK(h2d(s.wg, Wgsta_h, s.b_wg));
+    }
   }
+  // the scores straight into pinned host memory, as the last kernel makes them (it writes each once, 16 bytes at a time): 64 x 256
+  // candidates 1136 -> 1065 us per call, of which the copy behind the kernel was 77
+  void* z_alias = s.b_z > 0 && p.path != LASER_PATH_SIMT && gsta_mma_supported(p) ? device_alias(z_h) : nullptr;
   rc = forward_impl(p, ws + s.items, reinterpret_cast<const int32_t*>(ws + s.lengths), ws + s.cands,
                     reinterpret_cast<const int32_t*>(ws + s.offs), ws + s.wq, ws + s.wk, ws + s.wv, ws + s.wg, nullptr,
-                    ws + s.z, ws, st);
+                    z_alias ? z_alias : ws + s.z, ws, st);
   if (rc != LASER_OK) return rc;
-  if (s.b_z) LASER_CUDA_OK(cudaMemcpyAsync(z_h, ws + s.z, s.b_z, cudaMemcpyDeviceToHost, st));
+  if (s.b_z && !z_alias) LASER_CUDA_OK(cudaMemcpyAsync(z_h, ws + s.z, s.b_z, cudaMemcpyDeviceToHost, st));
   if (blocking) return laser_check_status(workspace, cuda_stream);
   return LASER_OK;
 }

@@ -358,11 +358,12 @@ __global__ void __launch_bounds__(kGThreads, BPS) gsta_mma_kernel(GstaParams P) 
   }
   cp_wait<0>();
 
-  for (int i = tid; i < kGT * (d / 2); i += kGThreads) {
-    const int r = i / (d / 2), q = i - r * (d / 2);
+  // (16 bytes at a time: z may be host memory)
+  for (int i = tid; i < kGT * (d / 8); i += kGThreads) {
+    const int r = i / (d / 8), c8 = (i - r * (d / 8)) * 8;
     if (c_base + r < c_end) {
-      const float2 v = *reinterpret_cast<const float2*>(Ts + r * TS + 2 * q);
-      *reinterpret_cast<uint32_t*>(P.z + (size_t)(c_base + r) * d + 2 * q) = pack2(v.x, v.y);
+      const float4 v = *reinterpret_cast<const float4*>(Ts + r * TS + c8), w = *reinterpret_cast<const float4*>(Ts + r * TS + c8 + 4);
+      *reinterpret_cast<uint4*>(P.z + (size_t)(c_base + r) * d + c8) = make_uint4(pack2(v.x, v.y), pack2(v.z, v.w), pack2(w.x, w.y), pack2(w.z, w.w));
     }
   }
 }

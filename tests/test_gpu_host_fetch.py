@@ -1,0 +1,54 @@
+"""The host entry point's ways of moving its arrays: pinned memory fetched by one kernel (odd byte counts, several blocks per array, row
+offsets over more users than a round of the scan), pageable or unaligned arrays by copies; scores into pinned memory in place or by a
+copy.  Always the device call's result, bit for bit."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2602_11562_b200 as P
+from workloads import make_custom
+
+pytestmark = pytest.mark.gpu
+
+CASES = [
+    dict(U=3, C=7, L=70, d=48, H=3, S=9, M=2, dtype="bf16"),                       # 12-byte lengths, 16-byte offsets; short padded items
+    dict(U=301, C=2, L=64, d=64, H=2, S=16, M=1, dtype="bf16"),                    # row offsets of two rounds of users, gathered items
+    dict(U=5, C=40, L=600, d=128, H=4, S=50, M=3, dtype="bf16", full=True),        # nothing to save: padded items, weights of 18 blocks
+    dict(U=20, C=9, L=900, d=128, H=4, S=50, M=1, dtype="bf16", full=True),        # padded items too long for the kernel
+    dict(U=2, C=9, L=50, d=32, H=2, S=10, M=0, dtype="bf16"),                      # no layer, no weights of one
+    dict(U=4, C=5, L=90, d=64, H=4, S=10, M=2, dtype="f32"),                       # scores by a copy
+    dict(U=40, C=1, L=300, d=64, H=2, S=10, M=1, dtype="bf16"),
+]
+
+
+@pytest.mark.parametrize("kind", ["pinned", "pageable", "unaligned"])
+@pytest.mark.parametrize("case", range(len(CASES)))
+def test_host_arrays(case, kind):
+    kw = dict(CASES[case])
+    if kw.pop("full", False):
+        kw["lengths"] = [kw["L"]] * kw["U"]
+    w = make_custom(seed=2900 + case, d_qh=16, emb_std="inv_sqrt_d", **kw)
+    dev = P.DeviceBatch.from_workload(w)
+    ws = torch.empty(P.laser_workspace_bytes(dev.cfg), dtype=torch.uint8, device="cuda")
+    want = P.laser_forward(dev.cfg, *dev.args(), dev.Wg, workspace=ws)
+    want = want[0] if isinstance(want, tuple) else want
+
+    def host(t):
+        t = t.cpu()
+        if kind == "pageable":
+            return t
+        if kind == "unaligned":                                    # pinned, but 4 (or 2) bytes off a 16-byte boundary
+            buf = torch.empty(t.numel() + 1, dtype=t.dtype).pin_memory()
+            view = buf[1:].view(t.shape)
+            view.copy_(t)
+            return view
+        return t.pin_memory()
+
+    args = [host(t) for t in dev.args()] + [host(dev.Wg)]
+    z = host(torch.zeros_like(want))
+    hws = torch.empty(P.laser_host_workspace_bytes(dev.cfg), dtype=torch.uint8, device="cuda")
+    for fill in (0xFF, 0x00):
+        hws.fill_(fill)
+        z.fill_(7.0)
+        P.laser_forward_host(dev.cfg, *args, z, hws)
+        assert torch.equal(z, want.cpu())
