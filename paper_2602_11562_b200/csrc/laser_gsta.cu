@@ -42,6 +42,7 @@ struct GstaParams {
   int* order;                  // [blocks] launch order, longest first (null: blocks run in candidate order)
   int* order_keys;             // [blocks] scratch of the sort that builds `order`
   int build_order;             // the set-up kernel's last block builds `order`
+  int release_early;           // the next kernel may start while this one runs
   int early_setup;             // images, counts and order come from a kernel at least two launches back (see the kernel)
   bf16* z;
   int* status;
@@ -90,7 +91,7 @@ __global__ void __launch_bounds__(kGThreads, BPS) gsta_mma_kernel(GstaParams P) 
   // predecessor and the wait comes first.
   if (!P.early_setup) {
     chain_wait();
-    chain_release();
+    if (P.release_early) chain_release();
   }
   // which 16 (or 8) candidates: in launch order when the set-up kernel sorted the blocks, else in candidate order
   const int blk = P.order ? min(max(P.order[blockIdx.x], 0), (int)gridDim.x - 1) : (int)blockIdx.x;
@@ -167,7 +168,7 @@ __global__ void __launch_bounds__(kGThreads, BPS) gsta_mma_kernel(GstaParams P) 
   int buf = 0;
   if (P.early_setup) {
     chain_wait();
-    chain_release();
+    if (P.release_early) chain_release();
   }
   if (f_valid) issue(0);
   cp_commit();
@@ -404,6 +405,15 @@ int gsta_candidates_per_block(const Plan& p) {
   return (p.N + 7) / 8 <= 2 * sms ? 8 : kGT;
 }
 
+// Blocks that could have an SM each, placed while the attention kernel runs, pile up on the few SMs that have no unit of it: one request
+// of 512 candidates (64 blocks) 26.6 -> 25.6 us with the blocks placed when it ends, 432 candidates (54) 31.0 -> 28.5.  A handful of blocks
+// does not crowd and gains from an early set-up (96 candidates, 12 blocks 21.8 against 22.6), and from about an SM's worth of blocks each
+// on there is nothing to spread (4400 candidates 62.9 against 64.5).
+bool gsta_prefers_idle_gpu(const Plan& p) {
+  const int cpb = gsta_candidates_per_block(p), blocks = (p.N + cpb - 1) / cpb;
+  return p.M > 0 && blocks >= 32 && blocks <= device_sms();
+}
+
 // Sorting the blocks pays only when the grid runs in more than one wave.
 bool gsta_wants_order(const Plan& p) {
   const int sms = device_sms();
@@ -432,6 +442,10 @@ int gsta_mma(const Plan& p, const void* Hprime, const int32_t* lengths, const in
   P.order_keys = order + (p.N + 7) / 8;
   P.build_order = ordered && !images_ready;
   P.early_setup = images_ready ? 1 : 0;
+  // A grid of one wave ends at once, and the next call's first blocks in its way cost more than their early start gains (4096
+  // candidates, one per user, 138.6 -> 136.0 us per call); several waves leave SMs idle at the end that they can use (16384 candidates,
+  // d = 128 152 against 158).
+  P.release_early = (p.N + P.cpb - 1) / P.cpb > 2 * device_sms() ? 1 : 0;
   if (p.M > 0 && !images_ready) {
     const int total = p.M * 3 * (p.d / 16) * (p.d / 16) * 32;
     LaunchScope ls("gsta_prep", st);

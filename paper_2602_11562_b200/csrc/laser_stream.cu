@@ -55,7 +55,7 @@ struct StreamParams {
   int* order;                     // [U] users by descending length (null: blocks take the users in index order)
   int* order_keys;                // [U] scratch of the sort
   int* status;
-  int chunk;                      // segments whose sums the attention kernel holds at a time
+  int chunk, parts;               // segments whose sums a block of the attention kernel holds at a time; blocks per user
   ZeroList zero;                  // backward pass: arrays that the pre kernel sets to zero, and what the stacked attention wants
   TrainPrep prep;                 // (img null: not wanted)
 };
@@ -203,12 +203,13 @@ __global__ void __launch_bounds__(kSThreads) stream_sta_kernel(const __grid_cons
   int len = 0;
   const int cand = user_candidate(P, u, &len);
   if (cand < 0) return;
-  const int nv = (len + P.S - 1) / P.S;          // non-empty segments
-  const int chunk = P.chunk;                     // segments whose sums are held at a time: all L', or a multiple of 16
+  const int nseg = (len + P.S - 1) / P.S;        // non-empty segments, and this block's share of them
+  const int per = (nseg + gridDim.y - 1) / gridDim.y, lo = min(nseg, (int)blockIdx.y * per), nv = min(nseg, lo + per);
+  const int chunk = P.chunk;                     // segments whose sums are held at a time: all of the block's, or a multiple of 16
   uint8_t* Rhi = smem;                           // [chunk][H] rows: bf16 high part of r_{i,h}
   uint8_t* Rlo = Rhi + (size_t)chunk * H * RS;   // same shape: bf16 low part
   uint8_t* ring = Rlo + (size_t)chunk * H * RS + (size_t)warp * kSStages * kSRows * RS;
-  // (the product with W_v reads segments in sixteens: where all L' are held, up to 15 H <= 120 rows past the end of Rlo lie in the
+  // (the product with W_v reads segments in sixteens: where all are held, up to 15 H <= 120 rows past the end of Rlo lie in the
   // ring's 256, which nothing writes by then, and what it makes of them is not stored)
   static_assert(kSW * kSStages * kSRows >= 15 * 8, "rows past the last segment stay inside the block's shared memory");
 
@@ -249,7 +250,7 @@ __global__ void __launch_bounds__(kSThreads) stream_sta_kernel(const __grid_cons
     }
   };
 
-  if (nv > 0) {
+  if (nv > lo) {
     // A fragments of U: row h = high part of u_h, row h + 8 = low part
     uint32_t ua[D16][4];
     {
@@ -271,8 +272,8 @@ __global__ void __launch_bounds__(kSThreads) stream_sta_kernel(const __grid_cons
 
     // fetch cursor over this warp's (segment, 16-row group) sequence.  A stage is kSRows rows of 2 D16 16-byte
     // pieces; lane l copies pieces l, l + 32, ...: their row, source offset and destination offset never change.
-    int f_seg = warp, f_grp = 0;
-    bool f_valid = warp < nv;
+    int f_seg = lo + warp, f_grp = 0;
+    bool f_valid = f_seg < nv;
     int p_row[D16], p_src[D16];
     uint32_t p_dst[D16];
 #pragma unroll
@@ -311,9 +312,9 @@ __global__ void __launch_bounds__(kSThreads) stream_sta_kernel(const __grid_cons
     const uint32_t off1 = ((lane & 7) + ((lane >> 4) & 1) * 8) * RS + ((lane >> 3) & 1) * 16;   // [item][k] operand
     const uint32_t off2 = ((lane & 7) + ((lane >> 3) & 1) * 8) * RS + (lane >> 4) * 16;         // [item][col], transposed
     // (a chunk of several is a multiple of the warps: a warp's segments, and the copies it has in flight, simply go on)
-    for (int s0 = 0; s0 < nv; s0 += chunk) {
+    for (int s0 = lo; s0 < nv; s0 += chunk) {
       const int s1 = kChunks ? min(nv, s0 + chunk) : nv;
-      if (kChunks && s0 > 0) __syncthreads();    // the previous chunk's sums have been read
+      if (kChunks && s0 > lo) __syncthreads();    // the previous chunk's sums have been read
       for (int seg = s0 + warp; seg < s1; seg += kSW) {
         float racc[2 * D16][4];
 #pragma unroll
@@ -375,12 +376,12 @@ __global__ void __launch_bounds__(kSThreads) stream_sta_kernel(const __grid_cons
   }
   if constexpr (!kChunks) {
     __syncthreads();
-    product(0, nv);
+    product(lo, nv);
   }
   if (P.zero_empty) {
     const int vec = d / 8;
-    for (int i = tid; i < (P.Lp - nv) * vec; i += kSThreads) {
-      const int seg = nv + i / vec, q = i % vec;
+    for (int i = blockIdx.y * kSThreads + tid; i < (P.Lp - nseg) * vec; i += gridDim.y * kSThreads) {
+      const int seg = nseg + i / vec, q = i % vec;
       *reinterpret_cast<uint4*>(P.Hp + ((size_t)cand * P.Lp + seg) * d + q * 8) = make_uint4(0, 0, 0, 0);
     }
   }
@@ -407,10 +408,10 @@ int stream_chunk(int d, int H, int Lp) {
 template <int D16>
 int launch_stream(const StreamParams& P, cudaStream_t st) {
   const size_t smem = stream_smem_bytes(P.d, P.H, P.chunk);
-  auto kernel = P.chunk < P.Lp ? stream_sta_kernel<D16, true> : stream_sta_kernel<D16, false>;
+  auto kernel = P.chunk < (P.Lp + P.parts - 1) / P.parts ? stream_sta_kernel<D16, true> : stream_sta_kernel<D16, false>;
   LASER_CUDA_OK(allow_smem(kernel, smem));
   LaunchScope ls("stream_sta", st);
-  LASER_CUDA_OK(launch_chained(kernel, dim3(P.U), dim3(kSThreads), smem, st, P));
+  LASER_CUDA_OK(launch_chained(kernel, dim3(P.U, P.parts), dim3(kSThreads), smem, st, P));
   return LASER_OK;
 }
 
@@ -512,7 +513,10 @@ int stream_sta(const Plan& p, const void* items, const int32_t* lengths, const v
                                      align_up((size_t)p.d * p.d * 2));
     P.order_keys = P.order + p.U;
   }
-  P.chunk = stream_chunk(p.d, p.H, p.Lp);
+  // Few users: a block per user leaves SMs idle, so a user's segments go to several blocks, four (one per warp) at least: 41 users of
+  // 2148 items, d = 96, six heads 37 -> 17 us, 27 of 5730, d = 64 41 -> 13 (CUDA events, about 6 too long)
+  P.parts = std::max(1, std::min((4 * device_sms() + p.U - 1) / p.U, p.Lp / kSW));
+  P.chunk = stream_chunk(p.d, p.H, (p.Lp + P.parts - 1) / P.parts);
   int rc = launch_pre(P, st);
   if (rc == LASER_OK && p.side) rc = p.side->launch(0);
   if (rc != LASER_OK) return rc;

@@ -61,6 +61,7 @@ struct TcParams {
   bf16 *imgK, *imgQ, *imgV;           // W_k^T, W_q^T [dqk x d], W_v^T [128 x d] in canonical K-major layout
   int* status;
   bf16* Hp;
+  int release_early;                  // the attention kernel lets its successor start while it runs
 };
 
 // Sanitised view of one user: invalid lengths / offsets behave like an empty user (and are reported by tc_prep_kernel).
@@ -706,7 +707,7 @@ __global__ void __launch_bounds__(kStaThreads, 1) tc_sta_kernel(TcParams P) {
   const int n_obuf = P.n_obuf;
   const bool two_epilogues = n_groups <= 2 && n_obuf == 2;    // gate warpgroup 2 has no head: it drains accumulator 1
   chain_wait();                         // K, V^T and Q tiles are complete
-  chain_release();
+  if (P.release_early) chain_release();
 
   // this block's contiguous range of units
   const int n_units = P.counters[0];
@@ -1207,6 +1208,7 @@ int tensor_sta(const Plan& p, const void* items, const int32_t* lengths, const v
   P.gimg = reinterpret_cast<uint4*>(ws + p.off_gimg);
   P.gnseg = reinterpret_cast<int*>(ws + p.off_gimg + gsta_nseg_offset(p));
   P.M = p.M;
+  P.release_early = !(P.Wg && !p.side && gsta_prefers_idle_gpu(p));
   P.gorder = nullptr;
   if (P.Wg && gsta_wants_order(p)) {
     P.gorder = reinterpret_cast<int*>(ws + p.off_gimg + gsta_order_offset(p));

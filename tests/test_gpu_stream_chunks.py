@@ -49,3 +49,18 @@ def test_segments_in_chunks(case):
 def test_asking_for_the_path_is_refused_as_before():
     w = make_custom(seed=1, dtype="bf16", d_qh=16, **dict(CASES[0], U=1, lengths=[500]))
     assert P.laser_workspace_bytes(P.DeviceBatch.from_workload(w, path=P.PATH_STREAM).cfg) == 0
+
+
+@pytest.mark.parametrize("kw", [
+    dict(U=1, C=1, L=640, d=64, H=2, S=10, M=1),                                # 64 segments over sixteen blocks
+    dict(U=3, C=1, L=200, d=32, H=1, S=3, M=1, lengths=[200, 5, 0]),            # shares of five, of none; a user without items
+    dict(U=7, C=1, L=330, d=128, H=8, S=5, M=1),                                # several blocks per user, several chunks per block
+])
+def test_segments_over_blocks(kw):
+    w = make_custom(seed=2800, dtype="bf16", d_qh=16, emb_std="inv_sqrt_d", **kw)
+    Hr, zr = oracle_forward(w)
+    b = P.DeviceBatch.from_workload(w)
+    ws = torch.empty(P.laser_workspace_bytes(b.cfg), dtype=torch.uint8, device="cuda")
+    Hp, z = P.laser_forward(b.cfg, *b.args(), b.Wg, workspace=ws, want_hprime=True)
+    assert P.laser_check_status(ws) == 0
+    assert err_metric(to_np(Hp), Hr) <= 2.0 ** -8 and err_metric(to_np(z), zr) <= 2e-2
