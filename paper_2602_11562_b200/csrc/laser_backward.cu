@@ -1096,12 +1096,15 @@ int backward_stream_all(const Plan& p, const T* items, const int32_t* lengths, c
   Z.add(dWq, (size_t)d * dqk); Z.add(dWk, (size_t)d * dqk); Z.add(dWv, (size_t)d * d); Z.add(dWg, (size_t)M * 3 * d * d);
   Z.add(backward_stream_sums(p, stream_scratch), (size_t)N * H * d);
   Z.add(ws + p.off_status, kStatusWords);
-  const TrainPrep prep = gsta_train_prep(p, 2, Wg, lengths, cand_offsets, train_scratch);
-  bf16 *Hhi = reinterpret_cast<bf16*>(s.Hp), *Hlo = Hhi + (size_t)N * p.Lp * d;
-  BWD_OK(backward_stream_forward(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, nullptr, Hhi, Hlo, ws, stream_scratch, st, &Z,
-                                 &prep));
+  const bool alus = gsta_train_f32_pays(p);
+  TrainPrep prep = {};
+  if (!alus) prep = gsta_train_prep(p, 2, Wg, lengths, cand_offsets, train_scratch);
+  bf16 *Hhi = alus ? nullptr : reinterpret_cast<bf16*>(s.Hp), *Hlo = alus ? nullptr : Hhi + (size_t)N * p.Lp * d;
+  BWD_OK(backward_stream_forward(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, alus ? s.Hp : nullptr, Hhi, Hlo, ws,
+                                 stream_scratch, st, &Z, &prep));
   const GstaPlanes G = train_planes(p, s);
-  BWD_OK(gsta_train(p, 2, Hhi, Hlo, lengths, cand_offsets, cands, Wg, dz, G, s.dHp, nullptr, train_scratch, st, true));
+  if (alus) BWD_OK(gsta_train_f32(p, s.Hp, lengths, cand_offsets, cands, Wg, dz, nullptr, &G, s.dHp, nullptr, st));
+  else BWD_OK(gsta_train(p, 2, Hhi, Hlo, lengths, cand_offsets, cands, Wg, dz, G, s.dHp, nullptr, train_scratch, st, true));
   const float* p_sums = nullptr;
   BWD_OK(backward_stream(p, items, lengths, cand_offsets, Wv, s.dHp, d_items, dWv, &p_sums, ws, stream_scratch, st));
 #undef BWD_OK
@@ -1138,6 +1141,12 @@ int lists_parts(const Plan& p) {
 int lists_attention(const Plan& p, int np, const BwdScratch& s, const int32_t* lengths, const int32_t* cand_offsets, const bf16* cands,
                     const bf16* Wg, const float* dz, const GstaPlanes& G, char* mma_scratch, char* train_scratch, cudaStream_t st,
                     bool prepared) {
+  if (gsta_train_f32_pays(p)) {
+    const int rc = sta_fwd_mma(p, lengths, cand_offsets, s.Hp, nullptr, nullptr, mma_scratch, st);
+    return rc != LASER_OK ? rc
+                          : gsta_train_f32(p, s.Hp, lengths, cand_offsets, cands, Wg, dz, nullptr, &G, nullptr,
+                                           sta_mma_segment_gradients(p, mma_scratch), st);
+  }
   bf16 *Hb = reinterpret_cast<bf16*>(s.Hp), *Hl = np == 2 ? Hb + (size_t)p.N * p.Lp * p.d : nullptr;
   int rc = sta_fwd_mma(p, lengths, cand_offsets, nullptr, Hb, Hl, mma_scratch, st);
   if (rc == LASER_OK)
@@ -1164,8 +1173,9 @@ int backward_lists(const Plan& p, const bf16* items, const int32_t* lengths, con
   Z.add(dWq, d * dqk); Z.add(dWk, d * dqk); Z.add(dWv, d * d); Z.add(dWg, M * 3 * d * d); Z.add(s.dQf, N * dqk);
   Z.add(ws + p.off_status, kStatusWords);
   const int np = lists_parts(p);
-  BWD_OK(rows_project(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, 0.5f * p.inv_gamma, Qb, Kb, Vb, Z,
-                      gsta_train_prep(p, np, Wg, lengths, cand_offsets, train_scratch), st));
+  TrainPrep prep = {};
+  if (!gsta_train_f32_pays(p)) prep = gsta_train_prep(p, np, Wg, lengths, cand_offsets, train_scratch);
+  BWD_OK(rows_project(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, 0.5f * p.inv_gamma, Qb, Kb, Vb, Z, prep, st));
   BWD_OK(lists_attention(p, np, s, lengths, cand_offsets, cands, Wg, dz, G, mma_scratch, train_scratch, st, true));
   BWD_OK(sta_bwd_mma_split(p, lengths, cand_offsets, s.dQf, dKh, dKl, dVh, dVl, mma_scratch, st));
   BWD_OK(rows_gradients(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, s.dQf, dKh, dKl, dVh, dVl, G.dT0, d_items, d_cands, dWq, dWk,
@@ -1181,7 +1191,13 @@ int backward_t(const Plan& p, const T* items, const int32_t* lengths, const T* c
                float* dWq, float* dWk, float* dWv, float* dWg, char* ws, cudaStream_t st, bool tensor) {
   const int N = p.N, d = p.d, H = p.H, Lp = p.Lp, M = p.M, dqk = p.dqk, dvh = p.dvh, U = p.U, L = p.L;
   const size_t UL = (size_t)U * L;
-  if (!tensor && N > 0 && U > 0 && gsta_train_simt_supported(p))
+  // Two to seven candidates per user in bf16: nothing of the tensor-core routes fits, and while the products over the item rows are
+  // small the FP32 route's five launches beat the general route's forty (and their TF32 products): 27 users x 7 candidates of 1578
+  // items, d = 64 387 -> 129 us, 64 x 5 of 2000, d = 96 (12 M elements of items) 1027 -> 810, 500 x 3 of 500, d = 64 (16 M) 570 -> 525; but
+  // 128 x 7 of 1100, d = 128 (18 M) 930 -> 1035, 1000 x 2 of 700, d = 128 (90 M) 1812 -> 3196.
+  const bool few = tensor && sizeof(T) == 2 && !backward_stream_supported(p) && !sta_bwd_mma_supported(p) && sta_bwd_f32_supported(p) &&
+                   (long long)UL * d <= 16ll << 20;
+  if ((!tensor || few) && N > 0 && U > 0 && gsta_train_simt_supported(p))
     return backward_simt<T>(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, Wg, dz, d_items, d_cands, dWq, dWk, dWv, dWg, ws, st);
   if (tensor && N > 0 && U > 0 && backward_stream_supported(p) && gsta_train_supported(p, 2))
     return backward_stream_all<T>(p, items, lengths, cands, cand_offsets, Wq, Wk, Wv, Wg, dz, d_items, d_cands, dWq, dWk, dWv, dWg, ws, st);

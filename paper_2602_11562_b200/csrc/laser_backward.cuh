@@ -23,19 +23,22 @@ bool gsta_train_simt_supported(const Plan& p);
 int gsta_train_simt(const Plan& p, const float* Hp, const int32_t* lengths, const int32_t* cand_offsets, const void* cands,
                     const void* Wg, const float* dz, const GstaTrain& G, float* dHp, cudaStream_t st);
 
-// The same for the widths in use (laser_backward_f32.cu), and the gates: every row of dK and dV, adds to dQf (zeroed before).
-// LASER_ERR_UNSUPPORTED for all other shapes.
-int gsta_train_f32(const Plan& p, const float* Hp, const int32_t* lengths, const int32_t* cand_offsets, const void* cands,
-                   const void* Wg, const float* dz, const GstaTrain& G, float* dHp, cudaStream_t st);
-bool sta_bwd_f32_supported(const Plan& p);
-int sta_bwd_f32(const Plan& p, const float* Qf, const float* Kf, const float* Vf, const float* dHp, const int32_t* lengths,
-                const int32_t* cand_offsets, float* dQf, float* dK, float* dV, cudaStream_t st);
-
 // The same for the tensor-core kernel, as bf16 high and low parts: arrays of [2][M, N, d] and [2][M, N, H, d].
 struct GstaPlanes {
   __nv_bfloat16 *T, *Q, *dT, *dQ, *Mh, *dQt;
   float* dT0;
 };
+
+// FP32 ALUs, the widths in use (laser_backward_f32.cu).  The stacked attention as gsta_train_simt, leaving G or the same as bf16 parts, dH'
+// in fp32 or rounded to bf16 (one of each pair is null); and the gates: every row of dK and dV, adds to dQf (zeroed before).
+// LASER_ERR_UNSUPPORTED for all other shapes.
+bool gsta_train_f32_pays(const Plan& p);      // in place of the tensor-core kernel
+int gsta_train_f32(const Plan& p, const float* Hp, const int32_t* lengths, const int32_t* cand_offsets, const void* cands,
+                   const void* Wg, const float* dz, const GstaTrain* G, const GstaPlanes* planes, float* dHp, __nv_bfloat16* dHp16,
+                   cudaStream_t st);
+bool sta_bwd_f32_supported(const Plan& p);
+int sta_bwd_f32(const Plan& p, const float* Qf, const float* Kf, const float* Vf, const float* dHp, const int32_t* lengths,
+                const int32_t* cand_offsets, float* dQf, float* dK, float* dV, cudaStream_t st);
 
 // Tensor cores (laser_backward_gsta.cu), bf16 inputs: np = 1: segment vectors S0 in bf16; np = 2: segment vectors S0 + S1 (bf16
 // high and low parts of fp32 values).  dS [N, Lp, d] leaves as fp32 in dS32 (np = 2) or rounded to bf16 in dS16, whichever is not

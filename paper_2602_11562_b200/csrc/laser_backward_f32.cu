@@ -28,7 +28,9 @@ struct TrainParams {
   const float* dz;
   const int *lengths, *cand_offsets;
   GstaTrain G;
+  GstaPlanes planes;                     // with planes.T: as bf16 high and low parts, instead of G
   float* dHp;
+  bf16* dHp16;                           // not null: dH' rounded to bf16, instead of dHp
   int U, L, S, Lp, LpP, M, N;            // LpP: L' rounded up to a multiple of 4
   float inv_tau;
 };
@@ -90,19 +92,33 @@ __global__ void __launch_bounds__(kThreads, 2) gsta_train_f32_kernel(const Train
   __syncthreads();
   stage_segments<float, D, CB, DS>(Hs, P.Hp, s_nv, c_base, Lp, tid);
 
-  auto keep = [&](float* dst, const float* src) {          // [CB][D] to the candidates' rows
-    for (int i = tid * 4; i < live; i += kThreads * 4)
-      *reinterpret_cast<float4*>(dst + (size_t)c_base * D + i) = *reinterpret_cast<const float4*>(src + i);
+  const size_t Nd = (size_t)P.N * D;
+  auto put_parts = [](bf16* hi, size_t lo, float4 v) {
+    const uint32_t a = mma::pack2(v.x, v.y), b = mma::pack2(v.z, v.w);
+    *reinterpret_cast<uint2*>(hi) = make_uint2(a, b);
+    *reinterpret_cast<uint2*>(hi + lo) = make_uint2(mma::pack2(v.x - mma::bf16_lo(a), v.y - mma::bf16_hi(a)),
+                                                    mma::pack2(v.z - mma::bf16_lo(b), v.w - mma::bf16_hi(b)));
   };
-  auto keep_heads = [&](float* dst, const float* src) {    // [CB][H][DS] to [N, H, D]
-    for (int i = tid; i < live * H / 4; i += kThreads)
-      *reinterpret_cast<float4*>(dst + (size_t)c_base * H * D + i * 4) =
-          *reinterpret_cast<const float4*>(src + i / kCols * DS + i % kCols * 4);
+  // layer l of an array: [CB][D] to the candidates' rows, in fp32 or in two parts
+  auto keep = [&](float* dst, bf16* parts, int l, const float* src) {
+    for (int i = tid * 4; i < live; i += kThreads * 4) {
+      const float4 v = *reinterpret_cast<const float4*>(src + i);
+      const size_t at = l * Nd + (size_t)c_base * D + i;
+      if (P.planes.T) put_parts(parts + at, M * Nd, v);
+      else *reinterpret_cast<float4*>(dst + at) = v;
+    }
+  };
+  auto keep_heads = [&](float* dst, bf16* parts, int l, const float* src) {    // [CB][H][DS] to [N, H, D]
+    for (int i = tid; i < live * H / 4; i += kThreads) {
+      const float4 v = *reinterpret_cast<const float4*>(src + i / kCols * DS + i % kCols * 4);
+      const size_t at = (l * Nd + (size_t)c_base * D) * H + i * 4;
+      if (P.planes.T) put_parts(parts + at, M * Nd * H, v);
+      else *reinterpret_cast<float4*>(dst + at) = v;
+    }
   };
   auto put4 = [&](float* y) {
     return [=](int i, const float (&s)[4]) { *reinterpret_cast<float4*>(y + i) = make_float4(s[0], s[1], s[2], s[3]); };
   };
-  const size_t Nd = (size_t)P.N * D;
 
   for (int l = 0; l < M; ++l) {
     const T *Wk = Wg + (size_t)(l * 3 + 1) * D * D, *Wv = Wk + D * D;
@@ -113,8 +129,8 @@ __global__ void __launch_bounds__(kThreads, 2) gsta_train_f32_kernel(const Train
     nn.finish(red, tid, put4(ql));
     __syncthreads();
     nt.run(ql, tid, [&](int c, int h, int i, float v) { qtl[(c * H + h) * DS + i] = v * P.inv_tau; });
-    keep(P.G.T + l * Nd, tl);
-    keep(P.G.Q + l * Nd, ql);
+    keep(P.G.T, P.planes.T, l, tl);
+    keep(P.G.Q, P.planes.Q, l, ql);
     __syncthreads();
     scores<D, H, CB, DS>(Hs, qtl, s_nv, Lp, LpP, 1.f, al, tid);
     __syncthreads();
@@ -127,7 +143,7 @@ __global__ void __launch_bounds__(kThreads, 2) gsta_train_f32_kernel(const Train
     __syncthreads();
     nn.run([&](int c, int j) { return (const float*)(ml + (c * H + j / (D / H)) * DS); }, red, tid);
     if (l + 1 < M) nn.load(Wv + D * D, tid);
-    keep_heads(P.G.Mh + l * Nd * H, ml);
+    keep_heads(P.G.Mh, P.planes.Mh, l, ml);
     __syncthreads();
     nn.finish(red, tid, [&](int i, const float (&s)[4]) {
       const float4 v = *reinterpret_cast<const float4*>(tl + i);
@@ -139,7 +155,7 @@ __global__ void __launch_bounds__(kThreads, 2) gsta_train_f32_kernel(const Train
   for (int l = M - 1; l >= 0; --l) {
     const T *Wq = Wg + (size_t)(l * 3) * D * D, *Wk = Wq + D * D;
     float *ml = m + l * CB * H * DS, *dml = dm + l * CB * H * DS, *al = a + l * CB * H * LpP, *del = de + l * CB * H * LpP;
-    keep(P.G.dT + l * Nd, dt);
+    keep(P.G.dT, P.planes.dT, l, dt);
     nt.run(dt, tid, [&](int c, int h, int i, float v) { dml[(c * H + h) * DS + i] = v; });
     __syncthreads();
     scores<D, H, CB, DS>(Hs, dml, s_nv, Lp, LpP, 1.f, del, tid);
@@ -164,7 +180,7 @@ __global__ void __launch_bounds__(kThreads, 2) gsta_train_f32_kernel(const Train
     __syncthreads();
     nn.run([&](int c, int j) { return (const float*)(dqt + (c * H + j / (D / H)) * DS); }, red, tid);
     ntf.load(Wq, tid);
-    keep_heads(P.G.dQt + l * Nd * H, dqt);
+    keep_heads(P.G.dQt, P.planes.dQt, l, dqt);
     __syncthreads();
     nn.finish(red, tid, [&](int i, const float (&s)[4]) {
       *reinterpret_cast<float4*>(dq + i) = make_float4(s[0] * P.inv_tau, s[1] * P.inv_tau, s[2] * P.inv_tau, s[3] * P.inv_tau);
@@ -172,7 +188,7 @@ __global__ void __launch_bounds__(kThreads, 2) gsta_train_f32_kernel(const Train
     __syncthreads();
     ntf.run(dq, tid, [&](int c, int h, int i, float v) { red[(h * CB + c) * D + i] = v; });
     if (l > 0) nt.load(Wq - D * D, tid);                   // W_v of the layer before
-    keep(P.G.dQ + l * Nd, dq);
+    keep(P.G.dQ, P.planes.dQ, l, dq);
     __syncthreads();
     for (int i = tid; i < CB * D; i += kThreads) {
       float v = dt[i];
@@ -182,12 +198,13 @@ __global__ void __launch_bounds__(kThreads, 2) gsta_train_f32_kernel(const Train
     }
     __syncthreads();
   }
-  keep(P.G.dT0, dt);
+  for (int i = tid * 4; i < live; i += kThreads * 4)
+    *reinterpret_cast<float4*>((P.planes.T ? P.planes.dT0 : P.G.dT0) + (size_t)c_base * D + i) = *reinterpret_cast<const float4*>(dt + i);
   // gradient of the segment vectors: thread = (eight segments, four features)
   constexpr int kJ = 8;
   for (int c = 0; c < CB && c_base + c < P.N; ++c) {
     const int nv = s_nv[c], groups = (Lp + kJ - 1) / kJ;
-    float* out = P.dHp + (size_t)(c_base + c) * Lp * D;
+    const size_t out = (size_t)(c_base + c) * Lp * D;
     for (int o = tid; o < groups * kCols; o += kThreads) {
       const int j0 = o / kCols * kJ, i = o % kCols * 4;
       float acc[kJ][4];
@@ -217,8 +234,10 @@ __global__ void __launch_bounds__(kThreads, 2) gsta_train_f32_kernel(const Train
       for (int j = 0; j < kJ; ++j)
         if (j0 + j < Lp) {
           const bool in = j0 + j < nv;                     // (rows of empty segments receive no gradient)
-          *reinterpret_cast<float4*>(out + (size_t)(j0 + j) * D + i) =
-              in ? make_float4(acc[j][0], acc[j][1], acc[j][2], acc[j][3]) : make_float4(0.f, 0.f, 0.f, 0.f);
+          const float4 v = in ? make_float4(acc[j][0], acc[j][1], acc[j][2], acc[j][3]) : make_float4(0.f, 0.f, 0.f, 0.f);
+          const size_t at = out + (size_t)(j0 + j) * D + i;
+          if (P.dHp16) *reinterpret_cast<uint2*>(P.dHp16 + at) = make_uint2(mma::pack2(v.x, v.y), mma::pack2(v.z, v.w));
+          else *reinterpret_cast<float4*>(P.dHp + at) = v;
         }
     }
   }
@@ -230,13 +249,17 @@ template <typename T, int D, int H, int CB>
 int launch_train_cb(const Plan& p, const TrainParams& P, cudaStream_t st) {
   const size_t smem = train_floats<D, H, CB>(P.Lp, P.LpP, P.M) * sizeof(float);
   LASER_CUDA_OK(allow_smem(gsta_train_f32_kernel<T, D, H, CB>, smem));
-  LaunchScope ls("gsta_train_simt", st);
+  LaunchScope ls(P.planes.T ? "gsta_train" : "gsta_train_simt", st);
   LASER_CUDA_OK(launch_chained(gsta_train_f32_kernel<T, D, H, CB>, dim3((p.N + CB - 1) / CB), dim3(kThreads), smem, st, P));
   return LASER_OK;
 }
 
 template <typename T, int D, int H>
-int launch_train(const Plan& p, const TrainParams& P, cudaStream_t st) {
+int launch_train(const Plan& p, const TrainParams& P, cudaStream_t st, int ask, size_t* smem) {
+  if (ask) {                             // only the shared memory of a block of one or two candidates
+    *smem = (ask == 2 ? train_floats<D, H, 2>(P.Lp, P.LpP, P.M) : train_floats<D, H, 1>(P.Lp, P.LpP, P.M)) * 4;
+    return LASER_OK;
+  }
   const int sms = device_sms();
   // Candidates per block as in the forward kernel (launch, laser_simt_gsta.cu).  us (CUDA events, about 6 too long; one | two | four):
   // 270 candidates, d = 64, two heads 17 | 19 | 25; 400, four heads 31 | 23 | 29; 992, d = 32 41 | 27 | 19; 1400, d = 64, four heads 64 | 48 |
@@ -248,19 +271,19 @@ int launch_train(const Plan& p, const TrainParams& P, cudaStream_t st) {
 }
 
 template <typename T>
-int dispatch_train(const Plan& p, const TrainParams& P, cudaStream_t st) {
+int dispatch_train(const Plan& p, const TrainParams& P, cudaStream_t st, int ask = 0, size_t* smem = nullptr) {
   switch (p.d * 16 + p.H) {
-    case 32 * 16 + 1: return launch_train<T, 32, 1>(p, P, st);
-    case 32 * 16 + 2: return launch_train<T, 32, 2>(p, P, st);
-    case 64 * 16 + 1: return launch_train<T, 64, 1>(p, P, st);
-    case 64 * 16 + 2: return launch_train<T, 64, 2>(p, P, st);
-    case 64 * 16 + 4: return launch_train<T, 64, 4>(p, P, st);
-    case 96 * 16 + 3: return launch_train<T, 96, 3>(p, P, st);
-    case 96 * 16 + 6: return launch_train<T, 96, 6>(p, P, st);
-    case 128 * 16 + 1: return launch_train<T, 128, 1>(p, P, st);
-    case 128 * 16 + 2: return launch_train<T, 128, 2>(p, P, st);
-    case 128 * 16 + 4: return launch_train<T, 128, 4>(p, P, st);
-    case 128 * 16 + 8: return launch_train<T, 128, 8>(p, P, st);
+    case 32 * 16 + 1: return launch_train<T, 32, 1>(p, P, st, ask, smem);
+    case 32 * 16 + 2: return launch_train<T, 32, 2>(p, P, st, ask, smem);
+    case 64 * 16 + 1: return launch_train<T, 64, 1>(p, P, st, ask, smem);
+    case 64 * 16 + 2: return launch_train<T, 64, 2>(p, P, st, ask, smem);
+    case 64 * 16 + 4: return launch_train<T, 64, 4>(p, P, st, ask, smem);
+    case 96 * 16 + 3: return launch_train<T, 96, 3>(p, P, st, ask, smem);
+    case 96 * 16 + 6: return launch_train<T, 96, 6>(p, P, st, ask, smem);
+    case 128 * 16 + 1: return launch_train<T, 128, 1>(p, P, st, ask, smem);
+    case 128 * 16 + 2: return launch_train<T, 128, 2>(p, P, st, ask, smem);
+    case 128 * 16 + 4: return launch_train<T, 128, 4>(p, P, st, ask, smem);
+    case 128 * 16 + 8: return launch_train<T, 128, 8>(p, P, st, ask, smem);
     default: return LASER_ERR_UNSUPPORTED;
   }
 }
@@ -502,10 +525,27 @@ bool gate_plan(const Plan& p, GateParams* params, int* split, size_t* smem) {
 
 }  // namespace
 
+// In place of the tensor-core kernel (laser_backward_gsta.cu), whose candidates go through their phases on one warp each: while few
+// candidates leave its SMs with a warp or two, a block per candidate or two is faster, as long as they all run at once.  us per call:
+// 99 candidates, d = 96, six heads, 121 segments 117 -> 76; 27, d = 64, 87 segments 54 -> 42; 300, d = 64, two heads 108 -> 89; 500, d = 128,
+// four heads 86 -> 72; but 1000, d = 64, four heads 53 -> 58, and 300, d = 128, eight heads, 100 segments (one block per SM) 112 -> 131.
+bool gsta_train_f32_pays(const Plan& p) {
+  if (p.M == 0 || p.N > 4 * device_sms()) return false;
+  TrainParams P = {};
+  P.Lp = p.Lp; P.LpP = (p.Lp + 3) & ~3; P.M = p.M;
+  const long long at_once = (long long)device_sms() * (p.N > 2 * device_sms() ? 2 : 1);      // candidates, one block per SM
+  size_t smem;
+  if (dispatch_train<float>(p, P, nullptr, p.N > 2 * device_sms() ? 2 : 1, &smem) != LASER_OK || smem > kMost) return false;
+  return p.N <= at_once * (smem <= kMost / 2 ? 2 : 1);
+}
+
 int gsta_train_f32(const Plan& p, const float* Hp, const int32_t* lengths, const int32_t* cand_offsets, const void* cands,
-                   const void* Wg, const float* dz, const GstaTrain& G, float* dHp, cudaStream_t st) {
-  TrainParams P;
-  P.Hp = Hp; P.cands = cands; P.Wg = Wg; P.dz = dz; P.lengths = lengths; P.cand_offsets = cand_offsets; P.G = G; P.dHp = dHp;
+                   const void* Wg, const float* dz, const GstaTrain* G, const GstaPlanes* planes, float* dHp, __nv_bfloat16* dHp16,
+                   cudaStream_t st) {
+  TrainParams P = {};
+  P.Hp = Hp; P.cands = cands; P.Wg = Wg; P.dz = dz; P.lengths = lengths; P.cand_offsets = cand_offsets; P.dHp = dHp; P.dHp16 = dHp16;
+  if (G) P.G = *G;
+  if (planes) P.planes = *planes;
   P.U = p.U; P.L = p.L; P.S = p.S; P.Lp = p.Lp; P.LpP = (p.Lp + 3) & ~3; P.M = p.M; P.N = p.N; P.inv_tau = p.inv_tau;
   return p.dtype == LASER_F32 ? dispatch_train<float>(p, P, st) : dispatch_train<bf16>(p, P, st);
 }

@@ -61,6 +61,7 @@ RowsPair pair_up(const RowsParams& items, const RowsParams& cands, long long mos
     P.first[r] = apart && r == 1 ? P.blocks[0] : 0;
   }
   *grid = apart ? P.blocks[0] + P.blocks[1] : std::max(P.blocks[0], P.blocks[1]);
+  if (!apart) P.first[1] = (int)*grid - P.blocks[1];      // few candidate tiles: to the last blocks, the first have the most item tiles
   return P;
 }
 
@@ -457,7 +458,7 @@ int launch_project(const ProjectJob& J, cudaStream_t st) {
   P.zero = J.zero;
   P.prep = J.prep;
   P.row_blocks = (int)grid;
-  P.prep_blocks = std::min((J.prep.M * 6 * D16 * D16 * 32 + kRThreads - 1) / kRThreads, sms);
+  P.prep_blocks = !J.prep.img ? 0 : std::min((J.prep.M * 6 * D16 * D16 * 32 + kRThreads - 1) / kRThreads, sms);
   LaunchScope ls("bwd_rows_project", st);
   LASER_CUDA_OK(launch_chained(rows_project_kernel<D16>, dim3(grid + P.prep_blocks + (J.prep.order ? 1 : 0)), dim3(kRThreads), smem, st, P));
   return LASER_OK;

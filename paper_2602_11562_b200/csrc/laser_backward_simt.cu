@@ -434,7 +434,7 @@ bool gsta_train_simt_supported(const Plan& p) { return p.M > 0 && train_simt_sme
 
 int gsta_train_simt(const Plan& p, const float* Hp, const int32_t* lengths, const int32_t* cand_offsets, const void* cands,
                     const void* Wg, const float* dz, const GstaTrain& G, float* dHp, cudaStream_t st) {
-  const int rc = gsta_train_f32(p, Hp, lengths, cand_offsets, cands, Wg, dz, G, dHp, st);
+  const int rc = gsta_train_f32(p, Hp, lengths, cand_offsets, cands, Wg, dz, &G, nullptr, dHp, nullptr, st);
   if (rc != LASER_ERR_UNSUPPORTED) return rc;
   if (p.dtype == LASER_F32)
     return train_t<float>(p, Hp, lengths, cand_offsets, (const float*)cands, (const float*)Wg, dz, G, dHp, st);

@@ -1,0 +1,62 @@
+"""bf16 backward on either side of the lines between its kernels: the stacked attention of few candidates (FP32 ALUs) and of more (tensor
+cores), two to seven candidates per user on the FP32 route and on the general one; against the float64 oracle."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2602_11562_b200 as P
+from oracle import backward_oracle
+from workloads import make_custom
+
+pytestmark = pytest.mark.gpu
+
+
+def _run(kw, seed, bar, launches=None):
+    w = make_custom(seed=seed, dtype="bf16", d_qh=16, emb_std="inv_sqrt_d", **kw)
+    s = w.spec
+    dz = np.random.default_rng(seed).standard_normal((w.N, s.d)).astype(np.float32)
+    ref = backward_oracle.backward(w.items, w.lengths, w.cands, w.cand_offsets, w.Wq, w.Wk, w.Wv, w.Wg, s.S, s.H, dz.astype(np.float64),
+                                   w.gamma, w.tau)
+    b = P.DeviceBatch.from_workload(w)
+    ws = torch.empty(P.laser_backward_workspace_bytes(b.cfg), dtype=torch.uint8, device="cuda")
+    ws.fill_(0xFF)
+    got = P.laser_backward(b.cfg, *b.args(), b.Wg, torch.from_numpy(dz).cuda(), workspace=ws)
+    assert P.laser_check_status(ws) == 0
+    if launches is not None:
+        assert P.laser_last_launch_count() <= launches
+    for k, r in ref.items():
+        g = got[k].cpu().numpy().astype(np.float64)
+        assert np.isfinite(g).all() and np.max(np.abs(g - r)) <= bar * max(float(np.max(np.abs(r))), 1e-30), k
+
+
+# the tensor-core stacked attention from 593 candidates on: one candidate per user on pairs (slots in several steps), lists on one part
+# and on pairs
+@pytest.mark.parametrize("kw", [
+    dict(U=593, C=1, L=20, d=96, H=6, S=4, M=3),
+    dict(U=600, C=1, L=18, d=128, H=8, S=3, M=2),
+    dict(U=3, C=200, L=64, d=64, H=4, S=8, M=2),
+    dict(U=4, C=150, L=90, d=96, H=6, S=9, M=2),
+    dict(U=2, C=300, L=90, d=128, H=8, S=3, M=1),
+])
+def test_many_candidates(kw):
+    _run(kw, 41, 2e-3 if kw["C"] == 1 else 2e-2)
+
+
+# ... and the FP32 one up to there: one, then two candidates per block; one block per SM where two do not fit
+@pytest.mark.parametrize("kw", [
+    dict(U=296, C=1, L=20, d=64, H=2, S=4, M=2),
+    dict(U=297, C=1, L=20, d=32, H=1, S=4, M=1),
+    dict(U=2, C=296, L=40, d=64, H=4, S=8, M=1),
+    dict(U=1, C=148, L=130, d=128, H=8, S=1, M=1),
+    dict(U=1, C=149, L=130, d=128, H=8, S=1, M=1),
+])
+def test_few_candidates(kw):
+    _run(kw, 42, 2e-3 if kw["C"] == 1 else 2e-2)
+
+
+# two to seven per user: sums of a few hundred fp32 terms, as for fp32 batches; the general route's products are TF32
+@pytest.mark.parametrize("kw", [dict(U=5, C=2, L=90, d=64, H=1, S=12, M=2), dict(U=3, C=7, L=70, d=128, H=8, S=9, M=1),
+                                dict(U=9, C=5, L=33, d=96, H=3, S=40, M=3)])
+def test_two_to_seven_candidates(kw):
+    _run(kw, 43, 1e-4, launches=5)
+    _run(dict(kw, U=2, L=90, d=48, H=3), 44, 2e-3)                   # (a width that neither new kernel takes)
