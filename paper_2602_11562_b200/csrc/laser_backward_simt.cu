@@ -4,6 +4,7 @@
 
 #include "laser_backward.cuh"
 #include "laser_common.cuh"
+#include "laser_mma.cuh"
 
 namespace laser {
 namespace {
@@ -317,22 +318,25 @@ int train_t(const Plan& p, const float* Hp, const int32_t* lengths, const int32_
 }
 
 // ------------------------------------------------------------------------------------------------ dense products
-// Every product of a list in one launch: C (64 x 64 tiles, 256 threads of 4 x 4) = D + alpha (A B + A2 B2), or C += by atomic
-// adds of slices of the contraction.  A block finds its product, tile, batch entry and slice from its index.  Tiles of 16
-// contraction steps are fetched a step ahead into registers, four consecutive elements at a time where the layout allows.
-// (One launch per product before: at a few hundred candidates each ran 2 to 12 blocks for 10 to 40 us.)
-constexpr int kTile = 64, kStep = 16;
+// Every product of a list in one launch: C = D + alpha (A B + A2 B2), or C += by atomic adds of slices of the contraction.  A block
+// finds its product, tile, batch entry and slice from its index.  Tiles of 64 rows x 64, 32 or 16 columns, as many as the product has:
+// a thread has 4 x 4 of them, and in the narrow ones (a head's 16 or 32 columns) two or four groups of threads take every second or
+// fourth step of the contraction (in 64-wide tiles three quarters of the weight sums of 16-wide heads were multiplications by zero).
+// Contraction steps come 32 at a time, fetched a round ahead into registers, four consecutive elements at a time where the layout
+// allows.  27 users x 49 candidates of 315 items, d = 96, six heads, two layers 62 -> 56 us, 75 x 23 of 169, d = 32
+// 19 -> 15, the two lists of 63 users with one candidate each, d = 96, six heads 11 + 9 -> 7 + 7.  Bound by issue (64 %) and shared-memory
+// reads (67 %).
+constexpr int kTile = 64, kStep = 32, kPitch = kTile + 4;
 struct ProductList {
   Product p[kMaxProducts];
   int first[kMaxProducts + 1];             // first block of each product
   int n;
 };
+__host__ __device__ inline int tile_cols(int N) { return N <= 16 ? 16 : (N + 31) % kTile < 32 ? kTile : 32; }
 
 template <typename TX>
-__device__ __forceinline__ void fetch4(float (&v)[4], const TX* X, int ld, bool k_major, int r0, int R, int k0, int K, int tid,
-                                       bool vec) {
-  // k_major: X[k ld + r], thread = (k, four rows); else X[r ld + k], thread = (row, four k)
-  const int r = r0 + (k_major ? (tid & 15) * 4 : tid >> 2), k = k0 + (k_major ? tid >> 4 : (tid & 3) * 4);
+__device__ __forceinline__ void fetch4(float (&v)[4], const TX* X, int ld, bool k_major, int r, int R, int k, int K, bool vec) {
+  // k_major: X[k ld + r], four rows; else X[r ld + k], four k
   const TX* src = k_major ? X + (size_t)k * ld + r : X + (size_t)r * ld + k;
   if (vec && r + (k_major ? 4 : 1) <= R && k + (k_major ? 1 : 4) <= K) {
     if constexpr (sizeof(TX) == 4) {
@@ -351,71 +355,124 @@ __device__ __forceinline__ void fetch4(float (&v)[4], const TX* X, int ld, bool 
     v[e] = in ? to_f32<TX>(src[e]) : 0.f;
   }
 }
-__device__ __forceinline__ void fetch4_any(float (&v)[4], const void* X, bool is16, int ld, bool k_major, int r0, int R, int k0,
-                                           int K, int tid) {
-  const bool vec = ld % 4 == 0 && (reinterpret_cast<uintptr_t>(X) & (is16 ? 7 : 15)) == 0;
-  if (is16) fetch4<bf16>(v, (const bf16*)X, ld, k_major, r0, R, k0, K, tid, vec);
-  else fetch4<float>(v, (const float*)X, ld, k_major, r0, R, k0, K, tid, vec);
-}
-// shared layout [k][64 + 4]
-__device__ __forceinline__ void put4(float* sm, const float (&v)[4], bool k_major, int tid) {
-  if (k_major) {
-    *reinterpret_cast<float4*>(sm + (tid >> 4) * (kTile + 4) + (tid & 15) * 4) = make_float4(v[0], v[1], v[2], v[3]);
-  } else {
+// A thread's share of a round: four elements of each half.  k_major: thread = (k, four rows), else (row, four k).
+struct Fetch {
+  const void* X;
+  int ld, r0, R;
+  bool is16, k_major, vec;
+  __device__ __forceinline__ Fetch(const void* x, bool b16, int l, bool km, int r, int rows)
+      : X(x), ld(l), r0(r), R(rows), is16(b16), k_major(km), vec(l % 4 == 0 && (reinterpret_cast<uintptr_t>(x) & (b16 ? 7 : 15)) == 0) {}
+  __device__ __forceinline__ void load(float (&v)[2][4], int k0, int K, int tid) const {
 #pragma unroll
-    for (int e = 0; e < 4; ++e) sm[((tid & 3) * 4 + e) * (kTile + 4) + (tid >> 2)] = v[e];
+    for (int half = 0; half < 2; ++half) {
+      const int r = r0 + (k_major ? (tid & 15) * 4 : tid >> 2), k = k0 + (k_major ? (tid >> 4) + 16 * half : ((tid & 3) + 4 * half) * 4);
+      if (is16) fetch4<bf16>(v[half], static_cast<const bf16*>(X), ld, k_major, r, R, k, K, vec);
+      else fetch4<float>(v[half], static_cast<const float*>(X), ld, k_major, r, R, k, K, vec);
+    }
+  }
+  // shared layout [k][64 + 4]
+  __device__ __forceinline__ void put(float* sm, const float (&v)[2][4], int tid) const {
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+      if (k_major) {
+        *reinterpret_cast<float4*>(sm + ((tid >> 4) + 16 * half) * kPitch + (tid & 15) * 4) = make_float4(v[half][0], v[half][1], v[half][2], v[half][3]);
+      } else {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) sm[(((tid & 3) + 4 * half) * 4 + e) * kPitch + (tid >> 2)] = v[half][e];
+      }
+    }
+  }
+};
+
+template <int COLS>
+__device__ __forceinline__ void multiply(float (&acc)[4][4], const float* As, const float* Bs, int tid) {
+  constexpr int kGroups = kTile / COLS, kTx = COLS / 4;
+  const int grp = tid / (16 * kTx), tx = tid % kTx, ty = tid / kTx % 16;
+#pragma unroll
+  for (int kk = 0; kk < kStep; kk += kGroups) {
+    const float4 a4 = *reinterpret_cast<const float4*>(As + (kk + grp) * kPitch + ty * 4);
+    const float4 b4 = *reinterpret_cast<const float4*>(Bs + (kk + grp) * kPitch + tx * 4);
+    const float a[4] = {a4.x, a4.y, a4.z, a4.w}, b[4] = {b4.x, b4.y, b4.z, b4.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
   }
 }
 
 __global__ void __launch_bounds__(256) products_kernel(const __grid_constant__ ProductList L) {
-  __shared__ __align__(16) float As[2][kStep * (kTile + 4)], Bs[2][kStep * (kTile + 4)];
+  __shared__ __align__(16) float sm[4 * kStep * kPitch];   // A and B, two buffers each; the groups' sums at the end
   chain_wait();
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int tid = threadIdx.x;
   int which = 0;
   while (which + 1 < L.n && (int)blockIdx.x >= L.first[which + 1]) ++which;
   const Product& P = L.p[which];
   int b = blockIdx.x - L.first[which];
-  const int tiles_n = (P.N + kTile - 1) / kTile, tiles = (P.M + kTile - 1) / kTile * tiles_n;
+  const int cols = tile_cols(P.N), tiles_n = (P.N + cols - 1) / cols, tiles = (P.M + kTile - 1) / kTile * tiles_n;
   const int slice = b / (tiles * P.batch);
   b -= slice * tiles * P.batch;
   const int bat = b / tiles, tile = b - bat * tiles;
-  const int m0 = tile / tiles_n * kTile, n0 = tile % tiles_n * kTile;
+  const int m0 = tile / tiles_n * kTile, n0 = tile % tiles_n * cols;
   float acc[4][4] = {};
   for (int seg = 0; seg < (P.A2 ? 2 : 1); ++seg) {
-    const void* A = seg ? P.A2 : (const char*)P.A + (size_t)bat * P.sa * (P.a16 ? 2 : 4);
-    const void* B = seg ? P.B2 : (const char*)P.B + (size_t)bat * P.sb * (P.b16 ? 2 : 4);
-    const int K = seg ? P.K2 : P.K, lda = seg ? P.lda2 : P.lda, ldb = seg ? P.ldb2 : P.ldb;
-    const int k_lo = slice * P.k_per, k_hi = seg ? K : min(K, k_lo + P.k_per);
-    float va[4], vb[4];
+    const Fetch A(seg ? P.A2 : (const char*)P.A + (size_t)bat * P.sa * (P.a16 ? 2 : 4), P.a16, seg ? P.lda2 : P.lda, P.ta, m0, P.M);
+    const Fetch B(seg ? P.B2 : (const char*)P.B + (size_t)bat * P.sb * (P.b16 ? 2 : 4), P.b16, seg ? P.ldb2 : P.ldb, !P.tb, n0, P.N);
+    const int K = seg ? P.K2 : P.K, k_lo = slice * P.k_per, k_hi = seg ? K : min(K, k_lo + P.k_per);
+    float va[2][4], vb[2][4];
     int buf = 0;
-    fetch4_any(va, A, P.a16, lda, P.ta, m0, P.M, k_lo, k_hi, tid);
-    fetch4_any(vb, B, P.b16, ldb, !P.tb, n0, P.N, k_lo, k_hi, tid);
+    A.load(va, k_lo, k_hi, tid);
+    B.load(vb, k_lo, k_hi, tid);
     for (int k0 = k_lo; k0 < k_hi; k0 += kStep, buf ^= 1) {
-      put4(As[buf], va, P.ta, tid);
-      put4(Bs[buf], vb, !P.tb, tid);
+      float *As = sm + buf * kStep * kPitch, *Bs = As + 2 * kStep * kPitch;
+      A.put(As, va, tid);
+      B.put(Bs, vb, tid);
       __syncthreads();
       if (k0 + kStep < k_hi) {
-        fetch4_any(va, A, P.a16, lda, P.ta, m0, P.M, k0 + kStep, k_hi, tid);
-        fetch4_any(vb, B, P.b16, ldb, !P.tb, n0, P.N, k0 + kStep, k_hi, tid);
+        A.load(va, k0 + kStep, k_hi, tid);
+        B.load(vb, k0 + kStep, k_hi, tid);
       }
-#pragma unroll
-      for (int kk = 0; kk < kStep; ++kk) {
-        const float4 a4 = *reinterpret_cast<const float4*>(As[buf] + kk * (kTile + 4) + ty * 4);
-        const float4 b4 = *reinterpret_cast<const float4*>(Bs[buf] + kk * (kTile + 4) + tx * 4);
-        const float a[4] = {a4.x, a4.y, a4.z, a4.w}, bb[4] = {b4.x, b4.y, b4.z, b4.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], bb[j], acc[i][j]);
-      }
+      if (cols == kTile) multiply<64>(acc, As, Bs, tid);
+      else if (cols == 32) multiply<32>(acc, As, Bs, tid);
+      else multiply<16>(acc, As, Bs, tid);
     }
-    __syncthreads();                       // (two buffers: one barrier per step, and one before the other pair of operands)
+    __syncthreads();                       // (two buffers: one barrier per round, and one before the other pair of operands)
+  }
+  const int tx = tid % (cols / 4), ty = tid / (cols / 4) % 16;
+  if (cols < kTile) {                      // the groups' sums, to the first group
+    const int groups = kTile / cols, per = 256 / groups, grp = tid / per;
+    float4* mine = reinterpret_cast<float4*>(sm) + (size_t)grp * per * 4 + tid % per;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) mine[i * per] = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+    __syncthreads();
+    if (grp > 0) return;
+    for (int k = 1; k < groups; ++k)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float4 v = mine[(k * 4 + i) * per];
+        acc[i][0] += v.x; acc[i][1] += v.y; acc[i][2] += v.z; acc[i][3] += v.w;
+      }
   }
   float* C = P.C + (size_t)bat * P.sc;
+  const bool whole = n0 + tx * 4 + 4 <= P.N && P.ldc % 4 == 0 && (reinterpret_cast<uintptr_t>(C) & 15) == 0 &&
+                     (reinterpret_cast<uintptr_t>(P.D) & 15) == 0;      // four columns with one access
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const int m = m0 + ty * 4 + i;
     if (m >= P.M) continue;
+    if (whole) {
+      const size_t at = (size_t)m * P.ldc + n0 + tx * 4;
+      float4 v = make_float4(P.alpha * acc[i][0], P.alpha * acc[i][1], P.alpha * acc[i][2], P.alpha * acc[i][3]);
+      if (P.atomic) {
+        mma::red_add4(C + at, v.x, v.y, v.z, v.w);
+      } else {
+        if (P.D) {
+          const float4 w = *reinterpret_cast<const float4*>(P.D + at);
+          v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
+        }
+        *reinterpret_cast<float4*>(C + at) = v;
+      }
+      continue;
+    }
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const int n = n0 + tx * 4 + j;
@@ -448,11 +505,12 @@ int run_products(Product* list, int n, cudaStream_t st) {
     long long blocks = 0;
     for (int i = 0; i < L.n; ++i) {
       Product& P = list[i0 + i];
-      const long long tiles = (long long)((P.M + kTile - 1) / kTile) * ((P.N + kTile - 1) / kTile) * P.batch;
+      const int cols = tile_cols(P.N);
+      const long long tiles = (long long)((P.M + kTile - 1) / kTile) * ((P.N + cols - 1) / cols) * P.batch;
       int slices = 1;
       P.k_per = std::max(P.K, 1);
       if (P.atomic) {                      // slices of at least 64 rows, longer when a product still gets about two blocks per SM
-        P.k_per = (int)std::min<long long>(std::max<long long>(64, ((long long)P.K * tiles / (2 * device_sms()) + 15) / 16 * 16), 1 << 24);
+        P.k_per = (int)std::min<long long>(std::max<long long>(64, ((long long)P.K * tiles / (2 * device_sms()) + kStep - 1) / kStep * kStep), 1 << 24);
         slices = (P.K + P.k_per - 1) / P.k_per;
       }
       L.p[i] = P;
