@@ -200,8 +200,10 @@ def _raw_stream(device_index: int) -> int:
     return torch._C._cuda_getCurrentRawStream(device_index)
 
 
+# (Sizes go to torch.empty one by one throughout this file: as a tuple each call takes 1 us longer, and a small call's time is the
+# host's: a training step of six outputs 15 us of 40.)
 def _dev(t: torch.Tensor, dtype, name: str) -> int:
-    if not (isinstance(t, torch.Tensor) and t.is_cuda and t.is_contiguous() and t.dtype == dtype):
+    if not (isinstance(t, torch.Tensor) and t.is_cuda and t.is_contiguous() and t.dtype is dtype):
         raise TypeError(f"{name}: expected a contiguous CUDA tensor of {dtype}")
     return t.data_ptr()
 
@@ -225,7 +227,7 @@ def laser_sta_forward(cfg, items, lengths, cands, cand_offsets, Wq, Wk, Wv, Hpri
     lib, dt = load_library(), cfg.torch_dtype()
     ws = _workspace(cfg, workspace, items.device)
     if Hprime is None:
-        Hprime = torch.empty((cfg.total_cands, cfg.n_seg, cfg.d_model), dtype=dt, device=items.device)
+        Hprime = torch.empty(cfg.total_cands, cfg.n_seg, cfg.d_model, dtype=dt, device=items.device)
     rc = lib.laser_sta_forward(ctypes.byref(cfg), _dev(items, dt, "items"), _dev(lengths, torch.int32, "lengths"),
                                _dev(cands, dt, "cands"), _dev(cand_offsets, torch.int32, "cand_offsets"),
                                _dev(Wq, dt, "Wq"), _dev(Wk, dt, "Wk"), _dev(Wv, dt, "Wv"), _dev(Hprime, dt, "Hprime"),
@@ -255,7 +257,7 @@ def laser_gsta_forward(cfg, Hprime, lengths, cand_offsets, cands, Wgsta, z=None,
     lib, dt = load_library(), cfg.torch_dtype()
     ws = _workspace(cfg, workspace, Hprime.device)
     if z is None:
-        z = torch.empty((cfg.total_cands, cfg.d_model), dtype=dt, device=Hprime.device)
+        z = torch.empty(cfg.total_cands, cfg.d_model, dtype=dt, device=Hprime.device)
     rc = lib.laser_gsta_forward(ctypes.byref(cfg), _dev(Hprime, dt, "Hprime"), _dev(lengths, torch.int32, "lengths"),
                                 _dev(cand_offsets, torch.int32, "cand_offsets"), _dev(cands, dt, "cands"),
                                 _dev(Wgsta, dt, "Wgsta"), _dev(z, dt, "z"), ws.data_ptr(), ws.numel(),
@@ -270,9 +272,9 @@ def laser_forward(cfg, items, lengths, cands, cand_offsets, Wq, Wk, Wv, Wgsta, H
     lib, dt = load_library(), cfg.torch_dtype()
     ws = _workspace(cfg, workspace, items.device)
     if z is None:
-        z = torch.empty((cfg.total_cands, cfg.d_model), dtype=dt, device=items.device)
+        z = torch.empty(cfg.total_cands, cfg.d_model, dtype=dt, device=items.device)
     if Hprime is None and want_hprime:
-        Hprime = torch.empty((cfg.total_cands, cfg.n_seg, cfg.d_model), dtype=dt, device=items.device)
+        Hprime = torch.empty(cfg.total_cands, cfg.n_seg, cfg.d_model, dtype=dt, device=items.device)
     rc = lib.laser_forward(ctypes.byref(cfg), _dev(items, dt, "items"), _dev(lengths, torch.int32, "lengths"),
                            _dev(cands, dt, "cands"), _dev(cand_offsets, torch.int32, "cand_offsets"),
                            _dev(Wq, dt, "Wq"), _dev(Wk, dt, "Wk"), _dev(Wv, dt, "Wv"), _dev(Wgsta, dt, "Wgsta"),
@@ -288,9 +290,9 @@ def laser_forward_packed(cfg, items_packed, item_offsets, lengths, cands, cand_o
     lib, dt = load_library(), cfg.torch_dtype()
     ws = _workspace(cfg, workspace, items_packed.device)
     if z is None:
-        z = torch.empty((cfg.total_cands, cfg.d_model), dtype=dt, device=items_packed.device)
+        z = torch.empty(cfg.total_cands, cfg.d_model, dtype=dt, device=items_packed.device)
     if Hprime is None and want_hprime:
-        Hprime = torch.empty((cfg.total_cands, cfg.n_seg, cfg.d_model), dtype=dt, device=items_packed.device)
+        Hprime = torch.empty(cfg.total_cands, cfg.n_seg, cfg.d_model, dtype=dt, device=items_packed.device)
     rc = lib.laser_forward_packed(ctypes.byref(cfg), _dev(items_packed, dt, "items_packed"),
                                   _dev(item_offsets, torch.int32, "item_offsets"), _dev(lengths, torch.int32, "lengths"),
                                   _dev(cands, dt, "cands"), _dev(cand_offsets, torch.int32, "cand_offsets"),
@@ -307,7 +309,7 @@ def laser_fusion_forward(cfg, Hprime, z, lengths, cand_offsets, num_recent, fuse
     if workspace is None:
         workspace = torch.empty(256, dtype=torch.uint8, device=Hprime.device)
     if fused is None:
-        fused = torch.empty((cfg.total_cands, (2 + num_recent) * cfg.d_model), dtype=dt, device=Hprime.device)
+        fused = torch.empty(cfg.total_cands, (2 + num_recent) * cfg.d_model, dtype=dt, device=Hprime.device)
     rc = lib.laser_fusion_forward(ctypes.byref(cfg), _dev(Hprime, dt, "Hprime"), _dev(z, dt, "z"),
                                   _dev(lengths, torch.int32, "lengths"), _dev(cand_offsets, torch.int32, "cand_offsets"),
                                   int(num_recent), _dev(fused, dt, "fused"), workspace.data_ptr(), workspace.numel(),
@@ -329,7 +331,7 @@ def laser_sta_softmax_forward(cfg, items, lengths, cands, cand_offsets, Wq, Wk, 
         raise LaserError(-1, "laser_sta_softmax_workspace_bytes (invalid or unsupported configuration)")
     ws = torch.empty(need, dtype=torch.uint8, device=items.device) if workspace is None else workspace
     if Hprime is None:
-        Hprime = torch.empty((cfg.total_cands, cfg.n_seg, cfg.d_model), dtype=dt, device=items.device)
+        Hprime = torch.empty(cfg.total_cands, cfg.n_seg, cfg.d_model, dtype=dt, device=items.device)
     rc = lib.laser_sta_softmax_forward(ctypes.byref(cfg), _dev(items, dt, "items"), _dev(lengths, torch.int32, "lengths"),
                                        _dev(cands, dt, "cands"), _dev(cand_offsets, torch.int32, "cand_offsets"),
                                        _dev(Wq, dt, "Wq"), _dev(Wk, dt, "Wk"), _dev(Wv, dt, "Wv"),
@@ -352,12 +354,12 @@ def laser_backward(cfg, items, lengths, cands, cand_offsets, Wq, Wk, Wv, Wg, dz,
     dev = items.device
     ws = torch.empty(need, dtype=torch.uint8, device=dev) if workspace is None else workspace
     f32 = torch.float32
-    out = {"d_items": torch.empty((cfg.num_users, cfg.max_len, cfg.d_model), dtype=f32, device=dev),
-           "d_cands": torch.empty((cfg.total_cands, cfg.d_model), dtype=f32, device=dev),
-           "dWq": torch.empty((cfg.d_model, cfg.d_qk), dtype=f32, device=dev),
-           "dWk": torch.empty((cfg.d_model, cfg.d_qk), dtype=f32, device=dev),
-           "dWv": torch.empty((cfg.d_model, cfg.d_model), dtype=f32, device=dev),
-           "dWg": torch.empty((cfg.num_gsta_layers, 3, cfg.d_model, cfg.d_model), dtype=f32, device=dev)}
+    out = {"d_items": torch.empty(cfg.num_users, cfg.max_len, cfg.d_model, dtype=f32, device=dev),
+           "d_cands": torch.empty(cfg.total_cands, cfg.d_model, dtype=f32, device=dev),
+           "dWq": torch.empty(cfg.d_model, cfg.d_qk, dtype=f32, device=dev),
+           "dWk": torch.empty(cfg.d_model, cfg.d_qk, dtype=f32, device=dev),
+           "dWv": torch.empty(cfg.d_model, cfg.d_model, dtype=f32, device=dev),
+           "dWg": torch.empty(cfg.num_gsta_layers, 3, cfg.d_model, cfg.d_model, dtype=f32, device=dev)}
     rc = lib.laser_backward(ctypes.byref(cfg), _dev(items, dt, "items"), _dev(lengths, torch.int32, "lengths"),
                             _dev(cands, dt, "cands"), _dev(cand_offsets, torch.int32, "cand_offsets"),
                             _dev(Wq, dt, "Wq"), _dev(Wk, dt, "Wk"), _dev(Wv, dt, "Wv"), _dev(Wg, dt, "Wg"),
@@ -407,9 +409,9 @@ def laser_forward_ffn(cfg, items, lengths, cands, cand_offsets, Wq, Wk, Wv, Wgst
     params, hid = _ffn_params(cfg, ffn, ln_eps)
     ws = _ffn_workspace(cfg, hid, workspace, items.device)
     if z is None:
-        z = torch.empty((cfg.total_cands, cfg.d_model), dtype=dt, device=items.device)
+        z = torch.empty(cfg.total_cands, cfg.d_model, dtype=dt, device=items.device)
     if Hprime is None and want_hprime:
-        Hprime = torch.empty((cfg.total_cands, cfg.n_seg, cfg.d_model), dtype=dt, device=items.device)
+        Hprime = torch.empty(cfg.total_cands, cfg.n_seg, cfg.d_model, dtype=dt, device=items.device)
     rc = lib.laser_forward_ffn(ctypes.byref(cfg), _dev(items, dt, "items"), _dev(lengths, torch.int32, "lengths"),
                                _dev(cands, dt, "cands"), _dev(cand_offsets, torch.int32, "cand_offsets"),
                                _dev(Wq, dt, "Wq"), _dev(Wk, dt, "Wk"), _dev(Wv, dt, "Wv"), _dev(Wgsta, dt, "Wgsta"),
