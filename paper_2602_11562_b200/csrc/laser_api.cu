@@ -777,6 +777,7 @@ int laser_forward_host(const laser_config* cfg, const void* items_h, const int32
   // the scores straight into pinned host memory, as the last kernel makes them (it writes each once, 16 bytes at a time): 64 x 256
   // candidates 1136 -> 1065 us per call, of which the copy behind the kernel was 77
   void* z_alias = s.b_z > 0 && p.path != LASER_PATH_SIMT && gsta_mma_supported(p) ? device_alias(z_h) : nullptr;
+  p.z_on_host = z_alias != nullptr;
   rc = forward_impl(p, ws + s.items, reinterpret_cast<const int32_t*>(ws + s.lengths), ws + s.cands,
                     reinterpret_cast<const int32_t*>(ws + s.offs), ws + s.wq, ws + s.wk, ws + s.wv, ws + s.wg, nullptr,
                     z_alias ? z_alias : ws + s.z, ws, st);

@@ -29,6 +29,7 @@ struct Plan {
   float inv_gamma, inv_tau;
   size_t esize;
   bool zero_in_ffn;                // the FFN kernel writes the zero rows of empty segments, STA's extra kernel does not
+  bool z_on_host;                  // the scores go straight to (pinned) host memory
   struct SideLaunches* side;       // launches that the STA path makes room for between its own (null: none)
   const int32_t* item_offsets;     // packed item layout: first row of every user ([U + 1]); null = padded [U, L, d]
   // workspace byte offsets

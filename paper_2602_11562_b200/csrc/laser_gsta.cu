@@ -66,7 +66,8 @@ __global__ void __launch_bounds__(256) gsta_prep_kernel(GstaParams P) {
 // shared memory per block) for grids of several waves, where the kernel is latency-bound and a third block's warps fill
 // issue slots (cfg4 49.5 -> 47.6 us); a grid of one wave keeps the two-block budget, whose code has the shorter
 // dependency chains.
-template <int D16, int BPS>
+// kHostZ: z is (pinned) host memory.
+template <int D16, int BPS, bool kHostZ>
 __global__ void __launch_bounds__(kGThreads, BPS) gsta_mma_kernel(GstaParams P) {
   constexpr int d = D16 * 16;
   constexpr int RS = 2 * d + 16;            // bytes per staged bf16 row (16 bytes of padding: conflict-free ldmatrix)
@@ -359,24 +360,36 @@ __global__ void __launch_bounds__(kGThreads, BPS) gsta_mma_kernel(GstaParams P) 
   }
   cp_wait<0>();
 
-  // (16 bytes at a time: z may be host memory)
-  for (int i = tid; i < kGT * (d / 8); i += kGThreads) {
-    const int r = i / (d / 8), c8 = (i - r * (d / 8)) * 8;
+  if constexpr (kHostZ) {                // 16 bytes at a time over the bus
+    for (int i = tid; i < kGT * (d / 8); i += kGThreads) {
+      const int r = i / (d / 8), c8 = (i - r * (d / 8)) * 8;
+      if (c_base + r < c_end) {
+        const float4 v = *reinterpret_cast<const float4*>(Ts + r * TS + c8), w = *reinterpret_cast<const float4*>(Ts + r * TS + c8 + 4);
+        *reinterpret_cast<uint4*>(P.z + (size_t)(c_base + r) * d + c8) = make_uint4(pack2(v.x, v.y), pack2(v.z, v.w), pack2(w.x, w.y), pack2(w.z, w.w));
+      }
+    }
+    return;
+  }
+  // all threads, 4 bytes each (16 at a time keep half of them idle and end a block later: 30,912 candidates, d = 64 94.3 against 92.9 us)
+  for (int i = tid; i < kGT * (d / 2); i += kGThreads) {
+    const int r = i / (d / 2), q = i - r * (d / 2);
     if (c_base + r < c_end) {
-      const float4 v = *reinterpret_cast<const float4*>(Ts + r * TS + c8), w = *reinterpret_cast<const float4*>(Ts + r * TS + c8 + 4);
-      *reinterpret_cast<uint4*>(P.z + (size_t)(c_base + r) * d + c8) = make_uint4(pack2(v.x, v.y), pack2(v.z, v.w), pack2(w.x, w.y), pack2(w.z, w.w));
+      const float2 v = *reinterpret_cast<const float2*>(Ts + r * TS + 2 * q);
+      *reinterpret_cast<uint32_t*>(P.z + (size_t)(c_base + r) * d + 2 * q) = pack2(v.x, v.y);
     }
   }
 }
 
 template <int D16>
-int launch_gsta(const GstaParams& P, cudaStream_t st) {
+int launch_gsta(const GstaParams& P, bool host_z, cudaStream_t st) {
   constexpr int d = D16 * 16, RS = 2 * d + 16, TS = d + 8;
   const size_t smem = (size_t)kGT * TS * 4 + (size_t)kGT * RS + (size_t)kGT * (P.H * RS + (P.H % 2 ? 0 : 16)) + RS + kGT * sizeof(int) +
                       (size_t)kGW * 2 * kChunk * RS;
   const int sms = device_sms();
   const int blocks = (P.N + P.cpb - 1) / P.cpb;
-  auto kernel = (D16 <= 4 && blocks > 2 * sms) ? gsta_mma_kernel<D16, (D16 <= 4 ? 3 : 2)> : gsta_mma_kernel<D16, 2>;
+  constexpr int kThree = D16 <= 4 ? 3 : 2;
+  auto kernel = blocks > 2 * sms ? (host_z ? gsta_mma_kernel<D16, kThree, true> : gsta_mma_kernel<D16, kThree, false>)
+                                 : (host_z ? gsta_mma_kernel<D16, 2, true> : gsta_mma_kernel<D16, 2, false>);
   LASER_CUDA_OK(allow_smem(kernel, smem));
   LaunchScope ls("gsta_mma", st);
   LASER_CUDA_OK(launch_chained(kernel, dim3(blocks), dim3(kGThreads), smem, st, P));
@@ -405,13 +418,15 @@ int gsta_candidates_per_block(const Plan& p) {
   return (p.N + 7) / 8 <= 2 * sms ? 8 : kGT;
 }
 
+constexpr int kFewBlocks = 32;
+
 // Blocks that could have an SM each, placed while the attention kernel runs, pile up on the few SMs that have no unit of it: one request
 // of 512 candidates (64 blocks) 26.6 -> 25.6 us with the blocks placed when it ends, 432 candidates (54) 31.0 -> 28.5.  A handful of blocks
 // does not crowd and gains from an early set-up (96 candidates, 12 blocks 21.8 against 22.6), and from about an SM's worth of blocks each
 // on there is nothing to spread (4400 candidates 62.9 against 64.5).
 bool gsta_prefers_idle_gpu(const Plan& p) {
   const int cpb = gsta_candidates_per_block(p), blocks = (p.N + cpb - 1) / cpb;
-  return p.M > 0 && blocks >= 32 && blocks <= device_sms();
+  return p.M > 0 && blocks >= kFewBlocks && blocks <= device_sms();
 }
 
 // Sorting the blocks pays only when the grid runs in more than one wave.
@@ -444,8 +459,9 @@ int gsta_mma(const Plan& p, const void* Hprime, const int32_t* lengths, const in
   P.early_setup = images_ready ? 1 : 0;
   // A grid of one wave ends at once, and the next call's first blocks in its way cost more than their early start gains (4096
   // candidates, one per user, 138.6 -> 136.0 us per call); several waves leave SMs idle at the end that they can use (16384 candidates,
-  // d = 128 152 against 158).
-  P.release_early = (p.N + P.cpb - 1) / P.cpb > 2 * device_sms() ? 1 : 0;
+  // d = 128 152 against 158), and a few blocks are in nobody's way (119 candidates 30.1 against 30.5).
+  const int blocks = (p.N + P.cpb - 1) / P.cpb;
+  P.release_early = blocks < kFewBlocks || blocks > 2 * device_sms() ? 1 : 0;
   if (p.M > 0 && !images_ready) {
     const int total = p.M * 3 * (p.d / 16) * (p.d / 16) * 32;
     LaunchScope ls("gsta_prep", st);
@@ -453,14 +469,14 @@ int gsta_mma(const Plan& p, const void* Hprime, const int32_t* lengths, const in
   }
   int rc;
   switch (p.d / 16) {
-    case 1: rc = launch_gsta<1>(P, st); break;
-    case 2: rc = launch_gsta<2>(P, st); break;
-    case 3: rc = launch_gsta<3>(P, st); break;
-    case 4: rc = launch_gsta<4>(P, st); break;
-    case 5: rc = launch_gsta<5>(P, st); break;
-    case 6: rc = launch_gsta<6>(P, st); break;
-    case 7: rc = launch_gsta<7>(P, st); break;
-    case 8: rc = launch_gsta<8>(P, st); break;
+    case 1: rc = launch_gsta<1>(P, p.z_on_host, st); break;
+    case 2: rc = launch_gsta<2>(P, p.z_on_host, st); break;
+    case 3: rc = launch_gsta<3>(P, p.z_on_host, st); break;
+    case 4: rc = launch_gsta<4>(P, p.z_on_host, st); break;
+    case 5: rc = launch_gsta<5>(P, p.z_on_host, st); break;
+    case 6: rc = launch_gsta<6>(P, p.z_on_host, st); break;
+    case 7: rc = launch_gsta<7>(P, p.z_on_host, st); break;
+    case 8: rc = launch_gsta<8>(P, p.z_on_host, st); break;
     default: return LASER_ERR_UNSUPPORTED;
   }
   if (rc != LASER_OK) return rc;
