@@ -61,7 +61,6 @@ struct TcParams {
   bf16 *imgK, *imgQ, *imgV;           // W_k^T, W_q^T [dqk x d], W_v^T [128 x d] in canonical K-major layout
   int* status;
   bf16* Hp;
-  int release_early;                  // the attention kernel lets its successor start while it runs
 };
 
 // Sanitised view of one user: invalid lengths / offsets behave like an empty user (and are reported by tc_prep_kernel).
@@ -656,7 +655,8 @@ constexpr uint32_t kColO = kColP + kGateGroups * (kItMax / 2);   // outputs [n_o
 // (any shift cancels in the quotient; this one keeps the sum >= 1) and capped at 2^60 above that shift.
 constexpr int kSumSlots = 4;
 constexpr float kExpCap = 60.f;
-template <bool kSoftmax>
+// kRelease: the next kernel may start while this one runs (a flag in its place made the kernel 0.3 .. 1 us slower, taken or not).
+template <bool kSoftmax, bool kRelease>
 __global__ void __launch_bounds__(kStaThreads, 1) tc_sta_kernel(TcParams P) {
   extern __shared__ __align__(128) uint8_t smem_raw[];
   __shared__ StaBars bars;
@@ -707,7 +707,7 @@ __global__ void __launch_bounds__(kStaThreads, 1) tc_sta_kernel(TcParams P) {
   const int n_obuf = P.n_obuf;
   const bool two_epilogues = n_groups <= 2 && n_obuf == 2;    // gate warpgroup 2 has no head: it drains accumulator 1
   chain_wait();                         // K, V^T and Q tiles are complete
-  if (P.release_early) chain_release();
+  if constexpr (kRelease) chain_release();
 
   // this block's contiguous range of units
   const int n_units = P.counters[0];
@@ -1208,7 +1208,6 @@ int tensor_sta(const Plan& p, const void* items, const int32_t* lengths, const v
   P.gimg = reinterpret_cast<uint4*>(ws + p.off_gimg);
   P.gnseg = reinterpret_cast<int*>(ws + p.off_gimg + gsta_nseg_offset(p));
   P.M = p.M;
-  P.release_early = !(P.Wg && !p.side && gsta_prefers_idle_gpu(p));
   P.gorder = nullptr;
   if (P.Wg && gsta_wants_order(p)) {
     P.gorder = reinterpret_cast<int*>(ws + p.off_gimg + gsta_order_offset(p));
@@ -1239,7 +1238,8 @@ int tensor_sta(const Plan& p, const void* items, const int32_t* lengths, const v
   {
     const size_t smem = sta_smem_bytes(p, P.IT, softmax);
     if (smem > 220 * 1024) return LASER_ERR_UNSUPPORTED;
-    auto kernel = softmax ? tc_sta_kernel<true> : tc_sta_kernel<false>;
+    const bool hold = P.Wg && !p.side && gsta_prefers_idle_gpu(p);
+    auto kernel = softmax ? tc_sta_kernel<true, true> : hold ? tc_sta_kernel<false, false> : tc_sta_kernel<false, true>;
     LASER_CUDA_OK(allow_smem(kernel, smem));
     LaunchScope ls(softmax ? "sta_tc_softmax" : "sta_tc", st);
     LASER_CUDA_OK(launch_chained(kernel, dim3(P.sta_grid), dim3(kStaThreads), smem, st, P));
